@@ -2,12 +2,13 @@
 import os
 import subprocess
 import sys
+import tempfile
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbifrost.so")
-SOURCES = ["api.cu", "ntt.cu", "kernels.cu", "encode.cu"]
-HEADERS = ["bf_common.cuh", "bf_host.h", os.path.join("..", "..", "include", "bifrost.h")]
+SOURCES = ["api.cu", "ntt.cu", "kernels.cu", "mac.cu", "mac_wide.cu", "encode.cu"]
+HEADERS = ["bf_common.cuh", "bf_host.h", "mac_kernel.cuh", os.path.join("..", "..", "include", "bifrost.h")]
 
 
 def _stale() -> bool:
@@ -22,13 +23,17 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
-           "-Xcompiler", "-fPIC,-O2,-fno-fast-math", "-shared", "-o", LIB]
+    flags = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
+             "-Xcompiler", "-fPIC,-O2,-fno-fast-math"]
     if verbose:
-        cmd += ["-Xptxas", "-v"]
-    cmd += [os.path.join(CSRC, f) for f in SOURCES]
-    cmd += ["-lcudart"]
-    subprocess.run(cmd, check=True)
+        flags += ["-Xptxas", "-v"]
+    with tempfile.TemporaryDirectory() as tmp:        # one compilation per source, side by side
+        objs = [os.path.join(tmp, f + ".o") for f in SOURCES]
+        jobs = [subprocess.Popen([nvcc, *flags, "-c", os.path.join(CSRC, f), "-o", o]) for f, o in zip(SOURCES, objs)]
+        failed = [f for f, j in zip(SOURCES, jobs) if j.wait() != 0]
+        if failed:
+            raise RuntimeError("nvcc failed on " + ", ".join(failed))
+        subprocess.run([nvcc, *flags, "-shared", "-o", LIB, *objs, "-lcudart"], check=True)
     return LIB
 
 

@@ -111,6 +111,7 @@ struct bf_ctx {
     std::map<u32, int> key_of_steps;
     u64* keys = nullptr;
     u32* perms = nullptr;            // [n_keys][N] pinv: where position n goes under the key's automorphism
+    std::vector<u32> gal, gal_inv;   // Galois element of each key's rotation, 5^steps mod 2N, and its inverse
     u32* perms_fwd = nullptr;        // [n_keys][N] perm: rotated[n] = unrotated[perm[n]] (per-output division by P)
     u32 n_keys = 0;
     // scratch (grow-only)
@@ -299,23 +300,27 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
         R.qinv_d[m] = 1.0 / (double)q;
         R.ninv_d[m] = (double)R.ninv[m];
         R.ninv_q[m] = (double)R.ninv[m] / (double)q;
-        R.ninvm_d[m] = (double)R.ninv_m[m];
-        R.ninvm_q[m] = (double)R.ninv_m[m] / (double)q;
+        R.dp[m] = q < (1ull << 40) ? 1u : 0u;
+        R.c40_d[m] = (double)((1ull << 40) % q);
+        R.c40_q[m] = R.c40_d[m] / (double)q;
+        R.ninvm_d[m] = (double)(R.dp[m] ? R.ninv[m] : R.ninv_m[m]);      // (plaintexts of these primes carry no factor)
+        R.ninvm_q[m] = R.ninvm_d[m] / (double)q;
         R.c30_d[m] = (double)((1ull << 30) % q);
         R.c30_q[m] = R.c30_d[m] / (double)q;
         R.k59_d[m] = (double)(2 * q - (1ull << 59) % q);
         R.pinv_d[m] = m < n_ct_primes ? (double)R.pinv[m] : 0.0;
         R.pinv_q[m] = m < n_ct_primes ? (double)R.pinv[m] / (double)q : 0.0;
         {   // constants of the encoder's fp64 load (see RingDev::enc_consts)
-            const u64 c96 = h_mulmod(R.c64[m], (1ull << 32) % q, q);
-            const u64 c127 = h_mulmod(R.c64[m], (1ull << 63) % q, q);
+            const u64 f = R.dp[m] ? 1 % q : R.c64[m];                    // the factor plaintexts are kept with
+            const u64 c96 = h_mulmod(f, (1ull << 32) % q, q);
+            const u64 c127 = h_mulmod(f, (1ull << 63) % q, q);
             const u64 neg = c127 ? q - c127 : 0;                         // -2^127 mod q in [0, q)
             double k = neg > q / 2 ? -(double)(q - neg) : (double)neg;    // centred
             if (q >> 41) k += 2.0 * (double)q;
             double* ec = &enc_consts[(size_t)m * ENC_CONSTS];
             ec[0] = (double)c96;
             ec[1] = ec[0] / (double)q;
-            ec[2] = (double)R.c64[m];
+            ec[2] = (double)f;
             ec[3] = ec[2] / (double)q;
             ec[4] = k;
         }
@@ -478,6 +483,7 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
     // the inner product run in the un-rotated index space; the rotation is applied at the very end
     // as the scatter out[pinv[i]] = v'[i], pinv = perm^{-1}.  Only pinv stays on the device.
     std::vector<u32> perms((size_t)n_keys * N), pinvs((size_t)n_keys * N);
+    std::vector<u32> gal(n_keys), gal_inv(n_keys);
     std::map<u32, int> key_of_steps;
     for (u32 t = 0; t < n_keys; ++t) {
         const u32 steps = rot_steps[t] % n;
@@ -490,6 +496,10 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
             pinvs[(size_t)t * N + pi] = i;
         }
         key_of_steps[steps] = (int)t;
+        u64 gi = 1;
+        for (u32 s = steps; s < n; ++s) gi = (gi * 5) % (2ull * N);      // 5 has order n
+        gal[t] = (u32)g;
+        gal_inv[t] = (u32)gi;
     }
     u32* perm_dev = nullptr;
     if (cudaMalloc(&perm_dev, perms.size() * sizeof(u32)) != cudaSuccess) return fail(BF_ERR_OOM);
@@ -524,6 +534,8 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
     }
     ctx->perms_fwd = perm_dev;
     ctx->key_of_steps.swap(key_of_steps);
+    ctx->gal.swap(gal);
+    ctx->gal_inv.swap(gal_inv);
     ctx->n_keys = n_keys;
     ctx->epoch++;
     return BF_OK;
@@ -946,13 +958,22 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     if (giant_per_lane > gb / (u32)lanes) giant_per_lane = gb / (u32)lanes;
     if (giant_per_lane < 1) giant_per_lane = 1;
     const u32 rot_per_lane = baby_per_lane > giant_per_lane ? baby_per_lane : giant_per_lane;
-    u32 n_dig_sets = giant_per_lane * (u32)lanes;       // digit sets alive at once
-    if (n_dig_sets < in_batch) n_dig_sets = in_batch;
     // double hoisting: the rotated inputs and the inner sums live in the extended basis {q_i, P}
     const bool dh = (ctx->plan.flags & BF_PLAN_DOUBLE_HOIST) != 0;
     const u32 nmp = mac_primes(ctx);                      // primes of X, of the plaintexts and of the inner sums
+    const u32 n_terms = n_in * b, n_pj = n_out * g;
+    // weights that are not resident in the transform domain are made in rounds of as many output groups as the scratch holds
+    const bool resident = pt_weights && pt_weights->pt;
+    const size_t groups_fit = ctx->encode_scratch_bytes / ((size_t)n_terms * nmp * N * 8);
+    const u32 groups = groups_fit < 1 ? 1u : groups_fit > (size_t)n_pj ? n_pj : (u32)groups_fit;
+    // the multiply-accumulate makes the rotated inputs itself, unless it runs in several rounds: each would stream the
+    // keys again, so that X is worth keeping in memory then
+    const bool rotate_in_mac = dh && (resident || groups == n_pj);
+    if (rotate_in_mac) in_batch = n_in;
+    u32 n_dig_sets = giant_per_lane * (u32)lanes;       // digit sets alive at once
+    if (n_dig_sets < in_batch) n_dig_sets = in_batch;
     const size_t xw = (size_t)2 * nmp * N;                // words per term of X / per inner sum
-    TRY(ensure(ctx, ctx->X, (size_t)n_in * b * xw * 8));
+    TRY(ensure(ctx, ctx->X, (size_t)n_in * (rotate_in_mac ? 1u : b) * xw * 8));
     if (dh) {
         TRY(ensure(ctx, ctx->X0, (size_t)n_in * ctw * 8));
         TRY(ensure(ctx, ctx->Aext, (size_t)n_out * g * xw * 8));
@@ -1004,7 +1025,8 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     PolyBatch B;
     memset(&B, 0, sizeof(B));
     // X[q][0] = NTT(ct_q): polynomial (q, component*r + prime).  Double hoisting keeps it apart (X0: the hoisted ModUp
-    // copies its c1 part) and puts P * NTT(ct_q), zero modulo P, into X
+    // copies its c1 part) and puts P * NTT(ct_q), zero modulo P, into X (term q*b, or term q where the
+    // multiply-accumulate makes the rotated ones itself)
     u64* X0 = dh ? (u64*)ctx->X0.p : X;
     const long long x0_stride = dh ? (long long)ctw : (long long)b * ctw;
     B.src = ct_in;
@@ -1016,9 +1038,9 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     B.mod_wrap = r;
     B.mod0 = 0;
     B.mod_step = 1;
-    if (dh) {                   // the transform's last store also writes P * NTT(ct_q) as term q*b of X
+    if (dh) {                   // the transform's last store also writes P * NTT(ct_q) into X
         B.lift_ptr = X;
-        B.lift_so = (long long)b * (long long)xw;
+        B.lift_so = (long long)(rotate_in_mac ? 1u : b) * (long long)xw;
     }
     CK(ntt_forward(ctx->ring, B, n_in, LOAD_PLAIN, ctx->stream));
     if (b > 1) {
@@ -1026,6 +1048,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
             const u32 qn = (n_in - q0 < in_batch) ? n_in - q0 : in_batch;
             TRY(modup(ctx, ctx->stream, ct_in + (size_t)q0 * ctw + (size_t)r * N, (long long)ctw, qn, Dig,
                       X0 + (size_t)q0 * x0_stride + (size_t)r * N, x0_stride));
+            if (rotate_in_mac) continue;
             // the rotations of the batch, key-major (rotation t = (k - 1) * qn + q: those that share a key follow one
             // another, so that an inner-product block loads the key once for all of them), dealt out to the lanes
             // in contiguous runs
@@ -1059,32 +1082,33 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     stamp(ctx, 1);
 
     // ---- multiply-accumulate over the encoded diagonals (double hoisting: over the extended basis, into Aext)
-    const u32 n_terms = n_in * b, n_pj = n_out * g;
     u64* mac_out = dh ? (u64*)ctx->Aext.p : A;
     MacScatter msc;
     memset(&msc, 0, sizeof(msc));
     if (assemble) {         // component 0 of the inner sums with j >= 1 is stored rotated (only the output assembly reads it)
-        msc.pinv = ctx->perms;
+        msc.on = 1;
         msc.n_out = n_out;
-        for (u32 j = 1; j < g; ++j) msc.key[j] = giant_key[j];
+        for (u32 j = 1; j < g; ++j) msc.gal_inv[j] = ctx->gal_inv[giant_key[j]];
     }
-    if (pt_weights && pt_weights->pt) {
-        // double hoisting: the launch for the special prime (one eighth of the words, on whole-word arithmetic) runs
-        // beside the launch for the ciphertext primes
-        // (also while single launches are being timed, chains serialised: the pair is then timed as one span, the way
-        // it runs)
-        const bool beside = dh && (lanes > 1 || ctx->prof.timing);
-        ProfSpan span(beside ? &ctx->prof : nullptr, CAT_MAC, ctx->stream);
-        if (beside) TRY(fork_lanes(ctx, 2));
-        CK(launch_mac(ctx->ring, pt_weights->pt, pt_weights->lay, X, mac_out, n_pj, n_terms, true, ctx->device_error, ctx->stream,
-                      beside ? ctx->side[0] : nullptr, &msc));
-        if (beside) TRY(join_lanes(ctx, 2));
+    BabySteps baby;
+    memset(&baby, 0, sizeof(baby));
+    if (rotate_in_mac) {
+        baby.n_in = n_in;
+        baby.b = b;
+        baby.keys = ctx->keys;
+        baby.dig = Dig;
+        for (u32 k = 1; k < b; ++k) {
+            baby.key[k] = (u32)baby_key[k];
+            baby.gal[k] = ctx->gal[baby_key[k]];
+            baby.gal_inv[k] = ctx->gal_inv[baby_key[k]];
+        }
+    }
+    const BabySteps* bsp = rotate_in_mac ? &baby : nullptr;
+    if (resident) {
+        CK(launch_mac(ctx->ring, pt_weights->pt, pt_weights->lay, X, mac_out, n_pj, n_terms, ctx->stream, msc, bsp));
     } else {
         // fallback: encode groups of (j, p) just in time into a scratch ring, then consume them (weights kept as
         // coefficients: the same without the encoder, only their transforms)
-        const size_t group_bytes = (size_t)n_terms * nmp * N * 8;
-        const size_t fit = ctx->encode_scratch_bytes / group_bytes;
-        const u32 groups = fit < 1 ? 1u : fit > (size_t)n_pj ? n_pj : (u32)fit;
         const TileLayout jl = mac_tile_layout(ctx->ring, groups, n_terms, nmp);
         TRY(ensure(ctx, ctx->ptjit, mac_tile_bytes(ctx->ring, jl)));
         for (u32 pj0 = 0; pj0 < n_pj; pj0 += groups) {
@@ -1092,8 +1116,8 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
             const TileLayout cl = mac_tile_layout(ctx->ring, cnt, n_terms, nmp);
             TRY(encode_range(ctx, W_raw, d_out, d_in, pj0 * n_terms, cnt * n_terms, (u64*)ctx->ptjit.p, cl, pj0, pt_weights));
             msc.pj0 = pj0;
-            CK(launch_mac(ctx->ring, (const u64*)ctx->ptjit.p, cl, X, mac_out + (size_t)pj0 * xw, cnt, n_terms, false,
-                          ctx->device_error, ctx->stream, nullptr, &msc));
+            CK(launch_mac(ctx->ring, (const u64*)ctx->ptjit.p, cl, X, mac_out + (size_t)pj0 * xw, cnt, n_terms, ctx->stream, msc,
+                          bsp));
         }
     }
     if (dh && !assemble) {

@@ -39,11 +39,15 @@ struct RingDev {
     double c30_d[MAX_MODULI], c30_q[MAX_MODULI];       // (double)(2^30 mod q) and that over q
     double k59_d[MAX_MODULI];    // 2q - (2^59 mod q): undoes the offset of a stored centred lift, keeps it positive
     double pinv_d[MAX_MODULI], pinv_q[MAX_MODULI];     // (double)(P^{-1} mod q_i) and that over q_i (i < r)
+    u32 dp[MAX_MODULI];          // modulus below 2^40: operands of the inner products (cached plaintexts, rotation keys, digits)
+                                 //   are kept as the bits of doubles and multiplied in fp64 (see DpAcc)
+    double c40_d[MAX_MODULI], c40_q[MAX_MODULI];       // (double)(2^40 mod q) and that over q
     // encoder output (signed 64-bit coefficients) into Montgomery form on the fp64 path: the word is
     // (hi' - 2^31) 2^32 + lo, so times 2^64 it is  hi' (2^96 mod q) + lo (2^64 mod q) - (2^127 mod q).
     // Five doubles per prime, in device memory (kernel parameters stay small): (double)(2^96 mod q), that
     // over q, (double)(2^64 mod q), that over q, and the centred residue of -2^127 (plus 2q for primes of
-    // 2^41 or more, whose values stay non-negative)
+    // 2^41 or more, whose values stay non-negative).  Primes with dp set keep plaintexts without the factor 2^64:
+    // 2^32, 1 and -2^63 instead
     const double* enc_consts;    // [r+1][ENC_CONSTS]
     const ulonglong2* tw_fwd;    // [r+1][N]  (psi^brev(k), companion), merged Cooley-Tukey order
     const ulonglong2* tw_inv;    // [r+1][N]  inverses of the above, for the Gentleman-Sande inverse
@@ -138,73 +142,6 @@ __device__ __forceinline__ void mac128(u64& hi, u64& lo, u64 a, u64 b) {
     hi += ph + (lo < pl ? 1ull : 0ull);
 }
 
-// Lazy sum of products of 64-bit words, kept as partial sums of 32-bit limb products so that one
-// term costs four 32x32->64 multiplies and no 64-bit high-product sequence:
-//   sum a*b = lo + mid * 2^32 + hi * 2^64,   lo = sum a0*b0,  mid = sum (a0*b1 + a1*b0),  hi = sum a1*b1.
-// lo and mid carry their overflow into 32-bit counters.  With words below 2^60 and at most 2^8 terms
-// hi stays below 2^64 and the total below 2^128.  SMALL drops the carry counter of mid: valid while
-// terms * 2 * 2^(bits-32) * 2^32 < 2^64, e.g. words below 2^50 and up to 2^13 terms.
-template <bool SMALL>
-struct LimbAcc {
-    u64 lo = 0, mid = 0, hi = 0;
-    u32 lo_c = 0, mid_c = 0;
-
-    __device__ __forceinline__ void mac(u64 a, u64 b) {
-        const u32 a0 = (u32)a, a1 = (u32)(a >> 32), b0 = (u32)b, b1 = (u32)(b >> 32);
-        if (SMALL) {
-            asm("{\n\t.reg .u64 p;\n\t"
-                "mul.wide.u32 p, %4, %6;\n\t"
-                "add.cc.u64 %0, %0, p;\n\t"
-                "addc.u32 %1, %1, 0;\n\t"
-                "mad.wide.u32 %2, %4, %7, %2;\n\t"
-                "mad.wide.u32 %2, %5, %6, %2;\n\t"
-                "mad.wide.u32 %3, %5, %7, %3;\n\t}"
-                : "+l"(lo), "+r"(lo_c), "+l"(mid), "+l"(hi)
-                : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
-        } else {
-            asm("{\n\t.reg .u64 p;\n\t"
-                "mul.wide.u32 p, %5, %7;\n\t"
-                "add.cc.u64 %0, %0, p;\n\t"
-                "addc.u32 %1, %1, 0;\n\t"
-                "mul.wide.u32 p, %5, %8;\n\t"
-                "add.cc.u64 %2, %2, p;\n\t"
-                "addc.u32 %3, %3, 0;\n\t"
-                "mul.wide.u32 p, %6, %7;\n\t"
-                "add.cc.u64 %2, %2, p;\n\t"
-                "addc.u32 %3, %3, 0;\n\t"
-                "mad.wide.u32 %4, %6, %8, %4;\n\t}"
-                : "+l"(lo), "+r"(lo_c), "+l"(mid), "+r"(mid_c), "+l"(hi)
-                : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
-        }
-    }
-
-    // the accumulated integer modulo q, in [0, q)
-    __device__ __forceinline__ u64 reduce(u64 q, u64 mu, u64 c64, u64 c64s) const {
-        const u64 L = lo + (mid << 32);
-        const u64 carry = L < lo ? 1ull : 0ull;
-        const u64 H = (u64)lo_c + (mid >> 32) + ((u64)mid_c << 32) + hi + carry;
-        return reduce128(H, L, q, mu, c64, c64s);
-    }
-
-    // Montgomery reduction of the accumulated integer V: V * 2^{-64} mod q, in [0, q).
-    // Requires V < q * 2^64 (number of terms times q below 2^64).  qneg = -q^{-1} mod 2^64.
-    __device__ __forceinline__ u64 reduce_mont(u64 q, u64 qneg) const {
-        const u64 L = lo + (mid << 32);
-        const u64 carry = L < lo ? 1ull : 0ull;
-        const u64 H = (u64)lo_c + (mid >> 32) + ((u64)mid_c << 32) + hi + carry;
-        const u64 m = L * qneg;
-        u64 t = H + __umul64hi(m, q) + (L != 0 ? 1ull : 0ull);   // L + lo(m*q) = 0 mod 2^64, carrying iff L != 0
-        return t >= q ? t - q : t;
-    }
-
-    // The same by two 32-bit rounds (redc_2x32 below): no 64-bit high product.
-    __device__ __forceinline__ u64 reduce_mont32(u64 q, u32 qneg32) const;
-
-    __device__ __forceinline__ void reset_to(u64 v) {
-        lo = v; mid = 0; hi = 0; lo_c = 0; mid_c = 0;
-    }
-};
-
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) {
     u64 v = a + b;
     return v >= q ? v - q : v;
@@ -276,12 +213,20 @@ struct ModDownEpilogue {
 };
 
 // Double hoisting with one division per output: component 0 of inner sum (j, p), j >= 1, is only ever used rotated
-// by giant step j, so the multiply-accumulate stores it through that rotation's permutation (group pj0 + pj has
-// j = (pj0 + pj) / n_out; pinv = null: plain stores).
+// by giant step j, so the multiply-accumulate stores it through that rotation (group pj0 + pj has j = (pj0 + pj) / n_out;
+// on = 0: plain stores).
 struct MacScatter {
-    const u32* pinv;              // [n_keys][N]
-    u32 n_out, pj0;
-    int key[MAX_ROT_BATCH + 1];   // key (permutation table) of giant step j
+    u32 on, n_out, pj0;
+    u32 gal_inv[MAX_ROT_BATCH + 1];     // inverse Galois element of giant step j
+};
+
+// Baby rotations computed inside the multiply-accumulate (double hoisting): input q's term k is its rotation by key[k].
+struct BabySteps {
+    u32 n_in, b;
+    u32 parts, per_part;                // how the inputs are dealt out to a block's lanes (set by the launcher)
+    const u64 *keys, *dig;              // resident keys; digit set q of input q (tile-major, see ks_tile_index)
+    u32 key[MAX_ROT_BATCH + 1];
+    u32 gal[MAX_ROT_BATCH + 1], gal_inv[MAX_ROT_BATCH + 1];
 };
 
 // Constants of a rescale from `level` primes: q_L^{-1} mod q_i with its Shoup companion, and q_L mod q_i (i < level - 1).
@@ -365,13 +310,10 @@ struct PolyBatch {
     u32 skip_diag;                // forward only: polynomial (o, m) with m < r and o % r == m (a digit in its own prime)
     const u64* diag_src;          //   is not transformed but copied from diag_src + (o / r)*diag_so + m*N, where its
     long long diag_so;            //   transform already exists
-    const u32* scatter;           // forward only: final store goes to scatter_dst[scatter[(o / scatter_div) * N + n]]
-    u32 scatter_div;              //   instead of dst[n] (same polynomial strides as dst)
-    u64* scatter_dst;
-    u32 scatter_mont;             //   and the stored value is the result times 2^64 mod q (rotation keys: the inner
-                                  //   product ends in a Montgomery reduction)
-    u32 split_bits;               // L > 0: the NTT-domain side of the transform is stored as two L-bit-aligned
-                                  // limbs per word, (v >> L) << 32 | (v & (2^L - 1)); forward writes, inverse reads it
+    const u32* scatter;           // forward only (rotation keys): coefficient n of the result goes to position
+    u32 scatter_div;              //   scatter[(o / scatter_div) * N + n] of dtile_ptr
+    u32 split_bits;               // tile-major side: 8-byte words modulo primes without RingDev::dp are stored as two limbs,
+                                  //   (v >> L) << 32 | (v & (2^L - 1)), L = split_bits below 2^50, else 30
     u64* lift_ptr;                // forward only, non-null (double hoisting): polynomial (o, m = comp * mod_wrap + i) is also
     long long lift_so;            //   stored times P mod q_i at lift_ptr + o*lift_so + (comp*(r+1) + i)*N, and zeros as the
                                   //   residue modulo P: the un-rotated input lifted to the extended basis
@@ -410,32 +352,6 @@ __device__ __forceinline__ size_t ks_tile_base(u32 N, u32 n_m, u32 div, u32 o_hi
 __device__ __forceinline__ u64 limb_split(u64 v, u32 L) { return ((v >> L) << 32) | (v & ((1ull << L) - 1)); }
 __device__ __forceinline__ u64 limb_join(u64 s, u32 L) { return ((s >> 32) << L) | (s & 0xffffffffull); }
 
-// Karatsuba accumulator for products of words given as two L-bit limbs (low limb in the low 32-bit
-// half, high limb in the high half), L <= 25:  three 32x32->64 multiply-adds per product and no
-// carries.  sum v*x = lo + (mid - lo - hi) * 2^L + hi * 2^(2L), with lo = sum v0*x0, hi = sum v1*x1,
-// mid = sum (v0+v1)*(x0+x1); every term of mid is below 2^(2L+2), so 2^(62-2L) terms fit.
-struct KaraAcc {
-    u64 lo = 0, mid = 0, hi = 0;
-    __device__ __forceinline__ void mac(u32 v0, u32 v1, u32 vs, u64 xsplit) {
-        const u32 x0 = (u32)xsplit, x1 = (u32)(xsplit >> 32);
-        lo += (u64)v0 * x0;
-        hi += (u64)v1 * x1;
-        mid += (u64)vs * (x0 + x1);
-    }
-    // the accumulated integer V as (H, L64)
-    __device__ __forceinline__ void value(u32 L, u64& H, u64& L64) const {
-        const u64 m = mid - lo - hi;
-        u64 l = lo, h = 0;
-        const u64 a = m << L;
-        l += a; h += (l < a) ? 1ull : 0ull;
-        h += m >> (64 - L);
-        const u64 b = hi << (2 * L);
-        l += b; h += (l < b) ? 1ull : 0ull;
-        h += hi >> (64 - 2 * L);
-        H = h; L64 = l;
-    }
-};
-
 // Montgomery reduction by two 32-bit rounds: V * 2^{-64} mod q in [0, q), for V = (H, L) < q * 2^64.
 // qneg32 = -q^{-1} mod 2^32.  Six 32-bit multiplies instead of a 64x64 high product.
 __device__ __forceinline__ u64 redc_2x32(u64 H, u64 L, u64 q, u32 qneg32) {
@@ -464,12 +380,94 @@ __device__ __forceinline__ u64 redc_2x32(u64 H, u64 L, u64 q, u32 qneg32) {
     return t >= q ? t - q : t;
 }
 
-template <bool SMALL>
-__device__ __forceinline__ u64 LimbAcc<SMALL>::reduce_mont32(u64 q, u32 qneg32) const {
-    const u64 L = lo + (mid << 32);
-    const u64 carry = L < lo ? 1ull : 0ull;
-    const u64 H = (u64)lo_c + (mid >> 32) + ((u64)mid_c << 32) + hi + carry;
-    return redc_2x32(H, L, q, qneg32);
+// ---- Sums of products of residues, three ways.  B200 issues 64 fp64 multiply-adds per SM and clock, but only 32
+// 32x32+64-bit integer ones, so the primes below 2^40 (all but one or two of a chain) multiply in fp64.
+enum OperandClass : int { OP_DP = 0, OP_NARROW = 1, OP_WIDE = 2 };
+constexpr u32 LIMB_NARROW = 25, LIMB_WIDE = 30;
+
+// Primes below 2^40, operands integer-valued doubles.  The running sum h sits at 1.5 * 2^92, where doubles are 2^40 apart:
+// h' = fma(a, b, h) adds a*b rounded to a multiple of 2^40 (exactly representable), h - h' is exact, and
+// fma(a, b, h - h') is the part rounded away, an integer of magnitude at most 2^39; l collects those.  Exact while
+// |sum| < 2^91 and |l| < 2^53: 2048 terms.
+struct DpAcc {
+    double h = 7427640236712282150480740352.0;       // 1.5 * 2^92
+    double l = 0.0;
+    __device__ __forceinline__ void mac(double a, double b) {
+        const double h2 = __fma_rn(a, b, h);
+        l = __dadd_rn(l, __fma_rn(a, b, __dsub_rn(h, h2)));
+        h = h2;
+    }
+    // the sum modulo q in [0, q), as an integer-valued double: (h / 2^40) (2^40 mod q) + l, h / 2^40 below 2^51
+    __device__ __forceinline__ double reduce(double q, double qinv, double c40, double c40q) const {
+        const double hi = __dmul_rn(__dsub_rn(h, 7427640236712282150480740352.0), 9.094947017729282379150390625e-13);   // 2^-40
+        const double v = __dadd_rn(fp_mul_centred_signed(fp_centre(hi, q, qinv), c40, c40q, q), l);
+        const double r = fp_centre(v, q, qinv);
+        return r < 0.0 ? __dadd_rn(r, q) : r;
+    }
+};
+
+// 64-bit words cut into two limbs, 25 bits below 2^50 (NARROW), 30 bits up to 2^60 (WIDE).  NARROW: Karatsuba, three
+// multiply-adds per product and no carries; a middle product is below 2^52, so the sums take 2^10 terms.  WIDE: four;
+// products are below 2^60, so 15 terms fit, and the sum of up to 2^7 such sums fits 128 bits.
+template <bool WIDE>
+struct LimbAcc {
+    u64 lo = 0, m0 = 0, m1 = 0, hi = 0;
+    __device__ __forceinline__ void mac(u32 a0, u32 a1, u32 as, u32 b0, u32 b1) {      // (as = a0 + a1)
+        lo += (u64)a0 * b0;
+        hi += (u64)a1 * b1;
+        if (WIDE) {
+            m0 += (u64)a0 * b1;
+            m1 += (u64)a1 * b0;
+        } else {
+            m0 += (u64)as * (b0 + b1);
+        }
+    }
+    __device__ __forceinline__ unsigned __int128 value() const {
+        typedef unsigned __int128 u128;
+        return WIDE ? (u128)lo + ((u128)m0 << 30) + ((u128)m1 << 30) + ((u128)hi << 60)
+                    : (u128)lo + ((u128)(m0 - lo - hi) << 25) + ((u128)hi << 50);
+    }
+    // times 2^-64, in [0, q)
+    __device__ __forceinline__ u64 reduce(u64 q, u32 qneg32) const {
+        const unsigned __int128 v = value();
+        return redc_2x32((u64)(v >> 64), (u64)v, q, qneg32);
+    }
+};
+__device__ __forceinline__ void cut_limbs(u32 lo, u32 hi, u32 L, u32& w0, u32& w1) {
+    w0 = lo & ((1u << L) - 1u);
+    w1 = __funnelshift_r(lo, hi, L);
 }
+
+// One output pair of the key-switch inner product: digit j (d[j * ds]) times key words (2j, 2j + 1) (k[s * ks]) summed
+// over r digits, in [0, q).  The keys carry a factor 2^64 except where the class is OP_DP.
+template <int CLS>
+struct KeyDot {
+    LimbAcc<CLS == OP_WIDE> a0, a1;
+    __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1, u32 l0, u32 l1) {     // (key limbs already cut)
+        u32 d0, d1;
+        cut_limbs(d.x, d.y, CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW, d0, d1);
+        a0.mac(d0, d1, d0 + d1, k0, k1);
+        a1.mac(d0, d1, d0 + d1, l0, l1);
+    }
+    static __device__ __forceinline__ void cut(u32& k0, u32& k1) { cut_limbs(k0, k1, CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW, k0, k1); }
+    __device__ __forceinline__ void reduce(const RingDev& R, u32 m, u64& v0, u64& v1) const {
+        v0 = a0.reduce(R.q[m], (u32)R.qneg[m]);
+        v1 = a1.reduce(R.q[m], (u32)R.qneg[m]);
+    }
+};
+template <>
+struct KeyDot<OP_DP> {
+    DpAcc a0, a1;
+    __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1, u32 l0, u32 l1) {
+        const double dd = __hiloint2double((int)d.y, (int)d.x);
+        a0.mac(dd, __hiloint2double((int)k1, (int)k0));
+        a1.mac(dd, __hiloint2double((int)l1, (int)l0));
+    }
+    static __device__ __forceinline__ void cut(u32&, u32&) {}
+    __device__ __forceinline__ void reduce(const RingDev& R, u32 m, u64& v0, u64& v1) const {
+        v0 = d2u(a0.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));
+        v1 = d2u(a1.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));
+    }
+};
 
 }  // namespace bf

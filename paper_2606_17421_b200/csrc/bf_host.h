@@ -31,7 +31,6 @@ struct Profiler {
     struct Rec { int cat; cudaEvent_t a, b; };
     std::vector<Rec> recs;            // event pairs recorded since the last collection
     std::vector<cudaEvent_t> pool;    // idle events
-    bool span_open = false;           // a ProfSpan is timing the launches inside it as one
     cudaEvent_t get();
 };
 
@@ -40,14 +39,6 @@ struct ProfScope {
     Profiler* p; int cat; cudaStream_t s; cudaEvent_t a = nullptr;
     ProfScope(Profiler* prof, int c, cudaStream_t st);
     ~ProfScope();
-};
-
-// Times a group of launches that run side by side as one span on stream st (from everything before the group to
-// everything after its join); the launches inside are still counted by their own ProfScope, but not timed singly.
-struct ProfSpan {
-    Profiler* p; int cat; cudaStream_t s; cudaEvent_t a = nullptr;
-    ProfSpan(Profiler* prof, int c, cudaStream_t st);
-    ~ProfSpan();
 };
 
 struct RingHost {
@@ -110,17 +101,15 @@ cudaError_t launch_pointwise_mul(const RingHost& ring, const u64* a, const u64* 
 // xext[rb.c0[rot]][0][m][n] : 0), terms of [2][r+1][N] words (term rb.c0[rot] holds P times the un-rotated input).
 cudaError_t launch_key_inner_product(const RingHost& ring, const RotBatch& rb, const u64* dig, const u64* keys, u64* u,
                                      int* error_flag, cudaStream_t stream, u64* xext = nullptr, const u32* pinv = nullptr);
-u32 mac_split_bits(const RingHost& ring);   // limb width of the cached plaintext format (0 = whole words)
+u32 mac_split_bits(const RingHost& ring);   // limb width of cached 8-byte words modulo primes below 2^50
 // layout of n_pj groups of n_terms diagonals held in n_primes primes (0 = the r ciphertext primes)
 TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_primes = 0);
 size_t mac_tile_bytes(const RingHost& ring, const TileLayout& t);           // bytes that layout occupies
-// x: [n_terms][2][lay.n_primes][N], a: [n_pj][2][lay.n_primes][N]; every prime of the layout is processed (the special
-// prime, when present, by a launch of its own on whole words)
-// special_stream non-null: the launch for the special prime goes there (the caller has ordered that stream after
-// everything the launch reads and joins it afterwards), beside the launch for the ciphertext primes on `stream`
+// a: [n_pj][2][lay.n_primes][N]; every prime of the layout is processed.  baby null: x holds all terms,
+// [n_terms][2][lay.n_primes][N].  baby non-null: x holds the un-rotated inputs, [n_in][2][lay.n_primes][N], and the
+// rotated terms are computed inside.
 cudaError_t launch_mac(const RingHost& ring, const u64* pt, const TileLayout& lay, const u64* x, u64* a, u32 n_pj,
-                       u32 n_terms, bool weights_static, int* error_flag, cudaStream_t stream,
-                       cudaStream_t special_stream = nullptr, const MacScatter* scatter = nullptr);
+                       u32 n_terms, cudaStream_t stream, const MacScatter& sc, const BabySteps* baby = nullptr);
 cudaError_t launch_rescale(const RingHost& ring, const u64* in, u64* out, u32 n_ct, u32 level, const u64* inv,
                            const u64* invs, const u64* qlmod, cudaStream_t stream);
 

@@ -1,0 +1,343 @@
+// Multiply-accumulate over encoded diagonals (the ciphertext x plaintext product of Sec. 3.5 / 4.2),
+//   A[pj][comp][i][n] = sum_{t < n_terms} Pt[pj][t][i][n] * X[t][comp][i][n]   (mod q_i),
+// with the baby rotations that make X computed in the same kernel where the plan allows (BABY: double hoisting).
+//
+// A block owns one prime i and a tile of TN adjacent coefficients, for all output groups.  It first fills the X tile of
+// all terms and both components in shared memory, then streams its contiguous region of the cached weights once.
+//
+// BABY: rotated input (q, k) is (P c0 + u0, u1) moved through the automorphism of its rotation, u the key-switch inner
+// product of the digits of input q with key k.  In the transform's bit-reversed order an automorphism maps every
+// aligned power-of-two block of positions onto another aligned block: position n holds the evaluation at exponent
+// 2 brev(n) + 1, adjacent positions differ in the exponent's top bits only, and multiplying by an odd number keeps
+// equal low bits equal.  So the tile of X needs exactly one tile of every key and of every digit; the block reads those
+// in place, coalesced, and permutes inside the tile on the way to shared memory.  X itself (2 (r+1) N words per term) is
+// never written to memory.
+//
+// What bounds it: HBM (keys and weights are read once, 8 bytes a word).  Loads go straight to registers: a stream that
+// every thread consumes in the pattern it loads needs no staging, no barriers and no producer; what hides the latency is
+// the number of independent loads per thread (2r key words at a time; two batches of 8 weights) times resident warps.
+#pragma once
+#include "bf_host.h"
+
+namespace bf {
+
+constexpr int MAC_THREADS = 256;
+
+// position of the evaluation that an automorphism X -> X^gal moves to position n (and, with the inverse exponent, where
+// position n goes)
+__device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
+    const u32 e = 2u * (__brev(n) >> (32u - logN)) + 1u;
+    return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
+}
+
+// words that are read exactly once: not kept in L1, first to leave L2
+__device__ __forceinline__ u64 stream_policy() {
+    u64 pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ void ld_stream(const void* p, u64 policy, u32& lo, u32& hi) {
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;" : "=r"(lo), "=r"(hi) : "l"(p), "l"(policy));
+}
+__device__ __forceinline__ u32 ld_stream32(const void* p, u64 policy) {
+    u32 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
+    return v;
+}
+__device__ __forceinline__ u32 ld_stream8(const void* p, u64 policy) {
+    u32 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u8 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
+    return v;
+}
+
+// Accumulator of one output word of the multiply-accumulate and the form its operands have: weights as stored (two
+// 32-bit halves), the X word as it sits in shared memory.
+template <int CLS>
+struct MacAcc {                                          // OP_NARROW
+    static constexpr u32 L = LIMB_NARROW;
+    LimbAcc<false> a;
+    __device__ __forceinline__ void mac(u32 w0, u32 w1, u64 x) { a.mac(w0, w1, w0 + w1, (u32)x, (u32)(x >> 32)); }
+    __device__ __forceinline__ void end_chunk(const RingDev&, u32, u32) {}
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const { return a.reduce(R.q[i], (u32)R.qneg[i]); }
+    static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
+    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) { cut_limbs(lo, hi, L, lo, hi); }   // (compact formats)
+};
+template <>
+struct MacAcc<OP_WIDE> {
+    // a chunk of 8 terms keeps every sum below 2^64 (16 middle products below 2^60), then it is folded into 128 bits;
+    // 128 terms of 120 bits fit there, and the reduction at the end wants the high half below q
+    static constexpr u32 L = LIMB_WIDE;
+    LimbAcc<true> a;
+    unsigned __int128 v = 0;
+    __device__ __forceinline__ void mac(u32 w0, u32 w1, u64 x) {
+        const u32 x0 = (u32)x, x1 = (u32)(x >> 32);
+        a.lo += (u64)w0 * x0;
+        a.m0 += (u64)w0 * x1;
+        a.m0 += (u64)w1 * x0;
+        a.hi += (u64)w1 * x1;
+    }
+    __device__ __forceinline__ void end_chunk(const RingDev& R, u32 i, u32 chunk) {
+        v += a.value();
+        a = {};
+        if ((chunk & 15u) == 15u) v = ((unsigned __int128)barrett64((u64)(v >> 64), R.q[i], R.mu[i]) << 64) | (u64)v;
+    }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const {
+        return redc_2x32(barrett64((u64)(v >> 64), R.q[i], R.mu[i]), (u64)v, R.q[i], (u32)R.qneg[i]);
+    }
+    static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
+    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) { cut_limbs(lo, hi, L, lo, hi); }
+};
+template <>
+struct MacAcc<OP_DP> {
+    DpAcc a;
+    __device__ __forceinline__ void mac(u32 w0, u32 w1, u64 x) {
+        a.mac(__hiloint2double((int)w1, (int)w0), __longlong_as_double((long long)x));
+    }
+    __device__ __forceinline__ void end_chunk(const RingDev&, u32, u32) {}
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const {
+        return d2u(a.reduce(R.qd[i], R.qinv_d[i], R.c40_d[i], R.c40_q[i]));
+    }
+    static __device__ __forceinline__ u64 x_word(u64 v) { return (u64)__double_as_longlong(u2d(v)); }
+    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) {
+        const double d = __dsub_rn(__hiloint2double((int)(hi | 0x43300000u), (int)lo), 4503599627370496.0);
+        lo = (u32)__double2loint(d);
+        hi = (u32)__double2hiint(d);
+    }
+};
+
+template <int CLS, int LOG_TN, bool BABY, bool COMPACT, int RC>
+__device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict__ pt, const TileLayout& lay,
+                                         const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 pj_begin, u32 pj_end,
+                                         u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, u64* xs) {
+    constexpr u32 TN = 1u << LOG_TN, PL = MAC_THREADS >> LOG_TN;
+    typedef MacAcc<CLS> Acc;
+    const u32 N = R.N, logN = R.logN;
+    const u32 np = lay.n_primes;
+    const u32 tid = threadIdx.x, c = tid & (TN - 1), l = tid >> LOG_TN;
+    const u32 n0 = tile << LOG_TN;
+    const u64 q = R.q[i];
+    const u64 pol = stream_policy();
+    if constexpr (BABY) {
+        const u32 r = R.r;
+        const u32 b = bs.b, n_in = bs.n_in;
+        // term (q, 0): P times the un-rotated input
+        for (u32 e = l; e < n_in * 2; e += PL)
+            xs[(size_t)((e >> 1) * b * 2 + (e & 1)) * TN + c] = Acc::x_word(__ldg(x + ((size_t)e * np + i) * N + n0 + c));
+        // rotations: an item is a key and a part of the inputs that share it
+        const u32 n_items = (b - 1) * bs.parts;
+        for (u32 it = l; it < n_items; it += PL) {
+            const u32 k = 1 + it / bs.parts, part = it % bs.parts;
+            const u32 q_end = min(n_in, (part + 1) * bs.per_part);
+            const u32 src = (automorphism_index(n0, bs.gal[k], logN) & ~(TN - 1)) + c;
+            const u32 cd = automorphism_index(src, bs.gal_inv[k], logN) & (TN - 1);
+            const u64* kp = bs.keys + ks_tile_base(N, r + 1, 2 * r, bs.key[k], 0u, i) + (size_t)(src / KS_TILE) * 2 * r * KS_TILE + src % KS_TILE;
+            const u64* dp = bs.dig + ks_tile_base(N, r + 1, r, part * bs.per_part, 0u, i) + (size_t)(src / KS_TILE) * r * KS_TILE + src % KS_TILE;
+            const size_t dig_stride = ks_tile_base(N, r + 1, r, 1u, 0u, 0u);
+            u32 k0[RC > 0 ? 2 * RC : 1], k1[RC > 0 ? 2 * RC : 1];
+            if constexpr (RC > 0) {
+#pragma unroll
+                for (int s = 0; s < 2 * RC; ++s) ld_stream(kp + s * KS_TILE, pol, k0[s], k1[s]);
+#pragma unroll
+                for (int s = 0; s < 2 * RC; ++s) KeyDot<CLS>::cut(k0[s], k1[s]);
+            }
+            for (u32 qi = part * bs.per_part; qi < q_end; ++qi, dp += dig_stride) {
+                KeyDot<CLS> dot;
+                const u64 pc0 = __ldg(x + ((size_t)qi * 2 * np + i) * N + src);
+                if constexpr (RC > 0) {
+                    uint2 dw[RC];
+#pragma unroll
+                    for (int j = 0; j < RC; ++j) dw[j] = __ldg((const uint2*)(dp + j * KS_TILE));
+#pragma unroll
+                    for (int j = 0; j < RC; ++j) dot.mac(dw[j], k0[2 * j], k1[2 * j], k0[2 * j + 1], k1[2 * j + 1]);
+                } else {
+#pragma unroll 4
+                    for (u32 j = 0; j < r; ++j) {
+                        uint2 ka = __ldg((const uint2*)(kp + (2 * j) * KS_TILE)), kb = __ldg((const uint2*)(kp + (2 * j + 1) * KS_TILE));
+                        KeyDot<CLS>::cut(ka.x, ka.y);
+                        KeyDot<CLS>::cut(kb.x, kb.y);
+                        dot.mac(__ldg((const uint2*)(dp + j * KS_TILE)), ka.x, ka.y, kb.x, kb.y);
+                    }
+                }
+                u64 v0, v1;
+                dot.reduce(R, i, v0, v1);
+                u64* xp = xs + (size_t)(qi * b + k) * 2 * TN + cd;
+                xp[0] = Acc::x_word(add_mod(v0, pc0, q));
+                xp[TN] = Acc::x_word(v1);
+            }
+        }
+    } else {
+        // X tile: all of a thread's words are requested in batches, one round trip each
+        const u64* xg = x + (size_t)i * N + n0 + c;
+        const u32 n_seg = n_terms * 2;
+        u32 e = l;
+        for (; e + 7 * PL < n_seg; e += 8 * PL) {
+            u64 v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = __ldg(xg + (size_t)(e + j * PL) * np * N);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) xs[(size_t)(e + j * PL) * TN + c] = Acc::x_word(v[j]);
+        }
+        for (; e < n_seg; e += PL) xs[(size_t)e * TN + c] = Acc::x_word(__ldg(xg + (size_t)e * np * N));
+    }
+    // terms up to a whole chunk are zero, and so are the padding words of a group's last stage once they are in registers
+    for (u32 e = 2 * n_terms + l; e < 2 * TILE_TS * lay.C; e += PL) xs[(size_t)e * TN + c] = 0;
+    __syncthreads();
+
+    // ---------------- the weight stream: a lane's words of successive stages lie one stage apart
+    if (pj_begin + l >= pj_end) return;
+    const u32 fmt = COMPACT ? tile_format(lay, i) : (u32)TILE_W64;
+    const u32 n_chunks = lay.C;
+    u32 left = ((pj_end - pj_begin - l + PL - 1) / PL) * n_chunks;      // stages to go
+    const u32 stage_bytes = tile_stage_bytes(fmt);
+    const unsigned char* stage = (const unsigned char*)pt + tile_prime_base(lay, i) +
+                                 ((size_t)tile * lay.G + pj_begin / PL) * n_chunks * stage_bytes;
+    const u32 at = l * TILE_TS * TN + c;
+    constexpr int TS = (int)TILE_TS;
+    // one stage's words of this thread, as they are stored
+    auto fetch = [&](u32 (&wa)[TS], u32 (&wb)[TS]) {
+        if (!COMPACT || fmt == TILE_W64) {
+            const u64* p = (const u64*)stage + at;
+#pragma unroll
+            for (int ts = 0; ts < TS; ++ts) ld_stream(p + ts * TN, pol, wa[ts], wb[ts]);
+        } else {
+            const u32* p = (const u32*)stage + at;
+            const unsigned char* ph = stage + TILE_STAGE_WORDS * 4u + at;
+#pragma unroll
+            for (int ts = 0; ts < TS; ++ts) wa[ts] = ld_stream32(p + ts * TN, pol);
+#pragma unroll
+            for (int ts = 0; ts < TS; ++ts) wb[ts] = fmt == TILE_W40 ? ld_stream8(ph + ts * TN, pol) : 0u;
+        }
+        stage += stage_bytes;
+    };
+    Acc a0, a1;
+    u32 pj = pj_begin + l, ch = 0;
+    const u64* xt = xs + c;
+    const u32 tail = n_terms % TILE_TS;
+    auto use = [&](u32 (&wa)[TS], u32 (&wb)[TS]) {
+        if (tail && ch + 1 == n_chunks) {
+#pragma unroll
+            for (int ts = 1; ts < TS; ++ts)
+                if ((u32)ts >= tail) wa[ts] = wb[ts] = 0;
+        }
+#pragma unroll
+        for (int ts = 0; ts < TS; ++ts) {
+            u32 w0 = wa[ts], w1 = wb[ts];
+            if (COMPACT && fmt != TILE_W64) Acc::narrow_word(w0, w1);
+            a0.mac(w0, w1, xt[(ts * 2) * TN]);
+            a1.mac(w0, w1, xt[(ts * 2 + 1) * TN]);
+        }
+        a0.end_chunk(R, i, ch);
+        a1.end_chunk(R, i, ch);
+        xt += TS * 2 * TN;
+        if (++ch == n_chunks) {
+            u64* ap = a + ((size_t)pj * 2 * np + i) * N;
+            u32 at0 = n0 + c;                                           // where component 0 goes (see MacScatter)
+            if (sc.on && sc.pj0 + pj >= sc.n_out) at0 = automorphism_index(at0, sc.gal_inv[(sc.pj0 + pj) / sc.n_out], logN);
+            ap[at0] = a0.reduce(R, i);
+            ap[(size_t)np * N + n0 + c] = a1.reduce(R, i);
+            a0 = {};
+            a1 = {};
+            pj += PL;
+            ch = 0;
+            xt = xs + c;
+        }
+    };
+    u32 wa[TS], wb[TS], va[TS], vb[TS];
+    fetch(wa, wb);
+    for (;;) {
+        if (left > 1) fetch(va, vb);
+        use(wa, wb);
+        if (left <= 1) break;
+        if (left > 2) fetch(wa, wb);
+        use(va, vb);
+        if (left <= 2) break;
+        left -= 2;
+    }
+}
+
+// grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
+// operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
+// Four blocks an SM (64 registers, a few spilled in the key part) because resident warps are what hides the latency: two,
+// three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
+// keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
+template <bool NARROW, int LOG_TN, bool BABY, bool COMPACT, int RC>
+__global__ void __launch_bounds__(MAC_THREADS, 4)
+mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const __grid_constant__ TileLayout lay,
+           const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 n_pj, u32 pj_per_block,
+           const __grid_constant__ MacScatter sc, const __grid_constant__ BabySteps bs) {
+    extern __shared__ __align__(128) u64 mac_xs[];
+    grid_dependency_enter();
+    const u32 tiles_log = R.logN - LOG_TN;
+    const u32 i = lay.n_primes - 1 - blockIdx.x % lay.n_primes;
+    const u32 tile = (blockIdx.x / lay.n_primes) & ((1u << tiles_log) - 1u), slice = (blockIdx.x / lay.n_primes) >> tiles_log;
+    const u32 pj_begin = slice * pj_per_block, pj_end = min(n_pj, pj_begin + pj_per_block);
+    if (R.dp[i]) mac_body<OP_DP, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    else if (NARROW && i < R.r) mac_body<OP_NARROW, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    else mac_body<OP_WIDE, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+}
+
+struct MacLaunch {
+    const RingHost* ring;
+    const u64* pt;
+    TileLayout lay;
+    const u64* x;
+    u64* a;
+    u32 n_pj, n_terms;
+    MacScatter sc;
+    BabySteps bs;
+    bool baby, compact;
+    cudaStream_t stream;
+};
+
+template <bool NARROW, int LOG_TN, bool BABY, bool COMPACT, int RC>
+static cudaError_t launch_mac_t(const MacLaunch& m) {
+    constexpr u32 TN = 1u << LOG_TN, PL = MAC_THREADS >> LOG_TN;
+    const RingHost& ring = *m.ring;
+    const size_t smem = (size_t)m.lay.C * TILE_TS * 2 * TN * 8;
+    if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    static bool attr_set[MAX_DEVICES] = {false};     // opt in once per device to the large dynamic shared-memory carve-out
+    if (!attr_set[device_slot(ring)]) {
+        cudaError_t e = cudaFuncSetAttribute(mac_kernel<NARROW, LOG_TN, BABY, COMPACT, RC>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (e != cudaSuccess) return e;
+        attr_set[device_slot(ring)] = true;
+    }
+    // slices over the output groups only where the tiles alone leave the machine short of blocks (every slice makes or
+    // reads the X tile again)
+    const u32 tiles = (ring.dev.N >> LOG_TN) * m.lay.n_primes;
+    u32 slices = BABY ? 1u : (148u * 3 + tiles - 1) / tiles;
+    const u32 max_slices = (m.n_pj + PL - 1) / PL;
+    if (slices > max_slices) slices = max_slices;
+    if (slices < 1) slices = 1;
+    u32 per = (m.n_pj + slices - 1) / slices;
+    per = (per + PL - 1) / PL * PL;
+    slices = (m.n_pj + per - 1) / per;
+    return launch_dependent(ring, mac_kernel<NARROW, LOG_TN, BABY, COMPACT, RC>, dim3(tiles * slices), dim3(MAC_THREADS), smem,
+                            m.stream, ring.dev, m.pt, m.lay, m.x, m.a, m.n_terms, m.n_pj, per, m.sc, m.bs);
+}
+
+template <bool NARROW, bool BABY, bool COMPACT, int RC>
+static cudaError_t launch_mac_tile(const MacLaunch& m) {
+    switch (m.lay.log_tn) {
+        case 7: return launch_mac_t<NARROW, 7, BABY, COMPACT, RC>(m);
+        case 6: return launch_mac_t<NARROW, 6, BABY, COMPACT, RC>(m);
+        case 5: return launch_mac_t<NARROW, 5, BABY, COMPACT, RC>(m);
+        default: return launch_mac_t<NARROW, 4, BABY, COMPACT, RC>(m);
+    }
+}
+
+template <bool NARROW>
+static cudaError_t launch_mac_ring(const MacLaunch& m) {
+    if (!m.baby) return m.compact ? launch_mac_tile<NARROW, false, true, 0>(m) : launch_mac_tile<NARROW, false, false, 0>(m);
+    // (digit counts of the shipped parameter sets: the key words of a rotation in registers)
+    switch (m.ring->dev.r) {
+        case 7: return m.compact ? launch_mac_tile<NARROW, true, true, 7>(m) : launch_mac_tile<NARROW, true, false, 7>(m);
+        case 9: return m.compact ? launch_mac_tile<NARROW, true, true, 9>(m) : launch_mac_tile<NARROW, true, false, 9>(m);
+        default: return m.compact ? launch_mac_tile<NARROW, true, true, 0>(m) : launch_mac_tile<NARROW, true, false, 0>(m);
+    }
+}
+
+cudaError_t launch_mac_narrow(const MacLaunch& m);      // every ciphertext prime below 2^50
+cudaError_t launch_mac_wide(const MacLaunch& m);
+
+}  // namespace bf

@@ -29,7 +29,7 @@ cudaEvent_t Profiler::get() {
 ProfScope::ProfScope(Profiler* prof, int c, cudaStream_t st) : p(prof), cat(c), s(st) {
     if (!p) return;
     p->launches[cat]++;
-    if (p->timing && !p->span_open) {
+    if (p->timing) {
         a = p->get();
         cudaEventRecord(a, s);
     }
@@ -40,21 +40,6 @@ ProfScope::~ProfScope() {
     cudaEvent_t b = p->get();
     cudaEventRecord(b, s);
     p->recs.push_back({cat, a, b});
-}
-
-ProfSpan::ProfSpan(Profiler* prof, int c, cudaStream_t st) : p(prof), cat(c), s(st) {
-    if (!p || !p->timing) return;
-    a = p->get();
-    cudaEventRecord(a, s);
-    p->span_open = true;
-}
-
-ProfSpan::~ProfSpan() {
-    if (!p || !a) return;
-    cudaEvent_t b = p->get();
-    cudaEventRecord(b, s);
-    p->recs.push_back({cat, a, b});
-    p->span_open = false;
 }
 
 struct LoadConsts {
@@ -484,6 +469,11 @@ __device__ __forceinline__ bool own_prime(const RingDev& R, const PolyBatch& B, 
     return lo == mod;
 }
 
+// a residue in the form the inner products read (see RingDev::dp)
+__device__ __forceinline__ u64 operand_word(const RingDev& R, u32 mod, u64 v) {
+    return R.dp[mod] ? (u64)__double_as_longlong(u2d(v)) : v;
+}
+
 template <bool FWD, int LOAD, int LOG_R, int LOG_LANES>
 __global__ void __launch_bounds__(((1 << (LOG_R + LOG_LANES)) / 8) < 32 ? 32 : ((1 << (LOG_R + LOG_LANES)) / 8),
                                   ((1 << (LOG_R + LOG_LANES)) / 8) >= 512 ? 2 : ((1 << (LOG_R + LOG_LANES)) / 8) >= 256 ? 4 : 8)
@@ -496,17 +486,12 @@ ntt_strided(const RingDev R, const PolyBatch B) {
     if (FWD && own_prime(R, B, o, mod)) {
         // this digit's transform in its own prime exists already: copy the tile instead
         const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
-        u64* dd = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
-        size_t tbase = 0;
-        if (B.dtile_ptr) {
-            u32 t_hi, t_lo;
-            split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
-            tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
-        }
+        u32 t_hi, t_lo;
+        split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
+        const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
         for (int w = threadIdx.x; w < (1 << (LOG_R + LOG_LANES)); w += blockDim.x) {
             const size_t gidx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * (1 << LOG_LANES) + (w & ((1 << LOG_LANES) - 1));
-            if (B.dtile_ptr) B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = ds[gidx];
-            else dd[gidx] = ds[gidx];
+            B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
         }
         return;
     }
@@ -584,17 +569,12 @@ ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
         if (own_prime(R, B, o, mod)) {
             // this digit's transform in its own prime exists already: copy the tile instead
             const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
-            u64* dd = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
-            size_t tbase = 0;
-            if (B.dtile_ptr) {
-                u32 t_hi, t_lo;
-                split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
-                tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
-            }
+            u32 t_hi, t_lo;
+            split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
+            const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
             for (int w = threadIdx.x; w < POINTS; w += blockDim.x) {
                 const size_t gidx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * LANES + (w & (LANES - 1));
-                if (B.dtile_ptr) B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = ds[gidx];
-                else dd[gidx] = ds[gidx];
+                B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
             }
             continue;
         }
@@ -634,6 +614,8 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
     const u32 a_near = slice + 8u * (u32)swz(4 * lane);                               // points 4 (lane + 32 it) + i
     T e[8];
+    const bool dp = R.dp[mod] != 0;         // (the operand arrays hold this prime's words as doubles)
+    (void)dp;
     size_t dtile_base = 0;
     if constexpr (DTILE) {
         u32 o_hi, o_lo;
@@ -729,7 +711,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 for (int i = 0; i < 4; ++i) {
                     double v = fp_centre(*(double*)&e[i], qd, qi);
                     if (v < 0.0) v = __dadd_rn(v, qd);
-                    v4[i] = d2u(v);
+                    v4[i] = DTILE && dp ? (u64)__double_as_longlong(v) : d2u(v);
                 }
             } else {
 #pragma unroll
@@ -784,10 +766,9 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const u32 at = tile_word_index(B.tile, pj, term, n);
                 const u32 fmt = tile_format(B.tile, mod);
                 if (fmt == TILE_W64) {
-                    if (B.split_bits && !(q >> 50)) {     // (the special prime of double hoisting stays in whole words)
+                    const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) v4[i] = limb_split(v4[i], B.split_bits);
-                    }
+                    for (int i = 0; i < 4; ++i) v4[i] = dp ? (u64)__double_as_longlong(u2d(v4[i])) : limb_split(v4[i], L);
                     ulonglong2* gp = (ulonglong2*)(stage + (size_t)at * 8);
                     gp[0] = make_ulonglong2(v4[0], v4[1]);
                     gp[1] = make_ulonglong2(v4[2], v4[3]);
@@ -817,29 +798,12 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     ((ulonglong2*)zp)[1] = make_ulonglong2(0, 0);
                 }
             }
-            if (B.split_bits) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v4[i] = limb_split(v4[i], B.split_bits);
-            }
-            if (B.dtile_ptr) {  // operands of the key-switch inner product: tile-major (keys also permuted, times 2^64)
-                if (B.scatter) {
-                    const u32* sc = B.scatter + (size_t)(o / B.scatter_div) * R.N + chunk * LEN + 4 * s;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        B.dtile_ptr[ks_tile_index(R.N, B.n_m, B.dtile_div, o, m, sc[i])] =
-                            B.scatter_mont ? mul_shoup(v4[i], R.c64[mod], R.c64s[mod], q) : v4[i];
-                } else {
-                    ulonglong2* gp = (ulonglong2*)(B.dtile_ptr + ks_tile_index(R.N, B.n_m, B.dtile_div, o, m, chunk * LEN + 4 * s));
-                    gp[0] = make_ulonglong2(v4[0], v4[1]);
-                    gp[1] = make_ulonglong2(v4[2], v4[3]);
-                }
-                continue;
-            }
-            if (B.scatter) {    // permuted store (keys are kept pre-permuted by their automorphism)
+            if (B.scatter) {    // rotation keys: tile-major, permuted by their automorphism, in the form the inner products read
                 const u32* sc = B.scatter + (size_t)(o / B.scatter_div) * R.N + chunk * LEN + 4 * s;
-                u64* sd = B.scatter_dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sd[sc[i]] = B.scatter_mont ? mul_shoup(v4[i], R.c64[mod], R.c64s[mod], q) : v4[i];
+                for (int i = 0; i < 4; ++i)
+                    B.dtile_ptr[ks_tile_index(R.N, B.n_m, B.dtile_div, o, m, sc[i])] =
+                        dp ? operand_word(R, mod, v4[i]) : mul_shoup(v4[i], R.c64[mod], R.c64s[mod], q);
                 continue;
             }
             ulonglong2* gp = (ulonglong2*)(gdst + 4 * s);
@@ -942,10 +906,9 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     const ulonglong2* gp = (const ulonglong2*)(stage + (size_t)at * 8);
                     const ulonglong2 a = gp[0], b = gp[1];
                     v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
-                    if (B.split_bits && !(q >> 50)) {
+                    const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) v4[i] = limb_join(v4[i], B.split_bits);
-                    }
+                    for (int i = 0; i < 4; ++i) v4[i] = dp ? d2u(__longlong_as_double((long long)v4[i])) : limb_join(v4[i], L);
                 } else {
                     const uint4 lo = *(const uint4*)(stage + (size_t)at * 4);
                     const u32 hi = fmt == TILE_W40 ? *(const u32*)(stage + TILE_STAGE_WORDS * 4u + at) : 0u;
@@ -958,10 +921,6 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const ulonglong2* gp = (const ulonglong2*)(gsrc + 4 * s);
                 const ulonglong2 a = gp[0], b = gp[1];
                 v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
-                if (B.split_bits) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) v4[i] = limb_join(v4[i], B.split_bits);
-                }
             }
             if (B.sum_terms) {      // the input is a sum of several arrays of the same shape
                 const u64* sp = B.sum_src + (size_t)o * B.src_so + (size_t)m * B.src_sm + (size_t)chunk * LEN + 4 * s;
@@ -1155,7 +1114,7 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
         if (B.tile_ptr)
             launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb,
                              no_rb, no_epi);
-        else if (FWD && B.dtile_ptr && !B.scatter && !B.lift_ptr && !B.split_bits)
+        else if (FWD && B.dtile_ptr && !B.scatter && !B.lift_ptr)
             launch_dependent(ring, ntt_contig<true, 0, false, true>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B,
                              cpb, no_rb, no_epi);
         else
@@ -1197,8 +1156,6 @@ cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B0, u32 n_o
     if (e != cudaSuccess) return e;
     B.scatter = scatter;
     B.scatter_div = scatter_div;
-    B.scatter_dst = final_dst;
-    B.scatter_mont = 1;           // (the only permuted store is that of the rotation keys)
     B.dtile_ptr = final_dst;      // tile-major: o = (key * r + digit) * 2 + component
     B.dtile_div = scatter_div;
     return launch_contig<true>(ring, B, n_polys, stream);

@@ -512,6 +512,26 @@ def test_random_small_ring_cases(case):
         g.close()
 
 
+@pytest.mark.parametrize("modes", [{}, dict(moddown="per_output", hoist="double")], ids=["plain", "extended"])
+@pytest.mark.parametrize("logN,bits,plan_t,shape", [
+    (10, [50, 45, 40, 30], (32, 2, 4, 4), (70, 90)),        # every operand class; 12 terms (a stage half empty), 3 inputs
+    (10, [59, 45, 38, 20], (64, 1, 16, 4), (64, 40)),       # a base prime beyond 2^50: 45 bits in 30-bit limbs
+    (11, [50] + [40] * 6, (32, 4, 2, 4), (33, 100)),        # 7 digits in registers; one key, four inputs in parts
+    (11, [50] + [40] * 8, (32, 2, 8, 2), (20, 60)),         # 9 digits, one output block, 16 terms
+    (12, [40, 40], (64, 8, 1, 8), (100, 64)),               # 2 digits, no baby step
+])
+def test_operand_classes_and_tile_edges(logN, bits, plan_t, shape, modes):
+    taken, primes = {}, []
+    for bt in bits:                                         # the largest primes below each power of two, all distinct
+        found = ckks.find_primes(1 << bt, 2 << logN, bits.count(bt))
+        primes.append(found[taken.setdefault(bt, 0)])
+        taken[bt] += 1
+    P = ckks.find_primes(1 << 60, 2 << logN, 1)[0]
+    par = ckks.Params(1 << logN, primes, P, 2.0 ** 40)
+    # (residues are compared exactly; the bound on the decrypted result only catches slips of scale or packing)
+    run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 31, 1e-2, "classes", tight=1e-2)
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
