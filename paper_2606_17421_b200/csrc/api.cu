@@ -97,6 +97,7 @@ struct bf_ctx {
     cudaStream_t stream;
     int device;
     ulonglong2 *tw_fwd = nullptr, *tw_inv = nullptr;
+    double *tw8_fwd = nullptr, *tw8_inv = nullptr;
     u32* slot_of_pos = nullptr;
     double2 *T = nullptr, *Z = nullptr;
     double* enc_consts = nullptr;   // per-prime constants of the encoder's fp64 load
@@ -115,7 +116,6 @@ struct bf_ctx {
     u32* perms_fwd = nullptr;        // [n_keys][N] perm: rotated[n] = unrotated[perm[n]] (per-output division by P)
     u32 n_keys = 0;
     // scratch (grow-only)
-    size_t dig_half = 0;            // words from a digit set in Dig to its staging twin
     DevBuf X, X0, Aext, Dig, U, Ubig, Tc, Tn, Cc, A, Rres, Lfull, fft, coef, ptnat, ptjit, stage_in, stage_out, nm_a, nm_b;
     u64 cache_budget = 0, cache_used = 0;
     std::vector<bf_weights*> weights;
@@ -260,10 +260,10 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     R.N = N;
     R.logN = ctx->logN;
     R.r = n_ct_primes;
-    ctx->ring.geom = ntt_geometry(ctx->logN);
     ctx->ring.q.assign(primes, primes + nb);
     const u64 P = primes[n_ct_primes];
     std::vector<ulonglong2> twf((size_t)nb * N), twi((size_t)nb * N);
+    std::vector<double> twf8((size_t)nb * N, 0.0), twi8((size_t)nb * N, 0.0);
     for (u32 m = 0; m < nb; ++m) {
         const u64 q = primes[m];
         R.q[m] = q;
@@ -339,6 +339,9 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
             const u32 e = h_brev(k, (int)ctx->logN);
             twf[(size_t)m * N + k] = entry(pw[e]);
             twi[(size_t)m * N + k] = entry(pwi[e]);
+            if (q >> 41) continue;
+            twf8[(size_t)m * N + k] = (double)pw[e];
+            twi8[(size_t)m * N + k] = (double)pwi[e];
         }
     }
     // encoder tables: twiddles from the host's libm so that results do not depend on the device's
@@ -378,6 +381,8 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     } while (0)
     CKC(cudaMalloc(&ctx->tw_fwd, twf.size() * sizeof(ulonglong2)));
     CKC(cudaMalloc(&ctx->tw_inv, twi.size() * sizeof(ulonglong2)));
+    CKC(cudaMalloc(&ctx->tw8_fwd, twf8.size() * sizeof(double)));
+    CKC(cudaMalloc(&ctx->tw8_inv, twi8.size() * sizeof(double)));
     CKC(cudaMalloc(&ctx->slot_of_pos, sop.size() * sizeof(u32)));
     CKC(cudaMalloc(&ctx->T, T.size() * sizeof(double2)));
     CKC(cudaMalloc(&ctx->Z, Z.size() * sizeof(double2)));
@@ -386,6 +391,8 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     ctx->device_error = ctx->overflow_flag + 1;
     CKC(cudaMemcpy(ctx->tw_fwd, twf.data(), twf.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->tw_inv, twi.data(), twi.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
+    CKC(cudaMemcpy(ctx->tw8_fwd, twf8.data(), twf8.size() * sizeof(double), cudaMemcpyHostToDevice));
+    CKC(cudaMemcpy(ctx->tw8_inv, twi8.data(), twi8.size() * sizeof(double), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->slot_of_pos, sop.data(), sop.size() * sizeof(u32), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->T, T.data(), T.size() * sizeof(double2), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->Z, Z.data(), Z.size() * sizeof(double2), cudaMemcpyHostToDevice));
@@ -395,6 +402,8 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
 #undef CKC
     R.tw_fwd = ctx->tw_fwd;
     R.tw_inv = ctx->tw_inv;
+    R.tw8_fwd = ctx->tw8_fwd;
+    R.tw8_inv = ctx->tw8_inv;
     R.enc_consts = ctx->enc_consts;
     *out = ctx;
     return BF_OK;
@@ -424,6 +433,8 @@ extern "C" void bf_ctx_destroy(bf_ctx* ctx) {
     for (DevBuf* b : bufs) free_buf(*b);
     cudaFree(ctx->tw_fwd);
     cudaFree(ctx->tw_inv);
+    cudaFree(ctx->tw8_fwd);
+    cudaFree(ctx->tw8_inv);
     cudaFree(ctx->slot_of_pos);
     cudaFree(ctx->T);
     cudaFree(ctx->Z);
@@ -834,10 +845,7 @@ static int moddown_batch(bf_ctx* ctx, const Lane& lane, const RotBatch& rb, cons
 
 static int ensure_rot_scratch(bf_ctx* ctx, u32 n_dig_sets, u32 n_rot) {
     const size_t N = ctx->N, r = ctx->r, nb = r + 1;
-    // digit sets, tile-major for the inner product, and behind them a staging area of the same size for the
-    // intermediate of their transforms (natural order)
-    TRY(ensure(ctx, ctx->Dig, (size_t)2 * n_dig_sets * r * nb * N * 8));
-    ctx->dig_half = ctx->Dig.cap / 16;
+    TRY(ensure(ctx, ctx->Dig, (size_t)n_dig_sets * r * nb * N * 8));       // digits between the passes of their transforms
     TRY(ensure(ctx, ctx->U, (size_t)n_rot * 2 * nb * N * 8));
     TRY(ensure(ctx, ctx->Tc, (size_t)n_rot * 2 * N * 8));
     TRY(ensure(ctx, ctx->Tn, (size_t)n_rot * 2 * r * N * 8));
@@ -854,12 +862,12 @@ static int find_key(bf_ctx* ctx, u32 steps, int* key) {
 // Digits of c1 (coefficient domain; set s at c1_coeff + s*set_stride, [r][N]) reduced into every prime
 // of the extended basis and transformed: dig[set][j][m] = NTT_m( c1_j mod m ).  The digit in its own
 // prime is the transform of c1 itself, which the caller already has (c1_ntt + s*c1_ntt_stride, [r][N]):
-// it is copied, not recomputed.
+// it is copied, not recomputed.  mid: room for what passes between the two halves of the transform.
 // div_t non-null: c1_coeff holds residues of polynomials of the extended basis and div_t + s*set_stride their
 // residues modulo P (centred): the digits are those of the polynomial divided by P (then c1_ntt is not used: no
 // transform of the quotient exists yet).
-static int modup(bf_ctx* ctx, cudaStream_t stream, const u64* c1_coeff, long long set_stride, u32 n_sets, u64* dig,
-                 const u64* c1_ntt, long long c1_ntt_stride, const u64* div_t = nullptr) {
+static PolyBatch modup_batch(bf_ctx* ctx, const u64* c1_coeff, long long set_stride, u64* mid, const u64* c1_ntt, long long c1_ntt_stride,
+                             const u64* div_t = nullptr) {
     const u32 N = ctx->N, r = ctx->r, nb = r + 1;
     PolyBatch B;
     memset(&B, 0, sizeof(B));
@@ -871,9 +879,7 @@ static int modup(bf_ctx* ctx, cudaStream_t stream, const u64* c1_coeff, long lon
     B.src_so2 = set_stride;
     B.src_so = N;
     B.src_sm = 0;
-    B.dst = dig + ctx->dig_half;         // staging between the two passes; the result goes to dig, tile-major
-    B.dtile_ptr = dig;
-    B.dtile_div = r;
+    B.dst = mid;                 // between the two passes
     B.dst_so = (long long)nb * N;
     B.dst_sm = N;
     B.skip_diag = div_t ? 0 : 1;
@@ -882,8 +888,7 @@ static int modup(bf_ctx* ctx, cudaStream_t stream, const u64* c1_coeff, long lon
     B.diag_so = c1_ntt_stride;
     B.div_t = div_t;
     B.div_so = set_stride;
-    CK(ntt_forward(ctx->ring, B, n_sets * r, LOAD_REDUCE, stream));
-    return BF_OK;
+    return B;
 }
 
 static void stamp(bf_ctx* ctx, int i) {
@@ -971,7 +976,9 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     const bool rotate_in_mac = dh && (resident || groups == n_pj);
     if (rotate_in_mac) in_batch = n_in;
     u32 n_dig_sets = giant_per_lane * (u32)lanes;       // digit sets alive at once
-    if (n_dig_sets < in_batch) n_dig_sets = in_batch;
+    // (the digits that the multiply-accumulate reads lie before those between the passes)
+    const u32 in_sets = rotate_in_mac ? 2 * in_batch : in_batch;
+    if (n_dig_sets < in_sets) n_dig_sets = in_sets;
     const size_t xw = (size_t)2 * nmp * N;                // words per term of X / per inner sum
     TRY(ensure(ctx, ctx->X, (size_t)n_in * (rotate_in_mac ? 1u : b) * xw * 8));
     if (dh) {
@@ -1046,34 +1053,40 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     if (b > 1) {
         for (u32 q0 = 0; q0 < n_in; q0 += in_batch) {
             const u32 qn = (n_in - q0 < in_batch) ? n_in - q0 : in_batch;
-            TRY(modup(ctx, ctx->stream, ct_in + (size_t)q0 * ctw + (size_t)r * N, (long long)ctw, qn, Dig,
-                      X0 + (size_t)q0 * x0_stride + (size_t)r * N, x0_stride));
-            if (rotate_in_mac) continue;
-            // the rotations of the batch, key-major (rotation t = (k - 1) * qn + q: those that share a key follow one
-            // another, so that an inner-product block loads the key once for all of them), dealt out to the lanes
-            // in contiguous runs
-            const u32 n_rot = qn * (b - 1);
-            const u32 per = cdiv(b - 1, (u32)lanes_baby) * qn;           // whole keys per lane: no key is streamed by two lanes
-            const int used = (int)cdiv(n_rot, per);
-            TRY(fork_lanes(ctx, used));
+            PolyBatch D0 = modup_batch(ctx, ct_in + (size_t)q0 * ctw + (size_t)r * N, (long long)ctw, Dig, X0 + (size_t)q0 * x0_stride + (size_t)r * N,
+                                       x0_stride);
+            if (rotate_in_mac) {            // the digits stay, in the form the multiply-accumulate reads
+                D0.dst = Dig + (size_t)qn * r * nb * N;
+                D0.dtile_ptr = Dig;
+                D0.dtile_div = r;
+                CK(ntt_forward(ctx->ring, D0, qn * r, LOAD_REDUCE, ctx->stream));
+                continue;
+            }
+            // the rotations of the batch, dealt out to the lanes by whole keys, so that no key is streamed by two lanes; the
+            // first pass of the digits' transforms is shared
+            const u32 per = cdiv(b - 1, (u32)lanes_baby);
+            const int used = (int)cdiv(b - 1, per);
+            if (used > 1) {
+                CK(ntt_forward_first(ctx->ring, D0, qn * r, ctx->stream));
+                TRY(fork_lanes(ctx, used));
+            }
             for (int c = 0; c < used; ++c) {
                 RotBatch rb;
                 memset(&rb, 0, sizeof(rb));
-                const u32 t_end = (u32)(c + 1) * per < n_rot ? (u32)(c + 1) * per : n_rot;
-                for (u32 t = (u32)c * per; t < t_end; ++t) {
-                    const u32 q = t % qn, k = t / qn + 1;
-                    const int i = rb.n++;
-                    rb.key[i] = baby_key[k];
-                    rb.dig[i] = (int)q;
-                    rb.c0[i] = (int)((q0 + q) * b);
-                    rb.out[i] = (int)((q0 + q) * b + k);
-                }
-                if (dh) {       // no division by P: the inner product's last step assembles the rotated input in X
-                    CK(launch_key_inner_product(ctx->ring, rb, Dig, ctx->keys, nullptr, ctx->device_error, lane[c].s, X,
-                                                ctx->perms));
-                    continue;
-                }
-                CK(launch_key_inner_product(ctx->ring, rb, Dig, ctx->keys, lane[c].U, ctx->device_error, lane[c].s));
+                const u32 k_end = (u32)(c + 1) * per < b - 1 ? (u32)(c + 1) * per : b - 1;
+                for (u32 q = 0; q < qn; ++q)
+                    for (u32 k = (u32)c * per + 1; k <= k_end; ++k) {
+                        const int i = rb.n++;
+                        rb.key[i] = baby_key[k];
+                        rb.dig[i] = (int)q;
+                        rb.c0[i] = (int)((q0 + q) * b);
+                        rb.out[i] = dh ? (int)((q0 + q) * b + k) : i;
+                    }
+                // double hoisting, no division by P: the product's last step assembles the rotated input in X
+                CK(ntt_forward_inner(ctx->ring, D0, used > 1 ? 0 : qn, rb, ctx->keys, dh ? nullptr : lane[c].U, dh ? X : nullptr,
+                                     dh ? ctx->perms : nullptr, lane[c].s));
+                if (dh) continue;
+                for (int i = 0; i < rb.n; ++i) rb.out[i] = (int)((q0 + i / (k_end - (u32)c * per)) * b + (u32)c * per + 1 + i % (k_end - (u32)c * per));
                 TRY(moddown_batch(ctx, lane[c], rb, X, (long long)ctw, X, (long long)ctw));
             }
             TRY(join_lanes(ctx, used));
@@ -1187,8 +1200,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
                     B.mod_step = 1;
                     B.store_centred = 2;
                     CK(ntt_inverse(ctx->ring, B, cnt, lane[c].s));
-                    TRY(modup(ctx, lane[c].s, lane[c].Cc, (long long)nb * N, cnt, lane[c].Dig, nullptr, 0,
-                              lane[c].Cc + (size_t)r * N));
+                    const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)nb * N, lane[c].Dig, nullptr, 0, lane[c].Cc + (size_t)r * N);
                     RotBatch rb;
                     memset(&rb, 0, sizeof(rb));
                     rb.n = (int)cnt;
@@ -1199,9 +1211,8 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
                         rb.out[t] = (int)t;
                     }
                     // (stored through the rotation: the output assembly reads plain sums)
-                    CK(launch_key_inner_product(ctx->ring, rb, lane[c].Dig, ctx->keys,
-                                                (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, ctx->device_error, lane[c].s,
-                                                nullptr, ctx->perms));
+                    CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, nullptr,
+                                         ctx->perms, lane[c].s));
                     continue;
                 }
                 const u64* Asrc = A + (size_t)(n_out + rho0) * ctw;      // ciphertexts with j >= 1 are contiguous
@@ -1216,7 +1227,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
                 B.mod0 = 0;
                 B.mod_step = 1;
                 CK(ntt_inverse(ctx->ring, B, cnt, lane[c].s));
-                TRY(modup(ctx, lane[c].s, lane[c].Cc, (long long)r * N, cnt, lane[c].Dig, Asrc + (size_t)r * N, (long long)ctw));
+                const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)r * N, lane[c].Dig, Asrc + (size_t)r * N, (long long)ctw);
                 RotBatch rb;
                 memset(&rb, 0, sizeof(rb));
                 rb.n = (int)cnt;
@@ -1228,11 +1239,11 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
                     rb.out[t] = (int)t;
                 }
                 if (per_output) {
-                    CK(launch_key_inner_product(ctx->ring, rb, lane[c].Dig, ctx->keys,
-                                                (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, ctx->device_error, lane[c].s));
+                    CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, nullptr, nullptr,
+                                         lane[c].s));
                     continue;
                 }
-                CK(launch_key_inner_product(ctx->ring, rb, lane[c].Dig, ctx->keys, lane[c].U, ctx->device_error, lane[c].s));
+                CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, lane[c].U, nullptr, nullptr, lane[c].s));
                 TRY(moddown_batch(ctx, lane[c], rb, Asrc, (long long)ctw, Rres + (size_t)rho0 * ctw, (long long)ctw));
             }
         }
@@ -1546,14 +1557,13 @@ extern "C" int bf_rotate(bf_ctx* ctx, const uint64_t* ct_in, uint32_t steps, uin
     B.n_m = r;
     B.mod_step = 1;
     CK(ntt_forward(ctx->ring, B, 2, LOAD_PLAIN, ctx->stream));
-    TRY(modup(ctx, ctx->stream, ct_in + (size_t)r * N, (long long)r * N, 1, (u64*)ctx->Dig.p, X + (size_t)r * N, 0));
+    const PolyBatch D0 = modup_batch(ctx, ct_in + (size_t)r * N, (long long)r * N, (u64*)ctx->Dig.p, X + (size_t)r * N, 0);
     RotBatch rb;
     memset(&rb, 0, sizeof(rb));
     rb.n = 1;
     rb.key[0] = key;
+    CK(ntt_forward_inner(ctx->ring, D0, 1, rb, ctx->keys, (u64*)ctx->U.p, nullptr, nullptr, ctx->stream));
     rb.out[0] = 1;
-    CK(launch_key_inner_product(ctx->ring, rb, (const u64*)ctx->Dig.p, ctx->keys, (u64*)ctx->U.p, ctx->device_error,
-                                ctx->stream));
     TRY(moddown_batch(ctx, main_lane(ctx), rb, X, (long long)ctw, X, (long long)ctw));
     memset(&B, 0, sizeof(B));
     B.src = X + ctw;
@@ -1603,8 +1613,7 @@ extern "C" int bf_fold(bf_ctx* ctx, uint64_t* ct, uint32_t n_ct) {
             B.mod_wrap = r;
             B.mod_step = 1;
             CK(ntt_forward(ctx->ring, B, cnt, LOAD_PLAIN, ctx->stream));
-            TRY(modup(ctx, ctx->stream, cts + (size_t)r * N, (long long)ctw, cnt, lane.Dig, X + (size_t)r * N,
-                      (long long)2 * ctw));
+            const PolyBatch D0 = modup_batch(ctx, cts + (size_t)r * N, (long long)ctw, lane.Dig, X + (size_t)r * N, (long long)2 * ctw);
             RotBatch rb;
             memset(&rb, 0, sizeof(rb));
             rb.n = (int)cnt;
@@ -1612,9 +1621,10 @@ extern "C" int bf_fold(bf_ctx* ctx, uint64_t* ct, uint32_t n_ct) {
                 rb.key[t] = key;
                 rb.dig[t] = (int)t;
                 rb.c0[t] = (int)(2 * t);
-                rb.out[t] = (int)(2 * t + 1);
+                rb.out[t] = (int)t;
             }
-            CK(launch_key_inner_product(ctx->ring, rb, lane.Dig, ctx->keys, lane.U, ctx->device_error, ctx->stream));
+            CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, lane.U, nullptr, nullptr, ctx->stream));
+            for (u32 t = 0; t < cnt; ++t) rb.out[t] = (int)(2 * t + 1);
             TRY(moddown_batch(ctx, lane, rb, X, (long long)ctw, X, (long long)ctw));
             memset(&B, 0, sizeof(B));
             B.src = X;

@@ -51,6 +51,7 @@ struct RingDev {
     const double* enc_consts;    // [r+1][ENC_CONSTS]
     const ulonglong2* tw_fwd;    // [r+1][N]  (psi^brev(k), companion), merged Cooley-Tukey order
     const ulonglong2* tw_inv;    // [r+1][N]  inverses of the above, for the Gentleman-Sande inverse
+    const double *tw8_fwd, *tw8_inv;   // [r+1][N]  (double)w alone, moduli below 2^41
 };
 
 // floor(x * w / 2^64)-based modular multiplication by a constant w with precomputed
@@ -168,8 +169,7 @@ struct RotBatch {                     // one key-switch launch over n rotations
     int dig[MAX_ROT_BATCH];           // which digit set the rotation reads
     int c0[MAX_ROT_BATCH];            // which source ciphertext is being rotated (its c0 is added)
     int out[MAX_ROT_BATCH];           // which output ciphertext slot receives the result
-    // runs of consecutive rotations that use the same key (filled in by the inner-product launcher): a block of the
-    // inner product takes one run, loads the key once and walks the run's digit sets
+    // runs of consecutive rotations that read the same digit set (filled in by the launcher): one block takes one run
     int n_groups;
     unsigned char grp_first[MAX_ROT_BATCH], grp_cnt[MAX_ROT_BATCH];
 };
@@ -285,7 +285,6 @@ __host__ __device__ __forceinline__ size_t tile_stage_of_word(const TileLayout& 
 // A batch of equally sized polynomials addressed as (outer index o, slot m):
 //   source  = src + o*src_so + m*src_sm      destination = dst + o*dst_so + m*dst_sm
 //   modulus index of polynomial (o, m) = mod0 + m*mod_step
-// blockIdx.y enumerates o*n_m + m.
 struct PolyBatch {
     const void* src;
     u64* dst;
@@ -319,9 +318,8 @@ struct PolyBatch {
                                   //   residue modulo P: the un-rotated input lifted to the extended basis
     u64* dtile_ptr;               // forward only, non-null: the final result goes there instead of dst, tile-major in tiles
     u32 dtile_div;                //   of KS_TILE coefficients (see ks_tile_index); with `scatter` the store is permuted
-    u32 grid3;                    // set by the launchers: the grid is (x, m, o) and no index has to be divided out
     u32 o_div_magic, dtile_magic; // ceil(2^32 / o_div), ceil(2^32 / dtile_div): o / d = umulhi(o, magic) for o < 2^16
-                                  //   (set by the launchers with grid3; 0 = divide)
+                                  //   (set by the launchers; 0 = divide)
     const u64* div_t;             // forward from a shared source, non-null (double hoisting): the source of digit
     long long div_so;             //   i = o % o_div of set s = o / o_div is the residue modulo q_i of a polynomial in the
                                   //   extended basis, coefficient domain, and t = div_t + s*div_so holds its residue
@@ -338,7 +336,7 @@ __host__ __device__ __forceinline__ size_t ks_tile_index(u32 N, u32 n_m, u32 div
     return ((((size_t)(o / div) * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + o % div) * KS_TILE + n % KS_TILE;
 }
 
-// o / d and o % d with a host-made reciprocal (see PolyBatch::grid3); magic = 0 divides
+// o / d and o % d with a host-made reciprocal (see PolyBatch::o_div_magic); magic = 0 divides
 __device__ __forceinline__ void split_index(u32 o, u32 d, u32 magic, u32& hi, u32& lo) {
     hi = magic ? __umulhi(o, magic) : o / d;
     lo = o - hi * d;
@@ -378,6 +376,16 @@ __device__ __forceinline__ u64 redc_2x32(u64 H, u64 L, u64 q, u32 qneg32) {
         : "r"(q0), "r"(q1), "r"(qneg32));
     const u64 t = ((u64)h1 << 32) | h0;
     return t >= q ? t - q : t;
+}
+
+// words that are read exactly once: not kept in L1, first to leave L2
+__device__ __forceinline__ u64 stream_policy() {
+    u64 pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ void ld_stream(const void* p, u64 policy, u32& lo, u32& hi) {
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;" : "=r"(lo), "=r"(hi) : "l"(p), "l"(policy));
 }
 
 // ---- Sums of products of residues, three ways.  B200 issues 64 fp64 multiply-adds per SM and clock, but only 32
@@ -437,6 +445,27 @@ __device__ __forceinline__ void cut_limbs(u32 lo, u32 hi, u32 L, u32& w0, u32& w
     w0 = lo & ((1u << L) - 1u);
     w1 = __funnelshift_r(lo, hi, L);
 }
+
+// One output word of the key-switch inner product: digits times key words (as stored), summed, in [0, q).  The keys carry a
+// factor 2^64 except where the class is OP_DP.
+template <int CLS>
+struct DigitDot {
+    static constexpr u32 L = CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW;
+    LimbAcc<CLS == OP_WIDE> a;
+    __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1) {
+        u32 d0, d1;
+        cut_limbs(d.x, d.y, L, d0, d1);
+        cut_limbs(k0, k1, L, k0, k1);
+        a.mac(d0, d1, d0 + d1, k0, k1);
+    }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const { return a.reduce(R.q[m], (u32)R.qneg[m]); }
+};
+template <>
+struct DigitDot<OP_DP> {
+    DpAcc a;
+    __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1) { a.mac(__hiloint2double((int)d.y, (int)d.x), __hiloint2double((int)k1, (int)k0)); }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const { return d2u(a.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m])); }
+};
 
 // One output pair of the key-switch inner product: digit j (d[j * ds]) times key words (2j, 2j + 1) (k[s * ks]) summed
 // over r digits, in [0, q).  The keys carry a factor 2^64 except where the class is OP_DP.

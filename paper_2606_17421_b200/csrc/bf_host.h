@@ -9,12 +9,6 @@
 
 namespace bf {
 
-struct NttGeometry {
-    int log_r, log_c;                 // N = 2^log_r rows x 2^log_c columns
-    int strided_lanes, strided_threads;
-    int contig_lanes, contig_threads, contig_pad;
-};
-
 // Kernel categories for launch counting and optional per-launch event timing.
 enum KernelCat : int {
     CAT_NTT_FWD_STRIDED = 0, CAT_NTT_FWD_CONTIG, CAT_NTT_INV_CONTIG, CAT_NTT_INV_STRIDED,
@@ -43,7 +37,6 @@ struct ProfScope {
 
 struct RingHost {
     RingDev dev;
-    NttGeometry geom;
     std::vector<u64> q;               // q_0..q_L, then P
     Profiler* prof = nullptr;
     bool dependent_launch = true;     // launch the kernels of a call with programmatic stream serialisation
@@ -73,7 +66,6 @@ static inline cudaError_t launch_dependent(const RingHost& ring, void (*kernel)(
 }
 
 // ---- ntt.cu
-NttGeometry ntt_geometry(u32 logN);
 cudaError_t ntt_forward(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, cudaStream_t stream);
 cudaError_t ntt_inverse(const RingHost& ring, const PolyBatch& B, u32 n_outer, cudaStream_t stream);
 // Forward transform of the centred lifts of P-residues with the ModDown epilogue fused into its last store.
@@ -90,17 +82,22 @@ cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, 
 cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, u64* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream);
 
+// First pass alone of a forward transform of digits (LOAD_REDUCE).
+cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_outer, cudaStream_t stream);
+// Digits of n_sets sets (B: LOAD_REDUCE from a shared source, B.dst = room for the [n_sets * r][r + 1][N] words between the
+// passes; n_sets = 0: they are there already) transformed and multiplied with the rotation keys (pre-permuted, tile-major):
+//   u[rb.out[rot]][comp][m][n] = sum_j NTT_m(digit j of set rb.dig[rot])[n] * key'[rb.key[rot]][j][comp][m][n]
+// stored at pinv[rb.key[rot]][n] where pinv is non-null.  xext non-null (double hoisting, with pinv): the result is finished
+// as a rotated input in the extended basis, xext[rb.out[rot]][comp][m][pinv[..][n]] = u'[comp][m][n] + (comp == 0 ?
+// xext[rb.c0[rot]][0][m][n] : 0), terms of [2][r+1][N] words (term rb.c0[rot] holds P times the un-rotated input).
+// Rotations of the same set have to be consecutive.
+cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B, u32 n_sets, const RotBatch& rb, const u64* keys, u64* u, u64* xext,
+                              const u32* pinv, cudaStream_t stream);
+
 // ---- kernels.cu : element-wise and streaming kernels of the linear layer
 // out[t] = a[t] * b[t] pointwise, polynomial t modulo basis prime mod0 + t % n_m
 cudaError_t launch_pointwise_mul(const RingHost& ring, const u64* a, const u64* b, u64* out, u32 n_polys, u32 n_m,
                                  u32 mod0, cudaStream_t stream);
-// u'[rot][comp][m][n] = sum_j dig[dig(rot)][j][m][n] * key'[key(rot)][j][comp][m][n]  (keys pre-permuted)
-// pinv non-null, xext null: u'[rot][comp][m] is stored through the rotation's permutation, at pinv[rb.key[rot]][n].
-// xext non-null (double hoisting): rotation `rot` is not stored to u but finished as a rotated input in the
-// extended basis: xext[rb.out[rot]][comp][m][pinv[rb.key[rot]][n]] = u'[comp][m][n] + (comp == 0 ?
-// xext[rb.c0[rot]][0][m][n] : 0), terms of [2][r+1][N] words (term rb.c0[rot] holds P times the un-rotated input).
-cudaError_t launch_key_inner_product(const RingHost& ring, const RotBatch& rb, const u64* dig, const u64* keys, u64* u,
-                                     int* error_flag, cudaStream_t stream, u64* xext = nullptr, const u32* pinv = nullptr);
 u32 mac_split_bits(const RingHost& ring);   // limb width of cached 8-byte words modulo primes below 2^50
 // layout of n_pj groups of n_terms diagonals held in n_primes primes (0 = the r ciphertext primes)
 TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_primes = 0);

@@ -1,5 +1,4 @@
-// Streaming and element-wise kernels of the encrypted linear layer: the key-switch inner product
-// (Sec. 4.2), the rescale (Sec. 2.1), width changes of cached coefficients.
+// Element-wise kernels of the encrypted linear layer: the rescale (Sec. 2.1), width changes of cached coefficients.
 #include "bf_host.h"
 
 #include <cstring>
@@ -25,235 +24,6 @@ cudaError_t launch_pointwise_mul(const RingHost& ring, const u64* a, const u64* 
     ProfScope prof(ring.prof, CAT_POINTWISE, stream);
     pointwise_mul_kernel<<<grid, 256, 0, stream>>>(ring.dev, a, b, out, n_m, mod0);
     return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------------------------------------
-// Asynchronous bulk copies (TMA, untiled form) and transaction barriers.
-__device__ __forceinline__ u32 smem_addr(const void* p) { return (u32)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(u64* bar, u32 count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(u64* bar, u32 bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-// global -> shared copy of `bytes` (multiple of 16, both addresses 16-byte aligned); completion is
-// signalled on the barrier as transferred bytes
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, u32 bytes, u64* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-// the same copy, with the lines marked "evict first" in L2: for streams that are read exactly once and must
-// not push reused operands (rotated inputs, digits, outputs) out of the cache
-__device__ __forceinline__ u64 l2_evict_first_policy() {
-    u64 pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void bulk_g2s_stream(void* dst, const void* src, u32 bytes, u64* bar, u64 policy) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar)), "l"(policy)
-        : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(u64* bar, u32 parity) {
-    u32 ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: gives up after a fixed number of polls (each poll may itself suspend for a while),
-// records the failure and lets the caller carry on so that the kernel always terminates.
-__device__ __forceinline__ void mbar_wait(u64* bar, u32 parity, int* error_flag) {
-    for (int it = 0; it < (1 << 22); ++it)
-        if (mbar_try_wait(bar, parity)) return;
-    atomicExch(error_flag, 1);
-}
-
-__device__ __forceinline__ void mbar_arrive(u64* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
-// ------------------------------------------------------------------------------------------------
-// Key-switch inner product over the extended basis (Sec. 4.2 "key-switching primitives").
-// The rotation keys are stored pre-permuted by their automorphism, so the product runs in the
-// un-rotated index space with fully coalesced operands:
-//   u'[rot][comp][m][n] = sum_j dig[dig(rot)][j][m][n] * key'[key(rot)][j][comp][m][n]
-// and the automorphism is applied once, as a scatter, when the rotated ciphertext is assembled.
-// Products accumulate as KeyDot says, one reduction per output word.
-//
-// A block owns one (run of rotations that share a key, modulus, tile of 128 coefficients): the baby rotations
-// of several input ciphertexts by the same amount, or the giant rotations of several output blocks by the same
-// amount.  Keys and digit sets are kept tile-major (see ks_tile_index): the key's 2r segments of the tile are one
-// contiguous block, fetched once by one asynchronous bulk copy, and stay in shared memory, so that the key stream
-// crosses HBM (and L2) once per run instead of once per rotation; the r digit segments of each rotation of the run
-// (one contiguous block as well) follow through two buffers, the next rotation's copy in flight while the current
-// one is multiplied.  The keys are resident in Montgomery form (times 2^64 mod q), so the sum
-// of the r products ends in the two-round 32-bit Montgomery reduction: r * max digit < 2^64 keeps it below
-// q * 2^64.  With double hoisting the block also finishes the rotated input (see launch_key_inner_product).
-// grid: x = run, y = tile, z = modulus of the extended basis.
-constexpr int KI_TILE = (int)KS_TILE;
-
-// sum over the r digits of digit x key for both key components, reduced; RC > 0: r == RC
-template <int CLS, int RC>
-__device__ __forceinline__ void ki_products(const RingDev& R, u32 m, const u64* sdc, const u64* sk, u32 r, u32 tid, u64& v0, u64& v1) {
-    KeyDot<CLS> dot;
-    auto term = [&](u32 j) {
-        uint2 ka = *(const uint2*)&sk[(j * 2) * KI_TILE + tid], kb = *(const uint2*)&sk[(j * 2 + 1) * KI_TILE + tid];
-        KeyDot<CLS>::cut(ka.x, ka.y);
-        KeyDot<CLS>::cut(kb.x, kb.y);
-        dot.mac(*(const uint2*)&sdc[j * KI_TILE + tid], ka.x, ka.y, kb.x, kb.y);
-    };
-    if constexpr (RC > 0) {
-#pragma unroll
-        for (int j = 0; j < RC; ++j) term(j);
-    } else {
-        for (u32 j = 0; j < r; ++j) term(j);
-    }
-    dot.reduce(R, m, v0, v1);
-}
-template <int CLS>
-__device__ __forceinline__ void ki_products(const RingDev& R, u32 m, const u64* sdc, const u64* sk, u32 r, u32 tid, u64& v0, u64& v1) {
-    // (digit counts of the shipped parameter sets with the loop unrolled: the launches where several rotations share a
-    // key are bound by instruction issue)
-    if (r == 7) ki_products<CLS, 7>(R, m, sdc, sk, r, tid, v0, v1);
-    else if (r == 9) ki_products<CLS, 9>(R, m, sdc, sk, r, tid, v0, v1);
-    else ki_products<CLS, 0>(R, m, sdc, sk, r, tid, v0, v1);
-}
-
-__global__ void __launch_bounds__(KI_TILE, 8) key_inner_bulk_kernel(const RingDev R, const RotBatch rb,
-                                                                   const u64* __restrict__ dig,
-                                                                   const u64* __restrict__ keys, u64* __restrict__ u,
-                                                                   int* __restrict__ error_flag,
-                                                                   u64* __restrict__ xext, const u32* __restrict__ pinv) {
-    extern __shared__ __align__(128) unsigned char ki_smem[];
-    const u32 grp = blockIdx.x, m = blockIdx.z;
-    const u32 first = rb.grp_first[grp], cnt = rb.grp_cnt[grp];      // this block's run of rotations: one key
-    const u32 N = R.N, r = R.r, nb = r + 1;
-    const u32 n0 = blockIdx.y * KI_TILE;
-    u64* sk = (u64*)ki_smem;                        // [r][2][KI_TILE] key components
-    u64* sd = sk + (size_t)2 * r * KI_TILE;         // [2][r][KI_TILE] digits of the current and the next rotation
-    u64* kbar = sd + (size_t)2 * r * KI_TILE;
-    u64* dbar = kbar + 1;                           // [2]
-    const u32 tid = threadIdx.x;
-    asm volatile("griddepcontrol.launch_dependents;");
-    if (tid == 0) {
-        mbar_init(kbar, 1);
-        mbar_init(&dbar[0], 1);
-        mbar_init(&dbar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    // digit segments of rotation `first + it` into buffer it & 1
-    auto fetch_digits = [&](u32 it) {
-        u64* buf = sd + (size_t)(it & 1) * r * KI_TILE;
-        if (tid == 0) mbar_expect_tx(&dbar[it & 1], r * KI_TILE * 8);
-        __syncwarp();
-        // the r digit segments of this set, modulus and tile are contiguous (see ks_tile_index): one copy
-        if (tid == 0)
-            bulk_g2s(buf, dig + ks_tile_base(N, nb, r, (u32)rb.dig[first + it], 0u, m) + (size_t)blockIdx.y * r * KI_TILE,
-                     r * KI_TILE * 8, &dbar[it & 1]);
-    };
-    if (tid < 32) {
-        if (tid == 0) mbar_expect_tx(kbar, 2 * r * KI_TILE * 8);
-        __syncwarp();
-        // the keys do not depend on the previous kernel: fetch them before waiting for it, the digits after
-        const u64 stream_policy = l2_evict_first_policy();      // keys stream through; digits and outputs stay in L2
-        if (tid == 0)       // the 2r key segments of this key, modulus and tile: one contiguous block
-            bulk_g2s_stream(sk, keys + ks_tile_base(N, nb, 2 * r, (u32)rb.key[first], 0u, m) + (size_t)blockIdx.y * 2 * r * KI_TILE,
-                            2 * r * KI_TILE * 8, kbar, stream_policy);
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        fetch_digits(0);
-        if (cnt > 1) fetch_digits(1);
-    } else {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-    }
-    const u64 q = R.q[m];
-    const size_t term_words = (size_t)2 * nb * N;
-    // double hoisting: what the last step of a rotation reads from global memory (where the coefficient goes under the
-    // rotation, and P*c0) is requested before the wait for the operands, so that it is not a second round trip
-    u32 dest = 0;
-    u64 pc0 = 0;
-    if (pinv) dest = __ldg(&pinv[(size_t)rb.key[first] * N + n0 + tid]);    // (the same for every rotation of the run)
-    if (xext) pc0 = xext[(size_t)rb.c0[first] * term_words + (size_t)m * N + n0 + tid];
-    mbar_wait(kbar, 0, error_flag);
-    for (u32 it = 0; it < cnt; ++it) {
-        const u32 rot = first + it;
-        const u64* sdc = sd + (size_t)(it & 1) * r * KI_TILE;
-        u64 pc0_next = 0;
-        if (xext && it + 1 < cnt) pc0_next = xext[(size_t)rb.c0[rot + 1] * term_words + (size_t)m * N + n0 + tid];
-        mbar_wait(&dbar[it & 1], (it >> 1) & 1, error_flag);
-        u64 v0, v1;
-        if (R.dp[m]) ki_products<OP_DP>(R, m, sdc, sk, r, tid, v0, v1);
-        else if (R.q[m] >> 50) ki_products<OP_WIDE>(R, m, sdc, sk, r, tid, v0, v1);
-        else ki_products<OP_NARROW>(R, m, sdc, sk, r, tid, v0, v1);
-        if (it + 2 < cnt) {                                  // the buffer is free once every thread has read it
-            __syncthreads();
-            if (tid < 32) fetch_digits(it + 2);
-        }
-        if (xext) {
-            // double hoisting: no division by P; the rotated input in the extended basis is (P*c0 + u0, u1) moved
-            // through the rotation's permutation; P*c0 (zero modulo P) was stored as the un-rotated term
-            v0 = add_mod(v0, pc0, q);
-            u64* xp = xext + (size_t)rb.out[rot] * term_words + (size_t)m * N + dest;
-            xp[0] = v0;
-            xp[(size_t)nb * N] = v1;
-            pc0 = pc0_next;
-        } else {
-            // (pinv without xext: the plain result, stored through the rotation's permutation)
-            u64* up = u + ((size_t)rot * 2 * nb + m) * N + (pinv ? dest : n0 + tid);
-            up[0] = v0;
-            up[(size_t)nb * N] = v1;
-        }
-    }
-}
-
-cudaError_t launch_key_inner_product(const RingHost& ring, const RotBatch& rb, const u64* dig, const u64* keys, u64* u,
-                                     int* error_flag, cudaStream_t stream, u64* xext, const u32* pinv) {
-    if (rb.n == 0) return cudaSuccess;
-    ProfScope prof(ring.prof, CAT_KEY_INNER, stream);
-    const u32 r = ring.dev.r;
-    if (ring.prof) {
-        const u64 key_bytes = (u64)r * 2 * (r + 1) * ring.dev.N * 8;
-        u32 distinct = 0;
-        for (int t = 0; t < rb.n; ++t) {
-            bool seen = false;
-            for (int k = 0; k < t && !seen; ++k) seen = rb.key[k] == rb.key[t];
-            distinct += seen ? 0u : 1u;
-        }
-        ring.prof->key_bytes_distinct += distinct * key_bytes;
-        ring.prof->key_bytes_per_rotation += (u64)rb.n * key_bytes;
-    }
-    const size_t smem = (size_t)4 * r * KI_TILE * 8 + 32;
-    // runs of consecutive rotations with the same key: one block per run, tile and modulus
-    RotBatch rbg = rb;
-    rbg.n_groups = 0;
-    for (int t = 0; t < rb.n; ++t) {
-        if (t > 0 && rb.key[t] == rb.key[t - 1]) {
-            rbg.grp_cnt[rbg.n_groups - 1]++;
-        } else {
-            rbg.grp_first[rbg.n_groups] = (unsigned char)t;
-            rbg.grp_cnt[rbg.n_groups] = 1;
-            rbg.n_groups++;
-        }
-    }
-    static bool attr_set[MAX_DEVICES] = {false};     // per device: the attribute belongs to the device's copy of the kernel
-    if (!attr_set[device_slot(ring)]) {
-        cudaError_t e = cudaFuncSetAttribute(key_inner_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_set[device_slot(ring)] = true;
-    }
-    dim3 grid(rbg.n_groups, ring.dev.N / KI_TILE, r + 1);
-    return launch_dependent(ring, key_inner_bulk_kernel, grid, dim3(KI_TILE), smem, stream, ring.dev, rbg, dig, keys, u,
-                            error_flag, xext, pinv);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -30,15 +30,6 @@ __device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
     return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
 }
 
-// words that are read exactly once: not kept in L1, first to leave L2
-__device__ __forceinline__ u64 stream_policy() {
-    u64 pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void ld_stream(const void* p, u64 policy, u32& lo, u32& hi) {
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;" : "=r"(lo), "=r"(hi) : "l"(p), "l"(policy));
-}
 __device__ __forceinline__ u32 ld_stream32(const void* p, u64 policy) {
     u32 v;
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));

@@ -8,10 +8,11 @@
 //
 // A transform of N = R*C points runs as two launches.  The strided pass transforms the R rows
 // (stride C) of a tile of adjacent columns; the contiguous pass transforms chunks of C adjacent
-// points.  Inside a pass every thread keeps a closed set of 4 or 8 points in registers for two or
-// three butterfly stages, and sets are exchanged through shared memory between stage groups.
-// Butterflies use Harvey's lazy reduction: forward values stay in [0, 4q), inverse in [0, 2q).
+// points.  Inside a pass every thread keeps a closed set of up to 16 points in registers for up to
+// four butterfly stages, and sets are exchanged through shared memory between stage groups.
 #include "bf_host.h"
+
+#include <type_traits>
 
 namespace bf {
 
@@ -49,13 +50,15 @@ struct LoadConsts {
     bool wide;          // target prime of 2^41 or more: values must stay in [0, 4q); otherwise they are signed
     bool src_small;     // LOAD_REDUCE: every source word is below 1.5 q already (block-uniform)
     bool src_fp;        // LOAD_REDUCE: every source word is below 2^51
+    bool staged_fp;     // LOAD_REDUCE: the source holds the bits of integer-valued doubles
 };
 
 template <int LOAD>
 __device__ __forceinline__ u64 load_src(const void* src, size_t idx, const LoadConsts& c) {
     if (LOAD == LOAD_PLAIN) return ((const u64*)src)[idx];
     if (LOAD == LOAD_REDUCE) {
-        const u64 t = ((const u64*)src)[idx];
+        u64 t = ((const u64*)src)[idx];
+        if (c.staged_fp) t = d2u(__longlong_as_double((long long)t));
         return c.src_small ? (t >= c.q ? t - c.q : t) : barrett64(t, c.q, c.mu);
     }
     if (LOAD == LOAD_I64 || LOAD == LOAD_I64_MONT) {
@@ -81,9 +84,10 @@ template <int LOAD>
 __device__ __forceinline__ double load_src_fp(const void* src, size_t idx, const LoadConsts& c) {
     if (LOAD == LOAD_REDUCE) {
         const u64 t = ((const u64*)src)[idx];
-        if (c.src_small) return u2d(t);
+        const double td = c.staged_fp ? __longlong_as_double((long long)t) : u2d(t);
+        if (c.src_small) return td;
         if (c.src_fp) {                                  // t - round(t / q) q, plus q where values must not be negative
-            const double v = fp_centre(u2d(t), c.qd, c.qinv);
+            const double v = fp_centre(td, c.qd, c.qinv);
             return c.wide ? __dadd_rn(v, c.qd) : v;
         }
         return u2d(barrett64(t, c.q, c.mu));
@@ -106,133 +110,164 @@ __device__ __forceinline__ double load_src_fp(const void* src, size_t idx, const
     return u2d(load_src<LOAD>(src, idx, c));
 }
 
-// Butterflies of one register-resident set of 2^K points over K consecutive stages.
-// tw_base = (blocks at the group's first forward stage) * mult, so that stage st, sub-block sub
-// uses twiddle (tw_base << st) + (blk << st) + sub.
-// Integer version: Harvey's lazy butterflies with Shoup products; forward values stay in [0, 4q),
-// inverse values in [0, 2q).
-// Twiddle (and companion) number idx: from the global table through the read-only path, or from a copy of
-// the table's head that the block staged in shared memory.
-template <bool TWSM>
-__device__ __forceinline__ ulonglong2 tw_fetch(const ulonglong2* tw, u32 idx) {
-    if (TWSM) return tw[idx];
-    return __ldg(&tw[idx]);
-}
-
-template <int K, bool FWD, bool TWSM = false>
-__device__ __forceinline__ void set_butterflies(u64 (&e)[8], const ulonglong2* __restrict__ tw, u32 tw_base, u32 blk,
-                                                u64 q, double) {
-    const u64 q2 = 2 * q;
-#pragma unroll
-    for (int s = 0; s < K; ++s) {
-        const int st = FWD ? s : (K - 1 - s);
-        const int d = (1 << K) >> (st + 1);
-#pragma unroll
-        for (int sub = 0; sub < (1 << st); ++sub) {
-            const ulonglong2 w = tw_fetch<TWSM>(tw, (tw_base << st) + (blk << st) + sub);
-#pragma unroll
-            for (int off = 0; off < d; ++off) {
-                const int i = sub * 2 * d + off;
-                if (FWD) {
-                    u64 x = e[i];
-                    if (x >= q2) x -= q2;
-                    u64 t = mul_shoup_lazy(e[i + d], w.x, w.y, q);
-                    e[i] = x + t;
-                    e[i + d] = x - t + q2;
-                } else {
-                    u64 a = e[i], b = e[i + d];
-                    u64 s2 = a + b;
-                    if (s2 >= q2) s2 -= q2;
-                    e[i] = s2;
-                    e[i + d] = mul_shoup_lazy(a - b + q2, w.x, w.y, q);
-                }
-            }
-        }
-    }
-}
-
-// fp64 version.  Primes below 2^41: values are signed integer-valued doubles, reduced lazily.
-//   Forward: (X, Y) -> (X + s, X - s), s = Y*w centred in (-0.54q, 0.54q): magnitudes grow by at most 0.54q
-//   per stage, from at most 3.6q after the load functors to below 13q after log2 N <= 16 stages; one
-//   reduction at the very end.
-//   Inverse: (a, b) -> (a + b, (a - b)*w centred): the sums double per stage and the product takes
-//   |a - b| < 2^47, i.e. magnitudes below 32q going into a stage.  From [0, q) the contiguous pass runs its
-//   first two groups (5 stages, sums up to 32q), centres the sums, and leaves at most 4.4q after its last
-//   group; the strided pass centres the sums after its first group when more groups follow, which keeps
-//   every later stage below 18q going in and the values handed to the final scaling below 35q.
-// WIDE (primes from 2^41 up to 2^50): the centred product lies in (-0.75q, 0.75q) and values must stay below
-// 4q < 2^52, so the forward butterfly keeps Harvey's invariant [0, 4q) with one conditional subtraction:
-// (X, Y) -> (X~ + T, X~ - T + 2q), X~ = X reduced below 2q, T = Y*w + q in (0.25q, 1.75q); the inverse is
-// (a, b) -> (a + b reduced below 2q, (a - b + 2q)*w + q in (0.25q, 1.75q)): values in [0, 2q).
-template <int K, bool FWD, bool WIDE, bool TWSM>
-__device__ __forceinline__ void set_butterflies_fp(double (&e)[8], const ulonglong2* __restrict__ tw, u32 tw_base,
-                                                   u32 blk, double q) {
-    const double q2 = __dadd_rn(q, q);
-#pragma unroll
-    for (int s = 0; s < K; ++s) {
-        const int st = FWD ? s : (K - 1 - s);
-        const int d = (1 << K) >> (st + 1);
-#pragma unroll
-        for (int sub = 0; sub < (1 << st); ++sub) {
-            const ulonglong2 wb = tw_fetch<TWSM>(tw, (tw_base << st) + (blk << st) + sub);
-            const double w = __longlong_as_double((long long)wb.x), wq = __longlong_as_double((long long)wb.y);
-#pragma unroll
-            for (int off = 0; off < d; ++off) {
-                const int i = sub * 2 * d + off;
-                if (FWD && WIDE) {
-                    double x = e[i];
-                    if (x >= q2) x = __dsub_rn(x, q2);
-                    const double t = __dadd_rn(fp_mul_centred(e[i + d], w, wq, q), q);
-                    e[i] = __dadd_rn(x, t);
-                    e[i + d] = __dadd_rn(__dsub_rn(x, t), q2);
-                } else if (FWD) {
-                    const double sv = fp_mul_centred_signed(e[i + d], w, wq, q);
-                    const double x = e[i];
-                    e[i] = __dadd_rn(x, sv);
-                    e[i + d] = __dsub_rn(x, sv);
-                } else if (WIDE) {
-                    const double a = e[i], b = e[i + d];
-                    double s2 = __dadd_rn(a, b);
-                    if (s2 >= q2) s2 = __dsub_rn(s2, q2);
-                    e[i] = s2;
-                    e[i + d] = __dadd_rn(fp_mul_centred(__dadd_rn(__dsub_rn(a, b), q2), w, wq, q), q);
-                } else {
-                    const double a = e[i], b = e[i + d];
-                    e[i] = __dadd_rn(a, b);
-                    e[i + d] = fp_mul_centred_signed(__dsub_rn(a, b), w, wq, q);
-                }
-            }
-        }
-    }
-}
-
-template <int K, bool FWD, bool TWSM = false>
-__device__ __forceinline__ void set_butterflies(double (&e)[8], const ulonglong2* __restrict__ tw, u32 tw_base,
-                                                u32 blk, u64 q_int, double q) {
-    if (q_int >> 41) set_butterflies_fp<K, FWD, true, TWSM>(e, tw, tw_base, blk, q);    // block-uniform
-    else set_butterflies_fp<K, FWD, false, TWSM>(e, tw, tw_base, blk, q);
-}
-
-// After an inverse group of K stages the first 2^(K-1) values of a set are sums (they doubled per stage),
-// the others fresh centred products: bring the sums back to |v| <= q/2.  Signed fp64 path only.
-template <int K>
-__device__ __forceinline__ void centre_sums(double (&e)[8], u64 q_int, double q, double qinv) {
-    if (q_int >> 41) return;
-#pragma unroll
-    for (int i = 0; i < (1 << K) / 2; ++i) e[i] = fp_centre(e[i], q, qinv);
-}
-template <int K>
-__device__ __forceinline__ void centre_sums(u64 (&)[8], u64, double, double) {}
-
-template <bool FP> struct Elem { typedef u64 T; };
-template <> struct Elem<true> { typedef double T; };
+// How a modulus is transformed.
+//   PATH_DP    primes below 2^41: signed integer-valued doubles, reduced lazily
+//   PATH_WIDE  primes from 2^41 up to 2^50: integer-valued doubles in [0, 4q) (forward) or [0, 2q) (inverse)
+//   PATH_INT   larger primes: 64-bit integers, Harvey's lazy butterflies with Shoup products, the same ranges
+enum Path : int { PATH_INT = 0, PATH_WIDE = 1, PATH_DP = 2 };
+__device__ __forceinline__ int path_of(const RingDev& R, u32 mod) { return !R.fp_ok[mod] ? PATH_INT : (R.q[mod] >> 41) ? PATH_WIDE : PATH_DP; }
+template <int PATH> struct Elem { typedef double T; };
+template <> struct Elem<PATH_INT> { typedef u64 T; };
 __device__ __forceinline__ void from_u64(u64& dst, u64 v) { dst = v; }
 __device__ __forceinline__ void from_u64(double& dst, u64 v) { dst = u2d(v); }
 
-// Stage groups of a local transform of 2^LOG_LEN points, in forward order.
+struct ModConsts {
+    u64 q;
+    double qd, qinv;
+};
+
+// 32 bytes at once (the widest global access of sm_100)
+__device__ __forceinline__ void ldg4(const double* p, double& a, double& b, double& c, double& d) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
+}
+__device__ __forceinline__ void stg4(u64* p, u64 a, u64 b, u64 c, u64 d) {
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+
+// The 2^ST twiddles of one stage of a register-resident set: entries idx .. idx + 2^ST - 1 (idx a multiple of 2^ST) of the
+// prime's table.  PATH_DP reads a table of plain doubles (half the bytes of the other paths' (w, companion) pairs: the
+// transforms are limited by what passes through L1 as much as by arithmetic) and makes w / q with one multiplication,
+// within 2^-52 relative.  SM: the table is a copy in shared memory.
+template <int ST, bool SM>
+__device__ __forceinline__ void load_twiddles(const double* tab, u32 idx, double (&w)[1 << ST]) {
+    const double* p = tab + idx;
+    if constexpr (ST == 0) {
+        w[0] = SM ? *p : __ldg(p);
+    } else if constexpr (ST == 1 || SM) {
+#pragma unroll
+        for (int i = 0; i < (1 << ST); i += 2) {
+            const double2 v = SM ? *(const double2*)(p + i) : __ldg((const double2*)(p + i));
+            w[i] = v.x;
+            w[i + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < (1 << ST); i += 4) ldg4(p + i, w[i], w[i + 1], w[i + 2], w[i + 3]);
+    }
+}
+
+// Butterflies of one register-resident set of 2^K points (e[OFF ..]) over K consecutive stages.  base = (blocks at the
+// group's first forward stage) + the set's block: stage st, sub-block sub uses twiddle (base << st) + sub.
+//
+// PATH_DP forward: (X, Y) -> (X + s, X - s), s = Y*w centred in (-0.54q, 0.54q): magnitudes grow by at most 0.54q per
+// stage, from at most 3.6q after the load functors to below 13q after log2 N <= 16 stages; one reduction at the very
+// end.  Inverse: (a, b) -> (a + b, (a - b)*w centred): the sums double per stage, the product takes |a - b| < 2^47, i.e.
+// magnitudes below 32q; see centre_sums.
+// PATH_WIDE: the centred product lies in (-0.75q, 0.75q) and values must stay below 4q < 2^52, so the forward butterfly
+// keeps Harvey's invariant [0, 4q) with one conditional subtraction: (X, Y) -> (X~ + T, X~ - T + 2q), X~ = X reduced
+// below 2q, T = Y*w + q in (0.25q, 1.75q); the inverse is (a, b) -> (a + b reduced below 2q, (a - b + 2q)*w + q in
+// (0.25q, 1.75q)): values in [0, 2q).
+template <int ST, int K, bool FWD, int PATH, bool SM, int OFF, typename T>
+__device__ __forceinline__ void stage_butterflies(T (&e)[8], const void* __restrict__ tab, u32 base, const ModConsts& c) {
+    constexpr int d = (1 << K) >> (ST + 1);
+    const u32 idx = base << ST;
+    if constexpr (PATH == PATH_DP) {
+        double w[1 << ST];
+        load_twiddles<ST, SM>((const double*)tab, idx, w);
+#pragma unroll
+        for (int sub = 0; sub < (1 << ST); ++sub) {
+            const double wq = __dmul_rn(w[sub], c.qinv);
+#pragma unroll
+            for (int off = 0; off < d; ++off) {
+                const int i = OFF + sub * 2 * d + off;
+                if (FWD) {
+                    const double sv = fp_mul_centred_signed(e[i + d], w[sub], wq, c.qd);
+                    const double x = e[i];
+                    e[i] = __dadd_rn(x, sv);
+                    e[i + d] = __dsub_rn(x, sv);
+                } else {
+                    const double a = e[i], b = e[i + d];
+                    e[i] = __dadd_rn(a, b);
+                    e[i + d] = fp_mul_centred_signed(__dsub_rn(a, b), w[sub], wq, c.qd);
+                }
+            }
+        }
+    } else {
+        const double q2d = __dadd_rn(c.qd, c.qd);
+        const u64 q = c.q, q2 = 2 * c.q;
+#pragma unroll
+        for (int sub = 0; sub < (1 << ST); ++sub) {
+            const ulonglong2 wb = SM ? ((const ulonglong2*)tab)[idx + sub] : __ldg((const ulonglong2*)tab + idx + sub);
+#pragma unroll
+            for (int off = 0; off < d; ++off) {
+                const int i = OFF + sub * 2 * d + off;
+                if constexpr (PATH == PATH_WIDE) {
+                    const double w = __longlong_as_double((long long)wb.x), wq = __longlong_as_double((long long)wb.y);
+                    if (FWD) {
+                        double x = e[i];
+                        if (x >= q2d) x = __dsub_rn(x, q2d);
+                        const double t = __dadd_rn(fp_mul_centred(e[i + d], w, wq, c.qd), c.qd);
+                        e[i] = __dadd_rn(x, t);
+                        e[i + d] = __dadd_rn(__dsub_rn(x, t), q2d);
+                    } else {
+                        const double a = e[i], b = e[i + d];
+                        double s2 = __dadd_rn(a, b);
+                        if (s2 >= q2d) s2 = __dsub_rn(s2, q2d);
+                        e[i] = s2;
+                        e[i + d] = __dadd_rn(fp_mul_centred(__dadd_rn(__dsub_rn(a, b), q2d), w, wq, c.qd), c.qd);
+                    }
+                } else if (FWD) {
+                    u64 x = e[i];
+                    if (x >= q2) x -= q2;
+                    const u64 t = mul_shoup_lazy(e[i + d], wb.x, wb.y, q);
+                    e[i] = x + t;
+                    e[i + d] = x - t + q2;
+                } else {
+                    const u64 a = e[i], b = e[i + d];
+                    u64 s2 = a + b;
+                    if (s2 >= q2) s2 -= q2;
+                    e[i] = s2;
+                    e[i + d] = mul_shoup_lazy(a - b + q2, wb.x, wb.y, q);
+                }
+            }
+        }
+    }
+}
+template <int K, bool FWD, int PATH, bool SM, int OFF = 0, typename T>
+__device__ __forceinline__ void set_butterflies(T (&e)[8], const void* __restrict__ tab, u32 base, const ModConsts& c) {
+    if constexpr (FWD) {
+        stage_butterflies<0, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+        if constexpr (K > 1) stage_butterflies<1, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+        if constexpr (K > 2) stage_butterflies<2, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+    } else {
+        if constexpr (K > 2) stage_butterflies<2, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+        if constexpr (K > 1) stage_butterflies<1, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+        stage_butterflies<0, K, FWD, PATH, SM, OFF>(e, tab, base, c);
+    }
+}
+// After an inverse group the points that were sums to the end have grown: point 0 by 2^K, point 1 to 2^(K-1) fresh
+// products (0.54q each), point 2 and 3 to 2^(K-2) of them, and so on.  Centring point 0 leaves every point within 2.2q, so
+// that a group of at most three stages starts below 2.2q and stays below 18q < 2^47.
+template <int K, int PATH, int OFF = 0, typename T>
+__device__ __forceinline__ void centre_sums(T (&e)[8], const ModConsts& c) {
+    if constexpr (PATH == PATH_DP) {
+        e[OFF] = fp_centre(e[OFF], c.qd, c.qinv);
+    }
+}
+
+constexpr int LOG_C = 8;              // contiguous pass: chunks of 256 points
+
+// Between the two passes of a transform the data sit in dst as lazily reduced values: 64-bit
+// integers for the integer path, fp64 bit patterns for the fp64 path (the modulus decides, so both
+// passes agree).
+
+// Geometry of the strided pass over 2^LOG_R rows (stride 256) of 2^LOG_LANES adjacent columns: up to three groups of at most
+// three stages, eight points a thread.  (Sixteen points and two groups execute a sixth fewer instructions, but half the
+// threads hide less latency and the integer path's blocks, which every launch waits for, take twice as long: the four calls
+// of a 0.6B decoder layer took 8 % longer.)
 __host__ __device__ constexpr int n_groups(int log_len) { return log_len <= 3 ? 1 : (log_len <= 6 ? 2 : 3); }
 __host__ __device__ constexpr int group_k(int log_len, int gi) {
-    // 1:{1} 2:{2} 3:{3} 4:{2,2} 5:{3,2} 6:{3,3} 7:{3,2,2} 8:{3,3,2}
+    // 2:{2} 3:{3} 4:{2,2} 5:{3,2} 6:{3,3} 7:{3,2,2} 8:{3,3,2}
     return log_len <= 3 ? log_len
          : log_len == 4 ? 2
          : log_len == 5 ? (gi == 0 ? 3 : 2)
@@ -245,6 +280,339 @@ __host__ __device__ constexpr int group_log_step(int log_len, int gi) {
     int done = 0;
     for (int i = 0; i <= gi; ++i) done += group_k(log_len, i);
     return log_len - done;
+}
+template <int LOG_R, int LOG_LANES>
+struct StridedGeo {
+    static constexpr int LEN = 1 << LOG_R, LANES = 1 << LOG_LANES, POINTS = LEN * LANES;
+    static constexpr int NT = POINTS / 8 < 32 ? 32 : POINTS / 8;
+    static constexpr int BLOCKS = NT >= 512 ? 2 : NT >= 256 ? 4 : 8;       // resident blocks per SM
+    static constexpr int TILES = (1 << LOG_C) / LANES;
+    static constexpr int TW_WORDS = 2 * LEN;                               // (w, companion) pairs, or half of it
+};
+
+__device__ __forceinline__ const void* twiddle_table(const RingDev& R, bool fwd, int path, u32 mod) {
+    return path == PATH_DP ? (const void*)((fwd ? R.tw8_fwd : R.tw8_inv) + (size_t)mod * R.N)
+                           : (const void*)((fwd ? R.tw_fwd : R.tw_inv) + (size_t)mod * R.N);
+}
+
+// A thread's share of the first 2^LOG_R twiddles of a prime, fetched early and put into shared memory later.
+template <int LOG_R>
+struct StridedTwiddles {
+    ulonglong2 mine;
+    __device__ __forceinline__ void fetch(const RingDev& R, bool fwd, int path, u32 mod) {
+        mine = make_ulonglong2(0, 0);
+        if (threadIdx.x < (1 << LOG_R)) {
+            const void* tab = twiddle_table(R, fwd, path, mod);
+            if (path == PATH_DP) mine.x = __ldg((const u64*)tab + threadIdx.x);
+            else mine = __ldg((const ulonglong2*)tab + threadIdx.x);
+        }
+    }
+    __device__ __forceinline__ void put(u64* tws, int path) const {
+        if (threadIdx.x < (1 << LOG_R)) {
+            if (path == PATH_DP) tws[threadIdx.x] = mine.x;
+            else ((ulonglong2*)tws)[threadIdx.x] = mine;
+        }
+    }
+};
+
+template <int LOAD>
+__device__ __forceinline__ LoadConsts load_consts(const RingDev& R, const PolyBatch& B, u32 o, u32 mod) {
+    LoadConsts lc;
+    const u64 q = R.q[mod], mu = R.mu[mod];
+    lc.q = q;
+    lc.mu = mu;
+    lc.lift_red = (LOAD == LOAD_CENTRED) ? barrett64(B.lift_mod, q, mu) : (LOAD == LOAD_I64_MONT) ? R.c64s[mod] : 0;
+    lc.lift_mod = (LOAD == LOAD_I64_MONT) ? R.c64[mod] : B.lift_mod;
+    lc.qd = R.qd[mod];
+    lc.qinv = R.qinv_d[mod];
+    lc.c30 = R.c30_d[mod];
+    lc.c30q = R.c30_q[mod];
+    lc.c64d = lc.c64q = 0.0;
+    lc.wide = (q >> 41) != 0;
+    // wide: 2q - (2^59 mod q) keeps the lifted value positive; otherwise the offset is just -(2^59 mod q)
+    lc.k59 = lc.wide ? R.k59_d[mod] : __dsub_rn(R.k59_d[mod], __dadd_rn(lc.qd, lc.qd));
+    if (LOAD == LOAD_I64_MONT) {
+        const double* ec = R.enc_consts + (size_t)mod * ENC_CONSTS;
+        lc.c30 = __ldg(ec);
+        lc.c30q = __ldg(ec + 1);
+        lc.c64d = __ldg(ec + 2);
+        lc.c64q = __ldg(ec + 3);
+        lc.k59 = __ldg(ec + 4);
+    }
+    u64 qs = ~(u64)0;
+    if (LOAD == LOAD_REDUCE && B.src_digits) {      // the prime the source digit belongs to
+        u32 s_hi, s_lo;
+        split_index(o, R.r, B.o_div == R.r ? B.o_div_magic : 0u, s_hi, s_lo);
+        qs = R.q[s_lo];
+    }
+    lc.src_small = qs <= q + (q >> 1);
+    lc.src_fp = qs < (1ull << 51);
+    lc.staged_fp = false;
+    return lc;
+}
+
+// Row `row` of the exchange buffer of a strided tile.  Tiles of 8 columns (64 bytes a row) swap the rows of a pair by bit 2
+// of the row number, so that the two rows a half-warp reads never share banks, whether they are neighbours or 4 apart.
+template <int LOG_LANES>
+__device__ __forceinline__ int exchange_row(int row) { return LOG_LANES == 3 ? row ^ ((row >> 2) & 1) : row; }
+
+// Strided pass: transforms the 2^LOG_R rows (stride 256) of a tile of adjacent columns.  Forward: first pass (reads the
+// batch source through the load functor, or from `staged`, [row][column], where several target primes of the same block
+// read it).  Inverse: second pass (in place, scales by N^{-1}).  tws: the prime's first 2^LOG_R twiddles, in shared memory.
+template <bool FWD, int LOAD, int LOG_R, int LOG_LANES, int PATH, bool STAGED = false>
+__device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u64* tws, u32 o,
+                                             u32 m, u32 mod, u32 tile, const LoadConsts& lc, const u64* staged,
+                                             const StridedTwiddles<LOG_R>& tw) {
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
+    typedef typename Elem<PATH>::T T;
+    constexpr int LEN = G::LEN, LANES = G::LANES, NT = G::NT, NG = n_groups(LOG_R);
+    T* sm = (T*)sm_raw;
+    ModConsts c;
+    c.q = R.q[mod];
+    c.qd = R.qd[mod];
+    c.qinv = R.qinv_d[mod];
+    u64* dst = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm + tile * LANES;
+    const char* src = nullptr;
+    if constexpr (FWD && !STAGED) {
+        u32 o_hi = 0, o_lo = o;
+        if (B.o_div) split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
+        const size_t src_off = B.o_div ? (size_t)o_hi * B.src_so2 + (size_t)o_lo * B.src_so : (size_t)o * B.src_so;
+        src = (const char*)B.src + (src_off + (size_t)m * B.src_sm + tile * LANES) * 8;
+    }
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int gi = 0; gi < NG; ++gi) {
+        const int fg = FWD ? gi : NG - 1 - gi;                 // group index in forward order
+        const int K = group_k(LOG_R, fg);
+        const int log_step = group_log_step(LOG_R, fg), step = 1 << log_step;
+        const u32 base0 = (u32)(LEN >> (log_step + K));        // blocks at the group's first forward stage
+        const int nsets = (LEN * LANES) >> K;
+        const bool g_first = (gi == 0), g_last = (gi == NG - 1);
+#pragma unroll
+        for (int w0 = 0; w0 < nsets; w0 += NT) {
+            const int w = w0 + tid;
+            if (NT > nsets && w >= nsets) break;
+            const int lane = w & (LANES - 1), u = w >> LOG_LANES;
+            const int blk = u >> log_step, off = u & (step - 1);
+            const int base = (blk << (log_step + K)) + off;
+            T e[8];
+#pragma unroll
+            for (int i = 0; i < (1 << K); ++i) {
+                const int row = base + i * step;
+                if (g_first) {
+                    const size_t gidx = ((size_t)row << LOG_C) + lane;
+                    if (FWD) {
+                        const void* from = STAGED ? (const void*)staged : (const void*)src;
+                        const size_t at = STAGED ? (size_t)(row * LANES + lane) : gidx;
+                        if constexpr (PATH != PATH_INT) e[i] = load_src_fp<LOAD>(from, at, lc);
+                        else e[i] = load_src<LOAD>(from, at, lc);
+                    } else {
+                        e[i] = ((const T*)dst)[gidx];
+                    }
+                } else {
+                    e[i] = sm[exchange_row<LOG_LANES>(row) * LANES + lane];
+                }
+            }
+            if (!STAGED && g_first && w0 == 0) {    // (the first sweep of the first group is full for every geometry)
+                static_assert(NT <= (G::POINTS >> group_k(LOG_R, FWD ? 0 : NG - 1)), "first sweep must be full");
+                tw.put(tws, PATH);
+                __syncthreads();
+            }
+            if (K == 3) set_butterflies<3, FWD, PATH, true>(e, tws, base0 + blk, c);
+            else if (K == 2) set_butterflies<2, FWD, PATH, true>(e, tws, base0 + blk, c);
+            else set_butterflies<1, FWD, PATH, true>(e, tws, base0 + blk, c);
+            if (!FWD && !g_last) centre_sums<1, PATH>(e, c);
+#pragma unroll
+            for (int i = 0; i < (1 << K); ++i) {
+                const int row = base + i * step;
+                if (g_last) {
+                    const size_t gidx = ((size_t)row << LOG_C) + lane;
+                    if (FWD) {
+                        ((T*)dst)[gidx] = e[i];                 // lazy; the contiguous pass finishes
+                    } else {                                    // scale by N^{-1}, to [0, q)
+                        const bool mont = B.from_mont != 0;
+                        u64 out;
+                        if constexpr (PATH != PATH_INT) {
+                            const double nv = mont ? R.ninvm_d[mod] : R.ninv_d[mod];
+                            const double nq = mont ? R.ninvm_q[mod] : R.ninv_q[mod];
+                            double v;
+                            if (PATH == PATH_WIDE) {
+                                v = __dadd_rn(fp_mul_centred(e[i], nv, nq, c.qd), c.qd);
+                                if (v >= c.qd) v = __dsub_rn(v, c.qd);
+                                if (v >= c.qd) v = __dsub_rn(v, c.qd);  // (the product can touch 2q for the 50-bit prime)
+                            } else {
+                                v = fp_mul_centred_signed(e[i], nv, nq, c.qd);
+                                if (v < 0.0) v = __dadd_rn(v, c.qd);
+                            }
+                            out = d2u(v);
+                        } else {
+                            out = mul_shoup(e[i], mont ? R.ninv_m[mod] : R.ninv[mod], mont ? R.ninv_ms[mod] : R.ninvs[mod], c.q);
+                        }
+                        if (B.store_centred == 1 || (B.store_centred == 2 && mod == R.r))
+                            out = (out > (c.q - 1) / 2 ? out - c.q : out) + (1ull << 59);
+                        dst[gidx] = out;
+                    }
+                } else {
+                    sm[exchange_row<LOG_LANES>(row) * LANES + lane] = e[i];
+                }
+            }
+        }
+        if (!g_last) __syncthreads();
+    }
+}
+
+// Blocks are dealt out in grid order: the last slot (the special prime, where a batch has it, on the long integer path) goes
+// first, so that nothing waits for its blocks at the end of the launch.
+__device__ __forceinline__ u32 slot_of_block(u32 y, u32 n_m) { return n_m - 1 - y; }
+// modulus index of slot m of a batch (n_m <= 2 * mod_wrap in every batch that wraps)
+__device__ __forceinline__ u32 batch_modulus(const PolyBatch& B, u32 m) {
+    return B.mod0 + ((B.mod_wrap && m >= B.mod_wrap) ? m - B.mod_wrap : m) * B.mod_step;
+}
+// a digit in its own prime (o = set * r + digit with digit == mod), which ModUp copies instead of transforming
+__device__ __forceinline__ bool own_prime(const RingDev& R, const PolyBatch& B, u32 o, u32 mod) {
+    if (!B.skip_diag || mod >= R.r) return false;
+    u32 hi, lo;
+    split_index(o, R.r, B.o_div == R.r ? B.o_div_magic : 0u, hi, lo);
+    return lo == mod;
+}
+
+// a residue in the form the inner products read (see RingDev::dp)
+__device__ __forceinline__ u64 operand_word(const RingDev& R, u32 mod, u64 v) {
+    return R.dp[mod] ? (u64)__double_as_longlong(u2d(v)) : v;
+}
+
+// the tile of a digit in its own prime: its transform exists already and is copied into the operand array
+template <int LOG_R, int LOG_LANES>
+__device__ __forceinline__ void copy_own_digit(const RingDev& R, const PolyBatch& B, u32 o, u32 m, u32 mod, u32 tile) {
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
+    const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
+    u32 t_hi, t_lo;
+    split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
+    const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
+#pragma unroll 4
+    for (int k = 0; k < G::POINTS / G::NT; ++k) {
+        const int w = threadIdx.x + k * G::NT;
+        const size_t gidx = ((size_t)(w / G::LANES) << LOG_C) + tile * G::LANES + w % G::LANES;
+        B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
+    }
+}
+
+// grid: x = tile, y = slot m, z = outer index.
+template <bool FWD, int LOAD, int LOG_R, int LOG_LANES>
+__global__ void __launch_bounds__(StridedGeo<LOG_R, LOG_LANES>::NT, StridedGeo<LOG_R, LOG_LANES>::BLOCKS)
+ntt_strided(const RingDev R, const PolyBatch B, u32 n_outer) {
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
+    __shared__ __align__(16) u64 sm[n_groups(LOG_R) > 1 ? G::POINTS : 1];
+    __shared__ __align__(16) u64 tws[G::TW_WORDS];
+    grid_dependency_enter();
+    const u32 m = slot_of_block(blockIdx.y, B.n_m), mod = batch_modulus(B, m);
+    const int path = path_of(R, mod);
+    StridedTwiddles<LOG_R> tw;
+    tw.fetch(R, FWD, path, mod);
+    for (u32 o = blockIdx.z; o < n_outer; o += gridDim.z) {
+        if (FWD && own_prime(R, B, o, mod)) {
+            if (B.dtile_ptr) copy_own_digit<LOG_R, LOG_LANES>(R, B, o, m, mod, blockIdx.x);
+            continue;
+        }
+        const LoadConsts lc = load_consts<LOAD>(R, B, o, mod);
+        if (path == PATH_DP) strided_body<FWD, LOAD, LOG_R, LOG_LANES, PATH_DP>(R, B, sm, tws, o, m, mod, blockIdx.x, lc, nullptr, tw);
+        else if (path == PATH_WIDE) strided_body<FWD, LOAD, LOG_R, LOG_LANES, PATH_WIDE>(R, B, sm, tws, o, m, mod, blockIdx.x, lc, nullptr, tw);
+        else strided_body<FWD, LOAD, LOG_R, LOG_LANES, PATH_INT>(R, B, sm, tws, o, m, mod, blockIdx.x, lc, nullptr, tw);
+        if (o + gridDim.z < n_outer) __syncthreads();
+    }
+}
+
+// Forward strided pass of a batch whose n_m target primes all read the same source polynomial (ModUp digits,
+// the P-residues of ModDown): a block stages the source tile in shared memory once and transforms it
+// into targets m_begin .. m_begin + m_count - 1, so the source crosses L2 once per block instead of once per
+// target (and a digit is made, or converted to fp64, once).  grid: x = tile, y = outer index o, z = slice of the targets.
+template <int LOAD, int LOG_R, int LOG_LANES>
+__global__ void __launch_bounds__(StridedGeo<LOG_R, LOG_LANES>::NT, StridedGeo<LOG_R, LOG_LANES>::BLOCKS)
+ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
+    constexpr int LANES = G::LANES, POINTS = G::POINTS, NT = G::NT;
+    extern __shared__ __align__(16) u64 shared_src_smem[];
+    u64* staged = shared_src_smem;                  // [POINTS] source: doubles where staged_fp, else raw words
+    u64* sm = shared_src_smem + POINTS;             // [POINTS] exchange between stage groups
+    u64* tws = sm + POINTS;                         // [2][TW_WORDS] twiddles of the current and the next target
+    grid_dependency_enter();
+    const u32 o = blockIdx.y, tile = blockIdx.x;
+    const u32 m_begin = slot_of_block(blockIdx.z, gridDim.z) * m_per_block;
+    const u32 m_end = min(B.n_m, m_begin + m_per_block);
+    StridedTwiddles<LOG_R> tw;
+    tw.fetch(R, true, path_of(R, batch_modulus(B, m_begin)), batch_modulus(B, m_begin));
+    u32 o_hi = 0, o_lo = o;
+    if (B.o_div) split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
+    // digits of primes on the fp64 path are staged as doubles
+    const bool staged_fp = LOAD == LOAD_REDUCE && B.src_digits && B.o_div == R.r && R.fp_ok[o_lo];
+    {
+        const size_t src_off = B.o_div ? (size_t)o_hi * B.src_so2 + (size_t)o_lo * B.src_so : (size_t)o * B.src_so;
+        const u64* src = (const u64*)B.src + src_off + tile * LANES;
+        auto at = [&](int w) { return ((size_t)(w / LANES) << LOG_C) + (w % LANES); };
+        if (B.div_t) {
+            // the digit is a division by P away: (source - t) * P^{-1} modulo the digit's own prime, t the centred lift
+            // of the polynomial's residue modulo P (exact: same value as dividing in the transform domain)
+            const u32 i = o_lo;
+            LoadConsts dc;
+            dc.q = R.q[i];
+            dc.mu = R.mu[i];
+            dc.lift_mod = R.q[R.r];
+            const u64* tp = B.div_t + (size_t)o_hi * B.div_so + tile * LANES;
+            if (R.fp_ok[i]) {
+                // in fp64 (every value an exact integer): t lazily reduced by the load functor, the difference times
+                // P^{-1} as a centred product, brought to [0, q) -- the digit must be the canonical residue, since it is
+                // reduced into the other primes next
+                const double qd = R.qd[i], pv = R.pinv_d[i], pq = R.pinv_q[i];
+                dc.qd = qd;
+                dc.c30 = R.c30_d[i];
+                dc.c30q = R.c30_q[i];
+                dc.wide = (dc.q >> 41) != 0;
+                dc.k59 = dc.wide ? R.k59_d[i] : __dsub_rn(R.k59_d[i], __dadd_rn(qd, qd));
+                const double q3 = __dadd_rn(__dadd_rn(qd, qd), qd);
+#pragma unroll 4
+                for (int k = 0; k < POINTS / NT; ++k) {
+                    const int w = threadIdx.x + k * NT;
+                    const double t = load_src_fp<LOAD_CENTRED>(tp, at(w), dc);     // (-1.75q, 0.76q), or (0.25q, 2.76q) when wide
+                    const double x = __dsub_rn(u2d(src[at(w)]), t);
+                    double s2 = dc.wide ? fp_mul_centred(__dadd_rn(x, q3), pv, pq, qd) : fp_mul_centred_signed(x, pv, pq, qd);
+                    if (s2 < 0.0) s2 = __dadd_rn(s2, qd);
+                    staged[w] = staged_fp ? (u64)__double_as_longlong(s2) : d2u(s2);
+                }
+            } else {
+                dc.lift_red = barrett64(dc.lift_mod, dc.q, dc.mu);
+                const u64 pinv = R.pinv[i], pinvs = R.pinvs[i];
+                for (int w = threadIdx.x; w < POINTS; w += NT) {
+                    const u64 t = load_src<LOAD_CENTRED>(tp, at(w), dc);
+                    staged[w] = mul_shoup(sub_mod(src[at(w)], t, dc.q), pinv, pinvs, dc.q);
+                }
+            }
+        } else {
+            u64 v[POINTS / NT];
+#pragma unroll
+            for (int k = 0; k < POINTS / NT; ++k) v[k] = src[at(threadIdx.x + k * NT)];
+#pragma unroll
+            for (int k = 0; k < POINTS / NT; ++k) staged[threadIdx.x + k * NT] = staged_fp ? (u64)__double_as_longlong(u2d(v[k])) : v[k];
+        }
+    }
+    u32 buf = 0;
+    for (u32 m = m_begin; m < m_end; ++m) {
+        const u32 mod = batch_modulus(B, m);
+        const int path = path_of(R, mod);
+        u64* tw_now = tws + buf * G::TW_WORDS;
+        tw.put(tw_now, path);
+        __syncthreads();            // (also: the source is staged, and the exchange buffer is free again)
+        if (m + 1 < m_end) tw.fetch(R, true, path_of(R, batch_modulus(B, m + 1)), batch_modulus(B, m + 1));
+        buf ^= 1;
+        if (own_prime(R, B, o, mod)) {
+            if (B.dtile_ptr) copy_own_digit<LOG_R, LOG_LANES>(R, B, o, m, mod, tile);
+            continue;
+        }
+        LoadConsts lc = load_consts<LOAD>(R, B, o, mod);
+        lc.staged_fp = staged_fp;
+        if (path == PATH_DP) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_DP, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+        else if (path == PATH_WIDE) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_WIDE, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+        else strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_INT, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+    }
 }
 
 // Shared-memory index swizzle for a 256-point chunk of 64-bit words: makes the three access
@@ -293,326 +661,72 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
     }
 }
 
-constexpr int LOG_C = 8;              // contiguous pass: chunks of 256 points, one warp each
-constexpr int CHUNKS_PER_BLOCK = 4;      // measured: 4 beats 8 by 4 % of the pass, 2 is no better
-
-// Between the two passes of a transform the data sit in dst as lazily reduced values: 64-bit
-// integers for the integer path, fp64 bit patterns for the fp64 path (the modulus decides, so both
-// passes agree).
-
-// Strided pass: transforms the 2^LOG_R rows (stride 256) of 2^LOG_LANES adjacent columns.
-// Forward: first pass (reads the batch source through the load functor).  Inverse: second pass
-// (in place, scales by N^{-1}).
-// STAGED: the source tile already sits in shared memory (`staged`, [row][lane], raw words) because several
-// target primes of the same block read it.
-template <bool FWD, int LOAD, int LOG_R, int LOG_LANES, bool FP, bool STAGED = false>
-__device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, ulonglong2* tws, u32 o,
-                                             u32 m, u32 mod, const u64* staged = nullptr) {
-    typedef typename Elem<FP>::T T;
-    constexpr int LEN = 1 << LOG_R, LANES = 1 << LOG_LANES;
-    constexpr int NT = (LEN * LANES / 8) < 32 ? 32 : (LEN * LANES / 8);
-    constexpr int NG = n_groups(LOG_R);
-    T* sm = (T*)sm_raw;
-    const u64 q = R.q[mod], mu = R.mu[mod];
-    const double qd = R.qd[mod];
-    // the strided pass uses the first LEN twiddles of the prime only: the block stages them in shared
-    // memory (the load is in flight together with the first data loads)
-    const ulonglong2* __restrict__ tw_global = (FWD ? R.tw_fwd : R.tw_inv) + (size_t)mod * R.N;
-    const ulonglong2* tw = tws;
-    ulonglong2 tw_mine = make_ulonglong2(0, 0);
-    if (threadIdx.x < LEN) tw_mine = __ldg(&tw_global[threadIdx.x]);
-    u64* dst = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
-    const char* src = nullptr;
-    if constexpr (!STAGED) {
-        u32 o_hi = 0, o_lo = o;
-        if (B.o_div) split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
-        const size_t src_off = B.o_div ? (size_t)o_hi * B.src_so2 + (size_t)o_lo * B.src_so : (size_t)o * B.src_so;
-        src = (const char*)B.src + (src_off + (size_t)m * B.src_sm) * 8;
-    }
-    LoadConsts lc;
-    lc.q = q;
-    lc.mu = mu;
-    lc.lift_red = (LOAD == LOAD_CENTRED) ? barrett64(B.lift_mod, q, mu) : (LOAD == LOAD_I64_MONT) ? R.c64s[mod] : 0;
-    lc.lift_mod = (LOAD == LOAD_I64_MONT) ? R.c64[mod] : B.lift_mod;
-    lc.qd = qd;
-    lc.qinv = R.qinv_d[mod];
-    lc.c30 = R.c30_d[mod];
-    lc.c30q = R.c30_q[mod];
-    lc.c64d = lc.c64q = 0.0;
-    lc.wide = (q >> 41) != 0;
-    // wide: 2q - (2^59 mod q) keeps the lifted value positive; otherwise the offset is just -(2^59 mod q)
-    lc.k59 = lc.wide ? R.k59_d[mod] : __dsub_rn(R.k59_d[mod], __dadd_rn(qd, qd));
-    if (LOAD == LOAD_I64_MONT) {
-        const double* ec = R.enc_consts + (size_t)mod * ENC_CONSTS;
-        lc.c30 = __ldg(ec);
-        lc.c30q = __ldg(ec + 1);
-        lc.c64d = __ldg(ec + 2);
-        lc.c64q = __ldg(ec + 3);
-        lc.k59 = __ldg(ec + 4);
-    }
-    {
-        u64 qs = ~(u64)0;
-        if (LOAD == LOAD_REDUCE && B.src_digits) {      // the prime the source digit belongs to
-            u32 s_hi, s_lo;
-            split_index(o, R.r, B.o_div == R.r ? B.o_div_magic : 0u, s_hi, s_lo);
-            qs = R.q[s_lo];
-        }
-        lc.src_small = qs <= q + (q >> 1);
-        lc.src_fp = qs < (1ull << 51);
-    }
-    const int col0 = blockIdx.x * LANES;
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int gi = 0; gi < NG; ++gi) {
-        const int fg = FWD ? gi : NG - 1 - gi;                 // group index in forward order
-        const int K = group_k(LOG_R, fg);
-        const int log_step = group_log_step(LOG_R, fg);
-        const int step = 1 << log_step, t0 = step << (K - 1);
-        const int m0 = LEN / (2 * t0);
-        const int nsets = (LEN * LANES) >> K;
-        const bool g_first = (gi == 0), g_last = (gi == NG - 1);
-#pragma unroll
-        for (int w0 = 0; w0 < nsets; w0 += NT) {
-            const int w = w0 + tid;
-            if (NT > nsets && w >= nsets) break;
-            const int lane = w & (LANES - 1), u = w >> LOG_LANES;
-            const int blk = u >> log_step, off = u & (step - 1);
-            const int base = blk * 2 * t0 + off;
-            T e[8];
-#pragma unroll
-            for (int i = 0; i < (1 << K); ++i) {
-                const int row = base + i * step;
-                if (g_first) {
-                    const size_t gidx = ((size_t)row << LOG_C) + col0 + lane;
-                    if (FWD) {
-                        const void* from = STAGED ? (const void*)staged : (const void*)src;
-                        const size_t at = STAGED ? (size_t)(row * LANES + lane) : gidx;
-                        if constexpr (FP) e[i] = load_src_fp<LOAD>(from, at, lc);
-                        else e[i] = load_src<LOAD>(from, at, lc);
-                    } else {
-                        e[i] = ((const T*)dst)[gidx];
-                    }
-                } else {
-                    e[i] = sm[row * LANES + lane];
-                }
-            }
-            if (g_first && w0 == 0) {       // (the first sweep of the first group is full for every geometry)
-                static_assert(NT <= ((LEN * LANES) >> group_k(LOG_R, FWD ? 0 : NG - 1)), "first sweep must be full");
-                if (threadIdx.x < LEN) tws[threadIdx.x] = tw_mine;
-                __syncthreads();
-            }
-            if (K == 3) set_butterflies<3, FWD, true>(e, tw, (u32)m0, (u32)blk, q, qd);
-            else if (K == 2) set_butterflies<2, FWD, true>(e, tw, (u32)m0, (u32)blk, q, qd);
-            else set_butterflies<1, FWD, true>(e, tw, (u32)m0, (u32)blk, q, qd);
-            if (!FWD && g_first && NG > 1) {
-                if (K == 3) centre_sums<3>(e, q, qd, R.qinv_d[mod]);
-                else if (K == 2) centre_sums<2>(e, q, qd, R.qinv_d[mod]);
-                else centre_sums<1>(e, q, qd, R.qinv_d[mod]);
-            }
-#pragma unroll
-            for (int i = 0; i < (1 << K); ++i) {
-                const int row = base + i * step;
-                if (g_last) {
-                    const size_t gidx = ((size_t)row << LOG_C) + col0 + lane;
-                    if (FWD) {
-                        ((T*)dst)[gidx] = e[i];                 // lazy; the contiguous pass finishes
-                    } else {                                    // scale by N^{-1}, to [0, q)
-                        const bool mont = B.from_mont != 0;
-                        u64 out;
-                        if constexpr (FP) {
-                            const double nv = mont ? R.ninvm_d[mod] : R.ninv_d[mod];
-                            const double nq = mont ? R.ninvm_q[mod] : R.ninv_q[mod];
-                            double v;
-                            if (q >> 41) {
-                                v = __dadd_rn(fp_mul_centred(e[i], nv, nq, qd), qd);
-                                if (v >= qd) v = __dsub_rn(v, qd);
-                                if (v >= qd) v = __dsub_rn(v, qd);  // (the product can touch 2q for the 50-bit prime)
-                            } else {
-                                v = fp_mul_centred_signed(e[i], nv, nq, qd);
-                                if (v < 0.0) v = __dadd_rn(v, qd);
-                            }
-                            out = d2u(v);
-                        } else {
-                            out = mul_shoup(e[i], mont ? R.ninv_m[mod] : R.ninv[mod], mont ? R.ninv_ms[mod] : R.ninvs[mod], q);
-                        }
-                        if (B.store_centred == 1 || (B.store_centred == 2 && mod == R.r))
-                            out = (out > (q - 1) / 2 ? out - q : out) + (1ull << 59);
-                        dst[gidx] = out;
-                    }
-                } else {
-                    sm[row * LANES + lane] = e[i];
-                }
-            }
-        }
-        if (!g_last) __syncthreads();
-    }
-}
-
-// Polynomial (o, m) of a block and its modulus: straight from the grid (x, m, o) when the launcher could lay it out
-// so, else divided out of blockIdx.y.  (n_m <= 2 * mod_wrap in every batch that wraps.)
-__device__ __forceinline__ void block_poly(const PolyBatch& B, u32& o, u32& m, u32& mod) {
-    if (B.grid3) {
-        m = blockIdx.y;
-        o = blockIdx.z;
-    } else {
-        o = blockIdx.y / B.n_m;
-        m = blockIdx.y - o * B.n_m;
-    }
-    const u32 mm = (B.mod_wrap && m >= B.mod_wrap) ? m - B.mod_wrap : m;
-    mod = B.mod0 + mm * B.mod_step;
-}
-// a digit in its own prime (o = set * r + digit with digit == mod), which ModUp copies instead of transforming
-__device__ __forceinline__ bool own_prime(const RingDev& R, const PolyBatch& B, u32 o, u32 mod) {
-    if (!B.skip_diag || mod >= R.r) return false;
-    u32 hi, lo;
-    split_index(o, R.r, B.o_div == R.r ? B.o_div_magic : 0u, hi, lo);
-    return lo == mod;
-}
-
-// a residue in the form the inner products read (see RingDev::dp)
-__device__ __forceinline__ u64 operand_word(const RingDev& R, u32 mod, u64 v) {
-    return R.dp[mod] ? (u64)__double_as_longlong(u2d(v)) : v;
-}
-
-template <bool FWD, int LOAD, int LOG_R, int LOG_LANES>
-__global__ void __launch_bounds__(((1 << (LOG_R + LOG_LANES)) / 8) < 32 ? 32 : ((1 << (LOG_R + LOG_LANES)) / 8),
-                                  ((1 << (LOG_R + LOG_LANES)) / 8) >= 512 ? 2 : ((1 << (LOG_R + LOG_LANES)) / 8) >= 256 ? 4 : 8)
-ntt_strided(const RingDev R, const PolyBatch B) {
-    __shared__ u64 sm[1 << (LOG_R + LOG_LANES)];
-    __shared__ ulonglong2 tws[1 << LOG_R];
-    grid_dependency_enter();
-    u32 o, m, mod;
-    block_poly(B, o, m, mod);
-    if (FWD && own_prime(R, B, o, mod)) {
-        // this digit's transform in its own prime exists already: copy the tile instead
-        const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
-        u32 t_hi, t_lo;
-        split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
-        const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
-        for (int w = threadIdx.x; w < (1 << (LOG_R + LOG_LANES)); w += blockDim.x) {
-            const size_t gidx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * (1 << LOG_LANES) + (w & ((1 << LOG_LANES) - 1));
-            B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
-        }
-        return;
-    }
-    if (R.fp_ok[mod]) strided_body<FWD, LOAD, LOG_R, LOG_LANES, true>(R, B, sm, tws, o, m, mod);
-    else strided_body<FWD, LOAD, LOG_R, LOG_LANES, false>(R, B, sm, tws, o, m, mod);
-}
-
-// Forward strided pass of a batch whose n_m target primes all read the same source polynomial (ModUp digits,
-// the P-residues of ModDown): a block stages the source tile in shared memory once and transforms it
-// into targets m_begin .. m_begin + m_count - 1, so the source crosses L2 once per block instead of once per
-// target.  grid: x = tile, y = outer index o, z = slice of the targets.
-template <int LOAD, int LOG_R, int LOG_LANES>
-__global__ void __launch_bounds__(((1 << (LOG_R + LOG_LANES)) / 8) < 32 ? 32 : ((1 << (LOG_R + LOG_LANES)) / 8),
-                                  ((1 << (LOG_R + LOG_LANES)) / 8) >= 512 ? 2 : ((1 << (LOG_R + LOG_LANES)) / 8) >= 256 ? 4 : 8)
-ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
-    constexpr int LANES = 1 << LOG_LANES, POINTS = 1 << (LOG_R + LOG_LANES);
-    extern __shared__ __align__(16) u64 shared_src_smem[];
-    u64* staged = shared_src_smem;                  // [POINTS] raw source words
-    u64* sm = shared_src_smem + POINTS;             // [POINTS] exchange between stage groups
-    ulonglong2* tws = (ulonglong2*)(shared_src_smem + 2 * POINTS);     // [2^LOG_R] twiddles of the current target
-    grid_dependency_enter();
-    const u32 o = blockIdx.y;
-    const u32 m_begin = blockIdx.z * m_per_block;
-    const u32 m_end = min(B.n_m, m_begin + m_per_block);
-    {
-        u32 o_hi = 0, o_lo = o;
-        if (B.o_div) split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
-        const size_t src_off = B.o_div ? (size_t)o_hi * B.src_so2 + (size_t)o_lo * B.src_so : (size_t)o * B.src_so;
-        const u64* src = (const u64*)B.src + src_off;
-        if (B.div_t) {
-            // the digit is a division by P away: (source - t) * P^{-1} modulo the digit's own prime, t the centred lift
-            // of the polynomial's residue modulo P (exact: same value as dividing in the transform domain)
-            const u32 i = o_lo;
-            LoadConsts dc;
-            dc.q = R.q[i];
-            dc.mu = R.mu[i];
-            dc.lift_mod = R.q[R.r];
-            const u64* tp = B.div_t + (size_t)o_hi * B.div_so;
-            if (R.fp_ok[i]) {
-                // in fp64 (every value an exact integer): t lazily reduced by the load functor, the difference times
-                // P^{-1} as a centred product, brought to [0, q) -- the digit must be the canonical residue, since it is
-                // reduced into the other primes next
-                const double qd = R.qd[i], pv = R.pinv_d[i], pq = R.pinv_q[i];
-                dc.qd = qd;
-                dc.c30 = R.c30_d[i];
-                dc.c30q = R.c30_q[i];
-                dc.wide = (dc.q >> 41) != 0;
-                dc.k59 = dc.wide ? R.k59_d[i] : __dsub_rn(R.k59_d[i], __dadd_rn(qd, qd));
-                const double q3 = __dadd_rn(__dadd_rn(qd, qd), qd);
-                for (int w = threadIdx.x; w < POINTS; w += blockDim.x) {
-                    const size_t idx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * LANES + (w & (LANES - 1));
-                    const double t = load_src_fp<LOAD_CENTRED>(tp, idx, dc);       // (-1.75q, 0.76q), or (0.25q, 2.76q) when wide
-                    const double x = __dsub_rn(u2d(src[idx]), t);
-                    double s2 = dc.wide ? fp_mul_centred(__dadd_rn(x, q3), pv, pq, qd) : fp_mul_centred_signed(x, pv, pq, qd);
-                    if (s2 < 0.0) s2 = __dadd_rn(s2, qd);
-                    staged[w] = d2u(s2);
-                }
-            } else {
-                dc.lift_red = barrett64(dc.lift_mod, dc.q, dc.mu);
-                const u64 pinv = R.pinv[i], pinvs = R.pinvs[i];
-                for (int w = threadIdx.x; w < POINTS; w += blockDim.x) {
-                    const size_t idx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * LANES + (w & (LANES - 1));
-                    const u64 t = load_src<LOAD_CENTRED>(tp, idx, dc);
-                    staged[w] = mul_shoup(sub_mod(src[idx], t, dc.q), pinv, pinvs, dc.q);
-                }
-            }
-        } else {
-            for (int w = threadIdx.x; w < POINTS; w += blockDim.x)
-                staged[w] = src[((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * LANES + (w & (LANES - 1))];
-        }
-    }
-    __syncthreads();
-    for (u32 m = m_begin; m < m_end; ++m) {
-        const u32 mod = B.mod0 + ((B.mod_wrap && m >= B.mod_wrap) ? m - B.mod_wrap : m) * B.mod_step;
-        if (own_prime(R, B, o, mod)) {
-            // this digit's transform in its own prime exists already: copy the tile instead
-            const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
-            u32 t_hi, t_lo;
-            split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
-            const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
-            for (int w = threadIdx.x; w < POINTS; w += blockDim.x) {
-                const size_t gidx = ((size_t)(w >> LOG_LANES) << LOG_C) + blockIdx.x * LANES + (w & (LANES - 1));
-                B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
-            }
-            continue;
-        }
-        if (R.fp_ok[mod]) strided_body<true, LOAD, LOG_R, LOG_LANES, true, true>(R, B, sm, tws, o, m, mod, staged);
-        else strided_body<true, LOAD, LOG_R, LOG_LANES, false, true>(R, B, sm, tws, o, m, mod, staged);
-        __syncthreads();            // the exchange buffer is free again
-    }
-}
-
 // Contiguous pass: every warp transforms one chunk of 256 adjacent points (8 per thread) through
 // the groups {3,3,2}; the chunk lives in the warp's own swizzled slice of shared memory between
-// groups, so only warp-level synchronisation is needed.
+// groups, so only warp-level synchronisation is needed.  The chunks of a block are consecutive in (chunk, outer index)
+// order: where a batch has several polynomials per prime, they share their twiddles through L1.
 // Forward: second pass (final reduction to [0, q), then the store functors).  Inverse: first pass
 // (reads the batch source: plain residues, tiled/limb-split plaintexts, or a sum of arrays).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
 // EPI: 0 = none; 1 = division by P per rotation (scatter through the rotation's permutation); 2 = per output
-// (sum over the output's giant rotations, gathered through their permutations); 3 = plain (see ModDownEpilogue).
+// (sum over the output's giant rotations, gathered through their permutations); 3 = plain; 4 = output assembly (see
+// ModDownEpilogue).
 // DTILE: the forward result goes to the tile-major operand array of the inner product and nowhere else (ModUp: the
 // hot case; its index arithmetic is hoisted out of the store loop and none of the other store functors is compiled in).
-template <bool FWD, int EPI, bool FP, bool TILED, bool DTILE = false>
+constexpr int CONTIG_THREADS = 128, CONTIG_SLOTS = CONTIG_THREADS / 32;
+
+// a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
+template <int PATH, typename T>
+__device__ __forceinline__ u64 canonical(T x, const ModConsts& c, bool bits) {
+    if constexpr (PATH == PATH_WIDE) {
+        return d2u(fp_reduce(x, c.qd, c.qinv));
+    } else if constexpr (PATH == PATH_DP) {
+        double v = fp_centre(x, c.qd, c.qinv);
+        if (v < 0.0) v = __dadd_rn(v, c.qd);
+        return bits ? (u64)__double_as_longlong(v) : d2u(v);
+    } else {
+        if (x >= 2 * c.q) x -= 2 * c.q;
+        return x >= c.q ? x - c.q : x;
+    }
+}
+
+// The first two groups of the forward pass over one chunk; the chunk is left in the warp's slice for the third, whose sets
+// are the 4 adjacent points at swizzled index 4 (lane + 32 it).
+template <int PATH, typename T>
+__device__ __forceinline__ void contig_forward_far(const T* gsrc, u32 slice, int lane, const void* tw, u32 mult, const ModConsts& c) {
+    const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
+    const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
+    T e[8];
+    // group 0: K = 3, spacing 32
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[i] = gsrc[lane + 32 * i];
+    set_butterflies<3, true, PATH, false>(e, tw, mult, c);
+    swz_store_set<8, 5>(a_far, e);
+    __syncwarp();
+    // group 1: K = 3, spacing 4
+    swz_load_set<8, 2>(a_mid, e);
+    set_butterflies<3, true, PATH, false>(e, tw, 8u * mult + (lane >> 2), c);
+    swz_store_set<8, 2>(a_mid, e);
+    __syncwarp();
+}
+
+template <bool FWD, int EPI, int PATH, bool TILED, bool DTILE = false>
 __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u32 o, u32 m, u32 mod,
                                             u32 chunk, int lane, const RotBatch& rb, const ModDownEpilogue& epi) {
-    typedef typename Elem<FP>::T T;
+    typedef typename Elem<PATH>::T T;
     constexpr int LEN = 1 << LOG_C;
     T* sm = (T*)sm_raw;
-    const u64 q = R.q[mod];
-    const double qd = R.qd[mod];
-    const ulonglong2* __restrict__ tw = (FWD ? R.tw_fwd : R.tw_inv) + (size_t)mod * R.N;
+    ModConsts c;
+    c.q = R.q[mod];
+    c.qd = R.qd[mod];
+    c.qinv = R.qinv_d[mod];
+    const u64 q = c.q;
+    const void* tw = twiddle_table(R, FWD, PATH, mod);
     u64* dst = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
     const u64* src = FWD ? dst : (const u64*)B.src + (size_t)o * B.src_so + (size_t)m * B.src_sm;
     const u32 mult = (R.N >> LOG_C) + chunk;                   // twiddle index multiplier of this chunk
     const u64* gsrc = src + (size_t)chunk * LEN;
     u64* gdst = dst + (size_t)chunk * LEN;
-    // byte addresses (shared window) of the thread's base point in each of the three access patterns
-    const u32 slice = (u32)__cvta_generic_to_shared(sm);
-    const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
-    const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
-    const u32 a_near = slice + 8u * (u32)swz(4 * lane);                               // points 4 (lane + 32 it) + i
     T e[8];
     const bool dp = R.dp[mod] != 0;         // (the operand arrays hold this prime's words as doubles)
     (void)dp;
@@ -623,21 +737,13 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
         dtile_base = ks_tile_base(R.N, B.n_m, B.dtile_div, o_hi, o_lo, m);
     }
     (void)dtile_base;
+    // byte addresses (shared window) of the thread's base point in each of the three access patterns
+    const u32 slice = (u32)__cvta_generic_to_shared(sm);
+    const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
+    const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
+    const u32 a_near = slice + 8u * (u32)swz(4 * lane);                               // points 4 (lane + 32 it) + i
     if (FWD) {
-        // group 0: K = 3, spacing 32
-#pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = ((const T*)gsrc)[lane + 32 * i];
-        set_butterflies<3, true>(e, tw, 1u * mult, 0u, q, qd);
-        swz_store_set<8, 5>(a_far, e);
-        __syncwarp();
-        // group 1: K = 3, spacing 4
-        {
-            const int blk = lane >> 2;
-            swz_load_set<8, 2>(a_mid, e);
-            set_butterflies<3, true>(e, tw, 8u * mult, (u32)blk, q, qd);
-            swz_store_set<8, 2>(a_mid, e);
-        }
-        __syncwarp();
+        contig_forward_far<PATH>((const T*)gsrc, slice, lane, tw, mult, c);
         // group 2: K = 2, adjacent points; two sets per thread
 #pragma unroll
         for (int it = 0; it < 2; ++it) {
@@ -655,28 +761,28 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     uint4 pv[3];
                     u64 uv[3][4], cv[3][4];
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t < epi.n_sum) pv[t] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + t] * R.N + n);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h < epi.n_sum) pv[h] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + h] * R.N + n);
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t) {
-                        if (j0 + t >= epi.n_sum) continue;
-                        const size_t rot = (size_t)(j0 + t) * epi.n_out + pp_out;
+                    for (u32 h = 0; h < 3; ++h) {
+                        if (j0 + h >= epi.n_sum) continue;
+                        const size_t rot = (size_t)(j0 + h) * epi.n_out + pp_out;
                         const u64* up = epi.u + ((rot * 2 + comp) * nb + ip) * R.N;
-                        uv[t][0] = __ldg(up + pv[t].x); uv[t][1] = __ldg(up + pv[t].y);
-                        uv[t][2] = __ldg(up + pv[t].z); uv[t][3] = __ldg(up + pv[t].w);
+                        uv[h][0] = __ldg(up + pv[h].x); uv[h][1] = __ldg(up + pv[h].y);
+                        uv[h][2] = __ldg(up + pv[h].z); uv[h][3] = __ldg(up + pv[h].w);
                         if (comp == 0) {
                             const u64* cp = epi.c0_base + rot * epi.c0_stride + (size_t)ip * R.N;
-                            cv[t][0] = __ldg(cp + pv[t].x); cv[t][1] = __ldg(cp + pv[t].y);
-                            cv[t][2] = __ldg(cp + pv[t].z); cv[t][3] = __ldg(cp + pv[t].w);
+                            cv[h][0] = __ldg(cp + pv[h].x); cv[h][1] = __ldg(cp + pv[h].y);
+                            cv[h][2] = __ldg(cp + pv[h].z); cv[h][3] = __ldg(cp + pv[h].w);
                         }
                     }
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t) {
-                        if (j0 + t >= epi.n_sum) continue;
+                    for (u32 h = 0; h < 3; ++h) {
+                        if (j0 + h >= epi.n_sum) continue;
 #pragma unroll
                         for (int w = 0; w < 4; ++w) {
-                            uu[w] = add_mod(uu[w], uv[t][w], q);
-                            if (comp == 0) cc[w] = add_mod(cc[w], cv[t][w], q);
+                            uu[w] = add_mod(uu[w], uv[h][w], q);
+                            if (comp == 0) cc[w] = add_mod(cc[w], cv[h][w], q);
                         }
                     }
                 }
@@ -700,42 +806,23 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const uint4 pv = *(const uint4*)(epi.pinv + (size_t)rb.key[rot] * R.N + n);
                 pp[0] = pv.x; pp[1] = pv.y; pp[2] = pv.z; pp[3] = pv.w;
             }
-            set_butterflies<2, true>(e, tw, 64u * mult, (u32)s, q, qd);
+            set_butterflies<2, true, PATH, false>(e, tw, 64u * mult + s, c);
+            // (doubles stay doubles where they are stored as such)
             u64 v4[4];
-            if (FP && (q >> 41)) {          // final reduction to [0, q)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v4[i] = d2u(fp_reduce(*(double*)&e[i], qd, R.qinv_d[mod]));
-            } else if (FP) {
-                const double qi = R.qinv_d[mod];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    double v = fp_centre(*(double*)&e[i], qd, qi);
-                    if (v < 0.0) v = __dadd_rn(v, qd);
-                    v4[i] = DTILE && dp ? (u64)__double_as_longlong(v) : d2u(v);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    u64 v = *(u64*)&e[i];
-                    if (v >= 2 * q) v -= 2 * q;
-                    if (v >= q) v -= q;
-                    v4[i] = v;
-                }
-            }
+            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, (DTILE || TILED) && dp);
             if constexpr (DTILE) {
                 // (4 adjacent coefficients never straddle a tile of 128)
                 const u32 n = chunk * LEN + 4 * s;
-                ulonglong2* gp = (ulonglong2*)(B.dtile_ptr + dtile_base + (size_t)(n / KS_TILE) * B.dtile_div * KS_TILE + n % KS_TILE);
-                gp[0] = make_ulonglong2(v4[0], v4[1]);
-                gp[1] = make_ulonglong2(v4[2], v4[3]);
+                stg4(B.dtile_ptr + dtile_base + (size_t)(n / KS_TILE) * B.dtile_div * KS_TILE + n % KS_TILE, v4[0], v4[1], v4[2], v4[3]);
                 continue;
             }
             if (EPI == 2) {
                 const u32 pp_out = o >> 1, comp = o & 1, ip = mod, r = R.r;
                 u64* op = epi.out_base + (size_t)pp_out * epi.out_stride + ((size_t)comp * r + ip) * R.N + (size_t)chunk * LEN + 4 * s;
 #pragma unroll
-                for (int t = 0; t < 4; ++t)
-                    v4[t] = add_mod(mul_shoup(sub_mod(uu[t], v4[t], q), R.pinv[ip], R.pinvs[ip], q), cc[t], q);
+                for (int i = 0; i < 4; ++i)
+                    v4[i] = add_mod(mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[ip], R.pinvs[ip], q), cc[i], q);
                 ((ulonglong2*)op)[0] = make_ulonglong2(v4[0], v4[1]);
                 ((ulonglong2*)op)[1] = make_ulonglong2(v4[2], v4[3]);
                 continue;
@@ -743,7 +830,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             if (EPI == 3) {
                 u64* op = epi.out_base + (size_t)o * epi.out_stride + (size_t)mod * R.N + (size_t)chunk * LEN + 4 * s;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) v4[t] = mul_shoup(sub_mod(uu[t], v4[t], q), R.pinv[mod], R.pinvs[mod], q);
+                for (int i = 0; i < 4; ++i) v4[i] = mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[mod], R.pinvs[mod], q);
                 ((ulonglong2*)op)[0] = make_ulonglong2(v4[0], v4[1]);
                 ((ulonglong2*)op)[1] = make_ulonglong2(v4[2], v4[3]);
                 continue;
@@ -752,10 +839,10 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const u32 rot = o >> 1, comp = o & 1, ip = mod, r = R.r;
                 u64* op = epi.out_base + (size_t)rb.out[rot] * epi.out_stride + ((size_t)comp * r + ip) * R.N;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    u64 v = mul_shoup(sub_mod(uu[t], v4[t], q), R.pinv[ip], R.pinvs[ip], q);
-                    v = add_mod(v, cc[t], q);
-                    op[pp[t]] = v;
+                for (int i = 0; i < 4; ++i) {
+                    u64 v = mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[ip], R.pinvs[ip], q);
+                    v = add_mod(v, cc[i], q);
+                    op[pp[i]] = v;
                 }
                 continue;
             }
@@ -766,13 +853,17 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const u32 at = tile_word_index(B.tile, pj, term, n);
                 const u32 fmt = tile_format(B.tile, mod);
                 if (fmt == TILE_W64) {
-                    const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
+                    if (!dp) {          // (else: the bits of doubles already)
+                        const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) v4[i] = dp ? (u64)__double_as_longlong(u2d(v4[i])) : limb_split(v4[i], L);
-                    ulonglong2* gp = (ulonglong2*)(stage + (size_t)at * 8);
-                    gp[0] = make_ulonglong2(v4[0], v4[1]);
-                    gp[1] = make_ulonglong2(v4[2], v4[3]);
+                        for (int i = 0; i < 4; ++i) v4[i] = limb_split(v4[i], L);
+                    }
+                    stg4((u64*)stage + at, v4[0], v4[1], v4[2], v4[3]);
                 } else {
+                    if (dp) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v4[i] = d2u(__longlong_as_double((long long)v4[i]));
+                    }
                     *(uint4*)(stage + (size_t)at * 4) = make_uint4((u32)v4[0], (u32)v4[1], (u32)v4[2], (u32)v4[3]);
                     if (fmt == TILE_W40)
                         *(u32*)(stage + TILE_STAGE_WORDS * 4u + at) = (u32)(v4[0] >> 32) | ((u32)(v4[1] >> 32) << 8) |
@@ -827,20 +918,20 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     uint4 pv[3];
                     u64 uv[3][4];
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t < epi.n_sum) pv[t] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + t] * R.N + n);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h < epi.n_sum) pv[h] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + h] * R.N + n);
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t) {
-                        if (j0 + t >= epi.n_sum) continue;
-                        const u64* up = epi.u + ((((size_t)(j0 + t) * epi.n_out + pp_out) * 2 + comp) * nb + mod) * R.N;
-                        uv[t][0] = __ldg(up + pv[t].x); uv[t][1] = __ldg(up + pv[t].y);
-                        uv[t][2] = __ldg(up + pv[t].z); uv[t][3] = __ldg(up + pv[t].w);
+                    for (u32 h = 0; h < 3; ++h) {
+                        if (j0 + h >= epi.n_sum) continue;
+                        const u64* up = epi.u + ((((size_t)(j0 + h) * epi.n_out + pp_out) * 2 + comp) * nb + mod) * R.N;
+                        uv[h][0] = __ldg(up + pv[h].x); uv[h][1] = __ldg(up + pv[h].y);
+                        uv[h][2] = __ldg(up + pv[h].z); uv[h][3] = __ldg(up + pv[h].w);
                     }
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t) {
-                        if (j0 + t >= epi.n_sum) continue;
+                    for (u32 h = 0; h < 3; ++h) {
+                        if (j0 + h >= epi.n_sum) continue;
 #pragma unroll
-                        for (int w = 0; w < 4; ++w) v4[w] = add_mod(v4[w], uv[t][w], q);
+                        for (int w = 0; w < 4; ++w) v4[w] = add_mod(v4[w], uv[h][w], q);
                     }
                 }
             } else if constexpr (EPI == 4) {   // output assembly in the extended basis (see ModDownEpilogue::assemble)
@@ -865,17 +956,17 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 for (u32 j0 = 1; j0 <= ju; j0 += 3) {
                     ulonglong2 a2[3], b2[3];
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t <= ju) {
-                            const u64* up = ub + (size_t)(j0 + t - 1) * u_step;
-                            a2[t] = *(const ulonglong2*)up;
-                            b2[t] = *(const ulonglong2*)(up + 2);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h <= ju) {
+                            const u64* up = ub + (size_t)(j0 + h - 1) * u_step;
+                            a2[h] = *(const ulonglong2*)up;
+                            b2[h] = *(const ulonglong2*)(up + 2);
                         }
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t <= ju) {
-                            v4[0] = add_mod(v4[0], a2[t].x, q); v4[1] = add_mod(v4[1], a2[t].y, q);
-                            v4[2] = add_mod(v4[2], b2[t].x, q); v4[3] = add_mod(v4[3], b2[t].y, q);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h <= ju) {
+                            v4[0] = add_mod(v4[0], a2[h].x, q); v4[1] = add_mod(v4[1], a2[h].y, q);
+                            v4[2] = add_mod(v4[2], b2[h].x, q); v4[3] = add_mod(v4[3], b2[h].y, q);
                         }
                 }
                 const u64* cb = epi.aext + (size_t)o * epi.aext_stride + (size_t)mod * R.N + n;  // inner sum (0, p), c0
@@ -883,17 +974,17 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 for (u32 j0 = jc_lo; j0 <= jc_hi; j0 += 3) {
                     ulonglong2 a2[3], b2[3];
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t <= jc_hi) {
-                            const u64* cp = cb + (size_t)(j0 + t) * c_step;
-                            a2[t] = *(const ulonglong2*)cp;
-                            b2[t] = *(const ulonglong2*)(cp + 2);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h <= jc_hi) {
+                            const u64* cp = cb + (size_t)(j0 + h) * c_step;
+                            a2[h] = *(const ulonglong2*)cp;
+                            b2[h] = *(const ulonglong2*)(cp + 2);
                         }
 #pragma unroll
-                    for (u32 t = 0; t < 3; ++t)
-                        if (j0 + t <= jc_hi) {
-                            v4[0] = add_mod(v4[0], a2[t].x, q); v4[1] = add_mod(v4[1], a2[t].y, q);
-                            v4[2] = add_mod(v4[2], b2[t].x, q); v4[3] = add_mod(v4[3], b2[t].y, q);
+                    for (u32 h = 0; h < 3; ++h)
+                        if (j0 + h <= jc_hi) {
+                            v4[0] = add_mod(v4[0], a2[h].x, q); v4[1] = add_mod(v4[1], a2[h].y, q);
+                            v4[2] = add_mod(v4[2], b2[h].x, q); v4[3] = add_mod(v4[3], b2[h].y, q);
                         }
                 }
             } else if constexpr (TILED) {  // read back from the tile-major plaintext cache
@@ -925,13 +1016,13 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             if (B.sum_terms) {      // the input is a sum of several arrays of the same shape
                 const u64* sp = B.sum_src + (size_t)o * B.src_so + (size_t)m * B.src_sm + (size_t)chunk * LEN + 4 * s;
                 // three arrays at a time, all their loads in flight together (g - 1 = 3 is the common case)
-                u32 t = 0;
-                for (; t + 3 <= B.sum_terms; t += 3) {
+                u32 h = 0;
+                for (; h + 3 <= B.sum_terms; h += 3) {
                     ulonglong2 a2[3], b2[3];
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
-                        a2[j] = *(const ulonglong2*)(sp + (size_t)(t + j) * B.sum_stride);
-                        b2[j] = *(const ulonglong2*)(sp + (size_t)(t + j) * B.sum_stride + 2);
+                        a2[j] = *(const ulonglong2*)(sp + (size_t)(h + j) * B.sum_stride);
+                        b2[j] = *(const ulonglong2*)(sp + (size_t)(h + j) * B.sum_stride + 2);
                     }
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
@@ -939,119 +1030,227 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                         v4[2] = add_mod(v4[2], b2[j].x, q); v4[3] = add_mod(v4[3], b2[j].y, q);
                     }
                 }
-                for (; t < B.sum_terms; ++t) {
-                    const ulonglong2 a2 = *(const ulonglong2*)(sp + (size_t)t * B.sum_stride);
-                    const ulonglong2 b2 = *(const ulonglong2*)(sp + (size_t)t * B.sum_stride + 2);
+                for (; h < B.sum_terms; ++h) {
+                    const ulonglong2 a2 = *(const ulonglong2*)(sp + (size_t)h * B.sum_stride);
+                    const ulonglong2 b2 = *(const ulonglong2*)(sp + (size_t)h * B.sum_stride + 2);
                     v4[0] = add_mod(v4[0], a2.x, q); v4[1] = add_mod(v4[1], a2.y, q);
                     v4[2] = add_mod(v4[2], b2.x, q); v4[3] = add_mod(v4[3], b2.y, q);
                 }
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) from_u64(e[i], v4[i]);
-            set_butterflies<2, false>(e, tw, 64u * mult, (u32)s, q, qd);
+            set_butterflies<2, false, PATH, false>(e, tw, 64u * mult + s, c);
             swz_store_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), e);
         }
         __syncwarp();
-        {
-            const int blk = lane >> 2;
-            swz_load_set<8, 2>(a_mid, e);
-            set_butterflies<3, false>(e, tw, 8u * mult, (u32)blk, q, qd);
-            centre_sums<3>(e, q, qd, R.qinv_d[mod]);
-            swz_store_set<8, 2>(a_mid, e);
-        }
+        swz_load_set<8, 2>(a_mid, e);
+        set_butterflies<3, false, PATH, false>(e, tw, 8u * mult + (lane >> 2), c);
+        centre_sums<3, PATH>(e, c);
+        swz_store_set<8, 2>(a_mid, e);
         __syncwarp();
         swz_load_set<8, 5>(a_far, e);
-        set_butterflies<3, false>(e, tw, 1u * mult, 0u, q, qd);
+        set_butterflies<3, false, PATH, false>(e, tw, mult, c);
+        centre_sums<3, PATH>(e, c);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) ((T*)gdst)[lane + 32 * i] = e[i];      // lazy, below 2q; the strided pass finishes
+        for (int i = 0; i < 8; ++i) ((T*)gdst)[lane + 32 * i] = e[i];      // lazy; the strided pass finishes
     }
 }
 
+// grid: x = groups of CONTIG_SLOTS chunks, y = slot m.
 // (the per-output forms run on a few polynomials per launch and hold the operands of three rotations at once: they
 // trade resident blocks for registers)
 template <bool FWD, int EPI, bool TILED, bool DTILE = false>
-__global__ void __launch_bounds__(32 * CHUNKS_PER_BLOCK, (EPI == 2 || EPI == 4) ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
-                                                                       u32 chunks_per_block, const RotBatch rb,
+__global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
+                                                                       u32 n_outer, const RotBatch rb,
                                                                        const ModDownEpilogue epi) {
-    __shared__ __align__(128) u64 sm_all[CHUNKS_PER_BLOCK << LOG_C];
+    __shared__ __align__(128) u64 sm_all[CONTIG_SLOTS << LOG_C];
     grid_dependency_enter();
-    u32 o, m, mod;
-    block_poly(B, o, m, mod);
+    const u32 m = slot_of_block(blockIdx.y, B.n_m), mod = batch_modulus(B, m);
+    const int slot = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const u32 g = blockIdx.x * CONTIG_SLOTS + slot;
+    const u32 chunk = g / n_outer, o = g - chunk * n_outer;
+    if (chunk >= (R.N >> LOG_C)) return;            // (whole warps leave)
     if (FWD && own_prime(R, B, o, mod)) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if ((u32)warp >= chunks_per_block) return;
-    const u32 chunk = blockIdx.x * chunks_per_block + warp;
-    u64* sm = sm_all + (warp << LOG_C);
-    if (R.fp_ok[mod]) contig_body<FWD, EPI, true, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else contig_body<FWD, EPI, false, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    u64* sm = sm_all + (slot << LOG_C);
+    const int path = path_of(R, mod);
+    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else contig_body<FWD, EPI, PATH_INT, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
 }
 
-NttGeometry ntt_geometry(u32 logN) {
-    NttGeometry g;
-    g.log_c = LOG_C;
-    g.log_r = (int)logN - LOG_C;
-    // strided tile: 2048 points (256 threads) unless the row count forces otherwise
-    int log_lanes = 11 - g.log_r;
-    if (log_lanes < 4) log_lanes = 4;
-    if (log_lanes > 8) log_lanes = 8;
-    g.strided_lanes = 1 << log_lanes;
-    g.strided_threads = ((1 << g.log_r) * g.strided_lanes) / 8 < 32 ? 32 : ((1 << g.log_r) * g.strided_lanes) / 8;
-    g.contig_lanes = (1 << g.log_r) < CHUNKS_PER_BLOCK ? (1 << g.log_r) : CHUNKS_PER_BLOCK;
-    g.contig_threads = 32 * CHUNKS_PER_BLOCK;
-    g.contig_pad = 0;
-    return g;
+// Key-switch products (Sec. 4.2 "key-switching primitives"): the contiguous pass of the digits' transforms and their inner
+// product with the rotation keys in one kernel.
+//   u'[rot][comp][m][n] = sum_j NTT_m(digit j of set dig(rot))[n] * key'[key(rot)][j][comp][m][n]
+// The rotation keys are stored pre-permuted by their automorphism, so the product runs in the un-rotated index space with
+// coalesced operands, and the automorphism is applied once, as a scatter, when the result is stored (pinv) or when the
+// rotated ciphertext is assembled.
+//
+// A block owns one run of rotations of the same digit set, one modulus m and CB chunks of 256 coefficients: warp w transforms
+// digit w % r of chunk w / r into its slice of shared memory, then every thread takes a coefficient, multiplies the r digits
+// with the 2r key words of each rotation of the run (straight from global memory: read once, coalesced) and reduces once per
+// output word.  The transformed digits, r (r+1) polynomials per set, never reach memory.
+// What bounds it: the key stream where the run is long (baby steps), the fp64 pipe and the latency of the transform elsewhere.
+// Measured over the giant steps of the four calls of a 0.6B decoder layer (N = 2^15, r = 7, 19 rotations): 302 us, where a
+// contiguous pass and an inner product of their own took 218 + 210 us; a projection's 15 baby and 9 giant rotations without
+// double hoisting: 291 us instead of 110 + 224 us.
+// grid: x = run, y = group of chunks, z = m: the runs that share a key's tile are adjacent.
+// (three blocks of 80 registers an SM instead of four of 64: 334 instead of 302 us)
+template <int RC>
+struct InnerGeo {
+    static constexpr int WARPS = RC > 8 ? RC : RC > 0 ? 8 : MAX_MODULI;    // (upper bound where r is not a constant)
+    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 0 ? 4 : 1;
+};
+template <int CLS, int RC>
+__device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch& rb, u32 first, u32 cnt, u32 m, u32 n, const u64* sd,
+                                               const u64* __restrict__ keys, u64* u, u64* xext,
+                                               const u32* __restrict__ pinv, u64 pol) {
+    const u32 N = R.N, r = RC > 0 ? RC : R.r, nb = r + 1;
+    const u32 at = (u32)swz((int)(n & 255u));
+    const size_t out_words = (size_t)2 * nb * N;
+    for (u32 rot = first; rot < first + cnt; ++rot) {
+        const u64* kp = keys + ks_tile_base(N, nb, 2 * r, (u32)rb.key[rot], 0u, m) + (size_t)(n / KS_TILE) * 2 * r * KS_TILE + n % KS_TILE;
+        u32 dest = n;
+        u64 pc0 = 0;
+        if (pinv) dest = __ldg(&pinv[(size_t)rb.key[rot] * N + n]);
+        if (xext) pc0 = xext[(size_t)rb.c0[rot] * out_words + (size_t)m * N + n];
+        // (one component at a time: with the key words of both in registers fewer blocks fit an SM)
+        auto component = [&](const u64* kc) -> u64 {
+            DigitDot<CLS> dot;
+            if constexpr (RC > 0) {
+                u32 k0[RC], k1[RC];
+#pragma unroll
+                for (int j = 0; j < RC; ++j) ld_stream(kc + 2 * j * KS_TILE, pol, k0[j], k1[j]);
+#pragma unroll
+                for (int j = 0; j < RC; ++j) dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
+            } else {
+#pragma unroll 4
+                for (u32 j = 0; j < r; ++j) {
+                    u32 k0, k1;
+                    ld_stream(kc + 2 * j * KS_TILE, pol, k0, k1);
+                    dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0, k1);
+                }
+            }
+            return dot.reduce(R, m);
+        };
+        const u64 v0 = component(kp), v1 = component(kp + KS_TILE);
+        // xext (double hoisting): the rotated input in the extended basis is (P*c0 + u0, u1) moved through the rotation's
+        // permutation; P*c0 (zero modulo P) was stored as the un-rotated term
+        u64* up = xext ? xext + (size_t)rb.out[rot] * out_words + (size_t)m * N + dest : u + (size_t)rb.out[rot] * out_words + (size_t)m * N + dest;
+        up[0] = xext ? add_mod(v0, pc0, R.q[m]) : v0;
+        up[(size_t)nb * N] = v1;
+    }
 }
 
-// Grid of a batch of n_polys = n_outer * n_m polynomials with x_blocks blocks each: (x, m, o) with the reciprocals
-// the kernels use instead of divisions, when the outer count fits the grid's z extent; else (x, o * n_m + m).
-static dim3 poly_grid(PolyBatch& B, u32 x_blocks, u32 n_polys) {
-    const u32 n_outer = n_polys / B.n_m;
-    B.grid3 = 0;
+template <int RC>
+__global__ void __launch_bounds__(32 * InnerGeo<RC>::WARPS, InnerGeo<RC>::BLOCKS)
+ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const u64* __restrict__ keys, u64* u, u64* xext,
+                 const u32* __restrict__ pinv, u32 cb) {
+    extern __shared__ __align__(128) u64 sm_all[];          // [cb][r] slices
+    grid_dependency_enter();
+    const u32 N = R.N, r = RC > 0 ? RC : R.r, nb = r + 1;
+    const u32 m = slot_of_block(blockIdx.z, nb), chunk0 = blockIdx.y * cb;
+    const u32 first = rb.grp_first[blockIdx.x], cnt = rb.grp_cnt[blockIdx.x], set = (u32)rb.dig[first];
+    const u32 warps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int path = path_of(R, m);
+    ModConsts c;
+    c.q = R.q[m];
+    c.qd = R.qd[m];
+    c.qinv = R.qinv_d[m];
+    const bool dp = R.dp[m] != 0;
+    if (threadIdx.x < cb * 2 && chunk0 + threadIdx.x / 2 < (N >> LOG_C)) {      // the first rotation's keys, on their way to L2
+        const u64* kp = keys + ks_tile_base(N, nb, 2 * r, (u32)rb.key[first], 0u, m) + (size_t)(chunk0 * 2 + threadIdx.x) * 2 * r * KS_TILE;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kp), "r"(2 * r * KS_TILE * 8) : "memory");
+    }
+    for (u32 w = threadIdx.x >> 5; w < cb * r; w += warps) {
+        const u32 chunk = chunk0 + w / r, j = w % r;
+        if (chunk >= (N >> LOG_C)) break;
+        u64* sm = sm_all + (w << LOG_C);
+        const u32 slice = (u32)__cvta_generic_to_shared(sm);
+        if (B.skip_diag && j == m) {            // a digit in its own prime: its transform exists already
+            const u64* ds = B.diag_src + (size_t)set * B.diag_so + (size_t)m * N + (chunk << LOG_C);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sm[swz(lane + 32 * i)] = operand_word(R, m, ds[lane + 32 * i]);
+            continue;
+        }
+        const u64* gsrc = B.dst + (size_t)(set * r + j) * B.dst_so + (size_t)m * B.dst_sm + (chunk << LOG_C);
+        const u32 mult = (N >> LOG_C) + chunk;
+        const void* tw = twiddle_table(R, true, path, m);
+        const u32 a_near = slice + 8u * (u32)swz(4 * lane);
+        auto finish = [&](auto path_c) {
+            constexpr int PATH = decltype(path_c)::value;
+            typedef typename Elem<PATH>::T T;
+            contig_forward_far<PATH>((const T*)gsrc, slice, lane, tw, mult, c);
+#pragma unroll
+            for (int it = 0; it < 2; ++it) {
+                T e[8];
+                swz_load_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), e);
+                set_butterflies<2, true, PATH, false>(e, tw, 64u * mult + lane + 32 * it, c);
+                u64 v[8];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = canonical<PATH>(e[i], c, dp);
+                swz_store_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), v);
+            }
+        };
+        if (path == PATH_DP) finish(std::integral_constant<int, PATH_DP>());
+        else if (path == PATH_WIDE) finish(std::integral_constant<int, PATH_WIDE>());
+        else finish(std::integral_constant<int, PATH_INT>());
+    }
+    __syncthreads();
+    const u64 pol = stream_policy();
+    for (u32 i = threadIdx.x; i < (cb << LOG_C); i += blockDim.x) {
+        const u32 n = (chunk0 << LOG_C) + i;
+        if (n >= N) break;
+        const u64* sd = sm_all + ((size_t)(i >> LOG_C) * r << LOG_C);
+        if (dp) inner_products<OP_DP, RC>(R, rb, first, cnt, m, n, sd, keys, u, xext, pinv, pol);
+        else if (R.q[m] >> 50) inner_products<OP_WIDE, RC>(R, rb, first, cnt, m, n, sd, keys, u, xext, pinv, pol);
+        else inner_products<OP_NARROW, RC>(R, rb, first, cnt, m, n, sd, keys, u, xext, pinv, pol);
+    }
+}
+
+// o / d by a reciprocal where the outer count allows it (see split_index)
+static void set_magics(PolyBatch& B, u32 n_outer) {
     B.o_div_magic = B.dtile_magic = 0;
-    if (n_outer * B.n_m != n_polys || n_outer > 65535u || B.n_m > 65535u) return dim3(x_blocks, n_polys);
-    B.grid3 = 1;
+    if (n_outer > 65535u) return;
     if (B.o_div) B.o_div_magic = (u32)((((u64)1 << 32) + B.o_div - 1) / B.o_div);
     if (B.dtile_div) B.dtile_magic = (u32)((((u64)1 << 32) + B.dtile_div - 1) / B.dtile_div);
-    return dim3(x_blocks, B.n_m, n_outer);
 }
 
 template <bool FWD, int LOAD, int LOG_R, int LOG_LANES>
 static void launch_strided_t(const RingHost& ring, const PolyBatch& B_in, u32 n_polys, cudaStream_t stream) {
-    constexpr int NT = ((1 << (LOG_R + LOG_LANES)) / 8) < 32 ? 32 : ((1 << (LOG_R + LOG_LANES)) / 8);
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
     PolyBatch B = B_in;
-    const dim3 grid = poly_grid(B, (1u << LOG_C) >> LOG_LANES, n_polys);
-    launch_dependent(ring, ntt_strided<FWD, LOAD, LOG_R, LOG_LANES>, grid, dim3(NT), 0, stream, ring.dev, B);
+    const u32 n_outer = n_polys / B.n_m;
+    set_magics(B, n_outer);
+    const dim3 grid(G::TILES, B.n_m, n_outer < 65535u ? n_outer : 65535u);
+    launch_dependent(ring, ntt_strided<FWD, LOAD, LOG_R, LOG_LANES>, grid, dim3(G::NT), 0, stream, ring.dev, B, n_outer);
 }
 
 template <int LOAD, int LOG_R, int LOG_LANES>
 static void launch_shared_src_t(const RingHost& ring, const PolyBatch& B_in, u32 n_outer, cudaStream_t stream) {
-    PolyBatch B = B_in;             // (its grid is (tile, o, slice of the targets): o is never divided out)
-    B.grid3 = 0;
-    B.dtile_magic = B.dtile_div ? (u32)((((u64)1 << 32) + B.dtile_div - 1) / B.dtile_div) : 0u;
-    B.o_div_magic = B.o_div ? (u32)((((u64)1 << 32) + B.o_div - 1) / B.o_div) : 0u;
-    constexpr int NT = ((1 << (LOG_R + LOG_LANES)) / 8) < 32 ? 32 : ((1 << (LOG_R + LOG_LANES)) / 8);
-    constexpr u32 S = (1u << LOG_C) >> LOG_LANES;
+    typedef StridedGeo<LOG_R, LOG_LANES> G;
+    PolyBatch B = B_in;
+    set_magics(B, n_outer);
     // targets per block: fewer blocks share the source better but quantise into waves; cost model =
     // waves x (targets per block + half a unit for staging the source)
-    const u32 slots = 148u * (NT >= 512 ? 2 : NT >= 256 ? 4 : 8);
+    const u32 slots = 148u * G::BLOCKS;
     u32 best = 1;
     double best_cost = 1e30;
     for (u32 per = 1; per <= B.n_m; ++per) {
         const u32 slices = (B.n_m + per - 1) / per;
         if ((B.n_m + slices - 1) / slices != per) continue;         // keep the slices balanced
-        const u32 blocks = S * n_outer * slices;
+        const u32 blocks = G::TILES * n_outer * slices;
         const double cost = (double)((blocks + slots - 1) / slots) * (per + 0.5);
         if (cost <= best_cost) { best_cost = cost; best = per; }
     }
-    dim3 grid(S, n_outer, (B.n_m + best - 1) / best);
-    constexpr size_t smem = (size_t)2 * 8 * (1u << (LOG_R + LOG_LANES)) + (size_t)16 * (1u << LOG_R);
+    const dim3 grid(G::TILES, n_outer, (B.n_m + best - 1) / best);
+    constexpr size_t smem = (size_t)8 * (2 * G::POINTS + 2 * G::TW_WORDS);
     static bool attr_set[MAX_DEVICES] = {false};     // opt in once per device to more than 48 KB of dynamic shared memory
     if (smem > 48 * 1024 && !attr_set[device_slot(ring)]) {
-        cudaFuncSetAttribute(ntt_strided_shared_src<LOAD, LOG_R, LOG_LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+        cudaFuncSetAttribute(ntt_strided_shared_src<LOAD, LOG_R, LOG_LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         attr_set[device_slot(ring)] = true;
     }
-    launch_dependent(ring, ntt_strided_shared_src<LOAD, LOG_R, LOG_LANES>, grid, dim3(NT), smem, stream, ring.dev, B, best);
+    launch_dependent(ring, ntt_strided_shared_src<LOAD, LOG_R, LOG_LANES>, grid, dim3(G::NT), smem, stream, ring.dev, B, best);
 }
 
 template <bool FWD, int LOAD>
@@ -1061,7 +1260,7 @@ static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 
     if constexpr (FWD && (LOAD == LOAD_REDUCE || LOAD == LOAD_CENTRED)) {
         const u32 n_outer = n_polys / B.n_m;
         if (B.src_sm == 0 && B.n_m > 1 && n_outer <= 65535 && !B.tile_ptr) {
-            switch (ring.geom.log_r) {
+            switch (ring.dev.logN - LOG_C) {
                 case 2: launch_shared_src_t<LOAD, 2, 8>(ring, B, n_outer, stream); break;
                 case 3: launch_shared_src_t<LOAD, 3, 8>(ring, B, n_outer, stream); break;
                 case 4: launch_shared_src_t<LOAD, 4, 7>(ring, B, n_outer, stream); break;
@@ -1074,7 +1273,7 @@ static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 
             return cudaGetLastError();
         }
     }
-    switch (ring.geom.log_r) {
+    switch (ring.dev.logN - LOG_C) {
         case 2: launch_strided_t<FWD, LOAD, 2, 8>(ring, B, n_polys, stream); break;
         case 3: launch_strided_t<FWD, LOAD, 3, 8>(ring, B, n_polys, stream); break;
         case 4: launch_strided_t<FWD, LOAD, 4, 7>(ring, B, n_polys, stream); break;
@@ -1092,33 +1291,34 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
                                  const RotBatch* rb = nullptr, const ModDownEpilogue* epi = nullptr) {
     if (n_polys == 0) return cudaSuccess;
     ProfScope prof(ring.prof, FWD ? CAT_NTT_FWD_CONTIG : CAT_NTT_INV_CONTIG, stream);
-    const u32 chunks = 1u << ring.geom.log_r;
-    const u32 cpb = (u32)ring.geom.contig_lanes;
     PolyBatch B = B_in;
-    const dim3 grid = poly_grid(B, chunks / cpb, n_polys);
+    const u32 n_outer = n_polys / B.n_m;
+    set_magics(B, n_outer);
+    const u32 groups = (u32)(((size_t)n_outer * (ring.dev.N >> LOG_C) + CONTIG_SLOTS - 1) / CONTIG_SLOTS);
+    const dim3 grid(groups, B.n_m);
     if (FWD && epi && epi->plain) {
-        launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
     } else if (!FWD && epi && epi->assemble) {
-        launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb, *rb,
+        launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
     } else if (epi && epi->n_sum) {
-        launch_dependent(ring, ntt_contig<FWD, 2, false>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 2, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
     } else if (FWD && epi) {
-        launch_dependent(ring, ntt_contig<FWD, 1, false>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 1, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
     } else {
         static const RotBatch no_rb = {};
         static const ModDownEpilogue no_epi = {};
         if (B.tile_ptr)
-            launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb,
+            launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
                              no_rb, no_epi);
         else if (FWD && B.dtile_ptr && !B.scatter && !B.lift_ptr)
-            launch_dependent(ring, ntt_contig<true, 0, false, true>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B,
-                             cpb, no_rb, no_epi);
+            launch_dependent(ring, ntt_contig<true, 0, false, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B,
+                             n_outer, no_rb, no_epi);
         else
-            launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(32 * CHUNKS_PER_BLOCK), 0, stream, ring.dev, B, cpb,
+            launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
                              no_rb, no_epi);
     }
     return cudaGetLastError();
@@ -1161,6 +1361,69 @@ cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B0, u32 n_o
     return launch_contig<true>(ring, B, n_polys, stream);
 }
 
+cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_outer, cudaStream_t stream) {
+    return launch_strided<true, LOAD_REDUCE>(ring, B, n_outer * B.n_m, stream);
+}
+
+template <int RC>
+static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const u64* keys, u64* u, u64* xext,
+                                         const u32* pinv, cudaStream_t stream) {
+    const u32 r = ring.dev.r, chunks = ring.dev.N >> LOG_C;
+    const u32 warps = r > 8 ? r : 8u;
+    u32 cb = warps / r;                         // chunks per block: few digits leave room for several
+    if (cb > chunks) cb = chunks;
+    return launch_dependent(ring, ntt_contig_inner<RC>, dim3(rb.n_groups, (chunks + cb - 1) / cb, r + 1), dim3(32 * warps),
+                            (size_t)8 * (cb * r << LOG_C), stream, ring.dev, B, rb, keys, u, xext, pinv, cb);
+}
+
+cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n_sets, const RotBatch& rb_in, const u64* keys, u64* u,
+                              u64* xext, const u32* pinv, cudaStream_t stream) {
+    const u32 r = ring.dev.r;
+    if (rb_in.n == 0) return cudaSuccess;
+    if (n_sets) {
+        const cudaError_t e = ntt_forward_first(ring, B_in, n_sets * r, stream);
+        if (e != cudaSuccess) return e;
+    }
+    // runs of consecutive rotations with the same digit set, cut into parts until the blocks fill the machine (every part
+    // transforms the digits again, which costs less than idle SMs)
+    RotBatch rb = rb_in;
+    const u32 warps = r > 8 ? r : 8u, cb = warps / r;
+    u32 runs = 0;
+    for (int t = 0; t < rb.n; ++t) runs += t == 0 || rb.dig[t] != rb.dig[t - 1];
+    const u32 blocks = runs * (((ring.dev.N >> LOG_C) + cb - 1) / cb) * (r + 1);
+    const u32 parts = blocks < 1776u ? 1776u / blocks : 1u;      // 148 SMs x 3 blocks x 4
+    rb.n_groups = 0;
+    for (int t = 0; t < rb.n;) {
+        int end = t + 1;
+        while (end < rb.n && rb.dig[end] == rb.dig[t]) ++end;
+        const int len = end - t, per = (len + (int)parts - 1) / (int)parts;
+        for (; t < end; t += per) {
+            rb.grp_first[rb.n_groups] = (unsigned char)t;
+            rb.grp_cnt[rb.n_groups++] = (unsigned char)(end - t < per ? end - t : per);
+        }
+        t = end;
+    }
+    if (ring.prof) {
+        const u64 key_bytes = (u64)r * 2 * (r + 1) * ring.dev.N * 8;
+        u32 distinct = 0;
+        for (int t = 0; t < rb.n; ++t) {
+            bool seen = false;
+            for (int k = 0; k < t && !seen; ++k) seen = rb.key[k] == rb.key[t];
+            distinct += seen ? 0u : 1u;
+        }
+        ring.prof->key_bytes_distinct += distinct * key_bytes;
+        ring.prof->key_bytes_per_rotation += (u64)rb.n * key_bytes;
+    }
+    ProfScope prof(ring.prof, CAT_KEY_INNER, stream);
+    switch (r) {                    // (digit counts of the shipped parameter sets)
+        case 3: return launch_contig_inner_t<3>(ring, B_in, rb, keys, u, xext, pinv, stream);
+        case 4: return launch_contig_inner_t<4>(ring, B_in, rb, keys, u, xext, pinv, stream);
+        case 7: return launch_contig_inner_t<7>(ring, B_in, rb, keys, u, xext, pinv, stream);
+        case 9: return launch_contig_inner_t<9>(ring, B_in, rb, keys, u, xext, pinv, stream);
+        default: return launch_contig_inner_t<0>(ring, B_in, rb, keys, u, xext, pinv, stream);
+    }
+}
+
 cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
                                   const ModDownEpilogue& epi, cudaStream_t stream) {
     const u32 n_polys = n_outer * B.n_m;
@@ -1175,11 +1438,11 @@ cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 
 //   ct[p][comp][i][n] = (ct[p][comp][i][n] - sum_terms t_term[n]) * P^{-1}  (mod q_i)
 // low non-null: the rescale (Sec. 2.1) follows in the same thread, which holds all residues of its coefficient: the
 // result goes to low[p][comp][r-1][N] as c'_i = (c_i - centred(c_{r-1})) * q_{r-1}^{-1} and ct only held the sums.
-__global__ void __launch_bounds__(256) finish_division_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
+__global__ void __launch_bounds__(128, 8) finish_division_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
                                                               const u64* __restrict__ T, u32 n_t, const RescaleConsts rc,
                                                               u64* __restrict__ low) {
     grid_dependency_enter();
-    const u32 n = blockIdx.x * 256 + threadIdx.x;
+    const u32 n = blockIdx.x * 128 + threadIdx.x;
     const u32 p = blockIdx.y >> 1, comp = blockIdx.y & 1;
     const u64* tp = T + (size_t)p * n_t * R.N + n;
     u64* cp = ct + (size_t)p * ct_stride + (size_t)comp * R.r * R.N + n;
@@ -1246,11 +1509,11 @@ __device__ __forceinline__ double fp_times_const(double x, bool wide, double w, 
     return s2 < 0.0 ? __dadd_rn(s2, q) : s2;
 }
 
-__global__ void __launch_bounds__(256) finish_division_fp_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
+__global__ void __launch_bounds__(128, 8) finish_division_fp_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
                                                                  const u64* __restrict__ T, u32 n_t, const RescaleConsts rc,
                                                                  u64* __restrict__ low) {
     grid_dependency_enter();
-    const u32 n = blockIdx.x * 256 + threadIdx.x;
+    const u32 n = blockIdx.x * 128 + threadIdx.x;
     const u32 p = blockIdx.y >> 1, comp = blockIdx.y & 1;
     const u64* tp = T + (size_t)p * n_t * R.N + n;
     u64* cp = ct + (size_t)p * ct_stride + (size_t)comp * R.r * R.N + n;
@@ -1315,11 +1578,11 @@ cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, 
     for (u32 i = 0; i < ring.dev.r; ++i) fp = fp && ring.dev.fp_ok[i];
     if (rc && ring.q[ring.dev.r - 1] >= (1ull << 46)) fp = false;
     if (fp) {
-        launch_dependent(ring, finish_division_fp_kernel, dim3(ring.dev.N / 256, n_out * 2), dim3(256), 0, stream, ring.dev,
+        launch_dependent(ring, finish_division_fp_kernel, dim3(ring.dev.N / 128, n_out * 2), dim3(128), 0, stream, ring.dev,
                          ct, ct_stride, T, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
         return cudaGetLastError();
     }
-    launch_dependent(ring, finish_division_kernel, dim3(ring.dev.N / 256, n_out * 2), dim3(256), 0, stream, ring.dev, ct,
+    launch_dependent(ring, finish_division_kernel, dim3(ring.dev.N / 128, n_out * 2), dim3(128), 0, stream, ring.dev, ct,
                      ct_stride, T, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
     return cudaGetLastError();
 }

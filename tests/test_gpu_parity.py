@@ -120,6 +120,26 @@ def test_rotate_matches_oracle(pkey):
         g.close()
 
 
+@pytest.mark.parametrize("logN,n_primes", [(10, 2), (10, 5), (11, 8), (10, 10), (10, 15)])
+def test_rotate_for_every_arrangement_of_digits_in_a_block(logN, n_primes):
+    # the fused transform and inner product gives each digit a warp: several chunks per block where digits are few (more
+    # than a small ring has), one chunk and 8 warps, one warp per digit beyond that
+    par = ckks.Params(1 << logN, ckks.find_primes(1 << 40, 2 << logN, n_primes), ckks.find_primes(1 << 60, 2 << logN, 1)[0], 2.0 ** 30)
+    plan = ckks.Plan(8, 1, 4, 2)
+    s = ckks.keygen(par, 5)
+    keys = ckks.make_rotation_keys(par, s, plan, 5)
+    g = GpuSide(par, plan)
+    try:
+        steps = g.load_keys(keys)
+        ct = ckks.encrypt(par, s, ckks.encode_coeffs(np.arange(par.n) % 7 - 3.0, par.N, par.scale), 6)
+        out = g.empty_u64(2, par.r, par.N)
+        for st in (steps[0], steps[-1]):
+            g.bf.bf_rotate(g.ctx, g.to_dev(ct), st, out)
+            assert np.array_equal(g.to_host_u64(out), ckks.rotate(par, ct, st, keys)), st
+    finally:
+        g.close()
+
+
 @pytest.mark.parametrize("pkey", ["n12", "n15"])
 def test_rescale_matches_oracle(pkey):
     par = oracle_params(pkey)
