@@ -324,6 +324,8 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
             ec[3] = ec[2] / (double)q;
             ec[4] = k;
         }
+        R.key_base[m] = R.key_bytes;
+        R.key_bytes += (u64)(N / KS_TILE) * key_tile_bytes(R.dp[m] != 0, n_ct_primes);
         auto dbits = [](double d) -> u64 {
             u64 bits;
             memcpy(&bits, &d, sizeof(bits));
@@ -486,7 +488,7 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
         return code;
     };
     const size_t key_words = (size_t)r * 2 * nb * N;
-    if (cudaMalloc(&ctx->keys, key_words * n_keys * sizeof(u64)) != cudaSuccess) { ctx->keys = nullptr; return fail(BF_ERR_OOM); }
+    if (cudaMalloc(&ctx->keys, (size_t)ctx->ring.dev.key_bytes * n_keys) != cudaSuccess) { ctx->keys = nullptr; return fail(BF_ERR_OOM); }
     if (cudaMalloc(&ctx->perms, (size_t)n_keys * N * sizeof(u32)) != cudaSuccess) { ctx->perms = nullptr; return fail(BF_ERR_OOM); }
     // permutation tables: position i of the transform holds the evaluation at psi^(2*brev(i)+1);
     // a(X) -> a(X^g) maps it to the evaluation at exponent (2*brev(i)+1)*g mod 2N, so the rotated

@@ -42,6 +42,8 @@ struct RingDev {
     u32 dp[MAX_MODULI];          // modulus below 2^40: operands of the inner products (cached plaintexts, rotation keys, digits)
                                  //   are kept as the bits of doubles and multiplied in fp64 (see DpAcc)
     double c40_d[MAX_MODULI], c40_q[MAX_MODULI];       // (double)(2^40 mod q) and that over q
+    u64 key_base[MAX_MODULI];    // resident rotation keys (see KeyTile): byte offset of modulus m inside a key
+    u64 key_bytes;               //   bytes of a key
     // encoder output (signed 64-bit coefficients) into Montgomery form on the fp64 path: the word is
     // (hi' - 2^31) 2^32 + lo, so times 2^64 it is  hi' (2^96 mod q) + lo (2^64 mod q) - (2^127 mod q).
     // Five doubles per prime, in device memory (kernel parameters stay small): (double)(2^96 mod q), that
@@ -224,7 +226,8 @@ struct MacScatter {
 struct BabySteps {
     u32 n_in, b;
     u32 parts, per_part;                // how the inputs are dealt out to a block's lanes (set by the launcher)
-    const u64 *keys, *dig;              // resident keys; digit set q of input q (tile-major, see ks_tile_index)
+    const void* keys;                   // resident keys
+    const u64* dig;                     // digit set q of input q (tile-major, see ks_tile_index)
     u32 key[MAX_ROT_BATCH + 1];
     u32 gal[MAX_ROT_BATCH + 1], gal_inv[MAX_ROT_BATCH + 1];
 };
@@ -327,10 +330,10 @@ struct PolyBatch {
 };
 
 // Operands of the key-switch inner product (digit sets and rotation keys) are kept tile-major, so that what a block
-// needs of one (outer index / div, modulus, tile) is contiguous and arrives by one bulk copy:
+// needs of one (outer index / div, modulus, tile) is contiguous:
 //   polynomial (o, m), coefficient n  ->  ((((o / div) * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + o % div) * KS_TILE + n % KS_TILE
 // digits: o = set * r + digit, div = r (a block reads the r digit segments of a set, modulus and tile);
-// keys: o = (key * r + digit) * 2 + component, div = 2r.
+// (keys: see KeyTile)
 constexpr u32 KS_TILE = 128;
 __host__ __device__ __forceinline__ size_t ks_tile_index(u32 N, u32 n_m, u32 div, u32 o, u32 m, u32 n) {
     return ((((size_t)(o / div) * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + o % div) * KS_TILE + n % KS_TILE;
@@ -386,6 +389,11 @@ __device__ __forceinline__ u64 stream_policy() {
 }
 __device__ __forceinline__ void ld_stream(const void* p, u64 policy, u32& lo, u32& hi) {
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;" : "=r"(lo), "=r"(hi) : "l"(p), "l"(policy));
+}
+__device__ __forceinline__ u32 ld_stream32(const void* p, u64 policy) {
+    u32 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
+    return v;
 }
 
 // ---- Sums of products of residues, three ways.  B200 issues 64 fp64 multiply-adds per SM and clock, but only 32
@@ -446,7 +454,49 @@ __device__ __forceinline__ void cut_limbs(u32 lo, u32 hi, u32 L, u32& w0, u32& w
     w1 = __funnelshift_r(lo, hi, L);
 }
 
-// One output word of the key-switch inner product: digits times key words (as stored), summed, in [0, q).  The keys carry a
+// Resident rotation keys: [key][modulus][tile of KS_TILE coefficients], a tile holding the 2r segments s = 2 digit + component
+// in turn.  The multiply-accumulate and the inner products read each key once and are bound by those bytes, so residues of
+// primes below 2^40 (RingDev::dp) take five: the low 32 bits, [2r][KS_TILE] words, then the high bytes of four segments at a
+// time, [(2r + 3) / 4][KS_TILE] words.  (Over the four calls of a 0.6B layer the keys are 60 % of the bytes.)  The others are
+// 8-byte words with a factor 2^64.
+__host__ __device__ __forceinline__ u32 key_tile_bytes(bool dp, u32 r) { return dp ? (2 * r + (2 * r + 3) / 4) * KS_TILE * 4 : 2 * r * KS_TILE * 8; }
+__device__ __forceinline__ const unsigned char* key_tile(const RingDev& R, const void* keys, u32 key, u32 m, u32 tile) {
+    return (const unsigned char*)keys + key * R.key_bytes + R.key_base[m] + (size_t)tile * key_tile_bytes(R.dp[m] != 0, R.r);
+}
+__device__ __forceinline__ void key_store(const RingDev& R, void* keys, u32 key, u32 m, u32 s, u32 n, u64 v) {      // v in [0, q)
+    unsigned char* t = const_cast<unsigned char*>(key_tile(R, keys, key, m, n / KS_TILE));
+    const u32 c = n % KS_TILE;
+    if (R.dp[m]) {
+        ((u32*)t)[s * KS_TILE + c] = (u32)v;
+        t[((size_t)(2 * R.r + s / 4) * KS_TILE + c) * 4 + s % 4] = (unsigned char)(v >> 32);
+    } else {
+        ((u64*)t)[s * KS_TILE + c] = mul_shoup(v, R.c64[m], R.c64s[m], R.q[m]);
+    }
+}
+// Coefficient c of a tile: the words of segments as they are stored (OP_DP: low words, and high[s / 4] with the high bytes),
+// cut into the form KeyDot and DigitDot multiply.
+template <int CLS>
+struct KeyTile {
+    const unsigned char* at;
+    u32 r;
+    __device__ __forceinline__ KeyTile(const unsigned char* tile, u32 c, u32 r_) : at(tile + (CLS == OP_DP ? 4 : 8) * c), r(r_) {}
+    __device__ __forceinline__ u32 high(u32 group, u64 pol) const { return CLS == OP_DP ? ld_stream32(at + (2 * r + group) * KS_TILE * 4, pol) : 0u; }
+    __device__ __forceinline__ void word(u32 s, u64 pol, u32& k0, u32& k1) const {
+        if (CLS == OP_DP) k0 = ld_stream32(at + s * KS_TILE * 4, pol);
+        else ld_stream(at + s * KS_TILE * 8, pol, k0, k1);
+    }
+    static __device__ __forceinline__ void cut(u32 s, u32 high, u32& k0, u32& k1) {
+        if (CLS == OP_DP) {                 // 2^52 + the 40-bit word, minus 2^52
+            const double d = __dsub_rn(__hiloint2double((int)__byte_perm(high, 0x43300000u, 0x7650u + s % 4), (int)k0), 4503599627370496.0);
+            k0 = (u32)__double2loint(d);
+            k1 = (u32)__double2hiint(d);
+        } else {
+            cut_limbs(k0, k1, CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW, k0, k1);
+        }
+    }
+};
+
+// One output word of the key-switch inner product: digits times key words (cut), summed, in [0, q).  The keys carry a
 // factor 2^64 except where the class is OP_DP.
 template <int CLS>
 struct DigitDot {
@@ -455,7 +505,6 @@ struct DigitDot {
     __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1) {
         u32 d0, d1;
         cut_limbs(d.x, d.y, L, d0, d1);
-        cut_limbs(k0, k1, L, k0, k1);
         a.mac(d0, d1, d0 + d1, k0, k1);
     }
     __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const { return a.reduce(R.q[m], (u32)R.qneg[m]); }
@@ -478,7 +527,6 @@ struct KeyDot {
         a0.mac(d0, d1, d0 + d1, k0, k1);
         a1.mac(d0, d1, d0 + d1, l0, l1);
     }
-    static __device__ __forceinline__ void cut(u32& k0, u32& k1) { cut_limbs(k0, k1, CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW, k0, k1); }
     __device__ __forceinline__ void reduce(const RingDev& R, u32 m, u64& v0, u64& v1) const {
         v0 = a0.reduce(R.q[m], (u32)R.qneg[m]);
         v1 = a1.reduce(R.q[m], (u32)R.qneg[m]);
@@ -492,7 +540,6 @@ struct KeyDot<OP_DP> {
         a0.mac(dd, __hiloint2double((int)k1, (int)k0));
         a1.mac(dd, __hiloint2double((int)l1, (int)l0));
     }
-    static __device__ __forceinline__ void cut(u32&, u32&) {}
     __device__ __forceinline__ void reduce(const RingDev& R, u32 m, u64& v0, u64& v1) const {
         v0 = d2u(a0.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));
         v1 = d2u(a1.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));

@@ -79,7 +79,7 @@ cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 
 // rc, low non-null: the rescale from r primes follows in the same kernel; the result goes to low ([n_out][2][r-1][N])
 cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_t, u32 n_out,
                             cudaStream_t stream, const RescaleConsts* rc = nullptr, u64* low = nullptr);
-cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, u64* final_dst,
+cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, void* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream);
 
 // First pass alone of a forward transform of digits (LOAD_REDUCE).
@@ -91,7 +91,7 @@ cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_ou
 // as a rotated input in the extended basis, xext[rb.out[rot]][comp][m][pinv[..][n]] = u'[comp][m][n] + (comp == 0 ?
 // xext[rb.c0[rot]][0][m][n] : 0), terms of [2][r+1][N] words (term rb.c0[rot] holds P times the un-rotated input).
 // Rotations of the same set have to be consecutive.
-cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B, u32 n_sets, const RotBatch& rb, const u64* keys, u64* u, u64* xext,
+cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B, u32 n_sets, const RotBatch& rb, const void* keys, u64* u, u64* xext,
                               const u32* pinv, cudaStream_t stream);
 
 // ---- kernels.cu : element-wise and streaming kernels of the linear layer

@@ -30,11 +30,6 @@ __device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
     return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
 }
 
-__device__ __forceinline__ u32 ld_stream32(const void* p, u64 policy) {
-    u32 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
-    return v;
-}
 __device__ __forceinline__ u32 ld_stream8(const void* p, u64 policy) {
     u32 v;
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u8 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
@@ -121,15 +116,18 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             const u32 q_end = min(n_in, (part + 1) * bs.per_part);
             const u32 src = (automorphism_index(n0, bs.gal[k], logN) & ~(TN - 1)) + c;
             const u32 cd = automorphism_index(src, bs.gal_inv[k], logN) & (TN - 1);
-            const u64* kp = bs.keys + ks_tile_base(N, r + 1, 2 * r, bs.key[k], 0u, i) + (size_t)(src / KS_TILE) * 2 * r * KS_TILE + src % KS_TILE;
+            const KeyTile<CLS> kt(key_tile(R, bs.keys, bs.key[k], i, src / KS_TILE), src % KS_TILE, r);
             const u64* dp = bs.dig + ks_tile_base(N, r + 1, r, part * bs.per_part, 0u, i) + (size_t)(src / KS_TILE) * r * KS_TILE + src % KS_TILE;
             const size_t dig_stride = ks_tile_base(N, r + 1, r, 1u, 0u, 0u);
             u32 k0[RC > 0 ? 2 * RC : 1], k1[RC > 0 ? 2 * RC : 1];
             if constexpr (RC > 0) {
+                u32 high[(2 * RC + 3) / 4];
 #pragma unroll
-                for (int s = 0; s < 2 * RC; ++s) ld_stream(kp + s * KS_TILE, pol, k0[s], k1[s]);
+                for (int s = 0; s < 2 * RC; ++s) kt.word(s, pol, k0[s], k1[s]);
 #pragma unroll
-                for (int s = 0; s < 2 * RC; ++s) KeyDot<CLS>::cut(k0[s], k1[s]);
+                for (int h = 0; h < (2 * RC + 3) / 4; ++h) high[h] = kt.high(h, pol);
+#pragma unroll
+                for (int s = 0; s < 2 * RC; ++s) KeyTile<CLS>::cut(s, high[s / 4], k0[s], k1[s]);
             }
             for (u32 qi = part * bs.per_part; qi < q_end; ++qi, dp += dig_stride) {
                 KeyDot<CLS> dot;
@@ -143,9 +141,12 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
                 } else {
 #pragma unroll 4
                     for (u32 j = 0; j < r; ++j) {
-                        uint2 ka = __ldg((const uint2*)(kp + (2 * j) * KS_TILE)), kb = __ldg((const uint2*)(kp + (2 * j + 1) * KS_TILE));
-                        KeyDot<CLS>::cut(ka.x, ka.y);
-                        KeyDot<CLS>::cut(kb.x, kb.y);
+                        uint2 ka, kb;
+                        kt.word(2 * j, pol, ka.x, ka.y);
+                        kt.word(2 * j + 1, pol, kb.x, kb.y);
+                        const u32 high = kt.high(j / 2, pol);
+                        KeyTile<CLS>::cut(2 * j, high, ka.x, ka.y);
+                        KeyTile<CLS>::cut(2 * j + 1, high, kb.x, kb.y);
                         dot.mac(__ldg((const uint2*)(dp + j * KS_TILE)), ka.x, ka.y, kb.x, kb.y);
                     }
                 }

@@ -889,12 +889,10 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     ((ulonglong2*)zp)[1] = make_ulonglong2(0, 0);
                 }
             }
-            if (B.scatter) {    // rotation keys: tile-major, permuted by their automorphism, in the form the inner products read
+            if (B.scatter) {    // rotation keys: permuted by their automorphism, in the form the inner products read
                 const u32* sc = B.scatter + (size_t)(o / B.scatter_div) * R.N + chunk * LEN + 4 * s;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    B.dtile_ptr[ks_tile_index(R.N, B.n_m, B.dtile_div, o, m, sc[i])] =
-                        dp ? operand_word(R, mod, v4[i]) : mul_shoup(v4[i], R.c64[mod], R.c64s[mod], q);
+                for (int i = 0; i < 4; ++i) key_store(R, B.dtile_ptr, o / B.scatter_div, m, o % B.scatter_div, sc[i], v4[i]);
                 continue;
             }
             ulonglong2* gp = (ulonglong2*)(gdst + 4 * s);
@@ -1098,41 +1096,50 @@ __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) 
 template <int RC>
 struct InnerGeo {
     static constexpr int WARPS = RC > 8 ? RC : RC > 0 ? 8 : MAX_MODULI;    // (upper bound where r is not a constant)
-    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 0 ? 4 : 1;
+    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 4 ? 4 : RC > 0 ? 3 : 1;
 };
 template <int CLS, int RC>
 __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch& rb, u32 first, u32 cnt, u32 m, u32 n, const u64* sd,
-                                               const u64* __restrict__ keys, u64* u, u64* xext,
+                                               const void* __restrict__ keys, u64* u, u64* xext,
                                                const u32* __restrict__ pinv, u64 pol) {
     const u32 N = R.N, r = RC > 0 ? RC : R.r, nb = r + 1;
     const u32 at = (u32)swz((int)(n & 255u));
     const size_t out_words = (size_t)2 * nb * N;
     for (u32 rot = first; rot < first + cnt; ++rot) {
-        const u64* kp = keys + ks_tile_base(N, nb, 2 * r, (u32)rb.key[rot], 0u, m) + (size_t)(n / KS_TILE) * 2 * r * KS_TILE + n % KS_TILE;
+        const KeyTile<CLS> kt(key_tile(R, keys, (u32)rb.key[rot], m, n / KS_TILE), n % KS_TILE, r);
         u32 dest = n;
         u64 pc0 = 0;
         if (pinv) dest = __ldg(&pinv[(size_t)rb.key[rot] * N + n]);
         if (xext) pc0 = xext[(size_t)rb.c0[rot] * out_words + (size_t)m * N + n];
         // (one component at a time: with the key words of both in registers fewer blocks fit an SM)
-        auto component = [&](const u64* kc) -> u64 {
+        u32 high[RC > 0 ? (2 * RC + 3) / 4 : 1];
+        if constexpr (RC > 0) {
+#pragma unroll
+            for (int h = 0; h < (2 * RC + 3) / 4; ++h) high[h] = kt.high(h, pol);
+        }
+        auto component = [&](u32 comp) -> u64 {
             DigitDot<CLS> dot;
             if constexpr (RC > 0) {
                 u32 k0[RC], k1[RC];
 #pragma unroll
-                for (int j = 0; j < RC; ++j) ld_stream(kc + 2 * j * KS_TILE, pol, k0[j], k1[j]);
+                for (int j = 0; j < RC; ++j) kt.word(2 * j + comp, pol, k0[j], k1[j]);
 #pragma unroll
-                for (int j = 0; j < RC; ++j) dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
+                for (int j = 0; j < RC; ++j) {
+                    KeyTile<CLS>::cut(2 * j + comp, high[j / 2], k0[j], k1[j]);
+                    dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
+                }
             } else {
 #pragma unroll 4
                 for (u32 j = 0; j < r; ++j) {
                     u32 k0, k1;
-                    ld_stream(kc + 2 * j * KS_TILE, pol, k0, k1);
+                    kt.word(2 * j + comp, pol, k0, k1);
+                    KeyTile<CLS>::cut(2 * j + comp, kt.high(j / 2, pol), k0, k1);
                     dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0, k1);
                 }
             }
             return dot.reduce(R, m);
         };
-        const u64 v0 = component(kp), v1 = component(kp + KS_TILE);
+        const u64 v0 = component(0), v1 = component(1);
         // xext (double hoisting): the rotated input in the extended basis is (P*c0 + u0, u1) moved through the rotation's
         // permutation; P*c0 (zero modulo P) was stored as the un-rotated term
         u64* up = xext ? xext + (size_t)rb.out[rot] * out_words + (size_t)m * N + dest : u + (size_t)rb.out[rot] * out_words + (size_t)m * N + dest;
@@ -1143,7 +1150,7 @@ __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch&
 
 template <int RC>
 __global__ void __launch_bounds__(32 * InnerGeo<RC>::WARPS, InnerGeo<RC>::BLOCKS)
-ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const u64* __restrict__ keys, u64* u, u64* xext,
+ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const void* __restrict__ keys, u64* u, u64* xext,
                  const u32* __restrict__ pinv, u32 cb) {
     extern __shared__ __align__(128) u64 sm_all[];          // [cb][r] slices
     grid_dependency_enter();
@@ -1159,8 +1166,8 @@ ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const u6
     c.qinv = R.qinv_d[m];
     const bool dp = R.dp[m] != 0;
     if (threadIdx.x < cb * 2 && chunk0 + threadIdx.x / 2 < (N >> LOG_C)) {      // the first rotation's keys, on their way to L2
-        const u64* kp = keys + ks_tile_base(N, nb, 2 * r, (u32)rb.key[first], 0u, m) + (size_t)(chunk0 * 2 + threadIdx.x) * 2 * r * KS_TILE;
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kp), "r"(2 * r * KS_TILE * 8) : "memory");
+        const unsigned char* kp = key_tile(R, keys, (u32)rb.key[first], m, chunk0 * 2 + threadIdx.x);
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kp), "r"(key_tile_bytes(dp, r)) : "memory");
     }
     for (u32 w = threadIdx.x >> 5; w < cb * r; w += warps) {
         const u32 chunk = chunk0 + w / r, j = w % r;
@@ -1346,7 +1353,7 @@ cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_
 
 // Forward transform whose final store is permuted: polynomial (o, m) ends up at
 // final[(o*dst_so + m*dst_sm) + scatter[(o / scatter_div)*N + n]].  B.dst is a staging buffer of the same shape.
-cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B0, u32 n_outer, int load, u64* final_dst,
+cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B0, u32 n_outer, int load, void* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream) {
     PolyBatch B = B0;
     const u32 n_polys = n_outer * B.n_m;
@@ -1356,8 +1363,7 @@ cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B0, u32 n_o
     if (e != cudaSuccess) return e;
     B.scatter = scatter;
     B.scatter_div = scatter_div;
-    B.dtile_ptr = final_dst;      // tile-major: o = (key * r + digit) * 2 + component
-    B.dtile_div = scatter_div;
+    B.dtile_ptr = (u64*)final_dst;
     return launch_contig<true>(ring, B, n_polys, stream);
 }
 
@@ -1366,7 +1372,7 @@ cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_ou
 }
 
 template <int RC>
-static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const u64* keys, u64* u, u64* xext,
+static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const void* keys, u64* u, u64* xext,
                                          const u32* pinv, cudaStream_t stream) {
     const u32 r = ring.dev.r, chunks = ring.dev.N >> LOG_C;
     const u32 warps = r > 8 ? r : 8u;
@@ -1376,7 +1382,7 @@ static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& 
                             (size_t)8 * (cb * r << LOG_C), stream, ring.dev, B, rb, keys, u, xext, pinv, cb);
 }
 
-cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n_sets, const RotBatch& rb_in, const u64* keys, u64* u,
+cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n_sets, const RotBatch& rb_in, const void* keys, u64* u,
                               u64* xext, const u32* pinv, cudaStream_t stream) {
     const u32 r = ring.dev.r;
     if (rb_in.n == 0) return cudaSuccess;
@@ -1404,7 +1410,7 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
         t = end;
     }
     if (ring.prof) {
-        const u64 key_bytes = (u64)r * 2 * (r + 1) * ring.dev.N * 8;
+        const u64 key_bytes = ring.dev.key_bytes;
         u32 distinct = 0;
         for (int t = 0; t < rb.n; ++t) {
             bool seen = false;
