@@ -149,7 +149,7 @@ struct bf_ctx {
     // on side streams between a fork and a join, so that one chain's HBM-bound inner product overlaps
     // another chain's arithmetic-bound transforms.  lane 0 is the context's stream.
     static constexpr int MAX_LANES = 4;
-    int n_lanes = 2;                // measured: two chains overlap best (0.651 -> 0.625 ms on the 768 x 2304 layer)
+    int n_lanes = 2;                // (set with the ring)
     cudaStream_t side[MAX_LANES - 1] = {nullptr, nullptr, nullptr};
     cudaEvent_t ev_fork = nullptr, ev_join[MAX_LANES - 1] = {nullptr, nullptr, nullptr};
     // stage timing
@@ -259,6 +259,10 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     memset(&R, 0, sizeof(R));
     R.N = N;
     R.logN = ctx->logN;
+    // two chains overlap where their kernels fill the GPU in part (N = 2^15, four calls of a 0.6B layer: 1385 us as one, 1371 as
+    // two); on small rings they are twice as many launches of the same length (N = 2^12, 64 x 64: 78 us as one, 84 as two;
+    // 300 x 1000 under double hoisting 57 and 59; N = 2^13, 768 x 2304: 296 and 297)
+    ctx->n_lanes = N >= (1u << 14) ? 2 : 1;
     R.r = n_ct_primes;
     ctx->ring.q.assign(primes, primes + nb);
     const u64 P = primes[n_ct_primes];
@@ -783,7 +787,7 @@ static Lane main_lane(bf_ctx* ctx) {
 
 static int ensure_lanes(bf_ctx* ctx) {
     if (!ctx->ev_fork) CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
-    const int n_side = ctx->n_lanes > 2 ? ctx->n_lanes - 1 : 1;       // (one side stream at least: the special prime's MAC)
+    const int n_side = ctx->n_lanes > 2 ? ctx->n_lanes - 1 : 1;
     for (int i = 0; i < n_side && i + 1 < bf_ctx::MAX_LANES; ++i) {
         if (!ctx->side[i]) CK(cudaStreamCreateWithFlags(&ctx->side[i], cudaStreamNonBlocking));
         if (!ctx->ev_join[i]) CK(cudaEventCreateWithFlags(&ctx->ev_join[i], cudaEventDisableTiming));
@@ -975,7 +979,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     const u32 groups = groups_fit < 1 ? 1u : groups_fit > (size_t)n_pj ? n_pj : (u32)groups_fit;
     // the multiply-accumulate makes the rotated inputs itself, unless it runs in several rounds: each would stream the
     // keys again, so that X is worth keeping in memory then
-    const bool rotate_in_mac = dh && (resident || groups == n_pj);
+    const bool rotate_in_mac = dh && b > 1 && (resident || groups == n_pj);
     if (rotate_in_mac) in_batch = n_in;
     u32 n_dig_sets = giant_per_lane * (u32)lanes;       // digit sets alive at once
     // (the digits that the multiply-accumulate reads lie before those between the passes)
@@ -984,7 +988,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     const size_t xw = (size_t)2 * nmp * N;                // words per term of X / per inner sum
     TRY(ensure(ctx, ctx->X, (size_t)n_in * (rotate_in_mac ? 1u : b) * xw * 8));
     if (dh) {
-        TRY(ensure(ctx, ctx->X0, (size_t)n_in * ctw * 8));
+        TRY(ensure(ctx, ctx->X0, (size_t)n_in * (rotate_in_mac ? ctw / 2 : ctw) * 8));
         TRY(ensure(ctx, ctx->Aext, (size_t)n_out * g * xw * 8));
     }
     TRY(ensure(ctx, ctx->A, (size_t)n_out * g * ctw * 8));
@@ -1034,36 +1038,49 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     PolyBatch B;
     memset(&B, 0, sizeof(B));
     // X[q][0] = NTT(ct_q): polynomial (q, component*r + prime).  Double hoisting keeps it apart (X0: the hoisted ModUp
-    // copies its c1 part) and puts P * NTT(ct_q), zero modulo P, into X (term q*b, or term q where the
-    // multiply-accumulate makes the rotated ones itself)
+    // copies its c1 part) and puts P * NTT(ct_q), zero modulo P, into X (term q*b).  Where the multiply-accumulate makes the
+    // rotated inputs itself, X holds the un-rotated terms only, and they and the digits come out of the same two launches
     u64* X0 = dh ? (u64*)ctx->X0.p : X;
     const long long x0_stride = dh ? (long long)ctw : (long long)b * ctw;
-    B.src = ct_in;
-    B.dst = X0;
-    B.src_so = (long long)ctw;
-    B.dst_so = x0_stride;
-    B.src_sm = B.dst_sm = N;
-    B.n_m = 2 * r;
-    B.mod_wrap = r;
-    B.mod0 = 0;
-    B.mod_step = 1;
-    if (dh) {                   // the transform's last store also writes P * NTT(ct_q) into X
+    if (rotate_in_mac) {
+        u64* mid = Dig + (size_t)n_in * r * nb * N;
+        B.src = ct_in;
+        B.o_div = r;                        // o = (input * 2 + component) * r + prime
+        B.src_so2 = (long long)r * N;
+        B.src_so = N;
+        B.dst = mid;
+        B.dst_so = (long long)nb * N;
+        B.dst_sm = N;
+        B.mod_step = 1;
+        B.src_digits = 1;
+        B.tail_dst = (u64*)ctx->X0.p;
+        B.dtile_ptr = Dig;
+        B.dtile_div = r;
         B.lift_ptr = X;
-        B.lift_so = (long long)(rotate_in_mac ? 1u : b) * (long long)xw;
+        B.lift_so = (long long)xw;
+        CK(ntt_forward_ingest(ctx->ring, B, n_in, ctx->stream));
+    } else {
+        B.src = ct_in;
+        B.dst = X0;
+        B.src_so = (long long)ctw;
+        B.dst_so = x0_stride;
+        B.src_sm = B.dst_sm = N;
+        B.n_m = 2 * r;
+        B.mod_wrap = r;
+        B.mod0 = 0;
+        B.mod_step = 1;
+        if (dh) {                   // the transform's last store also writes P * NTT(ct_q) into X
+            B.lift_ptr = X;
+            B.lift_so = (long long)b * (long long)xw;
+            B.lift_zero = 1;
+        }
+        CK(ntt_forward(ctx->ring, B, n_in, LOAD_PLAIN, ctx->stream));
     }
-    CK(ntt_forward(ctx->ring, B, n_in, LOAD_PLAIN, ctx->stream));
-    if (b > 1) {
+    if (b > 1 && !rotate_in_mac) {
         for (u32 q0 = 0; q0 < n_in; q0 += in_batch) {
             const u32 qn = (n_in - q0 < in_batch) ? n_in - q0 : in_batch;
-            PolyBatch D0 = modup_batch(ctx, ct_in + (size_t)q0 * ctw + (size_t)r * N, (long long)ctw, Dig, X0 + (size_t)q0 * x0_stride + (size_t)r * N,
-                                       x0_stride);
-            if (rotate_in_mac) {            // the digits stay, in the form the multiply-accumulate reads
-                D0.dst = Dig + (size_t)qn * r * nb * N;
-                D0.dtile_ptr = Dig;
-                D0.dtile_div = r;
-                CK(ntt_forward(ctx->ring, D0, qn * r, LOAD_REDUCE, ctx->stream));
-                continue;
-            }
+            const PolyBatch D0 = modup_batch(ctx, ct_in + (size_t)q0 * ctw + (size_t)r * N, (long long)ctw, Dig, X0 + (size_t)q0 * x0_stride + (size_t)r * N,
+                                             x0_stride);
             // the rotations of the batch, dealt out to the lanes by whole keys, so that no key is streamed by two lanes; the
             // first pass of the digits' transforms is shared
             const u32 per = cdiv(b - 1, (u32)lanes_baby);
@@ -1270,29 +1287,20 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
             epi.n_out = n_out;
             epi.assemble = 1;
             const u32 n_t = g + 3;
-            const bool beside = lanes > 1;
-            if (beside) TRY(fork_lanes(ctx, 2));
             memset(&B, 0, sizeof(B));
             B.src = epi.aext;                                   // (read through epi)
-            B.dst = (u64*)ctx->Tc.p;
-            B.dst_so = (long long)n_t * N;
-            B.dst_sm = N;
-            B.n_m = n_t;
-            B.mod0 = r;
-            B.mod_step = 0;
-            B.store_centred = 1;
-            CK(ntt_inverse_gathersum(ctx->ring, B, n_out, rb, epi, beside ? ctx->side[0] : ctx->stream));
-            memset(&B, 0, sizeof(B));
-            B.src = epi.aext;
             B.dst = ct_out;
             B.dst_so = (long long)ctw;
             B.dst_sm = N;
-            B.n_m = 2 * r;
+            B.n_m = 2 * r + n_t;
             B.mod_wrap = r;
             B.mod0 = 0;
             B.mod_step = 1;
+            B.tail_m = 2 * r;                                   // the residues modulo P
+            B.tail_dst = (u64*)ctx->Tc.p;
+            B.tail_so = (long long)n_t * N;
+            B.store_centred = 2;
             CK(ntt_inverse_gathersum(ctx->ring, B, n_out, rb, epi, ctx->stream));
-            if (beside) TRY(join_lanes(ctx, 2));
             CK(finish_division(ctx->ring, ct_out, (long long)ctw, (const u64*)ctx->Tc.p, n_t, n_out, ctx->stream,
                                ct_low ? &rcs : nullptr, ct_low));
             stamp(ctx, 3);

@@ -161,6 +161,7 @@ enum LoadMode : int {
     LOAD_I64 = 2,       // signed 64-bit integer coefficient: x mod q in [0, q)
     LOAD_CENTRED = 3,   // centred lift t' in (-M/2, M/2] of a residue of modulus M, stored as t' + 2^59: t' mod q
     LOAD_I64_MONT = 4,  // LOAD_I64, then times 2^64 mod q: the transform's output is in Montgomery form
+    LOAD_INGEST = 5,    // LOAD_REDUCE for an ingest batch (see PolyBatch::ingest)
 };
 
 constexpr int MAX_ROT_BATCH = 64; // rotations handled by one key-switch launch
@@ -310,17 +311,28 @@ struct PolyBatch {
     TileLayout tile;              //   (forward writes its final result there, inverse reads its input there);
     u32 tile_pj0, o_base;         //   diagonal o_base + o = pj*n_terms + t; the layout's group 0 is group tile_pj0
     u32 skip_diag;                // forward only: polynomial (o, m) with m < r and o % r == m (a digit in its own prime)
-    const u64* diag_src;          //   is not transformed but copied from diag_src + (o / r)*diag_so + m*N, where its
+    const u64* diag_src;          //   is not transformed but read from diag_src + (o / r)*diag_so + m*N, where its
     long long diag_so;            //   transform already exists
     const u32* scatter;           // forward only (rotation keys): coefficient n of the result goes to position
     u32 scatter_div;              //   scatter[(o / scatter_div) * N + n] of dtile_ptr
     u32 split_bits;               // tile-major side: 8-byte words modulo primes without RingDev::dp are stored as two limbs,
                                   //   (v >> L) << 32 | (v & (2^L - 1)), L = split_bits below 2^50, else 30
-    u64* lift_ptr;                // forward only, non-null (double hoisting): polynomial (o, m = comp * mod_wrap + i) is also
-    long long lift_so;            //   stored times P mod q_i at lift_ptr + o*lift_so + (comp*(r+1) + i)*N, and zeros as the
-                                  //   residue modulo P: the un-rotated input lifted to the extended basis
-    u64* dtile_ptr;               // forward only, non-null: the final result goes there instead of dst, tile-major in tiles
-    u32 dtile_div;                //   of KS_TILE coefficients (see ks_tile_index); with `scatter` the store is permuted
+    u64* lift_ptr;                // forward only, non-null (double hoisting): the transform of component comp of input o modulo
+    long long lift_so;            //   q_i is also stored times P mod q_i at lift_ptr + o*lift_so + (comp*(r+1) + i)*N: the
+                                  //   un-rotated input lifted to the extended basis (its residue modulo P is zero; it is only
+                                  //   written where lift_zero is set)
+    u32 lift_zero;
+    // inverse only, tail_m > 0: slots m >= tail_m are polynomials modulo the special prime with a destination of their own,
+    u32 tail_m;                   //   tail_dst + o*tail_so + (m - tail_m)*dst_sm
+    u64* tail_dst;
+    long long tail_so;
+    // forward only, ingest = 1 (the inputs of a double-hoisted call and their digits in one go): source o = (input, component,
+    // prime j).  Component 1 is transformed into every prime (digit j; n_m = r + 1 slots), component 0 into its own only, and
+    // passes through tail_dst + (input * r + j) * N between the passes.  The second pass takes outer index (input, j) and
+    // slots m <= r of component 1, m = r + 1 component 0; see EPI 5 of the contiguous pass
+    u32 ingest;
+    u64* dtile_ptr;               // ingest: the digits' transforms go there, tile-major in tiles of KS_TILE coefficients (see
+    u32 dtile_div;                //   ks_tile_index, div = r); with `scatter` the resident keys
     u32 o_div_magic, dtile_magic; // ceil(2^32 / o_div), ceil(2^32 / dtile_div): o / d = umulhi(o, magic) for o < 2^16
                                   //   (set by the launchers; 0 = divide)
     const u64* div_t;             // forward from a shared source, non-null (double hoisting): the source of digit

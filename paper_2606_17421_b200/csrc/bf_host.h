@@ -82,6 +82,8 @@ cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, 
 cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, void* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream);
 
+// The inputs of a double-hoisted call and their digits (see PolyBatch::ingest; B names source, buffers and outputs).
+cudaError_t ntt_forward_ingest(const RingHost& ring, const PolyBatch& B, u32 n_in, cudaStream_t stream);
 // First pass alone of a forward transform of digits (LOAD_REDUCE).
 cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_outer, cudaStream_t stream);
 // Digits of n_sets sets (B: LOAD_REDUCE from a shared source, B.dst = room for the [n_sets * r][r + 1][N] words between the

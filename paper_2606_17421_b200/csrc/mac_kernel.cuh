@@ -107,8 +107,8 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         const u32 r = R.r;
         const u32 b = bs.b, n_in = bs.n_in;
         // term (q, 0): P times the un-rotated input
-        for (u32 e = l; e < n_in * 2; e += PL)
-            xs[(size_t)((e >> 1) * b * 2 + (e & 1)) * TN + c] = Acc::x_word(__ldg(x + ((size_t)e * np + i) * N + n0 + c));
+        for (u32 e = l; e < n_in * 2; e += PL)      // (zero modulo P, and not stored there)
+            xs[(size_t)((e >> 1) * b * 2 + (e & 1)) * TN + c] = Acc::x_word(i < r ? __ldg(x + ((size_t)e * np + i) * N + n0 + c) : 0ull);
         // rotations: an item is a key and a part of the inputs that share it
         const u32 n_items = (b - 1) * bs.parts;
         for (u32 it = l; it < n_items; it += PL) {
@@ -131,7 +131,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             }
             for (u32 qi = part * bs.per_part; qi < q_end; ++qi, dp += dig_stride) {
                 KeyDot<CLS> dot;
-                const u64 pc0 = __ldg(x + ((size_t)qi * 2 * np + i) * N + src);
+                const u64 pc0 = i < r ? __ldg(x + ((size_t)qi * 2 * np + i) * N + src) : 0ull;
                 if constexpr (RC > 0) {
                     uint2 dw[RC];
 #pragma unroll

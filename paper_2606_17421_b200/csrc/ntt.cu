@@ -351,6 +351,17 @@ __device__ __forceinline__ LoadConsts load_consts(const RingDev& R, const PolyBa
     return lc;
 }
 
+template <bool TAIL>
+__device__ __forceinline__ u64* batch_dst(const PolyBatch& B, u32 o, u32 m) {
+    if (TAIL && B.tail_m && m >= B.tail_m) return B.tail_dst + (size_t)o * B.tail_so + (size_t)(m - B.tail_m) * B.dst_sm;
+    return B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
+}
+// the same for a source of an ingest batch (PolyBatch::ingest) and its target m
+__device__ __forceinline__ u64* ingest_dst(const RingDev& R, const PolyBatch& B, u32 o_hi, u32 o_lo, u32 m) {
+    const size_t set = (size_t)(o_hi >> 1) * R.r + o_lo;
+    return o_hi & 1 ? B.dst + set * B.dst_so + (size_t)m * B.dst_sm : B.tail_dst + set * R.N;
+}
+
 // Row `row` of the exchange buffer of a strided tile.  Tiles of 8 columns (64 bytes a row) swap the rows of a pair by bit 2
 // of the row number, so that the two rows a half-warp reads never share banks, whether they are neighbours or 4 apart.
 template <int LOG_LANES>
@@ -359,7 +370,7 @@ __device__ __forceinline__ int exchange_row(int row) { return LOG_LANES == 3 ? r
 // Strided pass: transforms the 2^LOG_R rows (stride 256) of a tile of adjacent columns.  Forward: first pass (reads the
 // batch source through the load functor, or from `staged`, [row][column], where several target primes of the same block
 // read it).  Inverse: second pass (in place, scales by N^{-1}).  tws: the prime's first 2^LOG_R twiddles, in shared memory.
-template <bool FWD, int LOAD, int LOG_R, int LOG_LANES, int PATH, bool STAGED = false>
+template <bool FWD, int LOAD, int LOG_R, int LOG_LANES, int PATH, bool STAGED = false, bool INGEST = false>
 __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u64* tws, u32 o,
                                              u32 m, u32 mod, u32 tile, const LoadConsts& lc, const u64* staged,
                                              const StridedTwiddles<LOG_R>& tw) {
@@ -371,7 +382,14 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
     c.q = R.q[mod];
     c.qd = R.qd[mod];
     c.qinv = R.qinv_d[mod];
-    u64* dst = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm + tile * LANES;
+    u64* dst = nullptr;
+    if constexpr (INGEST) {
+        u32 o_hi, o_lo;
+        split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
+        dst = ingest_dst(R, B, o_hi, o_lo, m) + tile * LANES;
+    } else {
+        dst = batch_dst<!FWD>(B, o, m) + tile * LANES;
+    }
     const char* src = nullptr;
     if constexpr (FWD && !STAGED) {
         u32 o_hi = 0, o_lo = o;
@@ -465,10 +483,12 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
 // first, so that nothing waits for its blocks at the end of the launch.
 __device__ __forceinline__ u32 slot_of_block(u32 y, u32 n_m) { return n_m - 1 - y; }
 // modulus index of slot m of a batch (n_m <= 2 * mod_wrap in every batch that wraps)
-__device__ __forceinline__ u32 batch_modulus(const PolyBatch& B, u32 m) {
+template <bool TAIL>
+__device__ __forceinline__ u32 batch_modulus(const RingDev& R, const PolyBatch& B, u32 m) {
+    if (TAIL && B.tail_m && m >= B.tail_m) return R.r;
     return B.mod0 + ((B.mod_wrap && m >= B.mod_wrap) ? m - B.mod_wrap : m) * B.mod_step;
 }
-// a digit in its own prime (o = set * r + digit with digit == mod), which ModUp copies instead of transforming
+// a digit in its own prime (o = set * r + digit with digit == mod), which ModUp does not transform
 __device__ __forceinline__ bool own_prime(const RingDev& R, const PolyBatch& B, u32 o, u32 mod) {
     if (!B.skip_diag || mod >= R.r) return false;
     u32 hi, lo;
@@ -481,22 +501,6 @@ __device__ __forceinline__ u64 operand_word(const RingDev& R, u32 mod, u64 v) {
     return R.dp[mod] ? (u64)__double_as_longlong(u2d(v)) : v;
 }
 
-// the tile of a digit in its own prime: its transform exists already and is copied into the operand array
-template <int LOG_R, int LOG_LANES>
-__device__ __forceinline__ void copy_own_digit(const RingDev& R, const PolyBatch& B, u32 o, u32 m, u32 mod, u32 tile) {
-    typedef StridedGeo<LOG_R, LOG_LANES> G;
-    const u64* ds = B.diag_src + (size_t)(o / R.r) * B.diag_so + (size_t)mod * R.N;
-    u32 t_hi, t_lo;
-    split_index(o, B.dtile_div, B.dtile_magic, t_hi, t_lo);
-    const size_t tbase = ks_tile_base(R.N, B.n_m, B.dtile_div, t_hi, t_lo, m);
-#pragma unroll 4
-    for (int k = 0; k < G::POINTS / G::NT; ++k) {
-        const int w = threadIdx.x + k * G::NT;
-        const size_t gidx = ((size_t)(w / G::LANES) << LOG_C) + tile * G::LANES + w % G::LANES;
-        B.dtile_ptr[tbase + (gidx / KS_TILE) * B.dtile_div * KS_TILE + gidx % KS_TILE] = operand_word(R, mod, ds[gidx]);
-    }
-}
-
 // grid: x = tile, y = slot m, z = outer index.
 template <bool FWD, int LOAD, int LOG_R, int LOG_LANES>
 __global__ void __launch_bounds__(StridedGeo<LOG_R, LOG_LANES>::NT, StridedGeo<LOG_R, LOG_LANES>::BLOCKS)
@@ -505,15 +509,12 @@ ntt_strided(const RingDev R, const PolyBatch B, u32 n_outer) {
     __shared__ __align__(16) u64 sm[n_groups(LOG_R) > 1 ? G::POINTS : 1];
     __shared__ __align__(16) u64 tws[G::TW_WORDS];
     grid_dependency_enter();
-    const u32 m = slot_of_block(blockIdx.y, B.n_m), mod = batch_modulus(B, m);
+    const u32 m = slot_of_block(blockIdx.y, B.n_m), mod = batch_modulus<!FWD>(R, B, m);
     const int path = path_of(R, mod);
     StridedTwiddles<LOG_R> tw;
     tw.fetch(R, FWD, path, mod);
     for (u32 o = blockIdx.z; o < n_outer; o += gridDim.z) {
-        if (FWD && own_prime(R, B, o, mod)) {
-            if (B.dtile_ptr) copy_own_digit<LOG_R, LOG_LANES>(R, B, o, m, mod, blockIdx.x);
-            continue;
-        }
+        if (FWD && own_prime(R, B, o, mod)) continue;
         const LoadConsts lc = load_consts<LOAD>(R, B, o, mod);
         if (path == PATH_DP) strided_body<FWD, LOAD, LOG_R, LOG_LANES, PATH_DP>(R, B, sm, tws, o, m, mod, blockIdx.x, lc, nullptr, tw);
         else if (path == PATH_WIDE) strided_body<FWD, LOAD, LOG_R, LOG_LANES, PATH_WIDE>(R, B, sm, tws, o, m, mod, blockIdx.x, lc, nullptr, tw);
@@ -526,9 +527,11 @@ ntt_strided(const RingDev R, const PolyBatch B, u32 n_outer) {
 // the P-residues of ModDown): a block stages the source tile in shared memory once and transforms it
 // into targets m_begin .. m_begin + m_count - 1, so the source crosses L2 once per block instead of once per
 // target (and a digit is made, or converted to fp64, once).  grid: x = tile, y = outer index o, z = slice of the targets.
-template <int LOAD, int LOG_R, int LOG_LANES>
+template <int LOAD_MODE, int LOG_R, int LOG_LANES>
 __global__ void __launch_bounds__(StridedGeo<LOG_R, LOG_LANES>::NT, StridedGeo<LOG_R, LOG_LANES>::BLOCKS)
 ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
+    constexpr bool INGEST = LOAD_MODE == LOAD_INGEST;
+    constexpr int LOAD = INGEST ? LOAD_REDUCE : LOAD_MODE;
     typedef StridedGeo<LOG_R, LOG_LANES> G;
     constexpr int LANES = G::LANES, POINTS = G::POINTS, NT = G::NT;
     extern __shared__ __align__(16) u64 shared_src_smem[];
@@ -537,12 +540,17 @@ ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
     u64* tws = sm + POINTS;                         // [2][TW_WORDS] twiddles of the current and the next target
     grid_dependency_enter();
     const u32 o = blockIdx.y, tile = blockIdx.x;
-    const u32 m_begin = slot_of_block(blockIdx.z, gridDim.z) * m_per_block;
-    const u32 m_end = min(B.n_m, m_begin + m_per_block);
-    StridedTwiddles<LOG_R> tw;
-    tw.fetch(R, true, path_of(R, batch_modulus(B, m_begin)), batch_modulus(B, m_begin));
     u32 o_hi = 0, o_lo = o;
     if (B.o_div) split_index(o, B.o_div, B.o_div_magic, o_hi, o_lo);
+    u32 m_begin = slot_of_block(blockIdx.z, gridDim.z) * m_per_block;
+    u32 m_end = min(B.n_m, m_begin + m_per_block);
+    if (INGEST && !(o_hi & 1)) {                  // component 0: into its own prime only
+        if (o_lo < m_begin || o_lo >= m_end) return;
+        m_begin = o_lo;
+        m_end = o_lo + 1;
+    }
+    StridedTwiddles<LOG_R> tw;
+    tw.fetch(R, true, path_of(R, batch_modulus<false>(R, B, m_begin)), batch_modulus<false>(R, B, m_begin));
     // digits of primes on the fp64 path are staged as doubles
     const bool staged_fp = LOAD == LOAD_REDUCE && B.src_digits && B.o_div == R.r && R.fp_ok[o_lo];
     {
@@ -596,22 +604,19 @@ ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
     }
     u32 buf = 0;
     for (u32 m = m_begin; m < m_end; ++m) {
-        const u32 mod = batch_modulus(B, m);
+        const u32 mod = batch_modulus<false>(R, B, m);
         const int path = path_of(R, mod);
         u64* tw_now = tws + buf * G::TW_WORDS;
         tw.put(tw_now, path);
         __syncthreads();            // (also: the source is staged, and the exchange buffer is free again)
-        if (m + 1 < m_end) tw.fetch(R, true, path_of(R, batch_modulus(B, m + 1)), batch_modulus(B, m + 1));
+        if (m + 1 < m_end) tw.fetch(R, true, path_of(R, batch_modulus<false>(R, B, m + 1)), batch_modulus<false>(R, B, m + 1));
         buf ^= 1;
-        if (own_prime(R, B, o, mod)) {
-            if (B.dtile_ptr) copy_own_digit<LOG_R, LOG_LANES>(R, B, o, m, mod, tile);
-            continue;
-        }
+        if (own_prime(R, B, o, mod)) continue;      // (its transform exists already)
         LoadConsts lc = load_consts<LOAD>(R, B, o, mod);
         lc.staged_fp = staged_fp;
-        if (path == PATH_DP) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_DP, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
-        else if (path == PATH_WIDE) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_WIDE, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
-        else strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_INT, true>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+        if (path == PATH_DP) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_DP, true, INGEST>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+        else if (path == PATH_WIDE) strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_WIDE, true, INGEST>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
+        else strided_body<true, LOAD, LOG_R, LOG_LANES, PATH_INT, true, INGEST>(R, B, sm, tw_now, o, m, mod, tile, lc, staged, tw);
     }
 }
 
@@ -670,9 +675,8 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
 // EPI: 0 = none; 1 = division by P per rotation (scatter through the rotation's permutation); 2 = per output
 // (sum over the output's giant rotations, gathered through their permutations); 3 = plain; 4 = output assembly (see
-// ModDownEpilogue).
-// DTILE: the forward result goes to the tile-major operand array of the inner product and nowhere else (ModUp: the
-// hot case; its index arithmetic is hoisted out of the store loop and none of the other store functors is compiled in).
+// ModDownEpilogue); 5 = ingest (see PolyBatch): the digits into the operand array, component c of the inputs times P into
+// lift_ptr.
 constexpr int CONTIG_THREADS = 128, CONTIG_SLOTS = CONTIG_THREADS / 32;
 
 // a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
@@ -688,6 +692,13 @@ __device__ __forceinline__ u64 canonical(T x, const ModConsts& c, bool bits) {
         if (x >= 2 * c.q) x -= 2 * c.q;
         return x >= c.q ? x - c.q : x;
     }
+}
+
+// v * P modulo q_m, v in [0, q_m)
+__device__ __forceinline__ u64 times_p(const RingDev& R, u32 m, u64 v) {
+    u64 hi = 0, lo = 0;
+    mac128(hi, lo, v, R.pmod[m]);
+    return reduce128(hi, lo, R.q[m], R.mu[m], R.c64[m], R.c64s[m]);
 }
 
 // The first two groups of the forward pass over one chunk; the chunk is left in the warp's slice for the third, whose sets
@@ -710,7 +721,7 @@ __device__ __forceinline__ void contig_forward_far(const T* gsrc, u32 slice, int
     __syncwarp();
 }
 
-template <bool FWD, int EPI, int PATH, bool TILED, bool DTILE = false>
+template <bool FWD, int EPI, int PATH, bool TILED>
 __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u32 o, u32 m, u32 mod,
                                             u32 chunk, int lane, const RotBatch& rb, const ModDownEpilogue& epi) {
     typedef typename Elem<PATH>::T T;
@@ -722,7 +733,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     c.qinv = R.qinv_d[mod];
     const u64 q = c.q;
     const void* tw = twiddle_table(R, FWD, PATH, mod);
-    u64* dst = B.dst + (size_t)o * B.dst_so + (size_t)m * B.dst_sm;
+    u64* dst = EPI == 5 && m > R.r ? B.tail_dst + (size_t)o * R.N : batch_dst<EPI == 4>(B, o, m);
     const u64* src = FWD ? dst : (const u64*)B.src + (size_t)o * B.src_so + (size_t)m * B.src_sm;
     const u32 mult = (R.N >> LOG_C) + chunk;                   // twiddle index multiplier of this chunk
     const u64* gsrc = src + (size_t)chunk * LEN;
@@ -730,13 +741,6 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     T e[8];
     const bool dp = R.dp[mod] != 0;         // (the operand arrays hold this prime's words as doubles)
     (void)dp;
-    size_t dtile_base = 0;
-    if constexpr (DTILE) {
-        u32 o_hi, o_lo;
-        split_index(o, B.dtile_div, B.dtile_magic, o_hi, o_lo);
-        dtile_base = ks_tile_base(R.N, B.n_m, B.dtile_div, o_hi, o_lo, m);
-    }
-    (void)dtile_base;
     // byte addresses (shared window) of the thread's base point in each of the three access patterns
     const u32 slice = (u32)__cvta_generic_to_shared(sm);
     const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
@@ -810,11 +814,18 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             // (doubles stay doubles where they are stored as such)
             u64 v4[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, (DTILE || TILED) && dp);
-            if constexpr (DTILE) {
-                // (4 adjacent coefficients never straddle a tile of 128)
-                const u32 n = chunk * LEN + 4 * s;
-                stg4(B.dtile_ptr + dtile_base + (size_t)(n / KS_TILE) * B.dtile_div * KS_TILE + n % KS_TILE, v4[0], v4[1], v4[2], v4[3]);
+            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, (TILED || EPI == 5) && dp);
+            if constexpr (EPI == 5) {
+                const u32 n = chunk * LEN + 4 * s, nbp = R.r + 1;
+                u32 q_in, j;
+                split_index(o, B.dtile_div, B.dtile_magic, q_in, j);
+                if (m <= R.r) stg4(B.dtile_ptr + ks_tile_base(R.N, nbp, R.r, q_in, j, m) + (size_t)(n / KS_TILE) * R.r * KS_TILE + n % KS_TILE, v4[0], v4[1], v4[2], v4[3]);
+                if (mod == j) {             // its own prime: the un-rotated input, times P
+                    u64 p4[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p4[i] = times_p(R, mod, dp ? d2u(__longlong_as_double((long long)v4[i])) : v4[i]);
+                    stg4(B.lift_ptr + (size_t)q_in * B.lift_so + ((size_t)(m <= R.r ? nbp : 0u) + mod) * R.N + n, p4[0], p4[1], p4[2], p4[3]);
+                }
                 continue;
             }
             if (EPI == 2) {
@@ -876,14 +887,10 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 u64* xp = B.lift_ptr + (size_t)o * B.lift_so + ((size_t)comp * nbp + mod) * R.N + (size_t)chunk * LEN + 4 * s;
                 u64 p4[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    u64 hi = 0, lo = 0;
-                    mac128(hi, lo, v4[i], R.pmod[mod]);
-                    p4[i] = reduce128(hi, lo, q, R.mu[mod], R.c64[mod], R.c64s[mod]);
-                }
+                for (int i = 0; i < 4; ++i) p4[i] = times_p(R, mod, v4[i]);
                 ((ulonglong2*)xp)[0] = make_ulonglong2(p4[0], p4[1]);
                 ((ulonglong2*)xp)[1] = make_ulonglong2(p4[2], p4[3]);
-                if (mod == 0) {     // the residue modulo P of P * ct is zero
+                if (B.lift_zero && mod == 0) {     // the residue modulo P of P * ct is zero
                     u64* zp = B.lift_ptr + (size_t)o * B.lift_so + ((size_t)comp * nbp + R.r) * R.N + (size_t)chunk * LEN + 4 * s;
                     ((ulonglong2*)zp)[0] = make_ulonglong2(0, 0);
                     ((ulonglong2*)zp)[1] = make_ulonglong2(0, 0);
@@ -933,14 +940,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     }
                 }
             } else if constexpr (EPI == 4) {   // output assembly in the extended basis (see ModDownEpilogue::assemble)
-                const u32 nb = R.r + 1, g1 = epi.n_sum;
+                const u32 nb = R.r + 1, g1 = epi.n_sum, mt = m - B.tail_m;
                 const size_t n = (size_t)chunk * LEN + 4 * s;
                 u32 comp = 0, ju = 0, jc_lo = 1, jc_hi = 0;    // u-terms of giant steps 1..ju, rotated c0 parts of jc_lo..jc_hi
                 bool ident = false;
                 if (mod < R.r) { comp = m / R.r; ident = true; ju = g1; if (comp == 0) jc_hi = g1; }
-                else if (m < 2) { comp = m; ju = g1; }
-                else if (m < 4) { comp = m - 2; ident = true; }
-                else { jc_lo = jc_hi = m - 3; }
+                else if (mt < 2) { comp = mt; ju = g1; }
+                else if (mt < 4) { comp = mt - 2; ident = true; }
+                else { jc_lo = jc_hi = mt - 3; }
                 v4[0] = v4[1] = v4[2] = v4[3] = 0;
                 if (ident) {
                     const u64* ap = epi.aext + (size_t)o * epi.aext_stride + ((size_t)comp * nb + mod) * R.N + n;
@@ -1057,23 +1064,25 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
 // grid: x = groups of CONTIG_SLOTS chunks, y = slot m.
 // (the per-output forms run on a few polynomials per launch and hold the operands of three rotations at once: they
 // trade resident blocks for registers)
-template <bool FWD, int EPI, bool TILED, bool DTILE = false>
+template <bool FWD, int EPI, bool TILED>
 __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
                                                                        u32 n_outer, const RotBatch rb,
                                                                        const ModDownEpilogue epi) {
     __shared__ __align__(128) u64 sm_all[CONTIG_SLOTS << LOG_C];
     grid_dependency_enter();
-    const u32 m = slot_of_block(blockIdx.y, B.n_m), mod = batch_modulus(B, m);
+    const u32 m = slot_of_block(blockIdx.y, B.n_m);
+    u32 mod = batch_modulus<EPI == 4>(R, B, m);
     const int slot = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const u32 g = blockIdx.x * CONTIG_SLOTS + slot;
     const u32 chunk = g / n_outer, o = g - chunk * n_outer;
     if (chunk >= (R.N >> LOG_C)) return;            // (whole warps leave)
+    if (EPI == 5 && m > R.r) mod = o % R.r;         // (component 0, in the prime it is a residue of)
     if (FWD && own_prime(R, B, o, mod)) return;
     u64* sm = sm_all + (slot << LOG_C);
     const int path = path_of(R, mod);
-    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else contig_body<FWD, EPI, PATH_INT, TILED, DTILE>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else contig_body<FWD, EPI, PATH_INT, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
 }
 
 // Key-switch products (Sec. 4.2 "key-switching primitives"): the contiguous pass of the digits' transforms and their inner
@@ -1096,7 +1105,7 @@ __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) 
 template <int RC>
 struct InnerGeo {
     static constexpr int WARPS = RC > 8 ? RC : RC > 0 ? 8 : MAX_MODULI;    // (upper bound where r is not a constant)
-    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 4 ? 4 : RC > 0 ? 3 : 1;
+    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 0 ? 4 : 1;
 };
 template <int CLS, int RC>
 __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch& rb, u32 first, u32 cnt, u32 m, u32 n, const u64* sd,
@@ -1264,7 +1273,7 @@ template <bool FWD, int LOAD>
 static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 n_polys, cudaStream_t stream) {
     if (n_polys == 0) return cudaSuccess;
     ProfScope prof(ring.prof, FWD ? CAT_NTT_FWD_STRIDED : CAT_NTT_INV_STRIDED, stream);
-    if constexpr (FWD && (LOAD == LOAD_REDUCE || LOAD == LOAD_CENTRED)) {
+    if constexpr (FWD && (LOAD == LOAD_REDUCE || LOAD == LOAD_CENTRED || LOAD == LOAD_INGEST)) {
         const u32 n_outer = n_polys / B.n_m;
         if (B.src_sm == 0 && B.n_m > 1 && n_outer <= 65535 && !B.tile_ptr) {
             switch (ring.dev.logN - LOG_C) {
@@ -1280,6 +1289,8 @@ static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 
             return cudaGetLastError();
         }
     }
+    if constexpr (LOAD == LOAD_INGEST) return cudaErrorInvalidValue;
+    else
     switch (ring.dev.logN - LOG_C) {
         case 2: launch_strided_t<FWD, LOAD, 2, 8>(ring, B, n_polys, stream); break;
         case 3: launch_strided_t<FWD, LOAD, 3, 8>(ring, B, n_polys, stream); break;
@@ -1306,6 +1317,10 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
     if (FWD && epi && epi->plain) {
         launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
+    } else if (FWD && B.ingest) {
+        static const RotBatch no_rb = {};
+        static const ModDownEpilogue no_epi = {};
+        launch_dependent(ring, ntt_contig<true, 5, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, no_rb, no_epi);
     } else if (!FWD && epi && epi->assemble) {
         launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
                          *epi);
@@ -1321,9 +1336,6 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
         if (B.tile_ptr)
             launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
                              no_rb, no_epi);
-        else if (FWD && B.dtile_ptr && !B.scatter && !B.lift_ptr)
-            launch_dependent(ring, ntt_contig<true, 0, false, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B,
-                             n_outer, no_rb, no_epi);
         else
             launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
                              no_rb, no_epi);
@@ -1341,6 +1353,17 @@ cudaError_t ntt_forward(const RingHost& ring, const PolyBatch& B, u32 n_outer, i
     else e = launch_strided<true, LOAD_CENTRED>(ring, B, n_polys, stream);
     if (e != cudaSuccess) return e;
     return launch_contig<true>(ring, B, n_polys, stream);
+}
+
+cudaError_t ntt_forward_ingest(const RingHost& ring, const PolyBatch& B0, u32 n_in, cudaStream_t stream) {
+    const u32 r = ring.dev.r;
+    PolyBatch B = B0;
+    B.ingest = 1;
+    B.n_m = r + 1;
+    cudaError_t e = launch_strided<true, LOAD_INGEST>(ring, B, n_in * 2 * r * B.n_m, stream);
+    if (e != cudaSuccess) return e;
+    B.n_m = r + 2;
+    return launch_contig<true>(ring, B, n_in * r * B.n_m, stream);
 }
 
 cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
