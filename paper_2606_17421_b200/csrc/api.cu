@@ -612,7 +612,7 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
     if (chunk < 32) chunk = 32;
     if (chunk > count) chunk = count > 0 ? count : 1;
     if (!stored) TRY(ensure(ctx, ctx->fft, (size_t)chunk * n * sizeof(double2)));
-    if (!coef_out && !(stored && stored->coef_bits == 64)) TRY(ensure(ctx, ctx->coef, (size_t)chunk * N * sizeof(i64)));
+    if (!coef_out && !stored) TRY(ensure(ctx, ctx->coef, (size_t)chunk * N * sizeof(i64)));
     if (!coef_out) TRY(ensure(ctx, ctx->ptnat, (size_t)chunk * r * N * sizeof(u64)));
     EncodeTables tab;
     tab.slot_of_pos = ctx->slot_of_pos;
@@ -635,11 +635,8 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
         db.d0 = d0 + lo;
         db.count = cnt;
         const void* coef_src = ctx->coef.p;
-        if (stored && stored->coef_bits == 64) {
-            coef_src = (const i64*)stored->coef + (size_t)(d0 + lo) * N;
-        } else if (stored) {
-            CK(launch_widen_i32(ctx->ring, (const int*)stored->coef + (size_t)(d0 + lo) * N, (i64*)ctx->coef.p, (size_t)cnt * N,
-                                ctx->stream));
+        if (stored) {
+            coef_src = (const char*)stored->coef + (size_t)(d0 + lo) * N * (stored->coef_bits / 8);
         } else {
             i64* into = coef_out ? coef_out + (size_t)lo * N : (i64*)ctx->coef.p;
             CK(launch_encode(ctx->ring, tab, db, (double2*)ctx->fft.p, into, ctx->overflow_flag, ctx->stream));
@@ -656,6 +653,7 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
         B.n_m = r;
         B.mod0 = 0;
         B.mod_step = 1;
+        B.src32 = stored && stored->coef_bits == 32;
         B.split_bits = mac_split_bits(ctx->ring);
         B.tile_ptr = dst;
         B.tile = lay;

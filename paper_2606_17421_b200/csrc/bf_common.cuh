@@ -80,6 +80,12 @@ __device__ __forceinline__ double u2d(u64 x) {          // exact for x < 2^52
 __device__ __forceinline__ u64 d2u(double d) {          // d an integer in [0, 2^52)
     return (u64)__double_as_longlong(d + 4503599627370496.0) - 0x4330000000000000ull;
 }
+__device__ __forceinline__ double i2d(i64 v) {          // exact for |v| < 2^51
+    return __longlong_as_double((long long)(v + 0x4338000000000000ll)) - 6755399441055744.0;
+}
+__device__ __forceinline__ i64 d2i(double d) {          // d an integer, |d| < 2^51
+    return (i64)__double_as_longlong(d + 6755399441055744.0) - 0x4338000000000000ll;
+}
 // x * w - round(x * w / q) * q for a non-negative integer-valued x and a constant 0 <= w < q given as
 // (double)w and wq = (double)w / q.  ph + pl = x*w exactly (FMA); the quotient estimate is within
 // 1/2 + x * 2^-52 of x*w/q; ph - qh*q is an integer far below 2^53 and therefore exact, and so is the final
@@ -302,6 +308,7 @@ struct PolyBatch {
     long long sum_stride;
     u32 sum_terms;
     u64 lift_mod;                 // LOAD_CENTRED: the modulus M the source residues live in
+    u32 src32;                    // LOAD_I64_MONT: the source words are 32-bit integers
     u32 src_digits;               // LOAD_REDUCE: the source of outer index o is a residue modulo prime o % r
     u32 store_centred;            // inverse transform: store the centred lift of each coefficient plus 2^59
                                   //   (the form LOAD_CENTRED reads) instead of the residue in [0, q); 2: only for the

@@ -50,7 +50,8 @@ struct LoadConsts {
     bool wide;          // target prime of 2^41 or more: values must stay in [0, 4q); otherwise they are signed
     bool src_small;     // LOAD_REDUCE: every source word is below 1.5 q already (block-uniform)
     bool src_fp;        // LOAD_REDUCE: every source word is below 2^51
-    bool staged_fp;     // LOAD_REDUCE: the source holds the bits of integer-valued doubles
+    bool staged_fp;     // the staged source holds the bits of integer-valued doubles
+                        //   (LOAD_I64_MONT: all below 2^40; src_small, src_fp: no factor 2^64, q from 2^39 or below)
 };
 
 template <int LOAD>
@@ -60,6 +61,11 @@ __device__ __forceinline__ u64 load_src(const void* src, size_t idx, const LoadC
         u64 t = ((const u64*)src)[idx];
         if (c.staged_fp) t = d2u(__longlong_as_double((long long)t));
         return c.src_small ? (t >= c.q ? t - c.q : t) : barrett64(t, c.q, c.mu);
+    }
+    if (LOAD == LOAD_I64_MONT && c.staged_fp) {             // |v| < 2^40 < q
+        const i64 v = d2i(((const double*)src)[idx]);
+        const u64 m = mul_shoup(v < 0 ? (u64)(-v) : (u64)v, c.lift_mod, c.lift_red, c.q);
+        return v < 0 && m != 0 ? c.q - m : m;
     }
     if (LOAD == LOAD_I64 || LOAD == LOAD_I64_MONT) {
         i64 v = ((const i64*)src)[idx];
@@ -98,6 +104,15 @@ __device__ __forceinline__ double load_src_fp(const void* src, size_t idx, const
         const u64 T = ((const u64*)src)[idx];
         const double hi = u2d(T >> 30), lo = u2d(T & ((1ull << 30) - 1));
         return __dadd_rn(__dadd_rn(fp_mul_centred(hi, c.c30, c.c30q, c.qd), lo), c.k59);   // (k59: see LoadConsts)
+    }
+    if (LOAD == LOAD_I64_MONT && c.staged_fp) {
+        // |v| < 2^40: as it is where plaintexts carry no factor and that is below 2q, else centred, or times 2^64 mod q
+        // (a centred product, within 0.51q; plus q where values must not be negative)
+        const double v = ((const double*)src)[idx];
+        if (c.src_small) return v;
+        if (c.src_fp) return fp_centre(v, c.qd, c.qinv);
+        const double m = fp_mul_centred_signed(v, c.c64d, c.c64q, c.qd);
+        return c.wide ? __dadd_rn(m, c.qd) : m;
     }
     if (LOAD == LOAD_I64_MONT) {
         // v = (hi' - 2^31) 2^32 + lo with hi' = (v >> 32) + 2^31 in [0, 2^32); two centred products (each
@@ -345,8 +360,8 @@ __device__ __forceinline__ LoadConsts load_consts(const RingDev& R, const PolyBa
         split_index(o, R.r, B.o_div == R.r ? B.o_div_magic : 0u, s_hi, s_lo);
         qs = R.q[s_lo];
     }
-    lc.src_small = qs <= q + (q >> 1);
-    lc.src_fp = qs < (1ull << 51);
+    lc.src_small = LOAD == LOAD_I64_MONT ? R.dp[mod] && (q >> 39) : qs <= q + (q >> 1);
+    lc.src_fp = LOAD == LOAD_I64_MONT ? R.dp[mod] != 0 : qs < (1ull << 51);
     lc.staged_fp = false;
     return lc;
 }
@@ -552,7 +567,7 @@ ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
     StridedTwiddles<LOG_R> tw;
     tw.fetch(R, true, path_of(R, batch_modulus<false>(R, B, m_begin)), batch_modulus<false>(R, B, m_begin));
     // digits of primes on the fp64 path are staged as doubles
-    const bool staged_fp = LOAD == LOAD_REDUCE && B.src_digits && B.o_div == R.r && R.fp_ok[o_lo];
+    bool staged_fp = LOAD == LOAD_REDUCE && B.src_digits && B.o_div == R.r && R.fp_ok[o_lo];
     {
         const size_t src_off = B.o_div ? (size_t)o_hi * B.src_so2 + (size_t)o_lo * B.src_so : (size_t)o * B.src_so;
         const u64* src = (const u64*)B.src + src_off + tile * LANES;
@@ -594,6 +609,25 @@ ntt_strided_shared_src(const RingDev R, const PolyBatch B, u32 m_per_block) {
                     staged[w] = mul_shoup(sub_mod(src[at(w)], t, dc.q), pinv, pinvs, dc.q);
                 }
             }
+        } else if constexpr (LOAD == LOAD_I64_MONT) {
+            // encoded coefficients: 64-bit integers, or 32-bit ones (src32).  Nearly all are small: a tile whose largest is
+            // below 2^40 is staged as doubles, which the primes below that take as they are
+            i64 v[POINTS / NT];
+            bool big = false;
+            if (B.src32) {
+                const int* src4 = (const int*)B.src + src_off + tile * LANES;
+#pragma unroll
+                for (int k = 0; k < POINTS / NT; ++k) v[k] = src4[at(threadIdx.x + k * NT)];
+            } else {
+#pragma unroll
+                for (int k = 0; k < POINTS / NT; ++k) v[k] = (i64)src[at(threadIdx.x + k * NT)];
+#pragma unroll
+                for (int k = 0; k < POINTS / NT; ++k) big = big || (u64)(v[k] + (1ll << 40)) >> 41;
+                big = __syncthreads_or(big) != 0;
+            }
+            staged_fp = !big;
+#pragma unroll
+            for (int k = 0; k < POINTS / NT; ++k) staged[threadIdx.x + k * NT] = big ? (u64)v[k] : (u64)__double_as_longlong(i2d(v[k]));
         } else {
             u64 v[POINTS / NT];
 #pragma unroll
@@ -1273,9 +1307,9 @@ template <bool FWD, int LOAD>
 static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 n_polys, cudaStream_t stream) {
     if (n_polys == 0) return cudaSuccess;
     ProfScope prof(ring.prof, FWD ? CAT_NTT_FWD_STRIDED : CAT_NTT_INV_STRIDED, stream);
-    if constexpr (FWD && (LOAD == LOAD_REDUCE || LOAD == LOAD_CENTRED || LOAD == LOAD_INGEST)) {
+    if constexpr (FWD && (LOAD == LOAD_REDUCE || LOAD == LOAD_CENTRED || LOAD == LOAD_INGEST || LOAD == LOAD_I64_MONT)) {
         const u32 n_outer = n_polys / B.n_m;
-        if (B.src_sm == 0 && B.n_m > 1 && n_outer <= 65535 && !B.tile_ptr) {
+        if (B.src_sm == 0 && B.n_m > 1 && n_outer <= 65535) {
             switch (ring.dev.logN - LOG_C) {
                 case 2: launch_shared_src_t<LOAD, 2, 8>(ring, B, n_outer, stream); break;
                 case 3: launch_shared_src_t<LOAD, 3, 8>(ring, B, n_outer, stream); break;
@@ -1289,7 +1323,7 @@ static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 
             return cudaGetLastError();
         }
     }
-    if constexpr (LOAD == LOAD_INGEST) return cudaErrorInvalidValue;
+    if constexpr (LOAD == LOAD_INGEST || LOAD == LOAD_I64_MONT) return cudaErrorInvalidValue;     // (always from a shared source)
     else
     switch (ring.dev.logN - LOG_C) {
         case 2: launch_strided_t<FWD, LOAD, 2, 8>(ring, B, n_polys, stream); break;
