@@ -261,6 +261,7 @@ struct TileLayout {
     u32 fmt_bits;                           // TileFormat of prime i in bits 2i, 2i+1
     u32 n_primes;                           // primes the plaintexts are held in: r, or r + 1 with double hoisting
                                             //   (the special prime last, always in 8-byte whole words)
+    size_t base[MAX_MODULI + 1];            // see tile_prime_base
 };
 constexpr u32 TILE_TS = 8;
 constexpr u32 TILE_STAGE_WORDS = 2048;
@@ -269,15 +270,8 @@ __host__ __device__ __forceinline__ u32 tile_format(const TileLayout& t, u32 i) 
 __host__ __device__ __forceinline__ u32 tile_stage_bytes(u32 fmt) {
     return TILE_STAGE_WORDS * (fmt == TILE_W64 ? 8u : fmt == TILE_W40 ? 5u : 4u);
 }
-// byte offset of prime i's first stage (i = r: total size): the primes' regions follow one another
-__host__ __device__ __forceinline__ size_t tile_prime_base(const TileLayout& t, u32 i) {
-    size_t words8 = 0;                      // in units of 2048 bytes: a stage is 8, 5 or 4 of them
-    for (u32 k = 0; k < i; ++k) {
-        const u32 f = tile_format(t, k);
-        words8 += f == TILE_W64 ? 8u : f == TILE_W40 ? 5u : 4u;
-    }
-    return words8 * TILE_STAGE_WORDS * (size_t)t.ntiles * t.G * t.C;
-}
+// byte offset of prime i's first stage (i = n_primes: total size): the primes' regions follow one another
+__host__ __device__ __forceinline__ size_t tile_prime_base(const TileLayout& t, u32 i) { return t.base[i]; }
 // byte offset of a stage
 __host__ __device__ __forceinline__ size_t tile_stage_offset(const TileLayout& t, u32 i, u32 tile, u32 g, u32 ch) {
     return tile_prime_base(t, i) + (((size_t)tile * t.G + g) * t.C + ch) * tile_stage_bytes(tile_format(t, i));

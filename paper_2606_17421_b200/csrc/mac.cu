@@ -35,6 +35,7 @@ TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_pr
         const u32 f = !ring.compact_cache || i >= ring.dev.r ? TILE_W64
                     : ring.q[i] < (1ull << 32) ? TILE_W32 : ring.q[i] < (1ull << 40) ? TILE_W40 : TILE_W64;
         t.fmt_bits |= f << (2 * i);
+        t.base[i + 1] = t.base[i] + (size_t)tile_stage_bytes(f) * t.ntiles * t.G * t.C;
     }
     return t;
 }

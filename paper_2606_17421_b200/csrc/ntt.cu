@@ -377,10 +377,17 @@ __device__ __forceinline__ u64* ingest_dst(const RingDev& R, const PolyBatch& B,
     return o_hi & 1 ? B.dst + set * B.dst_so + (size_t)m * B.dst_sm : B.tail_dst + set * R.N;
 }
 
-// Row `row` of the exchange buffer of a strided tile.  Tiles of 8 columns (64 bytes a row) swap the rows of a pair by bit 2
-// of the row number, so that the two rows a half-warp reads never share banks, whether they are neighbours or 4 apart.
+// Rows of the exchange buffer of a strided tile.  Tiles of 8 columns (64 bytes a row) swap the rows of a pair by bit 2 of the
+// row number, so that the two rows a half-warp touches never share banks, whether they are neighbours or 4 apart.  Row base +
+// i * step of a set then lies at (i odd ? odd : even) + i * step: two numbers per set, the rest are immediate offsets.
 template <int LOG_LANES>
-__device__ __forceinline__ int exchange_row(int row) { return LOG_LANES == 3 ? row ^ ((row >> 2) & 1) : row; }
+__device__ __forceinline__ void exchange_rows(int base, int log_step, int& even, int& odd) {
+    even = odd = base;
+    if (LOG_LANES != 3) return;
+    if (log_step > 2) even = odd = base ^ ((base >> 2) & 1);        // (bit 2 does not depend on i)
+    else if (log_step == 2) odd = base ^ 1;                         // (bit 2 of the row is bit 0 of i)
+    else { even += (base >> 2) & 1; odd -= (base >> 2) & 1; }       // (sets of 4 adjacent rows)
+}
 
 // Strided pass: transforms the 2^LOG_R rows (stride 256) of a tile of adjacent columns.  Forward: first pass (reads the
 // batch source through the load functor, or from `staged`, [row][column], where several target primes of the same block
@@ -428,6 +435,10 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
             const int lane = w & (LANES - 1), u = w >> LOG_LANES;
             const int blk = u >> log_step, off = u & (step - 1);
             const int base = (blk << (log_step + K)) + off;
+            int even, odd;
+            exchange_rows<LOG_LANES>(base, log_step, even, odd);
+            T* const sm_even = sm + even * LANES + lane;
+            T* const sm_odd = sm + odd * LANES + lane;
             T e[8];
 #pragma unroll
             for (int i = 0; i < (1 << K); ++i) {
@@ -443,7 +454,7 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
                         e[i] = ((const T*)dst)[gidx];
                     }
                 } else {
-                    e[i] = sm[exchange_row<LOG_LANES>(row) * LANES + lane];
+                    e[i] = (i & 1 ? sm_odd : sm_even)[i * step * LANES];
                 }
             }
             if (!STAGED && g_first && w0 == 0) {    // (the first sweep of the first group is full for every geometry)
@@ -486,7 +497,7 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
                         dst[gidx] = out;
                     }
                 } else {
-                    sm[exchange_row<LOG_LANES>(row) * LANES + lane] = e[i];
+                    (i & 1 ? sm_odd : sm_even)[i * step * LANES] = e[i];
                 }
             }
         }
@@ -775,6 +786,18 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     T e[8];
     const bool dp = R.dp[mod] != 0;         // (the operand arrays hold this prime's words as doubles)
     (void)dp;
+    // where the thread's words lie in the tile-major plaintext cache: points 4 lane.., and 128 further on
+    unsigned char* tile_stage = nullptr;
+    size_t tile_step = 0;
+    u32 tile_at = 0, tile_fmt = 0;
+    if constexpr (TILED) {
+        const u32 d = B.o_base + o, pj_all = d / B.tile.n_terms, term = d - pj_all * B.tile.n_terms, pj = pj_all - B.tile_pj0;
+        const u32 n = chunk * LEN + 4 * lane;
+        tile_stage = (unsigned char*)B.tile_ptr + tile_stage_of_word(B.tile, pj, term, mod, n);
+        tile_at = tile_word_index(B.tile, pj, term, n);
+        tile_fmt = tile_format(B.tile, mod);
+        tile_step = (size_t)((128u >> B.tile.log_tn) * B.tile.G * B.tile.C) * tile_stage_bytes(tile_fmt);
+    }
     // byte addresses (shared window) of the thread's base point in each of the three access patterns
     const u32 slice = (u32)__cvta_generic_to_shared(sm);
     const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
@@ -892,11 +915,8 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 continue;
             }
             if constexpr (TILED) {   // tile-major plaintext cache; 4 adjacent coefficients never straddle a tile (tiles hold >= 16)
-                const u32 pj = (B.o_base + o) / B.tile.n_terms - B.tile_pj0, term = (B.o_base + o) % B.tile.n_terms;
-                const u32 n = chunk * LEN + 4 * s;
-                unsigned char* stage = (unsigned char*)B.tile_ptr + tile_stage_of_word(B.tile, pj, term, mod, n);
-                const u32 at = tile_word_index(B.tile, pj, term, n);
-                const u32 fmt = tile_format(B.tile, mod);
+                unsigned char* stage = tile_stage + (size_t)it * tile_step;
+                const u32 at = tile_at, fmt = tile_fmt;
                 if (fmt == TILE_W64) {
                     if (!dp) {          // (else: the bits of doubles already)
                         const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
@@ -1027,11 +1047,8 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                         }
                 }
             } else if constexpr (TILED) {  // read back from the tile-major plaintext cache
-                const u32 pj = (B.o_base + o) / B.tile.n_terms - B.tile_pj0, term = (B.o_base + o) % B.tile.n_terms;
-                const u32 n = chunk * LEN + 4 * s;
-                const unsigned char* stage = (const unsigned char*)B.tile_ptr + tile_stage_of_word(B.tile, pj, term, mod, n);
-                const u32 at = tile_word_index(B.tile, pj, term, n);
-                const u32 fmt = tile_format(B.tile, mod);
+                const unsigned char* stage = tile_stage + (size_t)it * tile_step;
+                const u32 at = tile_at, fmt = tile_fmt;
                 if (fmt == TILE_W64) {
                     const ulonglong2* gp = (const ulonglong2*)(stage + (size_t)at * 8);
                     const ulonglong2 a = gp[0], b = gp[1];
