@@ -113,6 +113,13 @@ __device__ __forceinline__ double fp_centre(double v, double q, double qinv) {
     const double qh = __dsub_rn(__fma_rn(v, qinv, magic), magic);
     return __fma_rn(-qh, q, v);
 }
+// v mod q in [0, q) for a signed integer-valued |v| < 2^46, q < 2^41: (v + 1/2) / q is at least 2^-42 away from any integer,
+// which the errors of the product (2^-52 of at most 2^5 where v is within 32 q) do not bridge, so its floor is exact
+__device__ __forceinline__ double fp_canonical(double v, double q, double qinv) {
+    const double magic = 6755399441055744.0;
+    const double qh = __dsub_rn(__fma_rd(__dadd_rn(v, 0.5), qinv, magic), magic);
+    return __fma_rn(-qh, q, v);
+}
 // v mod q in [0, q) for an integer-valued 0 <= v < 2^46
 __device__ __forceinline__ double fp_reduce(double v, double q, double qinv) {
     const double magic = 4503599627370496.0;

@@ -713,8 +713,9 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 
 // Contiguous pass: every warp transforms one chunk of 256 adjacent points (8 per thread) through
 // the groups {3,3,2}; the chunk lives in the warp's own swizzled slice of shared memory between
-// groups, so only warp-level synchronisation is needed.  The chunks of a block are consecutive in (chunk, outer index)
-// order: where a batch has several polynomials per prime, they share their twiddles through L1.
+// groups, so only warp-level synchronisation is needed.
+// What bounds it: instruction issue.  An fp64 instruction takes two issue slots of its scheduler, any other one, and the
+// cycles per chunk are that sum (1020 of 324 fp64 and 367 other instructions, all primes below 2^41), with warps to spare.
 // Forward: second pass (final reduction to [0, q), then the store functors).  Inverse: first pass
 // (reads the batch source: plain residues, tiled/limb-split plaintexts, or a sum of arrays).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
@@ -722,7 +723,7 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // (sum over the output's giant rotations, gathered through their permutations); 3 = plain; 4 = output assembly (see
 // ModDownEpilogue); 5 = ingest (see PolyBatch): the digits into the operand array, component c of the inputs times P into
 // lift_ptr.
-constexpr int CONTIG_THREADS = 128, CONTIG_SLOTS = CONTIG_THREADS / 32;
+constexpr int CONTIG_THREADS = 128, CONTIG_WARPS = CONTIG_THREADS / 32;
 
 // a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
 template <int PATH, typename T>
@@ -730,8 +731,7 @@ __device__ __forceinline__ u64 canonical(T x, const ModConsts& c, bool bits) {
     if constexpr (PATH == PATH_WIDE) {
         return d2u(fp_reduce(x, c.qd, c.qinv));
     } else if constexpr (PATH == PATH_DP) {
-        double v = fp_centre(x, c.qd, c.qinv);
-        if (v < 0.0) v = __dadd_rn(v, c.qd);
+        const double v = fp_canonical(x, c.qd, c.qinv);
         return bits ? (u64)__double_as_longlong(v) : d2u(v);
     } else {
         if (x >= 2 * c.q) x -= 2 * c.q;
@@ -1112,24 +1112,24 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     }
 }
 
-// grid: x = groups of CONTIG_SLOTS chunks, y = slot m.
+// grid: x = group of 2^log_wo outer indices, y = slot m, z = group of chunks.
 // (the per-output forms run on a few polynomials per launch and hold the operands of three rotations at once: they
 // trade resident blocks for registers)
 template <bool FWD, int EPI, bool TILED>
 __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
-                                                                       u32 n_outer, const RotBatch rb,
+                                                                       u32 n_outer, u32 log_wo, const RotBatch rb,
                                                                        const ModDownEpilogue epi) {
-    __shared__ __align__(128) u64 sm_all[CONTIG_SLOTS << LOG_C];
+    __shared__ __align__(128) u64 sm_all[CONTIG_WARPS << LOG_C];
     grid_dependency_enter();
     const u32 m = slot_of_block(blockIdx.y, B.n_m);
     u32 mod = batch_modulus<EPI == 4>(R, B, m);
-    const int slot = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const u32 g = blockIdx.x * CONTIG_SLOTS + slot;
-    const u32 chunk = g / n_outer, o = g - chunk * n_outer;
-    if (chunk >= (R.N >> LOG_C)) return;            // (whole warps leave)
+    const u32 warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const u32 o = (blockIdx.x << log_wo) + (warp & ((1u << log_wo) - 1)), chunk = blockIdx.z * (CONTIG_WARPS >> log_wo) + (warp >> log_wo);
+    if (o >= n_outer || chunk >= (R.N >> LOG_C)) return;    // (whole warps leave)
     if (EPI == 5 && m > R.r) mod = o % R.r;         // (component 0, in the prime it is a residue of)
     if (FWD && own_prime(R, B, o, mod)) return;
-    u64* sm = sm_all + (slot << LOG_C);
+    u64* sm = sm_all + (warp << LOG_C);
     const int path = path_of(R, mod);
     if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
     else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
@@ -1363,32 +1363,35 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
     PolyBatch B = B_in;
     const u32 n_outer = n_polys / B.n_m;
     set_magics(B, n_outer);
-    const u32 groups = (u32)(((size_t)n_outer * (ring.dev.N >> LOG_C) + CONTIG_SLOTS - 1) / CONTIG_SLOTS);
-    const dim3 grid(groups, B.n_m);
+    // the four warps of a block take the same chunk of four polynomials where the batch has enough of them (one fetch of the
+    // chunk's twiddles serves them), else of two, else neighbouring chunks
+    const u32 log_wo = n_outer % 4 == 0 || n_outer >= 16 ? 2u : n_outer % 2 == 0 || n_outer >= 7 ? 1u : 0u;
+    const u32 per = CONTIG_WARPS >> log_wo, chunks = ring.dev.N >> LOG_C;
+    const dim3 grid((n_outer + (1u << log_wo) - 1) >> log_wo, B.n_m, (chunks + per - 1) / per);
     if (FWD && epi && epi->plain) {
-        launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
                          *epi);
     } else if (FWD && B.ingest) {
         static const RotBatch no_rb = {};
         static const ModDownEpilogue no_epi = {};
-        launch_dependent(ring, ntt_contig<true, 5, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, no_rb, no_epi);
+        launch_dependent(ring, ntt_contig<true, 5, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, no_rb, no_epi);
     } else if (!FWD && epi && epi->assemble) {
-        launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
+        launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
                          *epi);
     } else if (epi && epi->n_sum) {
-        launch_dependent(ring, ntt_contig<FWD, 2, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 2, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
                          *epi);
     } else if (FWD && epi) {
-        launch_dependent(ring, ntt_contig<FWD, 1, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, *rb,
+        launch_dependent(ring, ntt_contig<FWD, 1, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
                          *epi);
     } else {
         static const RotBatch no_rb = {};
         static const ModDownEpilogue no_epi = {};
         if (B.tile_ptr)
-            launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
+            launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo,
                              no_rb, no_epi);
         else
-            launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer,
+            launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo,
                              no_rb, no_epi);
     }
     return cudaGetLastError();
