@@ -294,10 +294,11 @@ static cudaError_t launch_mac_t(const MacLaunch& m) {
         if (e != cudaSuccess) return e;
         attr_set[device_slot(ring)] = true;
     }
-    // slices over the output groups only where the tiles alone leave the machine short of blocks (every slice makes or
-    // reads the X tile again)
+    // slices over the output groups where the tiles alone are fewer than three rounds of blocks (every slice reads the X tile
+    // again, which is little beside its weights; where the block makes X it is not): the primes beyond 2^50 take several times
+    // as long as the others, and one round ends with them alone (N = 2^13, 48 groups of 16 terms: 66 us in one, 50 us in three)
     const u32 tiles = (ring.dev.N >> LOG_TN) * m.lay.n_primes;
-    u32 slices = BABY ? 1u : (148u * 3 + tiles - 1) / tiles;
+    u32 slices = BABY ? 1u : (148u * 12 + tiles - 1) / tiles;
     const u32 max_slices = (m.n_pj + PL - 1) / PL;
     if (slices > max_slices) slices = max_slices;
     if (slices < 1) slices = 1;
