@@ -147,14 +147,13 @@ int bf_linear_rescaled(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const 
                        const float* W_raw, uint32_t d_out, uint32_t d_in, uint64_t* ct_low, uint32_t n_out,
                        double* scale_inout);
 
-/* Cache compression (Sec. 6.1 names the encoded-weight cache as the memory wall).  With
- * bf_set_compact_cache(ctx, 1) every weight encoded afterwards, cached or on the fallback path, is
- * held in the narrowest word format its prime allows: 4 bytes per word for primes below 2^32, 5
- * (low 32 bits and high bytes stored apart) below 2^40, 8 otherwise, instead of 8 throughout: with a
- * 50-bit and six 40-bit primes 38 of 56 bytes, i.e. 68 % of the resident size and of the
- * multiply-accumulate's HBM stream.  Results are identical; handles of both kinds can be used side by
- * side.  Default: off (the multiply-accumulate is no faster for it on B200, see the design notes;
- * the gain is capacity).  bf_weights_bytes reports sizes for the current setting. */
+/* Cache compression (Sec. 6.1 names the encoded-weight cache as the memory wall).  Encoded weights are held in the
+ * narrowest word format their primes allow: 4 bytes per word for primes below 2^32, 5 (low 32 bits and high bytes stored
+ * apart) below 2^40, 8 otherwise; with a 50-bit and six 40-bit primes that is 38 of 56 bytes, i.e. 68 % of the resident
+ * size and of the multiply-accumulate's HBM stream.  bf_set_compact_cache(ctx, 1) makes every weight encoded afterwards
+ * count for those bytes (cache budget, bf_cache_bytes_used, bf_weights_bytes); with the default, off, it counts for 8 bytes
+ * per word, an upper bound that does not depend on the primes.  Results are identical; handles of both kinds can be used
+ * side by side. */
 int bf_set_compact_cache(bf_ctx* ctx, int on);
 
 /* Coefficient form of the cache (the other answer to the memory wall of Sec. 6.1): with

@@ -582,7 +582,7 @@ static u64 weights_bytes(const bf_ctx* ctx, u32 d_out, u32 d_in, u32 b, u32 g) {
     if (ctx->coef_cache_bits)       // one rounded coefficient per diagonal and ring position, whatever the primes
         return (u64)n_in * n_out * (ctx->plan.tile_D / ctx->plan.tau) * ctx->N * (ctx->coef_cache_bits / 8);
     const TileLayout lay = mac_tile_layout(ctx->ring, n_out * g, n_in * b, mac_primes(ctx));
-    return mac_tile_bytes(ctx->ring, lay);
+    return mac_accounted_bytes(ctx->ring, lay);
 }
 
 extern "C" uint64_t bf_weights_bytes(const bf_ctx* ctx, uint32_t d_out, uint32_t d_in) {
@@ -729,13 +729,14 @@ extern "C" int bf_encode_weights_split(bf_ctx* ctx, const float* W, uint32_t d_o
             }
         }
     } else {
-        if (cudaMalloc(&w->pt, bytes) != cudaSuccess) {
+        const size_t occupied = mac_tile_bytes(w->lay);
+        if (cudaMalloc(&w->pt, occupied) != cudaSuccess) {
             cudaGetLastError();
             delete w;
             return BF_ERR_OOM;
         }
         // padding words of the layout are never read, but keep the allocation defined
-        if (cudaMemsetAsync(w->pt, 0, bytes, ctx->stream) != cudaSuccess) s = BF_ERR_CUDA;
+        if (cudaMemsetAsync(w->pt, 0, occupied, ctx->stream) != cudaSuccess) s = BF_ERR_CUDA;
         if (s == BF_OK) s = encode_range(ctx, W, d_out, d_in, 0, n_diag, w->pt, w->lay, 0, nullptr, nullptr, bsgs_b, bsgs_g);
     }
     if (s == BF_OK) s = check_overflow(ctx);
@@ -1140,7 +1141,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
         // fallback: encode groups of (j, p) just in time into a scratch ring, then consume them (weights kept as
         // coefficients: the same without the encoder, only their transforms)
         const TileLayout jl = mac_tile_layout(ctx->ring, groups, n_terms, nmp);
-        TRY(ensure(ctx, ctx->ptjit, mac_tile_bytes(ctx->ring, jl)));
+        TRY(ensure(ctx, ctx->ptjit, mac_tile_bytes(jl)));
         for (u32 pj0 = 0; pj0 < n_pj; pj0 += groups) {
             const u32 cnt = (n_pj - pj0 < groups) ? n_pj - pj0 : groups;
             const TileLayout cl = mac_tile_layout(ctx->ring, cnt, n_terms, nmp);
@@ -1502,7 +1503,7 @@ extern "C" int bf_set_coefficient_cache(bf_ctx* ctx, int bits) {
 
 extern "C" int bf_set_compact_cache(bf_ctx* ctx, int on) {
     if (!ctx) return BF_ERR_INVALID_ARG;
-    ctx->ring.compact_cache = on != 0;     // weights encoded from now on (and the fallback path's scratch) use it
+    ctx->ring.compact_cache = on != 0;     // (the words themselves are as narrow as their primes allow either way)
     return BF_OK;
 }
 

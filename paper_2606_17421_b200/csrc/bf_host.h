@@ -40,7 +40,7 @@ struct RingHost {
     std::vector<u64> q;               // q_0..q_L, then P
     Profiler* prof = nullptr;
     bool dependent_launch = true;     // launch the kernels of a call with programmatic stream serialisation
-    bool compact_cache = false;       // encode plaintexts in the narrowest word format each prime allows
+    bool compact_cache = false;       // cached plaintexts count for the bytes they occupy, not for 8 a word
     int device = 0;                   // the CUDA device of the context (kernel attributes are set once per device)
 };
 constexpr int MAX_DEVICES = 64;
@@ -103,7 +103,8 @@ cudaError_t launch_pointwise_mul(const RingHost& ring, const u64* a, const u64* 
 u32 mac_split_bits(const RingHost& ring);   // limb width of cached 8-byte words modulo primes below 2^50
 // layout of n_pj groups of n_terms diagonals held in n_primes primes (0 = the r ciphertext primes)
 TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_primes = 0);
-size_t mac_tile_bytes(const RingHost& ring, const TileLayout& t);           // bytes that layout occupies
+size_t mac_tile_bytes(const TileLayout& t);                                 // bytes that layout occupies
+size_t mac_accounted_bytes(const RingHost& ring, const TileLayout& t);      // bytes it counts for: 8 a word unless compact_cache
 // a: [n_pj][2][lay.n_primes][N]; every prime of the layout is processed.  baby null: x holds all terms,
 // [n_terms][2][lay.n_primes][N].  baby non-null: x holds the un-rotated inputs, [n_in][2][lay.n_primes][N], and the
 // rotated terms are computed inside.

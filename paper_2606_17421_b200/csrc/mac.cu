@@ -32,15 +32,18 @@ TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_pr
     t.C = (n_terms + TILE_TS - 1) / TILE_TS;
     t.ntiles = ring.dev.N >> t.log_tn;
     for (u32 i = 0; i < t.n_primes; ++i) {
-        const u32 f = !ring.compact_cache || i >= ring.dev.r ? TILE_W64
-                    : ring.q[i] < (1ull << 32) ? TILE_W32 : ring.q[i] < (1ull << 40) ? TILE_W40 : TILE_W64;
+        const u32 f = ring.q[i] < (1ull << 32) ? TILE_W32 : ring.q[i] < (1ull << 40) ? TILE_W40 : TILE_W64;
         t.fmt_bits |= f << (2 * i);
         t.base[i + 1] = t.base[i] + (size_t)tile_stage_bytes(f) * t.ntiles * t.G * t.C;
     }
     return t;
 }
 
-size_t mac_tile_bytes(const RingHost& ring, const TileLayout& t) { (void)ring; return tile_prime_base(t, t.n_primes); }
+size_t mac_tile_bytes(const TileLayout& t) { return tile_prime_base(t, t.n_primes); }
+
+size_t mac_accounted_bytes(const RingHost& ring, const TileLayout& t) {
+    return ring.compact_cache ? mac_tile_bytes(t) : (size_t)t.n_primes * t.ntiles * t.G * t.C * TILE_STAGE_WORDS * 8;
+}
 
 u32 mac_split_bits(const RingHost& ring) {
     u64 qmax = 0;
@@ -76,8 +79,6 @@ cudaError_t launch_mac(const RingHost& ring, const u64* pt, const TileLayout& la
         m.bs.per_part = (baby->n_in + parts - 1) / parts;
         m.bs.parts = (baby->n_in + m.bs.per_part - 1) / m.bs.per_part;
     }
-    m.compact = false;
-    for (u32 i = 0; i < lay.n_primes; ++i) m.compact = m.compact || tile_format(lay, i) != TILE_W64;
     m.stream = stream;
     ProfScope prof(ring.prof, CAT_MAC, stream);
     return mac_split_bits(ring) == LIMB_NARROW ? launch_mac_narrow(m) : launch_mac_wide(m);

@@ -13,7 +13,7 @@
 // in place, coalesced, and permutes inside the tile on the way to shared memory.  X itself (2 (r+1) N words per term) is
 // never written to memory.
 //
-// What bounds it: HBM (keys and weights are read once, 8 bytes a word).  Loads go straight to registers: a stream that
+// What bounds it: HBM (keys and weights are read once, 5 bytes a word modulo the primes below 2^40).  Loads go straight to registers: a stream that
 // every thread consumes in the pattern it loads needs no staging, no barriers and no producer; what hides the latency is
 // the number of independent loads per thread (2r key words at a time; two batches of 8 weights) times resident warps.
 #pragma once
@@ -30,11 +30,6 @@ __device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
     return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
 }
 
-__device__ __forceinline__ u32 ld_stream8(const void* p, u64 policy) {
-    u32 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u8 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
-    return v;
-}
 
 // Accumulator of one output word of the multiply-accumulate and the form its operands have: weights as stored (two
 // 32-bit halves), the X word as it sits in shared memory.
@@ -46,7 +41,6 @@ struct MacAcc {                                          // OP_NARROW
     __device__ __forceinline__ void end_chunk(const RingDev&, u32, u32) {}
     __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const { return a.reduce(R.q[i], (u32)R.qneg[i]); }
     static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
-    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) { cut_limbs(lo, hi, L, lo, hi); }   // (compact formats)
 };
 template <>
 struct MacAcc<OP_WIDE> {
@@ -71,7 +65,6 @@ struct MacAcc<OP_WIDE> {
         return redc_2x32(barrett64((u64)(v >> 64), R.q[i], R.mu[i]), (u64)v, R.q[i], (u32)R.qneg[i]);
     }
     static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
-    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) { cut_limbs(lo, hi, L, lo, hi); }
 };
 template <>
 struct MacAcc<OP_DP> {
@@ -84,14 +77,9 @@ struct MacAcc<OP_DP> {
         return d2u(a.reduce(R.qd[i], R.qinv_d[i], R.c40_d[i], R.c40_q[i]));
     }
     static __device__ __forceinline__ u64 x_word(u64 v) { return (u64)__double_as_longlong(u2d(v)); }
-    static __device__ __forceinline__ void narrow_word(u32& lo, u32& hi) {
-        const double d = __dsub_rn(__hiloint2double((int)(hi | 0x43300000u), (int)lo), 4503599627370496.0);
-        lo = (u32)__double2loint(d);
-        hi = (u32)__double2hiint(d);
-    }
 };
 
-template <int CLS, int LOG_TN, bool BABY, bool COMPACT, int RC>
+template <int CLS, int LOG_TN, bool BABY, int RC>
 __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict__ pt, const TileLayout& lay,
                                          const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 pj_begin, u32 pj_end,
                                          u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, u64* xs) {
@@ -177,27 +165,29 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
     // ---------------- the weight stream: a lane's words of successive stages lie one stage apart
     if (pj_begin + l >= pj_end) return;
-    const u32 fmt = COMPACT ? tile_format(lay, i) : (u32)TILE_W64;
+    // (primes of class OP_DP have 4 or 5 bytes a word, the others 8: see TileLayout)
+    constexpr bool PACKED = CLS == OP_DP;
+    const u32 fmt = tile_format(lay, i);
     const u32 n_chunks = lay.C;
     u32 left = ((pj_end - pj_begin - l + PL - 1) / PL) * n_chunks;      // stages to go
     const u32 stage_bytes = tile_stage_bytes(fmt);
     const unsigned char* stage = (const unsigned char*)pt + tile_prime_base(lay, i) +
                                  ((size_t)tile * lay.G + pj_begin / PL) * n_chunks * stage_bytes;
     const u32 at = l * TILE_TS * TN + c;
-    constexpr int TS = (int)TILE_TS;
+    constexpr int TS = (int)TILE_TS, TH = PACKED ? TS / 4 : TS;
     // one stage's words of this thread, as they are stored
-    auto fetch = [&](u32 (&wa)[TS], u32 (&wb)[TS]) {
-        if (!COMPACT || fmt == TILE_W64) {
-            const u64* p = (const u64*)stage + at;
-#pragma unroll
-            for (int ts = 0; ts < TS; ++ts) ld_stream(p + ts * TN, pol, wa[ts], wb[ts]);
-        } else {
+    auto fetch = [&](u32 (&wa)[TS], u32 (&wb)[TH]) {
+        if constexpr (PACKED) {
             const u32* p = (const u32*)stage + at;
-            const unsigned char* ph = stage + TILE_STAGE_WORDS * 4u + at;
+            const u32* ph = (const u32*)(stage + TILE_STAGE_WORDS * 4u) + l * 2 * TN + c;
 #pragma unroll
             for (int ts = 0; ts < TS; ++ts) wa[ts] = ld_stream32(p + ts * TN, pol);
 #pragma unroll
-            for (int ts = 0; ts < TS; ++ts) wb[ts] = fmt == TILE_W40 ? ld_stream8(ph + ts * TN, pol) : 0u;
+            for (int h = 0; h < TH; ++h) wb[h] = fmt == TILE_W40 ? ld_stream32(ph + h * TN, pol) : 0u;
+        } else {
+            const u64* p = (const u64*)stage + at;
+#pragma unroll
+            for (int ts = 0; ts < TS; ++ts) ld_stream(p + ts * TN, pol, wa[ts], wb[ts]);
         }
         stage += stage_bytes;
     };
@@ -205,16 +195,18 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
     u32 pj = pj_begin + l, ch = 0;
     const u64* xt = xs + c;
     const u32 tail = n_terms % TILE_TS;
-    auto use = [&](u32 (&wa)[TS], u32 (&wb)[TS]) {
-        if (tail && ch + 1 == n_chunks) {
+    auto use = [&](u32 (&wa)[TS], u32 (&wb)[TH]) {
+        if constexpr (!PACKED) {        // (packed padding is a finite number times a zero of X, whatever it is)
+            if (tail && ch + 1 == n_chunks) {
 #pragma unroll
-            for (int ts = 1; ts < TS; ++ts)
-                if ((u32)ts >= tail) wa[ts] = wb[ts] = 0;
+                for (int ts = 1; ts < TS; ++ts)
+                    if ((u32)ts >= tail) wa[ts] = wb[ts] = 0;
+            }
         }
 #pragma unroll
         for (int ts = 0; ts < TS; ++ts) {
-            u32 w0 = wa[ts], w1 = wb[ts];
-            if (COMPACT && fmt != TILE_W64) Acc::narrow_word(w0, w1);
+            u32 w0 = wa[ts], w1 = wb[PACKED ? ts / 4 : ts];
+            if constexpr (PACKED) unpack40(ts, w1, w0, w1);
             a0.mac(w0, w1, xt[(ts * 2) * TN]);
             a1.mac(w0, w1, xt[(ts * 2 + 1) * TN]);
         }
@@ -234,16 +226,19 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             xt = xs + c;
         }
     };
-    u32 wa[TS], wb[TS], va[TS], vb[TS];
-    fetch(wa, wb);
+    // batches in flight: packed words leave registers for a third
+    constexpr int NB = PACKED ? 3 : 2;
+    u32 wa[NB][TS], wb[NB][TH];
+#pragma unroll
+    for (int s = 0; s + 1 < NB; ++s)
+        if (left > (u32)s) fetch(wa[s], wb[s]);
     for (;;) {
-        if (left > 1) fetch(va, vb);
-        use(wa, wb);
-        if (left <= 1) break;
-        if (left > 2) fetch(wa, wb);
-        use(va, vb);
-        if (left <= 2) break;
-        left -= 2;
+#pragma unroll
+        for (int s = 0; s < NB; ++s) {
+            if (left > (u32)(NB - 1)) fetch(wa[(s + NB - 1) % NB], wb[(s + NB - 1) % NB]);
+            use(wa[s], wb[s]);
+            if (--left == 0) return;
+        }
     }
 }
 
@@ -252,7 +247,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 // Four blocks an SM (64 registers, a few spilled in the key part) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
-template <bool NARROW, int LOG_TN, bool BABY, bool COMPACT, int RC>
+template <bool NARROW, int LOG_TN, bool BABY, int RC>
 __global__ void __launch_bounds__(MAC_THREADS, 4)
 mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const __grid_constant__ TileLayout lay,
            const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 n_pj, u32 pj_per_block,
@@ -263,9 +258,9 @@ mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const 
     const u32 i = lay.n_primes - 1 - blockIdx.x % lay.n_primes;
     const u32 tile = (blockIdx.x / lay.n_primes) & ((1u << tiles_log) - 1u), slice = (blockIdx.x / lay.n_primes) >> tiles_log;
     const u32 pj_begin = slice * pj_per_block, pj_end = min(n_pj, pj_begin + pj_per_block);
-    if (R.dp[i]) mac_body<OP_DP, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
-    else if (NARROW && i < R.r) mac_body<OP_NARROW, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
-    else mac_body<OP_WIDE, LOG_TN, BABY, COMPACT, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    if (R.dp[i]) mac_body<OP_DP, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    else if (NARROW && i < R.r) mac_body<OP_NARROW, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    else mac_body<OP_WIDE, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
 }
 
 struct MacLaunch {
@@ -277,11 +272,11 @@ struct MacLaunch {
     u32 n_pj, n_terms;
     MacScatter sc;
     BabySteps bs;
-    bool baby, compact;
+    bool baby;
     cudaStream_t stream;
 };
 
-template <bool NARROW, int LOG_TN, bool BABY, bool COMPACT, int RC>
+template <bool NARROW, int LOG_TN, bool BABY, int RC>
 static cudaError_t launch_mac_t(const MacLaunch& m) {
     constexpr u32 TN = 1u << LOG_TN, PL = MAC_THREADS >> LOG_TN;
     const RingHost& ring = *m.ring;
@@ -289,7 +284,7 @@ static cudaError_t launch_mac_t(const MacLaunch& m) {
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
     static bool attr_set[MAX_DEVICES] = {false};     // opt in once per device to the large dynamic shared-memory carve-out
     if (!attr_set[device_slot(ring)]) {
-        cudaError_t e = cudaFuncSetAttribute(mac_kernel<NARROW, LOG_TN, BABY, COMPACT, RC>,
+        cudaError_t e = cudaFuncSetAttribute(mac_kernel<NARROW, LOG_TN, BABY, RC>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         attr_set[device_slot(ring)] = true;
@@ -305,28 +300,28 @@ static cudaError_t launch_mac_t(const MacLaunch& m) {
     u32 per = (m.n_pj + slices - 1) / slices;
     per = (per + PL - 1) / PL * PL;
     slices = (m.n_pj + per - 1) / per;
-    return launch_dependent(ring, mac_kernel<NARROW, LOG_TN, BABY, COMPACT, RC>, dim3(tiles * slices), dim3(MAC_THREADS), smem,
+    return launch_dependent(ring, mac_kernel<NARROW, LOG_TN, BABY, RC>, dim3(tiles * slices), dim3(MAC_THREADS), smem,
                             m.stream, ring.dev, m.pt, m.lay, m.x, m.a, m.n_terms, m.n_pj, per, m.sc, m.bs);
 }
 
-template <bool NARROW, bool BABY, bool COMPACT, int RC>
+template <bool NARROW, bool BABY, int RC>
 static cudaError_t launch_mac_tile(const MacLaunch& m) {
     switch (m.lay.log_tn) {
-        case 7: return launch_mac_t<NARROW, 7, BABY, COMPACT, RC>(m);
-        case 6: return launch_mac_t<NARROW, 6, BABY, COMPACT, RC>(m);
-        case 5: return launch_mac_t<NARROW, 5, BABY, COMPACT, RC>(m);
-        default: return launch_mac_t<NARROW, 4, BABY, COMPACT, RC>(m);
+        case 7: return launch_mac_t<NARROW, 7, BABY, RC>(m);
+        case 6: return launch_mac_t<NARROW, 6, BABY, RC>(m);
+        case 5: return launch_mac_t<NARROW, 5, BABY, RC>(m);
+        default: return launch_mac_t<NARROW, 4, BABY, RC>(m);
     }
 }
 
 template <bool NARROW>
 static cudaError_t launch_mac_ring(const MacLaunch& m) {
-    if (!m.baby) return m.compact ? launch_mac_tile<NARROW, false, true, 0>(m) : launch_mac_tile<NARROW, false, false, 0>(m);
+    if (!m.baby) return launch_mac_tile<NARROW, false, 0>(m);
     // (digit counts of the shipped parameter sets: the key words of a rotation in registers)
     switch (m.ring->dev.r) {
-        case 7: return m.compact ? launch_mac_tile<NARROW, true, true, 7>(m) : launch_mac_tile<NARROW, true, false, 7>(m);
-        case 9: return m.compact ? launch_mac_tile<NARROW, true, true, 9>(m) : launch_mac_tile<NARROW, true, false, 9>(m);
-        default: return m.compact ? launch_mac_tile<NARROW, true, true, 0>(m) : launch_mac_tile<NARROW, true, false, 0>(m);
+        case 7: return launch_mac_tile<NARROW, true, 7>(m);
+        case 9: return launch_mac_tile<NARROW, true, 9>(m);
+        default: return launch_mac_tile<NARROW, true, 0>(m);
     }
 }
 

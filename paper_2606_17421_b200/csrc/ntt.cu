@@ -789,13 +789,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     // where the thread's words lie in the tile-major plaintext cache: points 4 lane.., and 128 further on
     unsigned char* tile_stage = nullptr;
     size_t tile_step = 0;
-    u32 tile_at = 0, tile_fmt = 0;
+    u32 tile_at = 0, tile_fmt = 0, tile_high = 0;
     if constexpr (TILED) {
         const u32 d = B.o_base + o, pj_all = d / B.tile.n_terms, term = d - pj_all * B.tile.n_terms, pj = pj_all - B.tile_pj0;
         const u32 n = chunk * LEN + 4 * lane;
         tile_stage = (unsigned char*)B.tile_ptr + tile_stage_of_word(B.tile, pj, term, mod, n);
         tile_at = tile_word_index(B.tile, pj, term, n);
         tile_fmt = tile_format(B.tile, mod);
+        tile_high = tile_high_offset(B.tile, pj, term, n);
         tile_step = (size_t)((128u >> B.tile.log_tn) * B.tile.G * B.tile.C) * tile_stage_bytes(tile_fmt);
     }
     // byte addresses (shared window) of the thread's base point in each of the three access patterns
@@ -871,7 +872,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             // (doubles stay doubles where they are stored as such)
             u64 v4[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, (TILED || EPI == 5) && dp);
+            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, EPI == 5 && dp);
             if constexpr (EPI == 5) {
                 const u32 n = chunk * LEN + 4 * s, nbp = R.r + 1;
                 u32 q_in, j;
@@ -918,21 +919,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 unsigned char* stage = tile_stage + (size_t)it * tile_step;
                 const u32 at = tile_at, fmt = tile_fmt;
                 if (fmt == TILE_W64) {
-                    if (!dp) {          // (else: the bits of doubles already)
-                        const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) v4[i] = limb_split(v4[i], L);
-                    }
-                    stg4((u64*)stage + at, v4[0], v4[1], v4[2], v4[3]);
+                    const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
+                    stg4((u64*)stage + at, limb_split(v4[0], L), limb_split(v4[1], L), limb_split(v4[2], L), limb_split(v4[3], L));
                 } else {
-                    if (dp) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) v4[i] = d2u(__longlong_as_double((long long)v4[i]));
-                    }
                     *(uint4*)(stage + (size_t)at * 4) = make_uint4((u32)v4[0], (u32)v4[1], (u32)v4[2], (u32)v4[3]);
-                    if (fmt == TILE_W40)
-                        *(u32*)(stage + TILE_STAGE_WORDS * 4u + at) = (u32)(v4[0] >> 32) | ((u32)(v4[1] >> 32) << 8) |
-                                                                     ((u32)(v4[2] >> 32) << 16) | ((u32)(v4[3] >> 32) << 24);
+                    if (fmt == TILE_W40) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) stage[tile_high + 4 * i] = (unsigned char)(v4[i] >> 32);
+                    }
                 }
                 continue;
             }
@@ -1055,14 +1049,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                     v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
                     const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) v4[i] = dp ? d2u(__longlong_as_double((long long)v4[i])) : limb_join(v4[i], L);
+                    for (int i = 0; i < 4; ++i) v4[i] = limb_join(v4[i], L);
                 } else {
                     const uint4 lo = *(const uint4*)(stage + (size_t)at * 4);
-                    const u32 hi = fmt == TILE_W40 ? *(const u32*)(stage + TILE_STAGE_WORDS * 4u + at) : 0u;
-                    v4[0] = lo.x | ((u64)(hi & 255u) << 32);
-                    v4[1] = lo.y | ((u64)((hi >> 8) & 255u) << 32);
-                    v4[2] = lo.z | ((u64)((hi >> 16) & 255u) << 32);
-                    v4[3] = lo.w | ((u64)(hi >> 24) << 32);
+                    v4[0] = lo.x; v4[1] = lo.y; v4[2] = lo.z; v4[3] = lo.w;
+                    if (fmt == TILE_W40) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v4[i] |= (u64)stage[tile_high + 4 * i] << 32;
+                    }
                 }
             } else {
                 const ulonglong2* gp = (const ulonglong2*)(gsrc + 4 * s);
