@@ -6,9 +6,9 @@ timed beside it.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload qwen3_step@budget=60] [--impl reference]
 
 A step = one decode token's worth of the workload: the encrypted product and its rescale
-(bf_linear_rescaled: bf_linear + bf_rescale as one call) for every linear layer of the workload, cached encoded weights streamed from HBM (49 GB per step for the Qwen3-0.6B-shaped
-default, 352 MB for the single GPT-2 projection: always larger than L2, so consecutive steps cannot
-be served from cache).  The other configurations are timed after the main one and reported under
+(bf_linear_rescaled: bf_linear + bf_rescale as one call) for every linear layer of the workload, cached encoded weights
+streamed from HBM (27 GB per step for the Qwen3-0.6B-shaped default, 239 MB for the single GPT-2 projection, beside 0.3 GB
+of rotation keys a call: always larger than L2, so consecutive steps cannot be served from cache).  The other configurations are timed after the main one and reported under
 "other_workloads", each with its own rooflines.  Inputs are seeded and synthetic.
 """
 from __future__ import annotations
@@ -30,23 +30,17 @@ METRIC = "encrypted linear-layer ms per decode token"
 UNIT = "ms"
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) relative to the algorithmic bytes of the same launches,
-# from ncu captures summarised under profiles/.  The headline workload is too large for a multi-pass capture (37.6 GB on
-# the device), so the figures come from one GPT-2 layer under the same plan (same kernels, same call shapes), whose
-# traffic grows in proportion to the streamed bytes; `traffic` in the line = this ratio x the algorithmic bytes of a launch.
+# from an ncu capture summarised under profiles/ (the headline workload is too large for a multi-pass capture: one GPT-2
+# layer under the same plan, same kernel); `traffic` in the line = this ratio x the algorithmic bytes of a launch.
 NCU_TRAFFIC_RATIO = {
-    "mac": 1.32,                  # eight captured launches (four calls): 1417 MB for 1074 MB of cached words (rotated inputs, outputs)
-    "key_inner_product": 1.40,    # eight captured launches: 1352 MB for 33 distinct keys of 29.36 MB (digit sets, outputs)
+    "mac": 1.07,                  # the 768 -> 2304 call: 626 MB for 585 MB of keys and weights (digits, outputs)
 }
-# (ncu flushes the caches before every captured launch: rotated inputs and digit sets that a step finds in L2 count as
-# DRAM traffic in these ratios)
-# Executed warp instructions per butterfly by pipe, from the same captures (profiles/gpt2_layer_headline_plan_kernels_ncu.md),
-# to set beside the modelled 8 / 12 / 10 operations: the large fp64-path batches of each direction.
+# Executed warp instructions per butterfly by pipe, from the same captures (profiles/transform_passes_ncu.md), to set beside
+# the modelled 8 / 12 / 10 operations: 1024 transforms into six primes on the 8-operation fp64 path, one on the 12-operation
+# one, one on the 60-bit integer path.
 NCU_PIPE_INSTR = {
-    "ntt_forward": {"all": 24.7, "fp64": 8.3, "alu": 6.3, "fma_integer": 5.4, "lsu": 2.4,
-                    "from": "hoisted ModUp of three inputs (147 transforms: six primes on the 8-operation fp64 path, one "
-                            "on the 12-operation one, one on the 60-bit integer path), both passes"},
-    "ntt_inverse": {"all": 21.0, "fp64": 10.3, "alu": 3.9, "fma_integer": 2.0, "lsu": 2.3,
-                    "from": "c1 of 3 giant rotations x 7 primes, both passes (an earlier capture of the same kernels)"},
+    "ntt_forward": {"all": 24.4, "fp64": 8.7, "alu": 5.3, "fma_integer": 5.2, "lsu": 2.2,
+                    "from": "weights kept as coefficients, 128 diagonals into 8 primes, both passes"},
 }
 
 
@@ -173,17 +167,22 @@ def transform_counts(runner) -> dict:
     (at least 10 32-bit multiply-adds per butterfly)."""
     import math
     r, N = runner.r, runner.N
-    per = (N // 2) * int(math.log2(N))
+    per = (N // 2) * int(math.log2(N))           # butterflies of a transform
     moduli = list(runner.primes) + [runner.P]
     cost = [8 if q < (1 << 41) else 12 if q < (1 << 50) else 10 for q in moduli]
     fp = [q < (1 << 50) for q in moduli]
     fwd = [0] * (r + 1)
     inv = [0] * (r + 1)
+    fused = [0] * (r + 1)       # ModUp digits whose second pass (8 of the log2 N stages) is part of the key-switch product
     for e in runner.layers:
         n_in, n_out, b, g = e["n_in"], e["n_out"], e["b"], e["g"]
         n_giant = (g - 1) * n_out
         sets = (n_in if b > 1 else 0) + n_giant            # ModUp digit sets
-        rots = n_in * (b - 1) + n_giant                    # key switches
+        products = sets if runner.plan.hoist != "double" else n_giant      # digit sets multiplied in a launch of their own
+        in_place = r if runner.plan.hoist == "double" and runner.plan.moddown == "per_output" else r - 1
+        for i in range(r):
+            fused[i] += products * in_place
+        fused[r] += products * r
         # divisions by P: one per rotation and component, or (per_output) one per baby rotation and per output
         n_baby_lift = 2 * n_out * g if runner.plan.hoist == "double" else 2 * n_in * (b - 1)
         n_lift = n_baby_lift + 2 * (n_out if runner.plan.moddown == "per_output" and n_giant else n_giant)
@@ -207,8 +206,9 @@ def transform_counts(runner) -> dict:
             n_diag = n_in * n_out * b * g
             for i in range(r + (1 if runner.plan.hoist == "double" else 0)):
                 fwd[i] += n_diag
+    fwd = [c - f * 8.0 / math.log2(N) for c, f in zip(fwd, fused)]
     def summary(cnt):
-        return {"polys": sum(cnt), "fp64_polys": sum(c for c, f in zip(cnt, fp) if f),
+        return {"polys": round(sum(cnt), 1), "fp64_polys": round(sum(c for c, f in zip(cnt, fp) if f), 1),
                 "fp64_ops": sum(c * k for c, k, f in zip(cnt, cost, fp) if f),
                 "int_ops": sum(c * k for c, k, f in zip(cnt, cost, fp) if not f)}
     return {"fwd": summary(fwd), "inv": summary(inv), "per_poly": per}
@@ -305,18 +305,16 @@ class Measurement:
             return (ms / n) if n else None, n / K
 
         rl = {}
-        # weight-streaming multiply-accumulate: algorithmic bytes = every encoded word once
+        # weight-streaming multiply-accumulate: algorithmic bytes = every encoded word once, and under double hoisting the
+        # baby rotations' keys, whose inner products are part of it
         mac_ms, mac_n = avg_ms("mac")
         if mac_ms:
-            mac_bytes = R.total_pt_bytes() / max(1.0, mac_n)
+            mac_bytes = R.mac_stream_bytes() / max(1.0, mac_n)
             ach = mac_bytes / (mac_ms * 1e-3) / 1e9
             rl["mac"] = {"bound": "hbm", "achieved": round(ach, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(ach / hbm_peak, 4), "of": peak_kind, "traffic": traffic_of("mac", mac_bytes),
                          "launches_per_step": mac_n, "avg_ms": round(mac_ms, 5),
                          "bytes_per_launch": round(mac_bytes), "frac_of_nominal_8000": round(ach / 8000.0, 4)}
-            if R.plan.hoist == "double":
-                rl["mac"]["note"] = ("a call's two launches (ciphertext primes; the special prime beside it on a second "
-                                     "stream) are timed as one span, the way they run; avg_ms = that span / 2")
         # key-switch inner product: algorithmic bytes = every distinct key of a launch once
         ki_ms, ki_n = avg_ms("key_inner_product")
         if ki_ms:
@@ -331,7 +329,8 @@ class Measurement:
                                        "bytes_per_launch": round(distinct / n_launch),
                                        "achieved_counting_a_key_per_rotation": round(ach_rot, 1),
                                        "note": "bytes = the distinct keys of a launch, each once; the second figure "
-                                               "counts a key once per rotation (repeats are L2 hits)"}
+                                               "counts a key once per rotation (repeats are L2 hits); the "
+                                               "launch also does the second pass of its digits' transforms"}
         # transforms: bound by the arithmetic pipes (fp64 for the ciphertext primes, integer multiply-add for the
         # special prime); the peak uses the two rates measured in this run
         for cats, key, label in ((("ntt_fwd_strided", "ntt_fwd_contig"), "fwd", "ntt_forward"),

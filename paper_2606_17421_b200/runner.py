@@ -61,10 +61,13 @@ class WorkloadRunner:
         if coef_bits:               # weights resident as rounded 64- or 32-bit coefficients, transformed on every call
             bf.bf_set_coefficient_cache(self.ctx, coef_bits)
         self.coef_bits = coef_bits
-        # resident bytes per encoded coefficient over all primes (8 each, or 4 / 5 / 8 by prime size when compact)
+        # bytes an encoded coefficient counts for over all primes (8 each, or 4 / 5 / 8 by prime size when compact), and those
+        # it has
         self.word_bytes = sum((4 if q < 2 ** 32 else 5 if q < 2 ** 40 else 8) if compact_cache else 8 for q in self.primes)
+        self.stream_word_bytes = sum(4 if q < 2 ** 32 else 5 if q < 2 ** 40 else 8 for q in self.primes)
         if self.plan.hoist == "double":     # the residue modulo the special prime is kept too, always in 8 bytes
             self.word_bytes += 8
+            self.stream_word_bytes += 8
         budget = cache_budget_bytes if cache_budget_bytes is not None else self.w.cache_budget_bytes
         if budget:
             bf.bf_set_cache_budget(self.ctx, int(budget))
@@ -162,6 +165,15 @@ class WorkloadRunner:
 
     def total_pt_bytes(self):
         return sum(e["pt_bytes"] for e in self.layers)
+
+    def mac_stream_bytes(self):
+        """Bytes the multiply-accumulates of a step cannot do without: every encoded word once and, where they make the
+        baby rotations (double hoisting), every baby key of a call once."""
+        total = sum(e["pt_bytes"] for e in self.layers) * self.stream_word_bytes // self.word_bytes
+        if self.plan.hoist == "double":
+            words = sum(5 if q < 2 ** 40 else 8 for q in self.primes) + 8
+            total += sum(e["b"] - 1 for e in self.layers) * 2 * self.r * self.N * words
+        return total
 
     def n_fallback_layers(self):
         return sum(1 for e in self.layers if not e["handle"])
