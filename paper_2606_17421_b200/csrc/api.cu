@@ -605,10 +605,11 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
                         const TileLayout& lay, u32 pj0, const bf_weights* stored = nullptr, i64* coef_out = nullptr,
                         u32 split_b = 0, u32 split_g = 0) {
     const u32 N = ctx->N, r = lay.n_primes, n = N / 2;       // (r: primes each diagonal is reduced into)
-    // diagonals per pass: the encoder and the transforms gain from large batches (measured: 32 -> 128 per
-    // pass takes 6 to 8 % off a call that encodes on the fly); the scratch of a pass is held to about 0.5 GB
-    u32 chunk = (u32)(((size_t)512 << 20) / ((size_t)r * N * sizeof(u64))) & ~7u;
-    if (chunk > 256) chunk = 256;
+    // diagonals per pass: the encoder and the transforms gain from large batches (256 of them at N = 2^15: a coefficient layer
+    // in 2738 us, in passes of 64 2792, of 32 2874; 256 instead of 102 at N = 2^16: 2690 instead of 2792 us for a product
+    // encoded on the way); the scratch of a pass is held to about 1.5 GB
+    u32 chunk = (u32)(((size_t)1536 << 20) / ((size_t)r * N * sizeof(u64))) & ~7u;
+    if (chunk > 512) chunk = 512;
     if (chunk < 32) chunk = 32;
     if (chunk > count) chunk = count > 0 ? count : 1;
     if (!stored) TRY(ensure(ctx, ctx->fft, (size_t)chunk * n * sizeof(double2)));
