@@ -711,11 +711,11 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
     }
 }
 
-// Contiguous pass: every warp transforms one chunk of 256 adjacent points (8 per thread) through
-// the groups {3,3,2}; the chunk lives in the warp's own swizzled slice of shared memory between
-// groups, so only warp-level synchronisation is needed.
-// What bounds it: instruction issue.  An fp64 instruction takes two issue slots of its scheduler, any other one, and the
-// cycles per chunk are that sum (1020 of 324 fp64 and 367 other instructions, all primes below 2^41), with warps to spare.
+// Contiguous pass: a warp, or a block of 64 threads, transforms one chunk of 256 adjacent points (8 or 4 per thread, see
+// contig_forward_far); the chunk lives in a swizzled slice of shared memory between groups.
+// What bounds it: nothing alone.  In a launch of 1024 transforms modulo primes below 2^41 a chunk takes 255 cycles of an SM,
+// with 691 warp instructions (68 % of the issue slots), 324 of them fp64 (64 % of that pipe) and about 165 wavefronts of the
+// L1 pipe (65 %); small launches are bound by the latency of one chunk.
 // Forward: second pass (final reduction to [0, q), then the store functors).  Inverse: first pass
 // (reads the batch source: plain residues, tiled/limb-split plaintexts, or a sum of arrays).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
@@ -724,6 +724,7 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // ModDownEpilogue); 5 = ingest (see PolyBatch): the digits into the operand array, component c of the inputs times P into
 // lift_ptr.
 constexpr int CONTIG_THREADS = 128, CONTIG_WARPS = CONTIG_THREADS / 32;
+constexpr size_t CONTIG_SHORT_CHUNKS = 12000;       // forward launches of up to that many chunks: see ntt_contig_short
 
 // a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
 template <int PATH, typename T>
@@ -746,10 +747,30 @@ __device__ __forceinline__ u64 times_p(const RingDev& R, u32 m, u64 v) {
     return reduce128(hi, lo, R.q[m], R.mu[m], R.c64[m], R.c64s[m]);
 }
 
-// The first two groups of the forward pass over one chunk; the chunk is left in the warp's slice for the third, whose sets
-// are the 4 adjacent points at swizzled index 4 (lane + 32 it).
-template <int PATH, typename T>
+// All but the last group of the forward pass over one chunk; the chunk is left in its slice for the last, whose sets are the
+// 4 adjacent points at swizzled index 4 (lane + 32 it).
+// THREADS threads a chunk: 32 with 8 points each and groups {3,3,2}, or 64 with 4 points and groups of 2.
+template <int PATH, int THREADS = 32, typename T>
 __device__ __forceinline__ void contig_forward_far(const T* gsrc, u32 slice, int lane, const void* tw, u32 mult, const ModConsts& c) {
+    if constexpr (THREADS == 64) {
+        const u32 a0 = slice + 8u * (u32)swz(lane), a1 = slice + 8u * (u32)swz((lane >> 4) * 64 + (lane & 15)),
+                  a2 = slice + 8u * (u32)swz((lane >> 2) * 16 + (lane & 3));
+        T e[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e[i] = gsrc[lane + 64 * i];
+        set_butterflies<2, true, PATH, false>(e, tw, mult, c);
+        swz_store_set<4, 6>(a0, e);
+        __syncthreads();
+        swz_load_set<4, 4>(a1, e);
+        set_butterflies<2, true, PATH, false>(e, tw, 4u * mult + (lane >> 4), c);
+        swz_store_set<4, 4>(a1, e);
+        __syncthreads();
+        swz_load_set<4, 2>(a2, e);
+        set_butterflies<2, true, PATH, false>(e, tw, 16u * mult + (lane >> 2), c);
+        swz_store_set<4, 2>(a2, e);
+        __syncthreads();
+        return;
+    }
     const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
     const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
     T e[8];
@@ -766,7 +787,8 @@ __device__ __forceinline__ void contig_forward_far(const T* gsrc, u32 slice, int
     __syncwarp();
 }
 
-template <bool FWD, int EPI, int PATH, bool TILED>
+// (THREADS: see contig_forward_far; the inverse pass always has 64)
+template <bool FWD, int EPI, int PATH, bool TILED, int THREADS>
 __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u32 o, u32 m, u32 mod,
                                             u32 chunk, int lane, const RotBatch& rb, const ModDownEpilogue& epi) {
     typedef typename Elem<PATH>::T T;
@@ -799,16 +821,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
         tile_high = tile_high_offset(B.tile, pj, term, n);
         tile_step = (size_t)((128u >> B.tile.log_tn) * B.tile.G * B.tile.C) * tile_stage_bytes(tile_fmt);
     }
-    // byte addresses (shared window) of the thread's base point in each of the three access patterns
+    // byte addresses (shared window) of the thread's base points
     const u32 slice = (u32)__cvta_generic_to_shared(sm);
-    const u32 a_far = slice + 8u * (u32)swz(lane);                                    // points lane + 32 i
-    const u32 a_mid = slice + 8u * (u32)swz((lane >> 2) * 32 + (lane & 3));           // points base + 4 i
     const u32 a_near = slice + 8u * (u32)swz(4 * lane);                               // points 4 (lane + 32 it) + i
     if (FWD) {
-        contig_forward_far<PATH>((const T*)gsrc, slice, lane, tw, mult, c);
-        // group 2: K = 2, adjacent points; two sets per thread
+        contig_forward_far<PATH, THREADS>((const T*)gsrc, slice, lane, tw, mult, c);
+        // last group: K = 2, adjacent points; two sets per thread
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {
+        for (int it = 0; it < 64 / THREADS; ++it) {
             const int s = lane + 32 * it;
             swz_load_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), e);      // (swz(128) = 128: above the bits of 4 * lane)
             // the epilogue's operands do not depend on the transform: ask for them before the last butterflies
@@ -957,7 +977,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     } else {
         // inverse: groups in the opposite order
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {
+        for (int it = 0; it < 64 / THREADS; ++it) {
             const int s = lane + 32 * it;
             u64 v4[4];
             if constexpr (EPI == 2) {   // the residues of this output's giant rotations, each read through its rotation, summed
@@ -1092,42 +1112,69 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             set_butterflies<2, false, PATH, false>(e, tw, 64u * mult + s, c);
             swz_store_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), e);
         }
-        __syncwarp();
-        swz_load_set<8, 2>(a_mid, e);
-        set_butterflies<3, false, PATH, false>(e, tw, 8u * mult + (lane >> 2), c);
-        centre_sums<3, PATH>(e, c);
-        swz_store_set<8, 2>(a_mid, e);
-        __syncwarp();
-        swz_load_set<8, 5>(a_far, e);
-        set_butterflies<3, false, PATH, false>(e, tw, mult, c);
-        centre_sums<3, PATH>(e, c);
+        const u32 a0 = slice + 8u * (u32)swz(lane), a1 = slice + 8u * (u32)swz((lane >> 4) * 64 + (lane & 15)),
+                  a2 = slice + 8u * (u32)swz((lane >> 2) * 16 + (lane & 3));
+        __syncthreads();
+        swz_load_set<4, 2>(a2, e);
+        set_butterflies<2, false, PATH, false>(e, tw, 16u * mult + (lane >> 2), c);
+        centre_sums<2, PATH>(e, c);
+        swz_store_set<4, 2>(a2, e);
+        __syncthreads();
+        swz_load_set<4, 4>(a1, e);
+        set_butterflies<2, false, PATH, false>(e, tw, 4u * mult + (lane >> 4), c);
+        centre_sums<2, PATH>(e, c);
+        swz_store_set<4, 4>(a1, e);
+        __syncthreads();
+        swz_load_set<4, 6>(a0, e);
+        set_butterflies<2, false, PATH, false>(e, tw, mult, c);
+        centre_sums<2, PATH>(e, c);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) ((T*)gdst)[lane + 32 * i] = e[i];      // lazy; the strided pass finishes
+        for (int i = 0; i < 4; ++i) ((T*)gdst)[lane + 64 * i] = e[i];      // lazy; the strided pass finishes
     }
 }
 
 // grid: x = group of 2^log_wo outer indices, y = slot m, z = group of chunks.
 // (the per-output forms run on a few polynomials per launch and hold the operands of three rotations at once: they
 // trade resident blocks for registers)
-template <bool FWD, int EPI, bool TILED>
-__global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 || EPI == 4 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
+template <int EPI, bool TILED>
+__global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
                                                                        u32 n_outer, u32 log_wo, const RotBatch rb,
                                                                        const ModDownEpilogue epi) {
     __shared__ __align__(128) u64 sm_all[CONTIG_WARPS << LOG_C];
     grid_dependency_enter();
     const u32 m = slot_of_block(blockIdx.y, B.n_m);
-    u32 mod = batch_modulus<EPI == 4>(R, B, m);
+    u32 mod = batch_modulus<false>(R, B, m);
     const u32 warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const u32 o = (blockIdx.x << log_wo) + (warp & ((1u << log_wo) - 1)), chunk = blockIdx.z * (CONTIG_WARPS >> log_wo) + (warp >> log_wo);
     if (o >= n_outer || chunk >= (R.N >> LOG_C)) return;    // (whole warps leave)
     if (EPI == 5 && m > R.r) mod = o % R.r;         // (component 0, in the prime it is a residue of)
-    if (FWD && own_prime(R, B, o, mod)) return;
+    if (own_prime(R, B, o, mod)) return;
     u64* sm = sm_all + (warp << LOG_C);
     const int path = path_of(R, mod);
-    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else contig_body<FWD, EPI, PATH_INT, TILED>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    if (path == PATH_DP) contig_body<true, EPI, PATH_DP, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else if (path == PATH_WIDE) contig_body<true, EPI, PATH_WIDE, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else contig_body<true, EPI, PATH_INT, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+}
+
+// The same with a block of 64 threads per chunk, 4 points a thread: the inverse pass, and forward launches too small to run
+// in many rounds, whose time is that of one chunk, and of the integer path's in particular.  (Forward launches of up to 12000
+// chunks and all inverse ones: the calls of a 0.6B layer 1362 -> 1327 us, a 64 x 64 product on a ring of 2^12 70 -> 61 us.
+// Inverse launches of a LLaMA-3-8B layer, up to 36000 chunks: 549 -> 477 us.  Forward launches of 200000 chunks: 783 us with
+// 8 points, 938 us with 4, for an exchange through shared memory more.)  grid: x = outer index, y = slot m, z = chunk.
+template <bool FWD, int EPI, bool TILED>
+__global__ void __launch_bounds__(64, EPI == 2 || EPI == 4 ? 10 : 16) ntt_contig_short(const RingDev R, const PolyBatch B, const RotBatch rb,
+                                                                                    const ModDownEpilogue epi) {
+    __shared__ __align__(128) u64 sm[1 << LOG_C];
+    grid_dependency_enter();
+    const u32 m = slot_of_block(blockIdx.y, B.n_m), o = blockIdx.x, chunk = blockIdx.z;
+    u32 mod = batch_modulus<EPI == 4>(R, B, m);
+    if (EPI == 5 && m > R.r) mod = o % R.r;         // (component 0, in the prime it is a residue of)
+    if (FWD && own_prime(R, B, o, mod)) return;
+    const int path = path_of(R, mod), lane = threadIdx.x;
+    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    else contig_body<FWD, EPI, PATH_INT, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
 }
 
 // Key-switch products (Sec. 4.2 "key-switching primitives"): the contiguous pass of the digits' transforms and their inner
@@ -1359,37 +1406,35 @@ static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u3
     PolyBatch B = B_in;
     const u32 n_outer = n_polys / B.n_m;
     set_magics(B, n_outer);
+    const u32 chunks = ring.dev.N >> LOG_C;
+    static const RotBatch no_rb = {};
+    static const ModDownEpilogue no_epi = {};
+    const RotBatch& rots = rb ? *rb : no_rb;
+    const ModDownEpilogue& ep = epi ? *epi : no_epi;
     // the four warps of a block take the same chunk of four polynomials where the batch has enough of them (one fetch of the
     // chunk's twiddles serves them), else of two, else neighbouring chunks
     const u32 log_wo = n_outer % 4 == 0 || n_outer >= 16 ? 2u : n_outer % 2 == 0 || n_outer >= 7 ? 1u : 0u;
-    const u32 per = CONTIG_WARPS >> log_wo, chunks = ring.dev.N >> LOG_C;
-    const dim3 grid((n_outer + (1u << log_wo) - 1) >> log_wo, B.n_m, (chunks + per - 1) / per);
-    if (FWD && epi && epi->plain) {
-        launch_dependent(ring, ntt_contig<FWD, 3, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
-                         *epi);
-    } else if (FWD && B.ingest) {
-        static const RotBatch no_rb = {};
-        static const ModDownEpilogue no_epi = {};
-        launch_dependent(ring, ntt_contig<true, 5, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, no_rb, no_epi);
-    } else if (!FWD && epi && epi->assemble) {
-        launch_dependent(ring, ntt_contig<false, 4, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
-                         *epi);
-    } else if (epi && epi->n_sum) {
-        launch_dependent(ring, ntt_contig<FWD, 2, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
-                         *epi);
-    } else if (FWD && epi) {
-        launch_dependent(ring, ntt_contig<FWD, 1, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, *rb,
-                         *epi);
-    } else {
-        static const RotBatch no_rb = {};
-        static const ModDownEpilogue no_epi = {};
-        if (B.tile_ptr)
-            launch_dependent(ring, ntt_contig<FWD, 0, true>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo,
-                             no_rb, no_epi);
-        else
-            launch_dependent(ring, ntt_contig<FWD, 0, false>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo,
-                             no_rb, no_epi);
-    }
+    const u32 per = CONTIG_WARPS >> log_wo;
+    const dim3 grid((n_outer + (1u << log_wo) - 1) >> log_wo, B.n_m, (chunks + per - 1) / per), grid_short(n_outer, B.n_m, chunks);
+    auto go = [&](auto epi_c, auto tiled_c) {
+        constexpr int EPI = decltype(epi_c)::value;
+        constexpr bool TILED = decltype(tiled_c)::value;
+        if constexpr (FWD) {
+            if ((size_t)n_polys * chunks > CONTIG_SHORT_CHUNKS) {
+                launch_dependent(ring, ntt_contig<EPI, TILED>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, rots, ep);
+                return;
+            }
+        }
+        launch_dependent(ring, ntt_contig_short<FWD, EPI, TILED>, grid_short, dim3(64), 0, stream, ring.dev, B, rots, ep);
+    };
+    const std::integral_constant<bool, false> plain_store;
+    if (FWD && epi && epi->plain) go(std::integral_constant<int, FWD ? 3 : 0>(), plain_store);
+    else if (FWD && B.ingest) go(std::integral_constant<int, FWD ? 5 : 0>(), plain_store);
+    else if (!FWD && epi && epi->assemble) go(std::integral_constant<int, FWD ? 0 : 4>(), plain_store);
+    else if (epi && epi->n_sum) go(std::integral_constant<int, 2>(), plain_store);
+    else if (FWD && epi) go(std::integral_constant<int, FWD ? 1 : 0>(), plain_store);
+    else if (B.tile_ptr) go(std::integral_constant<int, 0>(), std::integral_constant<bool, true>());
+    else go(std::integral_constant<int, 0>(), plain_store);
     return cudaGetLastError();
 }
 
