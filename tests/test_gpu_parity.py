@@ -532,6 +532,13 @@ def test_random_small_ring_cases(case):
         g.close()
 
 
+@pytest.mark.parametrize("n_out", [124, 126])
+def test_one_division_per_output_on_both_sides_of_the_short_launches(n_out):
+    # forward passes of up to 12000 chunks have 4 points a thread, longer ones 8: n_out * 2 components * 3 primes * 16 chunks
+    par = oracle_params("n12")
+    run_case(par, ckks.Plan(16, 1, 8, 2, moddown="per_output"), n_out * 16, 16, 37, 1e-2, "short", tight=1e-2)
+
+
 @pytest.mark.parametrize("modes", [{}, dict(moddown="per_output", hoist="double")], ids=["plain", "extended"])
 @pytest.mark.parametrize("logN,bits,plan_t,shape", [
     (10, [50, 45, 40, 30], (32, 2, 4, 4), (70, 90)),        # every operand class; 12 terms (a stage half empty), 3 inputs
