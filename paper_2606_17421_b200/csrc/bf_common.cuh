@@ -269,7 +269,7 @@ struct TileLayout {
     u32 log_tn, n_terms, n_pj, G, C, ntiles;
     u32 fmt_bits;                           // TileFormat of prime i in bits 2i, 2i+1
     u32 n_primes;                           // primes the plaintexts are held in: r, or r + 1 with double hoisting
-                                            //   (the special prime last, always in 8-byte whole words)
+                                            //   (the special prime last, in the format its own size asks for)
     size_t base[MAX_MODULI + 1];            // see tile_prime_base
 };
 constexpr u32 TILE_TS = 8;

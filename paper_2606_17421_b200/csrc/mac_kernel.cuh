@@ -259,7 +259,9 @@ mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const 
     const u32 tile = (blockIdx.x / lay.n_primes) & ((1u << tiles_log) - 1u), slice = (blockIdx.x / lay.n_primes) >> tiles_log;
     const u32 pj_begin = slice * pj_per_block, pj_end = min(n_pj, pj_begin + pj_per_block);
     if (R.dp[i]) mac_body<OP_DP, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
-    else if (NARROW && i < R.r) mac_body<OP_NARROW, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
+    // (the class follows the words' limbs, as the tile store cuts them: 25 bits below 2^50 where every ciphertext prime is, the
+    // special prime included, else 30)
+    else if (NARROW && !(R.q[i] >> 50)) mac_body<OP_NARROW, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
     else mac_body<OP_WIDE, LOG_TN, BABY, RC>(R, pt, lay, x, a, n_terms, pj_begin, pj_end, tile, i, sc, bs, mac_xs);
 }
 

@@ -559,6 +559,25 @@ def test_operand_classes_and_tile_edges(logN, bits, plan_t, shape, modes):
     run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 31, 1e-2, "classes", tight=1e-2)
 
 
+@pytest.mark.parametrize("moddown", ["per_rotation", "per_output"])
+@pytest.mark.parametrize("plan_t", [(32, 2, 4, 4), (32, 4, 1, 8)], ids=["baby_steps", "none"])
+@pytest.mark.parametrize("bits,special_bits", [
+    ([50, 40, 40], 49),                     # the special prime below 2^50 among such primes: 25-bit limbs
+    ([45, 40, 39], 41),                     # ... below 2^41, the transforms' lazily reduced path
+    ([59, 45, 40], 45),                     # a ciphertext prime beyond 2^50: 30-bit limbs throughout
+    ([50, 40, 40], 38),                     # fp64 operands, 5-byte words
+    ([50, 40, 40], 31),                     # ... 4-byte words
+])
+def test_double_hoisting_with_a_special_prime_of_every_operand_class(bits, special_bits, plan_t, moddown):
+    two_n = 2 << 10
+    primes = [ckks.find_primes(1 << b, two_n, 2)[i] for i, b in enumerate(bits) if i < 2] + ckks.find_primes(1 << bits[2], two_n, 3)[2:]
+    P = ckks.find_primes(1 << special_bits, two_n, 1)[0]
+    assert len(set(primes + [P])) == 4
+    # (a special prime below the digits' primes: the key switch adds noise of about q / P times the usual, far below 2^80)
+    run_case(ckks.Params(1 << 10, primes, P, 2.0 ** 40), ckks.Plan(*plan_t, moddown=moddown, hoist="double"), 70, 90, 13, 1e-2,
+             "special", tight=1e-2)
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
