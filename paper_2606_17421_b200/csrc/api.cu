@@ -978,17 +978,21 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     const size_t groups_fit = ctx->encode_scratch_bytes / ((size_t)n_terms * nmp * N * 8);
     const u32 groups = groups_fit < 1 ? 1u : groups_fit > (size_t)n_pj ? n_pj : (u32)groups_fit;
     // the multiply-accumulate makes the rotated inputs itself, unless it runs in several rounds: each would stream the
-    // keys again, so that X is worth keeping in memory then
-    const bool rotate_in_mac = dh && b > 1 && (resident || groups == n_pj);
-    if (rotate_in_mac) in_batch = n_in;
-    u32 n_dig_sets = giant_per_lane * (u32)lanes;       // digit sets alive at once
-    // (the digits that the multiply-accumulate reads lie before those between the passes)
-    const u32 in_sets = rotate_in_mac ? 2 * in_batch : in_batch;
-    if (n_dig_sets < in_sets) n_dig_sets = in_sets;
+    // keys again, so that X is worth keeping in memory then.  It reads the digits of all inputs (r (r+1) polynomials each),
+    // where the other form keeps those of a batch and X; it is used where its scratch stays within that of the other form
+    // plus one more buffer of that one's digits (240 inputs, r = 15 and one rotation each, N = 2^10: 1139 MB in the one form,
+    // 350 MB in the other).  Their transforms run in batches of what giant_batch allows.
+    const u32 giant_sets = giant_per_lane * (u32)lanes, ingest_batch = gb < n_in ? gb : n_in;
+    const u32 other_sets = giant_sets > in_batch ? giant_sets : in_batch;
+    const bool rotate_in_mac = dh && b > 1 && (resident || groups == n_pj) &&
+                               ((u64)n_in + ingest_batch) * r <= (u64)2 * other_sets * r + (u64)2 * n_in * (b - 1);
+    // digit sets alive at once (those that the multiply-accumulate reads lie before those between the passes)
+    const u32 in_sets = rotate_in_mac ? n_in + ingest_batch : in_batch;
+    const u32 n_dig_sets = giant_sets > in_sets ? giant_sets : in_sets;
     const size_t xw = (size_t)2 * nmp * N;                // words per term of X / per inner sum
     TRY(ensure(ctx, ctx->X, (size_t)n_in * (rotate_in_mac ? 1u : b) * xw * 8));
     if (dh) {
-        TRY(ensure(ctx, ctx->X0, (size_t)n_in * (rotate_in_mac ? ctw / 2 : ctw) * 8));
+        TRY(ensure(ctx, ctx->X0, rotate_in_mac ? (size_t)ingest_batch * r * N * 8 : (size_t)n_in * ctw * 8));
         TRY(ensure(ctx, ctx->Aext, (size_t)n_out * g * xw * 8));
     }
     TRY(ensure(ctx, ctx->A, (size_t)n_out * g * ctw * 8));
@@ -1005,7 +1009,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     // (see below); their coefficient forms keep the residue modulo P
     const bool assemble = dh && per_output;
     const u32 cc_primes = assemble ? nb : r;
-    TRY(ensure(ctx, ctx->Cc, (size_t)n_dig_sets * cc_primes * N * 8));
+    TRY(ensure(ctx, ctx->Cc, (size_t)giant_sets * cc_primes * N * 8));
     {
         u32 rot_scratch = rot_per_lane * (u32)lanes;
         if (per_output && rot_scratch < n_out) rot_scratch = n_out;     // Tc, Tn of the per-output division
@@ -1044,7 +1048,6 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     const long long x0_stride = dh ? (long long)ctw : (long long)b * ctw;
     if (rotate_in_mac) {
         u64* mid = Dig + (size_t)n_in * r * nb * N;
-        B.src = ct_in;
         B.o_div = r;                        // o = (input * 2 + component) * r + prime
         B.src_so2 = (long long)r * N;
         B.src_so = N;
@@ -1054,11 +1057,14 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
         B.mod_step = 1;
         B.src_digits = 1;
         B.tail_dst = (u64*)ctx->X0.p;
-        B.dtile_ptr = Dig;
         B.dtile_div = r;
-        B.lift_ptr = X;
         B.lift_so = (long long)xw;
-        CK(ntt_forward_ingest(ctx->ring, B, n_in, ctx->stream));
+        for (u32 q0 = 0; q0 < n_in; q0 += ingest_batch) {
+            B.src = ct_in + (size_t)q0 * ctw;
+            B.dtile_ptr = Dig + (size_t)q0 * r * nb * N;
+            B.lift_ptr = X + (size_t)q0 * xw;
+            CK(ntt_forward_ingest(ctx->ring, B, n_in - q0 < ingest_batch ? n_in - q0 : ingest_batch, ctx->stream));
+        }
     } else {
         B.src = ct_in;
         B.dst = X0;

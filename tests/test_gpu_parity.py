@@ -578,6 +578,33 @@ def test_double_hoisting_with_a_special_prime_of_every_operand_class(bits, speci
              "special", tight=1e-2)
 
 
+@pytest.mark.parametrize("n_primes,n_in", [(3, 70), (15, 240)])
+def test_wide_inputs_take_no_more_scratch_than_the_batched_rotations(n_primes, n_in):
+    # 70 inputs: their digits in two batches, then rotated inside the multiply-accumulate.  240 inputs, 15 digits: the digits of
+    # all of them (15 x 16 polynomials each) and their intermediates would be 0.6 GB and more, far beyond the rotated inputs that
+    # this saves: in batches of 64 digits and rotated inputs are 0.25 GB, and the rest of a call's scratch is below 0.1 GB
+    import torch
+    par = ckks.Params(1 << 10, ckks.find_primes(1 << 40, 2 << 10, n_primes), ckks.find_primes(1 << 60, 2 << 10, 1)[0], 2.0 ** 30)
+    plan = ckks.Plan(4, 1, 2, 2, hoist="double", moddown="per_output")
+    d_in, d_out = n_in * 4, 4
+    s = ckks.keygen(par, 5)
+    keys = ckks.make_rotation_keys(par, s, plan, 5)
+    W, x = wl.gen_weights(5, "wide", d_out, d_in), wl.gen_activation(5, "wide", d_in)
+    cts = ckks.encrypt_vector(par, plan, s, x, 5)
+    expect = ckks.linear(par, plan, cts, W, keys)
+    g = GpuSide(par, plan)
+    try:
+        g.load_keys(keys)
+        w = g.bf.bf_encode_weights(g.ctx, g.to_dev(W), d_out, d_in)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        got = g.to_host_u64(g.linear(cts, W, d_out, d_in, weights=w))
+        assert free - torch.cuda.mem_get_info()[0] < 500 << 20
+        assert np.array_equal(got[0], expect[0])
+    finally:
+        g.close()
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
