@@ -1184,8 +1184,8 @@ __global__ void __launch_bounds__(64, EPI == 2 || EPI == 4 ? 10 : 16) ntt_contig
 // coalesced operands, and the automorphism is applied once, as a scatter, when the result is stored (pinv) or when the
 // rotated ciphertext is assembled.
 //
-// A block owns one run of rotations of the same digit set, one modulus m and CB chunks of 256 coefficients: warp w transforms
-// digit w % r of chunk w / r into its slice of shared memory, then every thread takes a coefficient, multiplies the r digits
+// A block owns one run of rotations of the same digit set, one modulus m and cb chunks of 256 coefficients: a warp transforms
+// digit w % r of chunk w / r (w = its number, then 8 more) into its slice of shared memory, then every thread takes a coefficient, multiplies the r digits
 // with the 2r key words of each rotation of the run (straight from global memory: read once, coalesced) and reduces once per
 // output word.  The transformed digits, r (r+1) polynomials per set, never reach memory.
 // What bounds it: the key stream where the run is long (baby steps), the fp64 pipe and the latency of the transform elsewhere.
@@ -1194,16 +1194,20 @@ __global__ void __launch_bounds__(64, EPI == 2 || EPI == 4 ? 10 : 16) ntt_contig
 // double hoisting: 291 us instead of 110 + 224 us.
 // grid: x = run, y = group of chunks, z = m: the runs that share a key's tile are adjacent.
 // (three blocks of 80 registers an SM instead of four of 64: 334 instead of 302 us)
+// An instance for every digit count: the key words of a component are all requested before the first is used, at immediate
+// offsets.  (A loop over the digits instead, four of them at a time, on a projection of 1024 -> 2048 with N = 2^15 without
+// double hoisting: 435 us for 6 digits, 800 for 10, 1394 for 15; with instances 356, 628, 1135.)  Eight warps for ten digits
+// and more: as many warps as digits leave fewer blocks to an SM (15 digits, loop: 1801 us).
 template <int RC>
 struct InnerGeo {
-    static constexpr int WARPS = RC > 8 ? RC : RC > 0 ? 8 : MAX_MODULI;    // (upper bound where r is not a constant)
-    static constexpr int BLOCKS = RC > 8 ? 3 : RC > 0 ? 4 : 1;
+    static constexpr int WARPS = RC == 9 ? 9 : 8, CHUNKS = RC > 8 ? 1 : WARPS / RC;    // (few digits leave room for several chunks)
+    static constexpr int BLOCKS = RC == 9 ? 3 : 4;
 };
 template <int CLS, int RC>
 __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch& rb, u32 first, u32 cnt, u32 m, u32 n, const u64* sd,
                                                const void* __restrict__ keys, u64* u, u64* xext,
                                                const u32* __restrict__ pinv, u64 pol) {
-    const u32 N = R.N, r = RC > 0 ? RC : R.r, nb = r + 1;
+    const u32 N = R.N, r = RC, nb = r + 1;
     const u32 at = (u32)swz((int)(n & 255u));
     const size_t out_words = (size_t)2 * nb * N;
     for (u32 rot = first; rot < first + cnt; ++rot) {
@@ -1213,30 +1217,18 @@ __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch&
         if (pinv) dest = __ldg(&pinv[(size_t)rb.key[rot] * N + n]);
         if (xext) pc0 = xext[(size_t)rb.c0[rot] * out_words + (size_t)m * N + n];
         // (one component at a time: with the key words of both in registers fewer blocks fit an SM)
-        u32 high[RC > 0 ? (2 * RC + 3) / 4 : 1];
-        if constexpr (RC > 0) {
+        u32 high[(2 * RC + 3) / 4];
 #pragma unroll
-            for (int h = 0; h < (2 * RC + 3) / 4; ++h) high[h] = kt.high(h, pol);
-        }
+        for (int h = 0; h < (2 * RC + 3) / 4; ++h) high[h] = kt.high(h, pol);
         auto component = [&](u32 comp) -> u64 {
             DigitDot<CLS> dot;
-            if constexpr (RC > 0) {
-                u32 k0[RC], k1[RC];
+            u32 k0[RC], k1[RC];
 #pragma unroll
-                for (int j = 0; j < RC; ++j) kt.word(2 * j + comp, pol, k0[j], k1[j]);
+            for (int j = 0; j < RC; ++j) kt.word(2 * j + comp, pol, k0[j], k1[j]);
 #pragma unroll
-                for (int j = 0; j < RC; ++j) {
-                    KeyTile<CLS>::cut(2 * j + comp, high[j / 2], k0[j], k1[j]);
-                    dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
-                }
-            } else {
-#pragma unroll 4
-                for (u32 j = 0; j < r; ++j) {
-                    u32 k0, k1;
-                    kt.word(2 * j + comp, pol, k0, k1);
-                    KeyTile<CLS>::cut(2 * j + comp, kt.high(j / 2, pol), k0, k1);
-                    dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0, k1);
-                }
+            for (int j = 0; j < RC; ++j) {
+                KeyTile<CLS>::cut(2 * j + comp, high[j / 2], k0[j], k1[j]);
+                dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
             }
             return dot.reduce(R, m);
         };
@@ -1255,7 +1247,7 @@ ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const vo
                  const u32* __restrict__ pinv, u32 cb) {
     extern __shared__ __align__(128) u64 sm_all[];          // [cb][r] slices
     grid_dependency_enter();
-    const u32 N = R.N, r = RC > 0 ? RC : R.r, nb = r + 1;
+    const u32 N = R.N, r = RC, nb = r + 1;
     const u32 m = slot_of_block(blockIdx.z, nb), chunk0 = blockIdx.y * cb;
     const u32 first = rb.grp_first[blockIdx.x], cnt = rb.grp_cnt[blockIdx.x], set = (u32)rb.dig[first];
     const u32 warps = blockDim.x >> 5;
@@ -1492,12 +1484,19 @@ cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_ou
 template <int RC>
 static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const void* keys, u64* u, u64* xext,
                                          const u32* pinv, cudaStream_t stream) {
-    const u32 r = ring.dev.r, chunks = ring.dev.N >> LOG_C;
-    const u32 warps = r > 8 ? r : 8u;
-    u32 cb = warps / r;                         // chunks per block: few digits leave room for several
-    if (cb > chunks) cb = chunks;
-    return launch_dependent(ring, ntt_contig_inner<RC>, dim3(rb.n_groups, (chunks + cb - 1) / cb, r + 1), dim3(32 * warps),
-                            (size_t)8 * (cb * r << LOG_C), stream, ring.dev, B, rb, keys, u, xext, pinv, cb);
+    typedef InnerGeo<RC> G;
+    const u32 chunks = ring.dev.N >> LOG_C, cb = (u32)G::CHUNKS < chunks ? (u32)G::CHUNKS : chunks;
+    return launch_dependent(ring, ntt_contig_inner<RC>, dim3(rb.n_groups, (chunks + cb - 1) / cb, RC + 1), dim3(32 * G::WARPS),
+                            (size_t)8 * (cb * RC << LOG_C), stream, ring.dev, B, rb, keys, u, xext, pinv, cb);
+}
+
+// (a context has 2 to MAX_MODULI - 1 digits: see bf_ctx_create)
+template <int RC>
+static cudaError_t launch_contig_inner(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const void* keys, u64* u, u64* xext,
+                                       const u32* pinv, cudaStream_t stream) {
+    if (ring.dev.r == RC) return launch_contig_inner_t<RC>(ring, B, rb, keys, u, xext, pinv, stream);
+    if constexpr (RC + 1 < MAX_MODULI) return launch_contig_inner<RC + 1>(ring, B, rb, keys, u, xext, pinv, stream);
+    else return cudaErrorInvalidValue;
 }
 
 cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n_sets, const RotBatch& rb_in, const void* keys, u64* u,
@@ -1511,11 +1510,11 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
     // runs of consecutive rotations with the same digit set, cut into parts until the blocks fill the machine (every part
     // transforms the digits again, which costs less than idle SMs)
     RotBatch rb = rb_in;
-    const u32 warps = r > 8 ? r : 8u, cb = warps / r;
+    const u32 cb = r > 8 ? 1u : 8u / r;
     u32 runs = 0;
     for (int t = 0; t < rb.n; ++t) runs += t == 0 || rb.dig[t] != rb.dig[t - 1];
     const u32 blocks = runs * (((ring.dev.N >> LOG_C) + cb - 1) / cb) * (r + 1);
-    const u32 parts = blocks < 1776u ? 1776u / blocks : 1u;      // 148 SMs x 3 blocks x 4
+    const u32 parts = blocks < 1776u ? 1776u / blocks : 1u;      // 148 SMs x 4 blocks x 3
     rb.n_groups = 0;
     for (int t = 0; t < rb.n;) {
         int end = t + 1;
@@ -1539,13 +1538,7 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
         ring.prof->key_bytes_per_rotation += (u64)rb.n * key_bytes;
     }
     ProfScope prof(ring.prof, CAT_KEY_INNER, stream);
-    switch (r) {                    // (digit counts of the shipped parameter sets)
-        case 3: return launch_contig_inner_t<3>(ring, B_in, rb, keys, u, xext, pinv, stream);
-        case 4: return launch_contig_inner_t<4>(ring, B_in, rb, keys, u, xext, pinv, stream);
-        case 7: return launch_contig_inner_t<7>(ring, B_in, rb, keys, u, xext, pinv, stream);
-        case 9: return launch_contig_inner_t<9>(ring, B_in, rb, keys, u, xext, pinv, stream);
-        default: return launch_contig_inner_t<0>(ring, B_in, rb, keys, u, xext, pinv, stream);
-    }
+    return launch_contig_inner<2>(ring, B_in, rb, keys, u, xext, pinv, stream);
 }
 
 cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,

@@ -140,6 +140,12 @@ def test_rotate_for_every_arrangement_of_digits_in_a_block(logN, n_primes):
         g.close()
 
 
+@pytest.mark.parametrize("n_primes", [3, 4, 6, 7, 9, 11, 12, 13, 14])
+def test_rotate_for_the_other_digit_counts(n_primes):
+    # (an instance of the fused transform and inner product each)
+    test_rotate_for_every_arrangement_of_digits_in_a_block(10, n_primes)
+
+
 @pytest.mark.parametrize("pkey", ["n12", "n15"])
 def test_rescale_matches_oracle(pkey):
     par = oracle_params(pkey)
