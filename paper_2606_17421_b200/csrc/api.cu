@@ -266,8 +266,24 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     R.r = n_ct_primes;
     ctx->ring.q.assign(primes, primes + nb);
     const u64 P = primes[n_ct_primes];
-    std::vector<ulonglong2> twf((size_t)nb * N), twi((size_t)nb * N);
-    std::vector<double> twf8((size_t)nb * N, 0.0), twi8((size_t)nb * N, 0.0);
+    // twiddles of one prime, in the form of its path: pairs, or plain doubles below 2^41 (see ntt.cu's twiddle_table; the part
+    // of the other form's array is never read)
+    std::vector<ulonglong2> twf(N), twi(N);
+    std::vector<double> twf8(N), twi8(N);
+    std::vector<u64> pw(N), pwi(N);
+#define CKC(call)                                                        \
+    do {                                                                 \
+        cudaError_t e__ = (call);                                        \
+        if (e__ != cudaSuccess) {                                        \
+            status = (e__ == cudaErrorMemoryAllocation) ? BF_ERR_OOM : BF_ERR_CUDA; \
+            cudaGetLastError();                                          \
+            return fail(status);                                         \
+        }                                                                \
+    } while (0)
+    CKC(cudaMalloc(&ctx->tw_fwd, (size_t)nb * N * sizeof(ulonglong2)));
+    CKC(cudaMalloc(&ctx->tw_inv, (size_t)nb * N * sizeof(ulonglong2)));
+    CKC(cudaMalloc(&ctx->tw8_fwd, (size_t)nb * N * sizeof(double)));
+    CKC(cudaMalloc(&ctx->tw8_inv, (size_t)nb * N * sizeof(double)));
     for (u32 m = 0; m < nb; ++m) {
         const u64 q = primes[m];
         R.q[m] = q;
@@ -292,7 +308,6 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
         const u64 psi = h_root_2n(q, N);
         if (!psi) return fail(BF_ERR_BAD_PRIME);
         const u64 psi_inv = h_invmod(psi, q);
-        std::vector<u64> pw(N), pwi(N);
         pw[0] = 1;
         pwi[0] = 1;
         for (u32 k = 1; k < N; ++k) {
@@ -341,13 +356,22 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
             if (!R.fp_ok[m]) return make_ulonglong2(w, h_shoup(w, q));
             return make_ulonglong2(dbits((double)w), dbits((double)w / (double)q));
         };
-        for (u32 k = 0; k < N; ++k) {
-            const u32 e = h_brev(k, (int)ctx->logN);
-            twf[(size_t)m * N + k] = entry(pw[e]);
-            twi[(size_t)m * N + k] = entry(pwi[e]);
-            if (q >> 41) continue;
-            twf8[(size_t)m * N + k] = (double)pw[e];
-            twi8[(size_t)m * N + k] = (double)pwi[e];
+        if (q >> 41) {
+            for (u32 k = 0; k < N; ++k) {
+                const u32 e = h_brev(k, (int)ctx->logN);
+                twf[k] = entry(pw[e]);
+                twi[k] = entry(pwi[e]);
+            }
+            CKC(cudaMemcpy(ctx->tw_fwd + (size_t)m * N, twf.data(), N * sizeof(ulonglong2), cudaMemcpyHostToDevice));
+            CKC(cudaMemcpy(ctx->tw_inv + (size_t)m * N, twi.data(), N * sizeof(ulonglong2), cudaMemcpyHostToDevice));
+        } else {
+            for (u32 k = 0; k < N; ++k) {
+                const u32 e = h_brev(k, (int)ctx->logN);
+                twf8[k] = (double)pw[e];
+                twi8[k] = (double)pwi[e];
+            }
+            CKC(cudaMemcpy(ctx->tw8_fwd + (size_t)m * N, twf8.data(), N * sizeof(double), cudaMemcpyHostToDevice));
+            CKC(cudaMemcpy(ctx->tw8_inv + (size_t)m * N, twi8.data(), N * sizeof(double), cudaMemcpyHostToDevice));
         }
     }
     // encoder tables: twiddles from the host's libm so that results do not depend on the device's
@@ -376,29 +400,12 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
             Z[k] = make_double2(cos(ang), -sin(ang));
         }
     }
-#define CKC(call)                                                        \
-    do {                                                                 \
-        cudaError_t e__ = (call);                                        \
-        if (e__ != cudaSuccess) {                                        \
-            status = (e__ == cudaErrorMemoryAllocation) ? BF_ERR_OOM : BF_ERR_CUDA; \
-            cudaGetLastError();                                          \
-            return fail(status);                                         \
-        }                                                                \
-    } while (0)
-    CKC(cudaMalloc(&ctx->tw_fwd, twf.size() * sizeof(ulonglong2)));
-    CKC(cudaMalloc(&ctx->tw_inv, twi.size() * sizeof(ulonglong2)));
-    CKC(cudaMalloc(&ctx->tw8_fwd, twf8.size() * sizeof(double)));
-    CKC(cudaMalloc(&ctx->tw8_inv, twi8.size() * sizeof(double)));
     CKC(cudaMalloc(&ctx->slot_of_pos, sop.size() * sizeof(u32)));
     CKC(cudaMalloc(&ctx->T, T.size() * sizeof(double2)));
     CKC(cudaMalloc(&ctx->Z, Z.size() * sizeof(double2)));
     CKC(cudaMalloc(&ctx->overflow_flag, 2 * sizeof(int)));
     CKC(cudaMalloc(&ctx->enc_consts, enc_consts.size() * sizeof(double)));
     ctx->device_error = ctx->overflow_flag + 1;
-    CKC(cudaMemcpy(ctx->tw_fwd, twf.data(), twf.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
-    CKC(cudaMemcpy(ctx->tw_inv, twi.data(), twi.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
-    CKC(cudaMemcpy(ctx->tw8_fwd, twf8.data(), twf8.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CKC(cudaMemcpy(ctx->tw8_inv, twi8.data(), twi8.size() * sizeof(double), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->slot_of_pos, sop.data(), sop.size() * sizeof(u32), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->T, T.data(), T.size() * sizeof(double2), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->Z, Z.data(), Z.size() * sizeof(double2), cudaMemcpyHostToDevice));
@@ -513,10 +520,8 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
             pinvs[(size_t)t * N + pi] = i;
         }
         key_of_steps[steps] = (int)t;
-        u64 gi = 1;
-        for (u32 s = steps; s < n; ++s) gi = (gi * 5) % (2ull * N);      // 5 has order n
         gal[t] = (u32)g;
-        gal_inv[t] = (u32)gi;
+        gal_inv[t] = (u32)h_powmod(5, n - steps, 2ull * N);              // 5 has order n
     }
     u32* perm_dev = nullptr;
     if (cudaMalloc(&perm_dev, perms.size() * sizeof(u32)) != cudaSuccess) return fail(BF_ERR_OOM);
