@@ -508,19 +508,19 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
     // as the scatter out[pinv[i]] = v'[i], pinv = perm^{-1}.  Only pinv stays on the device.
     std::vector<u32> perms((size_t)n_keys * N), pinvs((size_t)n_keys * N);
     std::vector<u32> gal(n_keys), gal_inv(n_keys);
+    std::vector<u32> brev(N);
+    for (u32 i = 0; i < N; ++i) brev[i] = h_brev(i, (int)ctx->logN);
     std::map<u32, int> key_of_steps;
     for (u32 t = 0; t < n_keys; ++t) {
         const u32 steps = rot_steps[t] % n;
-        u64 g = 1;
-        for (u32 s = 0; s < steps; ++s) g = (g * 5) % (2ull * N);
+        const u32 g = (u32)h_powmod(5, steps, 2ull * N);
         for (u32 i = 0; i < N; ++i) {
-            const u64 ex = ((2ull * h_brev(i, (int)ctx->logN) + 1) * g) % (2ull * N);
-            const u32 pi = h_brev((u32)((ex - 1) / 2), (int)ctx->logN);
+            const u32 pi = brev[(((2 * brev[i] + 1) * g) & (2 * N - 1)) >> 1];       // (exponents modulo 2N: a power of two)
             perms[(size_t)t * N + i] = pi;
             pinvs[(size_t)t * N + pi] = i;
         }
         key_of_steps[steps] = (int)t;
-        gal[t] = (u32)g;
+        gal[t] = g;
         gal_inv[t] = (u32)h_powmod(5, n - steps, 2ull * N);              // 5 has order n
     }
     u32* perm_dev = nullptr;
