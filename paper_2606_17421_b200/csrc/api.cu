@@ -170,6 +170,7 @@ struct bf_ctx {
 static int ensure(bf_ctx* ctx, DevBuf& b, size_t bytes) {
     if (b.cap >= bytes) return BF_OK;
     CK(cudaStreamSynchronize(ctx->stream));
+    ctx->epoch++;                  // captured launch sequences may point into the old buffer, whether a new one comes or not
     if (b.p) CK(cudaFree(b.p));
     b.p = nullptr;
     b.cap = 0;
@@ -180,7 +181,6 @@ static int ensure(bf_ctx* ctx, DevBuf& b, size_t bytes) {
         return BF_ERR_OOM;
     }
     b.cap = bytes;
-    ctx->epoch++;                  // captured launch sequences may point into the old buffer
     return BF_OK;
 }
 

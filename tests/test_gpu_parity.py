@@ -808,6 +808,56 @@ def test_repeated_calls_replay_a_graph_and_still_read_fresh_inputs():
         g.close()
 
 
+class _Device:
+    """A context on the N = 2^15 ring with uniform keys, and a device with little memory left."""
+
+    def __init__(self):
+        import torch
+        self.torch = torch
+        self.par, self.plan = oracle_params("n15"), ckks.Plan(1024, 16, 16, 4)
+        self.g = GpuSide(self.par, self.plan)
+        self.bf, self.ctx, self.hog = self.g.bf, self.g.ctx, None
+
+    def random_words(self, *shape):
+        return self.torch.randint(0, min(self.par.basis), shape, dtype=self.torch.int64, device="cuda")
+
+    def leave(self, nbytes):
+        self.torch.cuda.synchronize()
+        self.torch.cuda.empty_cache()
+        self.hog = self.torch.empty(self.torch.cuda.mem_get_info()[0] - nbytes, dtype=self.torch.uint8, device="cuda")
+
+    def close(self):
+        self.hog = None
+        self.torch.cuda.empty_cache()
+        self.g.close()
+
+
+def test_a_call_that_ran_out_of_memory_leaves_no_stale_launch_sequence():
+    # a larger call gives up the scratch of a captured one before its own allocation fails: the next small call has to
+    # allocate again, not replay a sequence that points into what was freed
+    d = _Device()
+    try:
+        par, steps = d.par, list(ckks.required_rotations(d.plan))
+        d.bf.bf_load_eval_keys(d.ctx, steps, len(steps), d.random_words(len(steps), par.r, 2, par.r + 1, par.N))
+        small, large = (d.torch.randn(rows, 1024, device="cuda") * 0.02 for rows in (1024, 8192))
+        ct, out, big = d.random_words(1, 2, par.r, par.N), d.g.empty_u64(1, 2, par.r, par.N), d.g.empty_u64(8, 2, par.r, par.N)
+        w = d.bf.bf_encode_weights(d.ctx, small, 1024, 1024)
+        call = lambda: d.bf.bf_linear(d.ctx, ct, 1, w, None, 1024, 1024, out, 1)
+        for _ in range(3):
+            call()
+        expect = d.g.to_host_u64(out)
+        d.leave(64 << 20)
+        with pytest.raises(d.bf.BifrostError) as ei:
+            d.bf.bf_linear(d.ctx, ct, 1, None, large, 8192, 1024, big, 8)
+        assert ei.value.code == d.bf.BF_ERR_OOM
+        for _ in range(3):
+            out.zero_()
+            call()
+        assert np.array_equal(d.g.to_host_u64(out), expect)
+    finally:
+        d.close()
+
+
 def test_unloading_keys_invalidates_replayed_launch_sequences():
     # after the keys are dropped, a call that was being replayed from its captured graph must be refused
     # (the graph holds the addresses of the freed key arrays), and reloading the keys must make it work again
