@@ -88,6 +88,8 @@ struct bf_weights {
     u32 coef_bits = 0;
 };
 
+constexpr size_t ENCODE_PASS_BYTES = (size_t)1536 << 20, ENCODE_PASS_BYTES_MIN = (size_t)512 << 20;
+
 struct bf_ctx {
     RingHost ring;
     Profiler prof;
@@ -105,6 +107,7 @@ struct bf_ctx {
     // multiply-accumulate (at least one group is always held).  Measured on a LLaMA-3-8B layer: 1 GiB 78 ms,
     // 2 GiB 73 ms, 4 GiB 70 ms, 8 GiB 69 ms: the rotated inputs are re-read once per round
     size_t encode_scratch_bytes = (size_t)4 << 30;
+    size_t encode_pass_bytes = ENCODE_PASS_BYTES;       // scratch of one pass of the encoder (see encode_range)
     u32 coef_cache_bits = 0;        // 64 / 32: weights encoded from now on are kept as rounded coefficients
     int* overflow_flag = nullptr;   // [0]: encoder range overflow; [1]: a bounded device-side wait gave up
     int* device_error = nullptr;
@@ -167,13 +170,25 @@ struct bf_ctx {
         }                                                                     \
     } while (0)
 
-static int ensure(bf_ctx* ctx, DevBuf& b, size_t bytes) {
-    if (b.cap >= bytes) return BF_OK;
-    CK(cudaStreamSynchronize(ctx->stream));
-    ctx->epoch++;                  // captured launch sequences may point into the old buffer, whether a new one comes or not
+#define TRY(call)                     \
+    do {                              \
+        int s__ = (call);             \
+        if (s__ != BF_OK) return s__; \
+    } while (0)
+
+// (the caller has waited for the stream)
+static int release(bf_ctx* ctx, DevBuf& b) {
+    ctx->epoch++;                  // captured launch sequences may point into it, whether a new buffer comes or not
     if (b.p) CK(cudaFree(b.p));
     b.p = nullptr;
     b.cap = 0;
+    return BF_OK;
+}
+
+static int ensure(bf_ctx* ctx, DevBuf& b, size_t bytes) {
+    if (b.cap >= bytes) return BF_OK;
+    CK(cudaStreamSynchronize(ctx->stream));
+    TRY(release(ctx, b));
     cudaError_t e = cudaMalloc(&b.p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -183,12 +198,6 @@ static int ensure(bf_ctx* ctx, DevBuf& b, size_t bytes) {
     b.cap = bytes;
     return BF_OK;
 }
-
-#define TRY(call)                     \
-    do {                              \
-        int s__ = (call);             \
-        if (s__ != BF_OK) return s__; \
-    } while (0)
 
 static bool is_pow2(u32 x) { return x && !(x & (x - 1)); }
 
@@ -612,14 +621,27 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
     const u32 N = ctx->N, r = lay.n_primes, n = N / 2;       // (r: primes each diagonal is reduced into)
     // diagonals per pass: the encoder and the transforms gain from large batches (256 of them at N = 2^15: a coefficient layer
     // in 2738 us, in passes of 64 2792, of 32 2874; 256 instead of 102 at N = 2^16: 2690 instead of 2792 us for a product
-    // encoded on the way); the scratch of a pass is held to about 1.5 GB
-    u32 chunk = (u32)(((size_t)1536 << 20) / ((size_t)r * N * sizeof(u64))) & ~7u;
-    if (chunk > 512) chunk = 512;
-    if (chunk < 32) chunk = 32;
-    if (chunk > count) chunk = count > 0 ? count : 1;
-    if (!stored) TRY(ensure(ctx, ctx->fft, (size_t)chunk * n * sizeof(double2)));
-    if (!coef_out && !stored) TRY(ensure(ctx, ctx->coef, (size_t)chunk * N * sizeof(i64)));
-    if (!coef_out) TRY(ensure(ctx, ctx->ptnat, (size_t)chunk * r * N * sizeof(u64)));
+    // encoded on the way); the scratch of a pass is held to about 1.5 GB, and to 0.5 GB once the device has not had the room
+    u32 chunk;
+    for (;;) {
+        const bool roomy = ctx->encode_pass_bytes > ENCODE_PASS_BYTES_MIN;
+        chunk = (u32)(ctx->encode_pass_bytes / ((size_t)r * N * sizeof(u64))) & ~7u;
+        if (chunk > (roomy ? 512u : 256u)) chunk = roomy ? 512u : 256u;
+        if (chunk < 32) chunk = 32;
+        if (chunk > count) chunk = count > 0 ? count : 1;
+        int s = BF_OK;
+        if (!stored) s = ensure(ctx, ctx->fft, (size_t)chunk * n * sizeof(double2));
+        if (s == BF_OK && !coef_out && !stored) s = ensure(ctx, ctx->coef, (size_t)chunk * N * sizeof(i64));
+        if (s == BF_OK && !coef_out) s = ensure(ctx, ctx->ptnat, (size_t)chunk * r * N * sizeof(u64));
+        if (s == BF_ERR_OOM && roomy) {
+            ctx->encode_pass_bytes = ENCODE_PASS_BYTES_MIN;
+            for (DevBuf* b : {&ctx->fft, &ctx->coef, &ctx->ptnat})
+                if (!(coef_out && b == &ctx->coef)) release(ctx, *b);       // (coef_out may lie there)
+            continue;
+        }
+        TRY(s);
+        break;
+    }
     EncodeTables tab;
     tab.slot_of_pos = ctx->slot_of_pos;
     tab.T = ctx->T;

@@ -858,6 +858,32 @@ def test_a_call_that_ran_out_of_memory_leaves_no_stale_launch_sequence():
         d.close()
 
 
+def test_encoding_needs_no_more_memory_than_small_passes_take():
+    # 512 diagonals in one pass of the encoder would take 1.3 GB beside 0.64 GB of weights; in passes of 256 it is 0.67 GB
+    d = _Device()
+    try:
+        W = d.torch.randn(8192, 1024, device="cuda") * 0.02
+        expect, got = d.g.empty_u64(d.par.r, d.par.N), d.g.empty_u64(d.par.r, d.par.N)
+        free = GpuSide(d.par, d.plan)               # (the same weights where memory is not short)
+        try:
+            w0 = free.bf.bf_encode_weights(free.ctx, W, 8192, 1024)
+            picks = [(0, 0, 0, 0), (3, 0, 3, 15), (7, 0, 1, 2), (7, 0, 3, 15)]
+            words = []
+            for at in picks:
+                free.bf.bf_weights_export(free.ctx, w0, *at, expect)
+                words.append(free.to_host_u64(expect).copy())
+        finally:
+            free.close()
+        d.torch.cuda.set_stream(d.g.stream)
+        d.leave(1640 << 20)
+        w = d.bf.bf_encode_weights(d.ctx, W, 8192, 1024)
+        for at, want in zip(picks, words):
+            d.bf.bf_weights_export(d.ctx, w, *at, got)
+            assert np.array_equal(d.g.to_host_u64(got), want), at
+    finally:
+        d.close()
+
+
 def test_unloading_keys_invalidates_replayed_launch_sequences():
     # after the keys are dropped, a call that was being replayed from its captured graph must be refused
     # (the graph holds the addresses of the freed key arrays), and reloading the keys must make it work again
