@@ -101,7 +101,8 @@ int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_t n_keys, c
 int bf_set_cache_budget(bf_ctx* ctx, uint64_t bytes);
 uint64_t bf_cache_bytes_used(const bf_ctx* ctx);
 
-/* Bytes bf_encode_weights would keep resident for a d_out x d_in projection under the plan. */
+/* Bytes bf_encode_weights would count against the budget for a d_out x d_in projection under the plan: its encoded words,
+ * with the terms rounded up to whole stages of 8 (see bf_set_compact_cache for the bytes of a word). */
 uint64_t bf_weights_bytes(const bf_ctx* ctx, uint32_t d_out, uint32_t d_in);
 
 /* EncodeWeights (Alg. 3, offline phase; Sec. 4.2): encode every generalised diagonal of

@@ -256,44 +256,45 @@ struct RescaleConsts {
 // each stream one contiguous region:  word (group pj, term t, prime i, coefficient n) has index
 //   ((pj%PL)*TS + t%TS)*TN + n%TN   inside stage   ((i, n/TN), pj/PL, t/TS)
 // with TN = 2^log_tn coefficients per tile, PL = 256/TN group lanes, TS = 8 terms per stage,
-// G = ceil(n_pj/PL), C = ceil(n_terms/TS); a stage holds 2048 words.  The stages of one prime are
+// G = ceil(n_pj/PL), C = ceil(n_terms/TS); a stage holds the words of min(PL, n_pj) lanes, 2048 of them where the groups fill
+// the lanes.  The stages of one prime are
 // contiguous, ordered (tile, pj/PL, t/TS), and every prime stores its words in the narrowest of three
 // formats its size allows, because the kernel that reads them is bound by HBM bytes:
-//   TILE_W64  8 bytes per word, two limbs (16 KB per stage)
-//   TILE_W40  primes below 2^40: the low 32 bits of all 2048 words, then their high bytes, those of four terms in one 32-bit
-//             word: byte t%4 of word (pj%PL * 2 + t%8 / 4) * TN + n%TN (10 KB per stage)
-//   TILE_W32  primes below 2^32: 32-bit words (8 KB per stage)
+//   TILE_W64  8 bytes per word, two limbs (16 KB per full stage)
+//   TILE_W40  primes below 2^40: a lane's TS rows of low 32 bits, then two rows of high bytes, those of four terms in one
+//             32-bit word: byte t%4 of word n%TN of row t%8 / 4 (10 KB per full stage)
+//   TILE_W32  primes below 2^32: 32-bit words (8 KB per full stage)
 // (Words of 8 bytes throughout: the four calls of a 0.6B layer stream 2.78 instead of 2.40 GB.)
 enum TileFormat : u32 { TILE_W64 = 0, TILE_W40 = 1, TILE_W32 = 2 };
 struct TileLayout {
     u32 log_tn, n_terms, n_pj, G, C, ntiles;
+    u32 stage_words;
     u32 fmt_bits;                           // TileFormat of prime i in bits 2i, 2i+1
     u32 n_primes;                           // primes the plaintexts are held in: r, or r + 1 with double hoisting
                                             //   (the special prime last, in the format its own size asks for)
     size_t base[MAX_MODULI + 1];            // see tile_prime_base
 };
 constexpr u32 TILE_TS = 8;
-constexpr u32 TILE_STAGE_WORDS = 2048;
 
 __host__ __device__ __forceinline__ u32 tile_format(const TileLayout& t, u32 i) { return (t.fmt_bits >> (2 * i)) & 3u; }
-__host__ __device__ __forceinline__ u32 tile_stage_bytes(u32 fmt) {
-    return TILE_STAGE_WORDS * (fmt == TILE_W64 ? 8u : fmt == TILE_W40 ? 5u : 4u);
+__host__ __device__ __forceinline__ u32 tile_stage_bytes(const TileLayout& t, u32 fmt) {
+    return t.stage_words * (fmt == TILE_W64 ? 8u : fmt == TILE_W40 ? 5u : 4u);
 }
 // byte offset of prime i's first stage (i = n_primes: total size): the primes' regions follow one another
 __host__ __device__ __forceinline__ size_t tile_prime_base(const TileLayout& t, u32 i) { return t.base[i]; }
 // byte offset of a stage
 __host__ __device__ __forceinline__ size_t tile_stage_offset(const TileLayout& t, u32 i, u32 tile, u32 g, u32 ch) {
-    return tile_prime_base(t, i) + (((size_t)tile * t.G + g) * t.C + ch) * tile_stage_bytes(tile_format(t, i));
+    return tile_prime_base(t, i) + (((size_t)tile * t.G + g) * t.C + ch) * tile_stage_bytes(t, tile_format(t, i));
 }
-// index of a word inside its stage
-__host__ __device__ __forceinline__ u32 tile_word_index(const TileLayout& t, u32 pj, u32 term, u32 n) {
+// byte offset of a word (TILE_W40: of its low half) inside its stage
+__host__ __device__ __forceinline__ u32 tile_word_offset(const TileLayout& t, u32 fmt, u32 pj, u32 term, u32 n) {
     const u32 TN = 1u << t.log_tn, PL = 256u >> t.log_tn;
-    return ((pj % PL) * TILE_TS + term % TILE_TS) * TN + (n & (TN - 1));
+    return ((pj % PL * (fmt == TILE_W40 ? TILE_TS + 2 : TILE_TS) + term % TILE_TS) * TN + (n & (TN - 1))) * (fmt == TILE_W64 ? 8 : 4);
 }
 // byte offset, inside its stage, of a word's high byte (TILE_W40)
 __host__ __device__ __forceinline__ u32 tile_high_offset(const TileLayout& t, u32 pj, u32 term, u32 n) {
     const u32 TN = 1u << t.log_tn, PL = 256u >> t.log_tn;
-    return TILE_STAGE_WORDS * 4u + (((pj % PL) * 2 + term % TILE_TS / 4) * TN + (n & (TN - 1))) * 4 + term % 4;
+    return ((pj % PL * (TILE_TS + 2) + TILE_TS + term % TILE_TS / 4) * TN + (n & (TN - 1))) * 4 + term % 4;
 }
 __host__ __device__ __forceinline__ size_t tile_stage_of_word(const TileLayout& t, u32 pj, u32 term, u32 i, u32 n) {
     const u32 PL = 256u >> t.log_tn;

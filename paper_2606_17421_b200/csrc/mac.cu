@@ -31,18 +31,25 @@ TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_pr
     t.G = (n_pj + PL - 1) / PL;
     t.C = (n_terms + TILE_TS - 1) / TILE_TS;
     t.ntiles = ring.dev.N >> t.log_tn;
+    t.stage_words = (n_pj < PL ? n_pj : PL) * TILE_TS << t.log_tn;
     for (u32 i = 0; i < t.n_primes; ++i) {
         const u32 f = ring.q[i] < (1ull << 32) ? TILE_W32 : ring.q[i] < (1ull << 40) ? TILE_W40 : TILE_W64;
         t.fmt_bits |= f << (2 * i);
-        t.base[i + 1] = t.base[i] + (size_t)tile_stage_bytes(f) * t.ntiles * t.G * t.C;
+        t.base[i + 1] = t.base[i] + (size_t)tile_stage_bytes(t, f) * t.ntiles * t.G * t.C;
     }
     return t;
 }
 
 size_t mac_tile_bytes(const TileLayout& t) { return tile_prime_base(t, t.n_primes); }
 
+// (of the groups there are: the last stages' idle lanes, at most PL - 1 groups, are left out)
 size_t mac_accounted_bytes(const RingHost& ring, const TileLayout& t) {
-    return ring.compact_cache ? mac_tile_bytes(t) : (size_t)t.n_primes * t.ntiles * t.G * t.C * TILE_STAGE_WORDS * 8;
+    size_t width = 0;
+    for (u32 i = 0; i < t.n_primes; ++i) {
+        const u32 f = tile_format(t, i);
+        width += !ring.compact_cache || f == TILE_W64 ? 8 : f == TILE_W40 ? 5 : 4;
+    }
+    return width * ring.dev.N * t.n_pj * t.C * TILE_TS;
 }
 
 u32 mac_split_bits(const RingHost& ring) {

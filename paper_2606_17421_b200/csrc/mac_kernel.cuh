@@ -170,22 +170,21 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
     const u32 fmt = tile_format(lay, i);
     const u32 n_chunks = lay.C;
     u32 left = ((pj_end - pj_begin - l + PL - 1) / PL) * n_chunks;      // stages to go
-    const u32 stage_bytes = tile_stage_bytes(fmt);
+    const u32 stage_bytes = tile_stage_bytes(lay, fmt);
     const unsigned char* stage = (const unsigned char*)pt + tile_prime_base(lay, i) +
                                  ((size_t)tile * lay.G + pj_begin / PL) * n_chunks * stage_bytes;
-    const u32 at = l * TILE_TS * TN + c;
+    stage += tile_word_offset(lay, fmt, l, 0, c);       // (the lane's words of a stage lie together)
     constexpr int TS = (int)TILE_TS, TH = PACKED ? TS / 4 : TS;
     // one stage's words of this thread, as they are stored
     auto fetch = [&](u32 (&wa)[TS], u32 (&wb)[TH]) {
         if constexpr (PACKED) {
-            const u32* p = (const u32*)stage + at;
-            const u32* ph = (const u32*)(stage + TILE_STAGE_WORDS * 4u) + l * 2 * TN + c;
+            const u32* p = (const u32*)stage;
 #pragma unroll
             for (int ts = 0; ts < TS; ++ts) wa[ts] = ld_stream32(p + ts * TN, pol);
 #pragma unroll
-            for (int h = 0; h < TH; ++h) wb[h] = fmt == TILE_W40 ? ld_stream32(ph + h * TN, pol) : 0u;
+            for (int h = 0; h < TH; ++h) wb[h] = fmt == TILE_W40 ? ld_stream32(p + (TS + h) * TN, pol) : 0u;
         } else {
-            const u64* p = (const u64*)stage + at;
+            const u64* p = (const u64*)stage;
 #pragma unroll
             for (int ts = 0; ts < TS; ++ts) ld_stream(p + ts * TN, pol, wa[ts], wb[ts]);
         }

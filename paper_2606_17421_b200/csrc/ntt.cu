@@ -816,10 +816,10 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
         const u32 d = B.o_base + o, pj_all = d / B.tile.n_terms, term = d - pj_all * B.tile.n_terms, pj = pj_all - B.tile_pj0;
         const u32 n = chunk * LEN + 4 * lane;
         tile_stage = (unsigned char*)B.tile_ptr + tile_stage_of_word(B.tile, pj, term, mod, n);
-        tile_at = tile_word_index(B.tile, pj, term, n);
         tile_fmt = tile_format(B.tile, mod);
+        tile_at = tile_word_offset(B.tile, tile_fmt, pj, term, n);
         tile_high = tile_high_offset(B.tile, pj, term, n);
-        tile_step = (size_t)((128u >> B.tile.log_tn) * B.tile.G * B.tile.C) * tile_stage_bytes(tile_fmt);
+        tile_step = (size_t)((128u >> B.tile.log_tn) * B.tile.G * B.tile.C) * tile_stage_bytes(B.tile, tile_fmt);
     }
     // byte addresses (shared window) of the thread's base points
     const u32 slice = (u32)__cvta_generic_to_shared(sm);
@@ -940,9 +940,9 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const u32 at = tile_at, fmt = tile_fmt;
                 if (fmt == TILE_W64) {
                     const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
-                    stg4((u64*)stage + at, limb_split(v4[0], L), limb_split(v4[1], L), limb_split(v4[2], L), limb_split(v4[3], L));
+                    stg4((u64*)(stage + at), limb_split(v4[0], L), limb_split(v4[1], L), limb_split(v4[2], L), limb_split(v4[3], L));
                 } else {
-                    *(uint4*)(stage + (size_t)at * 4) = make_uint4((u32)v4[0], (u32)v4[1], (u32)v4[2], (u32)v4[3]);
+                    *(uint4*)(stage + at) = make_uint4((u32)v4[0], (u32)v4[1], (u32)v4[2], (u32)v4[3]);
                     if (fmt == TILE_W40) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) stage[tile_high + 4 * i] = (unsigned char)(v4[i] >> 32);
@@ -1064,14 +1064,14 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const unsigned char* stage = tile_stage + (size_t)it * tile_step;
                 const u32 at = tile_at, fmt = tile_fmt;
                 if (fmt == TILE_W64) {
-                    const ulonglong2* gp = (const ulonglong2*)(stage + (size_t)at * 8);
+                    const ulonglong2* gp = (const ulonglong2*)(stage + at);
                     const ulonglong2 a = gp[0], b = gp[1];
                     v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
                     const u32 L = q >> 50 ? LIMB_WIDE : B.split_bits;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) v4[i] = limb_join(v4[i], L);
                 } else {
-                    const uint4 lo = *(const uint4*)(stage + (size_t)at * 4);
+                    const uint4 lo = *(const uint4*)(stage + at);
                     v4[0] = lo.x; v4[1] = lo.y; v4[2] = lo.z; v4[3] = lo.w;
                     if (fmt == TILE_W40) {
 #pragma unroll

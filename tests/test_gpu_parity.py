@@ -91,6 +91,31 @@ def test_encode_weights_matches_oracle(pkey, plan_t, shape, compact, pack):
         g.close()
 
 
+@pytest.mark.parametrize("d_out,plan_t", [(16, (16, 1, 16, 1)), (16, (16, 1, 8, 2)), (40, (16, 1, 16, 1)), (100, (16, 1, 4, 4))])
+def test_weights_of_few_output_groups_count_for_their_words_only(d_out, plan_t):
+    # 1, 2, 3 and 28 groups, where a small ring's tiles have 8 lanes: idle lanes are neither counted nor, where one stage has
+    # them all, stored
+    import torch
+    par, plan = oracle_params("n12"), ckks.Plan(*plan_t)
+    g = GpuSide(par, plan)
+    try:
+        W = torch.randn(d_out, 16 * 40, device="cuda") * 0.02
+        groups, terms = plan.n_out(d_out) * plan.g, 40 * plan.b
+        widths = {False: 8 * par.r, True: sum(5 if q < 2 ** 40 else 8 for q in par.primes)}
+        for compact in (False, True):
+            g.bf.bf_set_compact_cache(g.ctx, compact)
+            assert g.bf.bf_weights_bytes(g.ctx, d_out, 16 * 40) == widths[compact] * par.N * groups * terms
+        g.bf.bf_weights_free(g.ctx, g.bf.bf_encode_weights(g.ctx, W, d_out, 16 * 40))       # (scratch, code)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        handles = [g.bf.bf_encode_weights(g.ctx, W, d_out, 16 * 40) for _ in range(4)]
+        stored = (free - torch.cuda.mem_get_info()[0]) / 4
+        assert stored <= widths[True] * par.N * (groups if groups <= 8 else groups + 4) * terms + (3 << 20)
+        assert len(handles) == 4
+    finally:
+        g.close()
+
+
 # ------------------------------------------------------------------ key switch, rescale
 
 @pytest.mark.parametrize("pkey", ["n12", "n15"])
