@@ -39,7 +39,7 @@ enum {
     BF_ERR_CUDA = -7,          /* a CUDA call failed; see bf_last_cuda_error() */
     BF_ERR_RANGE = -8,         /* an encoded coefficient does not fit 2^62 (scale too large for the data) */
     BF_ERR_TOO_LARGE = -9,     /* more work than the fixed scratch of an allocation-free entry point holds */
-    BF_ERR_TIMEOUT = -10       /* a device-side wait on an asynchronous copy hit its poll limit */
+    BF_ERR_TIMEOUT = -10       /* reserved, not returned: no kernel waits on anything but the end of the one before it */
 };
 
 typedef struct bf_ctx bf_ctx;          /* ring tables, rotation keys, scratch memory */
@@ -263,17 +263,15 @@ int bf_weights_export(bf_ctx* ctx, const bf_weights* w, uint32_t p, uint32_t q, 
 
 /* Per-stage device time of the last bf_linear on this context, in milliseconds, when stage timing
  * was switched on with bf_set_stage_timing(ctx, 1) (adds event records; off by default).
- * stages: 0 input transforms + hoisted ModUp + baby steps, 1 multiply-accumulate (on the fallback
- * path: with the on-the-fly encoding), 2 giant steps, 3 output transform.
+ * stages: 0 input transforms + hoisted ModUp + baby steps, 1 multiply-accumulate (with the baby
+ * steps where it makes them, and on the fallback path with the on-the-fly encoding), 2 giant steps, 3 output transform.
  * bf_get_stage_ms synchronises the stream. */
 int bf_set_stage_timing(bf_ctx* ctx, int on);
 int bf_get_stage_ms(bf_ctx* ctx, float* ms_out /* host, 4 values */);
 
-/* Kernels that wait on asynchronous copies poll with a limit; when a wait gives up the kernel
- * records it and still terminates.  bf_device_status synchronises the stream and returns
- * BF_ERR_TIMEOUT if that happened since the last check (the affected call's results are invalid),
- * BF_ERR_RANGE for an encoder overflow on the fallback path, else BF_OK.  bf_linear_host performs
- * this check itself. */
+/* Synchronises the stream and returns BF_ERR_RANGE if the encoder met a coefficient out of range since the last check (the
+ * affected call's results are invalid), else BF_OK.  bf_linear with raw weights and bf_linear_host perform this check
+ * themselves. */
 int bf_device_status(bf_ctx* ctx);
 
 /* Launch accounting.  The library counts its kernel launches per category; with

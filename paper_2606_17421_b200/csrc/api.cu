@@ -109,8 +109,7 @@ struct bf_ctx {
     size_t encode_scratch_bytes = (size_t)4 << 30;
     size_t encode_pass_bytes = ENCODE_PASS_BYTES;       // scratch of one pass of the encoder (see encode_range)
     u32 coef_cache_bits = 0;        // 64 / 32: weights encoded from now on are kept as rounded coefficients
-    int* overflow_flag = nullptr;   // [0]: encoder range overflow; [1]: a bounded device-side wait gave up
-    int* device_error = nullptr;
+    int* overflow_flag = nullptr;   // encoder range overflow
     // rotation keys
     std::map<u32, int> key_of_steps;
     u64* keys = nullptr;
@@ -212,7 +211,7 @@ extern "C" const char* bf_strerror(int code) {
         case BF_ERR_OOM: return "out of memory or over the cache budget";
         case BF_ERR_CUDA: return "CUDA error";
         case BF_ERR_RANGE: return "encoded coefficient out of range";
-        case BF_ERR_TIMEOUT: return "a bounded device-side wait gave up (results of that call are invalid)";
+        case BF_ERR_TIMEOUT: return "a device-side wait gave up (reserved: no kernel waits)";
         case BF_ERR_TOO_LARGE: return "request exceeds the fixed capacity of the allocation-free entry point";
         default: return "unknown error";
     }
@@ -412,14 +411,13 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
     CKC(cudaMalloc(&ctx->slot_of_pos, sop.size() * sizeof(u32)));
     CKC(cudaMalloc(&ctx->T, T.size() * sizeof(double2)));
     CKC(cudaMalloc(&ctx->Z, Z.size() * sizeof(double2)));
-    CKC(cudaMalloc(&ctx->overflow_flag, 2 * sizeof(int)));
+    CKC(cudaMalloc(&ctx->overflow_flag, sizeof(int)));
     CKC(cudaMalloc(&ctx->enc_consts, enc_consts.size() * sizeof(double)));
-    ctx->device_error = ctx->overflow_flag + 1;
     CKC(cudaMemcpy(ctx->slot_of_pos, sop.data(), sop.size() * sizeof(u32), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->T, T.data(), T.size() * sizeof(double2), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->Z, Z.data(), Z.size() * sizeof(double2), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(ctx->enc_consts, enc_consts.data(), enc_consts.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CKC(cudaMemset(ctx->overflow_flag, 0, 2 * sizeof(int)));
+    CKC(cudaMemset(ctx->overflow_flag, 0, sizeof(int)));
     CKC(cudaDeviceSynchronize());
 #undef CKC
     R.tw_fwd = ctx->tw_fwd;
@@ -692,14 +690,14 @@ static int encode_range(bf_ctx* ctx, const float* W, u32 d_out, u32 d_in, u32 d0
     return BF_OK;
 }
 
-// Reads the two device-side flags (encoder range overflow; a bounded wait that gave up).  Synchronises.
+// Reads the device-side flag of the encoder (a coefficient out of range).  Synchronises.
 static int check_overflow(bf_ctx* ctx) {
-    int flags[2] = {0, 0};
-    CK(cudaMemcpyAsync(flags, ctx->overflow_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    int flag = 0;
+    CK(cudaMemcpyAsync(&flag, ctx->overflow_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    if (flags[0] || flags[1]) {
-        CK(cudaMemsetAsync(ctx->overflow_flag, 0, 2 * sizeof(int), ctx->stream));
-        return flags[1] ? BF_ERR_TIMEOUT : BF_ERR_RANGE;
+    if (flag) {
+        CK(cudaMemsetAsync(ctx->overflow_flag, 0, sizeof(int), ctx->stream));
+        return BF_ERR_RANGE;
     }
     return BF_OK;
 }
@@ -1579,7 +1577,7 @@ extern "C" int bf_linear_host(bf_ctx* ctx, const uint64_t* host_ct_in, uint32_t 
                            n_out, nullptr));
     const size_t out_bytes = (size_t)n_out * 2 * (ctx->r - 1) * ctx->N * 8;
     CK(cudaMemcpyAsync(host_ct_out, ctx->stage_out.p, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
-    return check_overflow(ctx);          // synchronises; reports a device-side wait that gave up
+    return check_overflow(ctx);          // synchronises
 }
 
 extern "C" int bf_rotate(bf_ctx* ctx, const uint64_t* ct_in, uint32_t steps, uint64_t* ct_out) {

@@ -241,7 +241,7 @@ struct BabySteps {
     u32 n_in, b;
     u32 parts, per_part;                // how the inputs are dealt out to a block's lanes (set by the launcher)
     const void* keys;                   // resident keys
-    const u64* dig;                     // digit set q of input q (tile-major, see ks_tile_index)
+    const u64* dig;                     // digit set q of input q (tile-major, see KS_TILE)
     u32 key[MAX_ROT_BATCH + 1];
     u32 gal[MAX_ROT_BATCH + 1], gal_inv[MAX_ROT_BATCH + 1];
 };
@@ -347,8 +347,8 @@ struct PolyBatch {
     // passes through tail_dst + (input * r + j) * N between the passes.  The second pass takes outer index (input, j) and
     // slots m <= r of component 1, m = r + 1 component 0; see EPI 5 of the contiguous pass
     u32 ingest;
-    u64* dtile_ptr;               // ingest: the digits' transforms go there, tile-major in tiles of KS_TILE coefficients (see
-    u32 dtile_div;                //   ks_tile_index, div = r); with `scatter` the resident keys
+    u64* dtile_ptr;               // ingest: the digits' transforms go there, tile-major (see
+    u32 dtile_div;                //   KS_TILE, div = r); with `scatter` the resident keys
     u32 o_div_magic, dtile_magic; // ceil(2^32 / o_div), ceil(2^32 / dtile_div): o / d = umulhi(o, magic) for o < 2^16
                                   //   (set by the launchers; 0 = divide)
     const u64* div_t;             // forward from a shared source, non-null (double hoisting): the source of digit
@@ -357,22 +357,18 @@ struct PolyBatch {
                                   //   modulo P as a centred lift plus 2^59: the digit is (source - t) * P^{-1} mod q_i
 };
 
-// Operands of the key-switch inner product (digit sets and rotation keys) are kept tile-major, so that what a block
-// needs of one (outer index / div, modulus, tile) is contiguous:
-//   polynomial (o, m), coefficient n  ->  ((((o / div) * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + o % div) * KS_TILE + n % KS_TILE
-// digits: o = set * r + digit, div = r (a block reads the r digit segments of a set, modulus and tile);
+// The digit sets that the multiply-accumulate reads are kept tile-major, so that what a block needs of one (set, modulus,
+// tile) is contiguous.  Polynomial (o, m), o = set * div + digit, div = r; coefficient n:
+//   (((set * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + digit) * KS_TILE + n % KS_TILE
 // (keys: see KeyTile)
 constexpr u32 KS_TILE = 128;
-__host__ __device__ __forceinline__ size_t ks_tile_index(u32 N, u32 n_m, u32 div, u32 o, u32 m, u32 n) {
-    return ((((size_t)(o / div) * n_m + m) * (N / KS_TILE) + n / KS_TILE) * div + o % div) * KS_TILE + n % KS_TILE;
-}
 
 // o / d and o % d with a host-made reciprocal (see PolyBatch::o_div_magic); magic = 0 divides
 __device__ __forceinline__ void split_index(u32 o, u32 d, u32 magic, u32& hi, u32& lo) {
     hi = magic ? __umulhi(o, magic) : o / d;
     lo = o - hi * d;
 }
-// ks_tile_index of coefficient 0 of polynomial (o = o_hi * div + o_lo, m); coefficient n then sits at
+// that index for coefficient 0 of polynomial (o = o_hi * div + o_lo, m); coefficient n then sits at
 // base + (n / KS_TILE) * div * KS_TILE + n % KS_TILE
 __device__ __forceinline__ size_t ks_tile_base(u32 N, u32 n_m, u32 div, u32 o_hi, u32 o_lo, u32 m) {
     return (((size_t)o_hi * n_m + m) * (N / KS_TILE) * div + o_lo) * KS_TILE;
