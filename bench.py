@@ -8,8 +8,10 @@ timed beside it.
 A step = one decode token's worth of the workload: the encrypted product and its rescale
 (bf_linear_rescaled: bf_linear + bf_rescale as one call) for every linear layer of the workload, cached encoded weights
 streamed from HBM (27 GB per step for the Qwen3-0.6B-shaped default, 239 MB for the single GPT-2 projection, beside 0.3 GB
-of rotation keys a call: always larger than L2, so consecutive steps cannot be served from cache).  The other configurations are timed after the main one and reported under
-"other_workloads", each with its own rooflines.  Inputs are seeded and synthetic.
+of rotation keys a call: always larger than L2, so consecutive steps cannot be served from cache).  The other
+configurations are timed after the main one and reported under
+"other_workloads", each with its own rooflines: --details FILE writes all of it, the line that is printed names each
+workload's time.  Inputs are seeded and synthetic.
 """
 from __future__ import annotations
 
@@ -101,7 +103,11 @@ class ClockSampler(threading.Thread):
                 "power_w": max(power) if power else None, "samples": len(sm), "reasons": sorted(reasons)}
 
 
-DEFAULT_LANES = 2       # the library's default number of concurrent key-switch chains
+def default_lanes(ring_n):
+    """The library's default number of concurrent key-switch chains."""
+    return 2 if ring_n >= 1 << 14 else 1
+
+
 MIN_REGION_S = 0.5      # every timed region lasts at least this long (steps are repeated inside it)
 
 # Workload specifications: "<workload>[@option[,option...]]".  Options: budget=<GB> (cache budget, so that
@@ -275,12 +281,14 @@ class Measurement:
         bf.bf_set_kernel_timing(R.ctx, True)
         bf.bf_set_lanes(R.ctx, 1)
         bf.bf_get_key_stream_bytes(R.ctx)
+        bf.bf_get_mac_key_bytes(R.ctx)
         self.timed(R.step, k_steps)
         out["kstats"] = bf.bf_get_kernel_stats(R.ctx)
         out["key_bytes"] = bf.bf_get_key_stream_bytes(R.ctx)
+        out["mac_key_bytes"] = bf.bf_get_mac_key_bytes(R.ctx)
         out["k_steps"] = k_steps
         bf.bf_set_kernel_timing(R.ctx, False)
-        bf.bf_set_lanes(R.ctx, DEFAULT_LANES)
+        bf.bf_set_lanes(R.ctx, default_lanes(R.N))
         if e2e:
             # end to end through the host-buffer entry point (pinned host ciphertexts in and out)
             R.make_host_buffers()
@@ -305,11 +313,11 @@ class Measurement:
             return (ms / n) if n else None, n / K
 
         rl = {}
-        # weight-streaming multiply-accumulate: algorithmic bytes = every encoded word once, and under double hoisting the
-        # baby rotations' keys, whose inner products are part of it
+        # weight-streaming multiply-accumulate: algorithmic bytes = every encoded word once, and the keys of the baby
+        # rotations where it makes them (counted by the library)
         mac_ms, mac_n = avg_ms("mac")
         if mac_ms:
-            mac_bytes = R.mac_stream_bytes() / max(1.0, mac_n)
+            mac_bytes = (R.total_pt_bytes() + m["mac_key_bytes"] / K) / max(1.0, mac_n)
             ach = mac_bytes / (mac_ms * 1e-3) / 1e9
             rl["mac"] = {"bound": "hbm", "achieved": round(ach, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(ach / hbm_peak, 4), "of": peak_kind, "traffic": traffic_of("mac", mac_bytes),
@@ -448,9 +456,8 @@ def run_ours(args):
                    "plan": desc["plan"], "layers": len(R.layers),
                    "encoded_weight_bytes_per_step": R.total_pt_bytes(),
                    "encoded_weight_bytes_cached": R.cached_pt_bytes(), "fallback_layers": R.n_fallback_layers(),
-                   "l2": "inputs larger than L2: the encoded weights streamed each step exceed 126 MB",
-                   "timed_region": f"{args.steps} steps x {m['repeats_per_step']} repeats, at least {MIN_REGION_S} s",
-                   "multi_gpu": "replicas: every rank decodes its own token, no data-path collective"},
+                   "l2": "inputs larger than L2: the encoded weights of a step exceed 126 MB",
+                   "multi_gpu": "replicas: a token per rank, no collective on the data path"},
         "tokens_per_s": round(world * 1e3 / ms_per_step, 3),
         "clocks": clocks,
         "e2e": {"value": round(job_ms_per_token(m["e2e_ms"], world), 5), "unit": UNIT, "h2d_bytes_per_step": h2d,
@@ -461,7 +468,7 @@ def run_ours(args):
         "kernel_time_share": shares,
         "kernel_ms_per_step": info["kernel_ms_per_step"],
         "kernel_timing": "event pair around every launch with the key-switch chains serialised (1 lane); "
-                         f"value and e2e are timed with {DEFAULT_LANES} concurrent chains and no per-launch events",
+                         f"value and e2e are timed with {default_lanes(R.N)} concurrent chains and no per-launch events",
         "measured_rates": {"imad_per_sm_clk": round(imad_rate / 148 / (sm_mhz * 1e6), 2),
                            "fma64_per_sm_clk": round(fma_rate / 148 / (sm_mhz * 1e6), 2),
                            "imad_per_s": imad_rate, "fma64_per_s": fma_rate},
@@ -487,9 +494,30 @@ def run_ours(args):
         line["cpu_baseline"] = cpu_baseline(args.workload, budget_s=20.0)
     elif world == 1:
         line["cpu_baseline"] = None
-    print(json.dumps(line))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(short_line(line)))
     if world > 1:
         dist.destroy_process_group()
+
+
+def short_line(line: dict) -> dict:
+    """The line that is printed: the contract's keys and one figure for each kernel and each further workload, below 3000
+    characters, which is what survives of a longer one where only the end of the output is kept (--details writes it all)."""
+    out = {k: v for k, v in line.items() if k not in ("rooflines", "kernel_ms_per_step", "kernel_timing", "other_workloads",
+                                                      "roofline", "kernel_time_share", "measured_rates", "cpu_baseline")}
+    out["config"] = dict(line["config"], plan="%(pack)s, %(moddown)s, %(hoist)s; D %(D)d, tau %(tau)d, %(b)dx%(g)d" % line["config"]["plan"])
+    out["roofline"] = {k: line["roofline"].get(k) for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic")}
+    out["frac"] = {k: v["frac"] for k, v in line["rooflines"].items()}
+    out["time_share"] = {k: round(v, 3) for k, v in line["kernel_time_share"].items()}
+    out["rates"] = {k: line["measured_rates"][k] for k in ("imad_per_sm_clk", "fma64_per_sm_clk")}
+    if line.get("cpu_baseline"):
+        out["cpu_baseline"] = {k: line["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    if "other_workloads" in line:
+        out["other_ms"] = {k.replace(BEST, "best"): round(v.get("ms_per_token", v.get("ms_per_call")), 3)
+                           for k, v in line["other_workloads"].items()}
+    return out
 
 
 # ------------------------------------------------------------------------------------------------
@@ -682,6 +710,7 @@ def main():
     ap.add_argument("--extra", default=DEFAULT_EXTRA,
                     help="comma-separated further workload specs timed after the main one (N=1 only); '' for none; "
                          "tiles = the tile-size study and the paper's own parameter set")
+    ap.add_argument("--details", default="", help="file for every workload's plan, rooflines and kernel times")
     args = ap.parse_args()
     if args.extra == "tiles":     # tile-size study and the paper's own parameter set
         args.extra = ("gemm1024_D1024,gemm1024_D512,gemm1024_D256,gemm1024_D128,gpt2_qkv_paper_params,"

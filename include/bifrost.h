@@ -297,8 +297,13 @@ int bf_measure_fma64_rate(bf_ctx* ctx, double* fma_per_second_out);
 /* Bytes of rotation keys the key-switch inner products launched since the previous call had to stream:
  * counted once per distinct key of each launch (distinct_out, host: what must come from HBM; Sec. 4.2
  * "key-switching primitives") and once per rotation (per_rotation_out, host: what the launches read,
- * L2 hits included).  Resets both counters.  Does not synchronise. */
+ * L2 hits included).  Keys that a multiply-accumulate reads because it makes the baby rotations itself
+ * (double hoisting) are not among them: see bf_get_mac_key_bytes.  Resets both counters.  Does not
+ * synchronise. */
 int bf_get_key_stream_bytes(bf_ctx* ctx, uint64_t* distinct_out, uint64_t* per_rotation_out);
+/* Bytes of rotation keys that the multiply-accumulates launched since the previous call had to stream (out, host; a key
+ * once per launch).  Resets the counter.  Does not synchronise. */
+int bf_get_mac_key_bytes(bf_ctx* ctx, uint64_t* out);
 
 const char* bf_strerror(int code);
 const char* bf_last_cuda_error(const bf_ctx* ctx);

@@ -84,6 +84,7 @@ _SIGNATURES = {
     "bf_measure_imad_rate": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double)]),
     "bf_measure_fma64_rate": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double)]),
     "bf_get_key_stream_bytes": (ctypes.c_int, [_vp, ctypes.POINTER(_u64), ctypes.POINTER(_u64)]),
+    "bf_get_mac_key_bytes": (ctypes.c_int, [_vp, ctypes.POINTER(_u64)]),
     "bf_strerror": (ctypes.c_char_p, [ctypes.c_int]),
     "bf_last_cuda_error": (ctypes.c_char_p, [_vp]),
 }
@@ -310,3 +311,10 @@ def bf_get_key_stream_bytes(ctx) -> tuple[int, int]:
     a, b = _u64(0), _u64(0)
     _check(load().bf_get_key_stream_bytes(ctx, ctypes.byref(a), ctypes.byref(b)), "bf_get_key_stream_bytes", ctx)
     return int(a.value), int(b.value)
+
+
+def bf_get_mac_key_bytes(ctx) -> int:
+    """Bytes of rotation keys that multiply-accumulates read since the previous call, once per key and launch."""
+    a = _u64(0)
+    _check(load().bf_get_mac_key_bytes(ctx, ctypes.byref(a)), "bf_get_mac_key_bytes", ctx)
+    return int(a.value)

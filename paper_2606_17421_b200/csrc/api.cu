@@ -129,7 +129,7 @@ struct bf_ctx {
         u32 seen = 0;
         bool unusable = false;
         uint64_t launches[CAT_COUNT] = {0};
-        uint64_t key_bytes_distinct = 0, key_bytes_per_rotation = 0;
+        uint64_t key_bytes_distinct = 0, key_bytes_per_rotation = 0, mac_key_bytes = 0;
     };
     struct GraphKey {
         const void *ct_in, *weights, *ct_out;
@@ -1454,6 +1454,7 @@ static int linear_call(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const 
         for (int c = 0; c < (int)CAT_COUNT; ++c) ctx->prof.launches[c] += ge.launches[c];
         ctx->prof.key_bytes_distinct += ge.key_bytes_distinct;
         ctx->prof.key_bytes_per_rotation += ge.key_bytes_per_rotation;
+        ctx->prof.mac_key_bytes += ge.mac_key_bytes;
         return BF_OK;
     }
     if (ge.exec) {                       // stale: buffers, keys or weights changed since the capture
@@ -1471,7 +1472,7 @@ static int linear_call(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const 
     // second call: capture, instantiate, launch
     uint64_t before[CAT_COUNT];
     for (int c = 0; c < (int)CAT_COUNT; ++c) before[c] = ctx->prof.launches[c];
-    const uint64_t kd_before = ctx->prof.key_bytes_distinct, kr_before = ctx->prof.key_bytes_per_rotation;
+    const uint64_t kd_before = ctx->prof.key_bytes_distinct, kr_before = ctx->prof.key_bytes_per_rotation, km_before = ctx->prof.mac_key_bytes;
     if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         ge.unusable = true;
@@ -1490,6 +1491,7 @@ static int linear_call(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const 
         for (int c = 0; c < (int)CAT_COUNT; ++c) ctx->prof.launches[c] = before[c];
         ctx->prof.key_bytes_distinct = kd_before;
         ctx->prof.key_bytes_per_rotation = kr_before;
+        ctx->prof.mac_key_bytes = km_before;
         ge.unusable = true;
         if (rc != BF_OK) return rc;      // argument errors are reported as usual
         return linear_enqueue(ctx, ct_in, n_in, pt_weights, W_raw, d_out, d_in, rescaled ? nullptr : ct_out, n_out, rescaled ? ct_out : nullptr);
@@ -1502,12 +1504,14 @@ static int linear_call(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const 
         for (int c = 0; c < (int)CAT_COUNT; ++c) ctx->prof.launches[c] = before[c];
         ctx->prof.key_bytes_distinct = kd_before;
         ctx->prof.key_bytes_per_rotation = kr_before;
+        ctx->prof.mac_key_bytes = km_before;
         ge.unusable = true;
         return linear_enqueue(ctx, ct_in, n_in, pt_weights, W_raw, d_out, d_in, rescaled ? nullptr : ct_out, n_out, rescaled ? ct_out : nullptr);
     }
     for (int c = 0; c < (int)CAT_COUNT; ++c) ge.launches[c] = ctx->prof.launches[c] - before[c];
     ge.key_bytes_distinct = ctx->prof.key_bytes_distinct - kd_before;
     ge.key_bytes_per_rotation = ctx->prof.key_bytes_per_rotation - kr_before;
+    ge.mac_key_bytes = ctx->prof.mac_key_bytes - km_before;
     ge.exec = exec;
     ge.epoch = ctx->epoch;
     CK(cudaGraphLaunch(ge.exec, ctx->stream));
@@ -1817,6 +1821,13 @@ extern "C" int bf_get_key_stream_bytes(bf_ctx* ctx, uint64_t* distinct_out, uint
     *distinct_out = ctx->prof.key_bytes_distinct;
     *per_rotation_out = ctx->prof.key_bytes_per_rotation;
     ctx->prof.key_bytes_distinct = ctx->prof.key_bytes_per_rotation = 0;
+    return BF_OK;
+}
+
+extern "C" int bf_get_mac_key_bytes(bf_ctx* ctx, uint64_t* out) {
+    if (!ctx || !out) return BF_ERR_INVALID_ARG;
+    *out = ctx->prof.mac_key_bytes;
+    ctx->prof.mac_key_bytes = 0;
     return BF_OK;
 }
 

@@ -22,6 +22,7 @@ struct Profiler {
     // key-switch inner products: bytes of rotation keys counted once per distinct key of a launch (what must come
     // from HBM) and once per rotation (what the launch reads, L2 hits included)
     uint64_t key_bytes_distinct = 0, key_bytes_per_rotation = 0;
+    uint64_t mac_key_bytes = 0;       // the baby keys that multiply-accumulates read, once per key and launch
     struct Rec { int cat; cudaEvent_t a, b; };
     std::vector<Rec> recs;            // event pairs recorded since the last collection
     std::vector<cudaEvent_t> pool;    // idle events
@@ -40,7 +41,7 @@ struct RingHost {
     std::vector<u64> q;               // q_0..q_L, then P
     Profiler* prof = nullptr;
     bool dependent_launch = true;     // launch the kernels of a call with programmatic stream serialisation
-    bool compact_cache = false;       // cached plaintexts count for the bytes they occupy, not for 8 a word
+    bool compact_cache = false;       // cached plaintexts count for the bytes of their words, not for 8 a word
     int device = 0;                   // the CUDA device of the context (kernel attributes are set once per device)
 };
 constexpr int MAX_DEVICES = 64;
@@ -104,7 +105,7 @@ u32 mac_split_bits(const RingHost& ring);   // limb width of cached 8-byte words
 // layout of n_pj groups of n_terms diagonals held in n_primes primes (0 = the r ciphertext primes)
 TileLayout mac_tile_layout(const RingHost& ring, u32 n_pj, u32 n_terms, u32 n_primes = 0);
 size_t mac_tile_bytes(const TileLayout& t);                                 // bytes that layout occupies
-size_t mac_accounted_bytes(const RingHost& ring, const TileLayout& t);      // bytes it counts for: 8 a word unless compact_cache
+size_t mac_accounted_bytes(const RingHost& ring, const TileLayout& t);      // bytes its words count for: 8 each unless compact_cache
 // a: [n_pj][2][lay.n_primes][N]; every prime of the layout is processed.  baby null: x holds all terms,
 // [n_terms][2][lay.n_primes][N].  baby non-null: x holds the un-rotated inputs, [n_in][2][lay.n_primes][N], and the
 // rotated terms are computed inside.

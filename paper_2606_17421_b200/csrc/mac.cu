@@ -85,6 +85,7 @@ cudaError_t launch_mac(const RingHost& ring, const u64* pt, const TileLayout& la
         if (parts < 1) parts = 1;
         m.bs.per_part = (baby->n_in + parts - 1) / parts;
         m.bs.parts = (baby->n_in + m.bs.per_part - 1) / m.bs.per_part;
+        if (ring.prof) ring.prof->mac_key_bytes += (u64)(baby->b - 1) * ring.dev.key_bytes;
     }
     m.stream = stream;
     ProfScope prof(ring.prof, CAT_MAC, stream);

@@ -53,7 +53,7 @@ class WorkloadRunner:
                                                (bf.BF_PLAN_MODDOWN_PER_OUTPUT if self.plan.moddown == "per_output" else 0) |
                                                (bf.BF_PLAN_DOUBLE_HOIST if self.plan.hoist == "double" else 0)),
                                     self.stream.cuda_stream)
-        if compact_cache:           # narrower resident words per prime: 68 % of the cache for the 50 + 6 x 40-bit chain
+        if compact_cache:           # weights count for the bytes of their words in the cache budget, not for 8 a word
             bf.bf_set_compact_cache(self.ctx, True)
         self.compact_cache = compact_cache
         if lanes:                   # concurrent key-switch chains (the library's default otherwise)
@@ -61,13 +61,9 @@ class WorkloadRunner:
         if coef_bits:               # weights resident as rounded 64- or 32-bit coefficients, transformed on every call
             bf.bf_set_coefficient_cache(self.ctx, coef_bits)
         self.coef_bits = coef_bits
-        # bytes an encoded coefficient counts for over all primes (8 each, or 4 / 5 / 8 by prime size when compact), and those
-        # it has
-        self.word_bytes = sum((4 if q < 2 ** 32 else 5 if q < 2 ** 40 else 8) if compact_cache else 8 for q in self.primes)
-        self.stream_word_bytes = sum(4 if q < 2 ** 32 else 5 if q < 2 ** 40 else 8 for q in self.primes)
-        if self.plan.hoist == "double":     # the residue modulo the special prime is kept too, always in 8 bytes
-            self.word_bytes += 8
-            self.stream_word_bytes += 8
+        # bytes an encoded coefficient has over all primes it is held in (with double hoisting the special prime too)
+        held = self.primes + ([self.P] if self.plan.hoist == "double" else [])
+        self.word_bytes = sum(4 if q < 2 ** 32 else 5 if q < 2 ** 40 else 8 for q in held)
         budget = cache_budget_bytes if cache_budget_bytes is not None else self.w.cache_budget_bytes
         if budget:
             bf.bf_set_cache_budget(self.ctx, int(budget))
@@ -95,7 +91,7 @@ class WorkloadRunner:
             keys = _uniform_residues(self.gen, basis, (len(self.rot_steps), self.r, 2), self.N, self.device)
             bf.bf_load_eval_keys(self.ctx, self.rot_steps, len(self.rot_steps), keys)
             del keys
-        self.key_bytes = len(self.rot_steps) * self.r * 2 * (self.r + 1) * self.N * 8
+        self.key_bytes = len(self.rot_steps) * self.r * 2 * self.N * sum(5 if q < 2 ** 40 else 8 for q in basis)
         # layers
         self.layers = []
         for rep in range(self.w.n_repeat):
@@ -160,20 +156,11 @@ class WorkloadRunner:
         return sum(e["pt_bytes"] for e in self.layers if e["handle"])
 
     def resident_bytes(self):
-        """Bytes the cached weights occupy (differs from the streamed bytes when they are kept as coefficients)."""
+        """Bytes the cached weights have (differs from the streamed bytes when they are kept as coefficients)."""
         return sum(e["resident_bytes"] for e in self.layers)
 
     def total_pt_bytes(self):
         return sum(e["pt_bytes"] for e in self.layers)
-
-    def mac_stream_bytes(self):
-        """Bytes the multiply-accumulates of a step cannot do without: every encoded word once and, where they make the
-        baby rotations (double hoisting), every baby key of a call once."""
-        total = sum(e["pt_bytes"] for e in self.layers) * self.stream_word_bytes // self.word_bytes
-        if self.plan.hoist == "double":
-            words = sum(5 if q < 2 ** 40 else 8 for q in self.primes) + 8
-            total += sum(e["b"] - 1 for e in self.layers) * 2 * self.r * self.N * words
-        return total
 
     def n_fallback_layers(self):
         return sum(1 for e in self.layers if not e["handle"])
