@@ -420,8 +420,10 @@ __device__ __forceinline__ u32 ld_stream32(const void* p, u64 policy) {
     return v;
 }
 
-// ---- Sums of products of residues, three ways.  B200 issues 64 fp64 multiply-adds per SM and clock, but only 32
-// 32x32+64-bit integer ones, so the primes below 2^40 (all but one or two of a chain) multiply in fp64.
+// ---- Sums of products of residues, three ways.  fp64 multiply-adds and 32x32+64-bit integer ones issue at the same measured
+// rate (62 and 63 per SM and clock), but a product takes four fp64 operations, on a pipe that these kernels leave idle
+// otherwise, against three or four integer multiply-adds beside the cutting and adding of limbs, on the pipes that do the
+// address arithmetic too: so the primes below 2^40 (all but one or two of a chain) multiply in fp64.
 enum OperandClass : int { OP_DP = 0, OP_NARROW = 1, OP_WIDE = 2 };
 constexpr u32 LIMB_NARROW = 25, LIMB_WIDE = 30;
 

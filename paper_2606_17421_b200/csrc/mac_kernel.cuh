@@ -13,9 +13,12 @@
 // in place, coalesced, and permutes inside the tile on the way to shared memory.  X itself (2 (r+1) N words per term) is
 // never written to memory.
 //
-// What bounds it: HBM (keys and weights are read once, 5 bytes a word modulo the primes below 2^40).  Loads go straight to registers: a stream that
-// every thread consumes in the pattern it loads needs no staging, no barriers and no producer; what hides the latency is
-// the number of independent loads per thread (2r key words at a time; two batches of 8 weights) times resident warps.
+// What bounds it: no resource alone.  The 768 -> 2304 call of a GPT-2 layer (510 MB of keys and weights, read once, 5 bytes a
+// word modulo the primes below 2^40) takes 126 us: 4.3 TB/s of DRAM traffic, 61 % of the issue slots, 45 % of the warps
+// resident, waits for loads ahead of every other stall; weights in 5 bytes instead of 8 took 13 % of its bytes and none of its
+// time.  Loads go straight to registers: a stream that every thread consumes in the pattern it loads needs no staging, no
+// barriers and no producer; what hides the latency is the number of independent loads per thread (2r key words at a time;
+// two batches of 8 weights, three where they are packed) times resident warps.
 #pragma once
 #include "bf_host.h"
 
@@ -243,7 +246,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
 // grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
 // operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
-// Four blocks an SM (64 registers, a few spilled in the key part) because resident warps are what hides the latency: two,
+// Four blocks an SM (64 registers; the key part spills 80 bytes at r = 7, 236 at r = 9) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
 template <bool NARROW, int LOG_TN, bool BABY, int RC>

@@ -8,8 +8,8 @@
 //
 // A transform of N = R*C points runs as two launches.  The strided pass transforms the R rows
 // (stride C) of a tile of adjacent columns; the contiguous pass transforms chunks of C adjacent
-// points.  Inside a pass every thread keeps a closed set of up to 16 points in registers for up to
-// four butterfly stages, and sets are exchanged through shared memory between stage groups.
+// points.  Inside a pass every thread keeps a closed set of up to 8 points in registers for up to
+// three butterfly stages, and sets are exchanged through shared memory between stage groups.
 #include "bf_host.h"
 
 #include <type_traits>
@@ -262,7 +262,8 @@ __device__ __forceinline__ void set_butterflies(T (&e)[8], const void* __restric
 }
 // After an inverse group the points that were sums to the end have grown: point 0 by 2^K, point 1 to 2^(K-1) fresh
 // products (0.54q each), point 2 and 3 to 2^(K-2) of them, and so on.  Centring point 0 leaves every point within 2.2q, so
-// that a group of at most three stages starts below 2.2q and stays below 18q < 2^47.
+// that a group of at most three stages that starts there stays below 18q < 2^47.  (The contiguous pass starts from canonical
+// residues and does not centre after its first group of two stages: the second starts below 4q and stays below 16q.)
 template <int K, int PATH, int OFF = 0, typename T>
 __device__ __forceinline__ void centre_sums(T (&e)[8], const ModConsts& c) {
     if constexpr (PATH == PATH_DP) {
@@ -724,7 +725,11 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // ModDownEpilogue); 5 = ingest (see PolyBatch): the digits into the operand array, component c of the inputs times P into
 // lift_ptr.
 constexpr int CONTIG_THREADS = 128, CONTIG_WARPS = CONTIG_THREADS / 32;
-constexpr size_t CONTIG_SHORT_CHUNKS = 12000;       // forward launches of up to that many chunks: see ntt_contig_short
+// Forward launches of up to that many chunks: see ntt_contig_short.  Plain forward launches over 6 primes of 40 bits, one of 50 and
+// one of 60 (N = 2^15), with 4 and with 8 points a thread: 7168 chunks 15.1 and 15.0 us, 10240 19.0 and 18.4, 13312 22.8 and 21.3,
+// 17408 27.1 and 25.8, 23552 33.3 and 31.4; on a ring of 2^12 8000 17.3 and 18.2, 10944 21.0 and 21.1, 13952 25.1 and 24.6.
+// Whole calls do not tell lines from 7000 to 40000 apart (within 1 % but for 768 -> 2304 without flags: 477, 485, 485 us).
+constexpr size_t CONTIG_SHORT_CHUNKS = 12000;
 
 // a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
 template <int PATH, typename T>

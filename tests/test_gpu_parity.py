@@ -147,8 +147,8 @@ def test_rotate_matches_oracle(pkey):
 
 @pytest.mark.parametrize("logN,n_primes", [(10, 2), (10, 5), (11, 8), (10, 10), (10, 15)])
 def test_rotate_for_every_arrangement_of_digits_in_a_block(logN, n_primes):
-    # the fused transform and inner product gives each digit a warp: several chunks per block where digits are few (more
-    # than a small ring has), one chunk and 8 warps, one warp per digit beyond that
+    # the fused transform and inner product: several chunks per block where digits are few (all that the smallest ring has),
+    # one chunk and idle warps, a warp per digit, digits in two rounds of 8 warps
     par = ckks.Params(1 << logN, ckks.find_primes(1 << 40, 2 << logN, n_primes), ckks.find_primes(1 << 60, 2 << logN, 1)[0], 2.0 ** 30)
     plan = ckks.Plan(8, 1, 4, 2)
     s = ckks.keygen(par, 5)
