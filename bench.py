@@ -35,7 +35,7 @@ UNIT = "ms"
 # from an ncu capture summarised under profiles/ (the headline workload is too large for a multi-pass capture: one GPT-2
 # layer under the same plan, same kernel); `traffic` in the line = this ratio x the algorithmic bytes of a launch.
 NCU_TRAFFIC_RATIO = {
-    "mac": 1.07,                  # the 768 -> 2304 call: 626 MB for 585 MB of keys and weights (digits, outputs)
+    "mac": 1.06,                  # the 768 -> 2304 call: 542 MB for 510 MB of keys and weights (digits, outputs)
 }
 # Executed warp instructions per butterfly by pipe, from the same captures (profiles/transform_passes_ncu.md), to set beside
 # the modelled 8 / 12 / 10 operations: 1024 transforms into six primes on the 8-operation fp64 path, one on the 12-operation
@@ -456,7 +456,8 @@ def run_ours(args):
                    "plan": desc["plan"], "layers": len(R.layers),
                    "encoded_weight_bytes_per_step": R.total_pt_bytes(),
                    "encoded_weight_bytes_cached": R.cached_pt_bytes(), "fallback_layers": R.n_fallback_layers(),
-                   "l2": "inputs larger than L2: the encoded weights of a step exceed 126 MB",
+                   "l2": "inputs larger than L2: the encoded weights of a step exceed 126 MB" if R.total_pt_bytes() > 126e6
+                   else "the encoded weights of a step fit L2 (126 MB): a repeated small call",
                    "multi_gpu": "replicas: a token per rank, no collective on the data path"},
         "tokens_per_s": round(world * 1e3 / ms_per_step, 3),
         "clocks": clocks,

@@ -107,15 +107,18 @@ WORKLOADS = {
     # M = 64 diagonals per tile split as 16 baby x 4 giant steps: measured fastest on B200 (fewer full
     # key switches than 8 x 8 at the price of four more rotation keys)
     "gpt2_qkv": Workload("gpt2_qkv", "n15", PlanSpec(1024, 16, 16, 4), (GPT2_LAYER[0],)),
-    # (per call, ms on B200 for 16x4 / 32x2 / 8x8: ffn_down 0.507 / 0.872 / 0.490; the other three are fastest at 16x4)
+    # (the splits were chosen when an inner product was a launch of its own: ms per call for 16x4 / 32x2 / 8x8, ffn_down
+    # 0.507 / 0.872 / 0.490.  Now that the multiply-accumulate makes the baby rotations: qkv 0.310 / 0.286 / 0.446, ffn_down
+    # 0.358 / 0.485 / 0.382)
     "gpt2_step": Workload("gpt2_step", "n15", PlanSpec(1024, 16, 16, 4), GPT2_LAYER, n_repeat=12,
                           splits={"ffn_down": (8, 8)}),
-    # (16x4 / 32x2 / 8x8: q+k+v 0.380 / 0.395 / 0.534, o 0.384 / 0.535 / 0.401, gate+up 0.483 / 0.454 / 0.729,
-    # down 0.507 / 0.872 / 0.490)
+    # (16x4 / 32x2 / 8x8 when they were chosen: q+k+v 0.380 / 0.395 / 0.534, o 0.384 / 0.535 / 0.401, gate+up 0.483 / 0.454 /
+    # 0.729, down 0.507 / 0.872 / 0.490; now 0.311 / 0.286 / 0.446, 0.290 / 0.372 / 0.327, 0.397 / 0.342 / 0.627, 0.358 /
+    # 0.485 / 0.381)
     "qwen3_step": Workload("qwen3_step", "n15", PlanSpec(1024, 16, 16, 4), QWEN3_LAYER, n_repeat=28,
                            cache_budget_bytes=60 * 10 ** 9, splits={"gate+up": (32, 2), "down": (8, 8)}),
-    # (8x4 / 16x2 / 4x8: q+k+v 1.79 / 1.79 / 2.49, o 1.43 / 1.56 / 1.84, gate+up 5.88 / 4.25 / 9.86,
-    # down 3.78 / 6.29 / 3.44)
+    # (8x4 / 16x2 / 4x8 when they were chosen: q+k+v 1.79 / 1.79 / 2.49, o 1.43 / 1.56 / 1.84, gate+up 5.88 / 4.25 / 9.86,
+    # down 3.78 / 6.29 / 3.44; now 1.49 / 1.44 / 2.11, 1.19 / 1.28 / 1.56, 4.90 / 3.42 / 8.43, 3.03 / 4.13 / 2.86)
     "llama3_layer": Workload("llama3_layer", "n16", PlanSpec(1024, 32, 8, 4), LLAMA3_8B_LAYER,
                              splits={"gate+up": (16, 2), "down": (4, 8)}),
 }
