@@ -1006,7 +1006,9 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     // keys again, so that X is worth keeping in memory then.  It reads the digits of all inputs (r (r+1) polynomials each),
     // where the other form keeps those of a batch and X; it is used where its scratch stays within that of the other form
     // plus one more buffer of that one's digits (240 inputs, r = 15 and one rotation each, N = 2^10: 1139 MB in the one form,
-    // 350 MB in the other).  Their transforms run in batches of what giant_batch allows.
+    // 350 MB in the other; beyond that line the two are as fast: N = 2^15, r = 7, 60 inputs of 3 rotations 2540 us with 3.1 GB and
+    // 2593 us with 2.3 GB, 160 inputs of one rotation 5302 us with 7.4 GB and 4835 us with 4.0 GB).  Their transforms run in
+    // batches of what giant_batch allows.
     const u32 giant_sets = giant_per_lane * (u32)lanes, ingest_batch = gb < n_in ? gb : n_in;
     const u32 other_sets = giant_sets > in_batch ? giant_sets : in_batch;
     const bool rotate_in_mac = dh && b > 1 && (resident || groups == n_pj) &&
