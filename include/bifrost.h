@@ -141,8 +141,8 @@ int bf_linear(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const bf_weight
 
 /* bf_linear followed by bf_rescale from the full level (Sec. 2.1 rescaling; the decode loop of Alg. 3 rescales every
  * product), as one call: ct_low receives n_out ciphertexts of r-1 primes, boundary layout [2][r-1][N], the same residues
- * as the two calls in turn.  Where the plan ends the product in an element-wise kernel (double hoisting with one
- * division per output) the rescale happens inside it; the full-level result then never reaches memory the caller sees.
+ * as the two calls in turn.  Where the product ends in an element-wise kernel (every plan with giant steps or
+ * double hoisting) the rescale happens inside it; the full-level result then never reaches memory the caller sees.
  * scale_inout (host, may be NULL) is divided by the dropped prime.  Same errors as bf_linear; BF_ERR_LEVEL if r < 2. */
 int bf_linear_rescaled(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, const bf_weights* pt_weights,
                        const float* W_raw, uint32_t d_out, uint32_t d_in, uint64_t* ct_low, uint32_t n_out,

@@ -115,10 +115,9 @@ struct bf_ctx {
     u64* keys = nullptr;
     u32* perms = nullptr;            // [n_keys][N] pinv: where position n goes under the key's automorphism
     std::vector<u32> gal, gal_inv;   // Galois element of each key's rotation, 5^steps mod 2N, and its inverse
-    u32* perms_fwd = nullptr;        // [n_keys][N] perm: rotated[n] = unrotated[perm[n]] (per-output division by P)
     u32 n_keys = 0;
     // scratch (grow-only)
-    DevBuf X, X0, Aext, Dig, U, Ubig, Tc, Tn, Cc, A, Rres, Lfull, fft, coef, ptnat, ptjit, stage_in, stage_out, nm_a, nm_b;
+    DevBuf X, X0, Aext, Dig, U, Ubig, Tc, Tn, Cc, A, Lfull, fft, coef, ptnat, ptjit, stage_in, stage_out, nm_a, nm_b;
     u64 cache_budget = 0, cache_used = 0;
     std::vector<bf_weights*> weights;
     std::string cuda_msg;
@@ -448,7 +447,7 @@ extern "C" void bf_ctx_destroy(bf_ctx* ctx) {
             delete w;
         }
     }
-    DevBuf* bufs[] = {&ctx->X, &ctx->X0, &ctx->Aext, &ctx->Dig, &ctx->U, &ctx->Ubig, &ctx->Tc, &ctx->Tn, &ctx->Cc, &ctx->A, &ctx->Rres, &ctx->Lfull,
+    DevBuf* bufs[] = {&ctx->X, &ctx->X0, &ctx->Aext, &ctx->Dig, &ctx->U, &ctx->Ubig, &ctx->Tc, &ctx->Tn, &ctx->Cc, &ctx->A, &ctx->Lfull,
                       &ctx->fft, &ctx->coef, &ctx->ptnat, &ctx->ptjit, &ctx->stage_in, &ctx->stage_out, &ctx->nm_a, &ctx->nm_b};
     for (DevBuf* b : bufs) free_buf(*b);
     cudaFree(ctx->tw_fwd);
@@ -467,7 +466,6 @@ extern "C" void bf_ctx_destroy(bf_ctx* ctx) {
     cudaFree(ctx->overflow_flag);
     cudaFree(ctx->keys);
     cudaFree(ctx->perms);
-    cudaFree(ctx->perms_fwd);
     for (cudaEvent_t& e : ctx->ev)
         if (e) cudaEventDestroy(e);
     for (auto& rec : ctx->prof.recs) { cudaEventDestroy(rec.a); cudaEventDestroy(rec.b); }
@@ -484,10 +482,8 @@ static void drop_eval_keys(bf_ctx* ctx) {
     ctx->epoch++;
     cudaFree(ctx->keys);
     cudaFree(ctx->perms);
-    cudaFree(ctx->perms_fwd);
     ctx->keys = nullptr;
     ctx->perms = nullptr;
-    ctx->perms_fwd = nullptr;
     ctx->key_of_steps.clear();
     ctx->n_keys = 0;
 }
@@ -556,12 +552,11 @@ extern "C" int bf_load_eval_keys(bf_ctx* ctx, const uint32_t* rot_steps, uint32_
     cudaError_t ne = ntt_forward_split(ctx->ring, B, n_keys * r * 2, LOAD_REDUCE, ctx->keys, perm_dev, 2 * r, ctx->stream);
     cudaError_t se = cudaStreamSynchronize(ctx->stream);
     cudaFree(stage);
+    cudaFree(perm_dev);
     if (ne != cudaSuccess || se != cudaSuccess) {
-        cudaFree(perm_dev);
         ctx->cuda_msg = std::string("key transform: ") + cudaGetErrorString(ne != cudaSuccess ? ne : se);
         return fail(BF_ERR_CUDA);
     }
-    ctx->perms_fwd = perm_dev;
     ctx->key_of_steps.swap(key_of_steps);
     ctx->gal.swap(gal);
     ctx->gal_inv.swap(gal_inv);
@@ -874,11 +869,11 @@ static int moddown_batch(bf_ctx* ctx, const Lane& lane, const RotBatch& rb, cons
     return BF_OK;
 }
 
-static int ensure_rot_scratch(bf_ctx* ctx, u32 n_dig_sets, u32 n_rot) {
+// for n_rot rotations whose results are divided in the transform domain (Tc: at least n_tc polynomials)
+static int ensure_rot_scratch(bf_ctx* ctx, u32 n_rot, u32 n_tc = 0) {
     const size_t N = ctx->N, r = ctx->r, nb = r + 1;
-    TRY(ensure(ctx, ctx->Dig, (size_t)n_dig_sets * r * nb * N * 8));       // digits between the passes of their transforms
     TRY(ensure(ctx, ctx->U, (size_t)n_rot * 2 * nb * N * 8));
-    TRY(ensure(ctx, ctx->Tc, (size_t)n_rot * 2 * N * 8));
+    TRY(ensure(ctx, ctx->Tc, (size_t)(2 * n_rot > n_tc ? 2 * n_rot : n_tc) * N * 8));
     TRY(ensure(ctx, ctx->Tn, (size_t)n_rot * 2 * r * N * 8));
     return BF_OK;
 }
@@ -993,7 +988,6 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     // and a launch takes at most MAX_ROT_BATCH)
     if (giant_per_lane > gb / (u32)lanes) giant_per_lane = gb / (u32)lanes;
     if (giant_per_lane < 1) giant_per_lane = 1;
-    const u32 rot_per_lane = baby_per_lane > giant_per_lane ? baby_per_lane : giant_per_lane;
     // double hoisting: the rotated inputs and the inner sums live in the extended basis {q_i, P}
     const bool dh = (ctx->plan.flags & BF_PLAN_DOUBLE_HOIST) != 0;
     const u32 nmp = mac_primes(ctx);                      // primes of X, of the plaintexts and of the inner sums
@@ -1022,41 +1016,47 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
         TRY(ensure(ctx, ctx->X0, rotate_in_mac ? (size_t)ingest_batch * r * N * 8 : (size_t)n_in * ctw * 8));
         TRY(ensure(ctx, ctx->Aext, (size_t)n_out * g * xw * 8));
     }
-    TRY(ensure(ctx, ctx->A, (size_t)n_out * g * ctw * 8));
+    else TRY(ensure(ctx, ctx->A, (size_t)n_out * g * ctw * 8));
     if (ct_low) {                   // the full-level result is an intermediate
         TRY(ensure(ctx, ctx->Lfull, (size_t)n_out * ctw * 8));
         ct_out = (u64*)ctx->Lfull.p;
     }
     RescaleConsts rcs;
     if (ct_low) rescale_consts(ctx, r, rcs);
-    // one division by P per output: the inner products of all giant rotations stay alive until every chain is done
-    const bool per_output = (ctx->plan.flags & BF_PLAN_MODDOWN_PER_OUTPUT) && n_giant > 0;
-    TRY(ensure(ctx, ctx->Rres, (size_t)(per_output ? n_out : n_giant ? n_giant : 1) * ctw * 8));
-    // double hoisting with one division per output: the giant steps' inputs are never divided in the transform domain
-    // (see below); their coefficient forms keep the residue modulo P
-    const bool assemble = dh && per_output;
-    const u32 cc_primes = assemble ? nb : r;
-    TRY(ensure(ctx, ctx->Cc, (size_t)giant_sets * cc_primes * N * 8));
+    // Divisions by P behind the multiply-accumulate happen in the coefficient domain, which the giant steps' digits and the
+    // outputs need anyway: of the inner sums of the extended basis in the ModUp of the giant steps, of everything else in the
+    // output assembly.  The inner products of all giant rotations stay alive until then.  (Dividing each giant rotation in the
+    // transform domain takes 2r forward transforms of lifted residues more.  768 -> 2304 without flags: N = 2^15, 9 giant
+    // rotations, 493 -> 463 us; N = 2^13, 45 of them, 253 -> 234 us; 64 x 64 on 2^12, 61.7 -> 59.4 us)
+    const bool assemble = dh || n_giant > 0;
+    const u32 mid_primes = dh ? nb : r;                     // of the giant steps' inputs in the coefficient domain
+    OutputAssembly as;
+    memset(&as, 0, sizeof(as));
+    as.a_stride = (long long)xw;
+    as.g1 = g - 1;
+    as.n_out = n_out;
+    as.ext = dh;
+    as.each = !(ctx->plan.flags & BF_PLAN_MODDOWN_PER_OUTPUT);
+    TRY(ensure(ctx, ctx->Cc, (size_t)giant_sets * mid_primes * N * 8));
     {
-        u32 rot_scratch = rot_per_lane * (u32)lanes;
-        if (per_output && rot_scratch < n_out) rot_scratch = n_out;     // Tc, Tn of the per-output division
-        if (dh && rot_scratch < n_out * g) rot_scratch = n_out * g;     // Tc, Tn of the division of the inner sums
-        if (assemble && rot_scratch * 2 < n_out * (g + 3)) rot_scratch = cdiv(n_out * (g + 3), 2u);   // Tc of the output assembly
-        TRY(ensure_rot_scratch(ctx, n_dig_sets, rot_scratch));
+        const u32 rot = dh ? 0u : baby_per_lane * (u32)lanes;          // rotations divided in the transform domain
+        TRY(ensure(ctx, ctx->Dig, (size_t)n_dig_sets * r * nb * N * 8));       // digits between the passes of their transforms
+        TRY(ensure_rot_scratch(ctx, rot, n_out * as.n_t()));
     }
-    if (per_output) TRY(ensure(ctx, ctx->Ubig, (size_t)n_giant * 2 * nb * N * 8));
+    TRY(ensure(ctx, ctx->Ubig, (size_t)n_giant * 2 * nb * N * 8));
     Lane lane[bf_ctx::MAX_LANES];
     for (int c = 0; c < lanes; ++c) {
         lane[c].s = c == 0 ? ctx->stream : ctx->side[c - 1];
         lane[c].Dig = (u64*)ctx->Dig.p + (size_t)c * giant_per_lane * r * nb * N;
-        lane[c].U = (u64*)ctx->U.p + (size_t)c * rot_per_lane * 2 * nb * N;
-        lane[c].Tc = (u64*)ctx->Tc.p + (size_t)c * rot_per_lane * 2 * N;
-        lane[c].Tn = (u64*)ctx->Tn.p + (size_t)c * rot_per_lane * 2 * r * N;
-        lane[c].Cc = (u64*)ctx->Cc.p + (size_t)c * giant_per_lane * cc_primes * N;
+        lane[c].U = (u64*)ctx->U.p + (size_t)c * baby_per_lane * 2 * nb * N;
+        lane[c].Tc = (u64*)ctx->Tc.p + (size_t)c * baby_per_lane * 2 * N;
+        lane[c].Tn = (u64*)ctx->Tn.p + (size_t)c * baby_per_lane * 2 * r * N;
+        lane[c].Cc = (u64*)ctx->Cc.p + (size_t)c * giant_per_lane * mid_primes * N;
     }
     u64* X = (u64*)ctx->X.p;
-    u64* A = (u64*)ctx->A.p;
-    u64* Rres = (u64*)ctx->Rres.p;
+    u64* A = dh ? (u64*)ctx->Aext.p : (u64*)ctx->A.p;      // inner sums
+    as.a = A;
+    as.u = (const u64*)ctx->Ubig.p;
     u64* Dig = (u64*)ctx->Dig.p;
     if (ctx->timing) {
         for (cudaEvent_t& e : ctx->ev)
@@ -1147,14 +1147,11 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     stamp(ctx, 1);
 
     // ---- multiply-accumulate over the encoded diagonals (double hoisting: over the extended basis, into Aext)
-    u64* mac_out = dh ? (u64*)ctx->Aext.p : A;
-    MacScatter msc;
+    MacScatter msc;         // component 0 of the inner sums with j >= 1 is stored rotated (only the output assembly reads it)
     memset(&msc, 0, sizeof(msc));
-    if (assemble) {         // component 0 of the inner sums with j >= 1 is stored rotated (only the output assembly reads it)
-        msc.on = 1;
-        msc.n_out = n_out;
-        for (u32 j = 1; j < g; ++j) msc.gal_inv[j] = ctx->gal_inv[giant_key[j]];
-    }
+    msc.on = n_giant > 0;
+    msc.n_out = n_out;
+    if (n_giant) msc.gal_inv = ctx->gal_inv[giant_key[1]];
     BabySteps baby;
     memset(&baby, 0, sizeof(baby));
     if (rotate_in_mac) {
@@ -1170,7 +1167,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     }
     const BabySteps* bsp = rotate_in_mac ? &baby : nullptr;
     if (resident) {
-        CK(launch_mac(ctx->ring, pt_weights->pt, pt_weights->lay, X, mac_out, n_pj, n_terms, ctx->stream, msc, bsp));
+        CK(launch_mac(ctx->ring, pt_weights->pt, pt_weights->lay, X, A, n_pj, n_terms, ctx->stream, msc, bsp));
     } else {
         // fallback: encode groups of (j, p) just in time into a scratch ring, then consume them (weights kept as
         // coefficients: the same without the encoder, only their transforms)
@@ -1181,44 +1178,9 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
             const TileLayout cl = mac_tile_layout(ctx->ring, cnt, n_terms, nmp);
             TRY(encode_range(ctx, W_raw, d_out, d_in, pj0 * n_terms, cnt * n_terms, (u64*)ctx->ptjit.p, cl, pj0, pt_weights));
             msc.pj0 = pj0;
-            CK(launch_mac(ctx->ring, (const u64*)ctx->ptjit.p, cl, X, mac_out + (size_t)pj0 * xw, cnt, n_terms, ctx->stream, msc,
+            CK(launch_mac(ctx->ring, (const u64*)ctx->ptjit.p, cl, X, A + (size_t)pj0 * xw, cnt, n_terms, ctx->stream, msc,
                           bsp));
         }
-    }
-    if (dh && !assemble) {
-        // one division by P per inner sum and component: A[pj][comp][i] = (Aext[pj][comp][i] - t) * P^{-1}, t the
-        // centred lift of the residue modulo P
-        const u64* Aext = (const u64*)ctx->Aext.p;
-        memset(&B, 0, sizeof(B));
-        B.src = Aext + (size_t)r * N;
-        B.dst = (u64*)ctx->Tc.p;
-        B.src_so = (long long)nb * N;
-        B.dst_so = N;
-        B.n_m = 1;
-        B.mod0 = r;
-        B.mod_step = 0;
-        B.store_centred = 1;
-        CK(ntt_inverse(ctx->ring, B, n_pj * 2, ctx->stream));
-        memset(&B, 0, sizeof(B));
-        B.src = (const u64*)ctx->Tc.p;
-        B.dst = (u64*)ctx->Tn.p;
-        B.src_so = N;
-        B.src_sm = 0;
-        B.dst_so = (long long)r * N;
-        B.dst_sm = N;
-        B.n_m = r;
-        B.mod0 = 0;
-        B.mod_step = 1;
-        B.lift_mod = ctx->ring.q[r];
-        RotBatch no_rb;
-        memset(&no_rb, 0, sizeof(no_rb));
-        ModDownEpilogue epi;
-        memset(&epi, 0, sizeof(epi));
-        epi.u = Aext;
-        epi.out_base = A;
-        epi.out_stride = (long long)r * N;
-        epi.plain = 1;
-        CK(ntt_forward_moddown(ctx->ring, B, n_pj * 2, no_rb, epi, ctx->stream));
     }
     stamp(ctx, 2);
 
@@ -1234,160 +1196,46 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
             for (u32 rho0 = (u32)c * per; rho0 < lane_end; rho0 += giant_chunk) {
                 const u32 cnt = (lane_end - rho0 < giant_chunk) ? lane_end - rho0 : giant_chunk;
                 if (cnt > (u32)MAX_ROT_BATCH) return BF_ERR_INVALID_ARG;   // (cannot happen: see giant_per_lane)
-                if (assemble) {
-                    // The inner sums stay in the extended basis.  A giant step needs the digits of c1 / P: both happen
-                    // in the coefficient domain, where the division is element-wise, so one inverse transform over all
-                    // r + 1 primes feeds the hoisted ModUp, whose first load divides (no transform of the lift of the
-                    // P-residue, none of the quotient back and forth)
-                    const u64* Esrc = (const u64*)ctx->Aext.p + (size_t)(n_out + rho0) * xw + (size_t)nmp * N;   // c1 of each
-                    memset(&B, 0, sizeof(B));
-                    B.src = Esrc;
-                    B.dst = lane[c].Cc;
-                    B.src_so = (long long)xw;
-                    B.src_sm = N;
-                    B.dst_so = (long long)nb * N;
-                    B.dst_sm = N;
-                    B.n_m = nb;
-                    B.mod0 = 0;
-                    B.mod_step = 1;
-                    B.store_centred = 2;
-                    CK(ntt_inverse(ctx->ring, B, cnt, lane[c].s));
-                    const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)nb * N, lane[c].Dig, nullptr, 0, lane[c].Cc + (size_t)r * N);
-                    RotBatch rb;
-                    memset(&rb, 0, sizeof(rb));
-                    rb.n = (int)cnt;
-                    for (u32 t = 0; t < cnt; ++t) {
-                        rb.key[t] = giant_key[(rho0 + t) / n_out + 1];
-                        rb.dig[t] = (int)t;
-                        rb.c0[t] = (int)t;
-                        rb.out[t] = (int)t;
-                    }
-                    // (stored through the rotation: the output assembly reads plain sums)
-                    CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, nullptr,
-                                         ctx->perms, lane[c].s));
-                    continue;
-                }
-                const u64* Asrc = A + (size_t)(n_out + rho0) * ctw;      // ciphertexts with j >= 1 are contiguous
+                // c1 of each, in the coefficient domain.  Inner sums of the extended basis are not divided by P yet: a giant step
+                // needs the digits of c1 / P, and the hoisted ModUp's first load divides, element-wise (no transform of the lift
+                // of the P-residue, none of the quotient back and forth).  Else the transform of a digit in its own prime is
+                // what the inverse transform reads
+                const u64* c1 = A + (size_t)(n_out + rho0) * xw + (size_t)nmp * N;
                 memset(&B, 0, sizeof(B));
-                B.src = Asrc + (size_t)r * N;                            // c1 of each
+                B.src = c1;
                 B.dst = lane[c].Cc;
-                B.src_so = (long long)ctw;
+                B.src_so = (long long)xw;
                 B.src_sm = N;
-                B.dst_so = (long long)r * N;
+                B.dst_so = (long long)mid_primes * N;
                 B.dst_sm = N;
-                B.n_m = r;
+                B.n_m = mid_primes;
                 B.mod0 = 0;
                 B.mod_step = 1;
+                B.store_centred = 2;
                 CK(ntt_inverse(ctx->ring, B, cnt, lane[c].s));
-                const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)r * N, lane[c].Dig, Asrc + (size_t)r * N, (long long)ctw);
+                const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)mid_primes * N, lane[c].Dig, c1, (long long)xw,
+                                                 dh ? lane[c].Cc + (size_t)r * N : nullptr);
                 RotBatch rb;
                 memset(&rb, 0, sizeof(rb));
                 rb.n = (int)cnt;
                 for (u32 t = 0; t < cnt; ++t) {
-                    const u32 j = (rho0 + t) / n_out + 1;
-                    rb.key[t] = giant_key[j];
+                    rb.key[t] = giant_key[(rho0 + t) / n_out + 1];
                     rb.dig[t] = (int)t;
                     rb.c0[t] = (int)t;
                     rb.out[t] = (int)t;
                 }
-                if (per_output) {
-                    CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, nullptr, nullptr,
-                                         lane[c].s));
-                    continue;
-                }
-                CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, lane[c].U, nullptr, nullptr, lane[c].s));
-                TRY(moddown_batch(ctx, lane[c], rb, Asrc, (long long)ctw, Rres + (size_t)rho0 * ctw, (long long)ctw));
+                // (stored through the rotation: the output assembly reads plain sums)
+                CK(ntt_forward_inner(ctx->ring, D0, cnt, rb, ctx->keys, (u64*)ctx->Ubig.p + (size_t)rho0 * 2 * nb * N, nullptr, ctx->perms,
+                                     lane[c].s));
             }
         }
         TRY(join_lanes(ctx, used));
-        if (assemble) {
-            // Output p, component by component, is a sum of terms of the extended basis, each divided by P by itself
-            // (the inner sum of giant step 0, the rotated c0 parts of the other inner sums) or once for their sum (the
-            // key-switch results).  The result is wanted in the coefficient domain, where the division is element-
-            // wise: so the terms' residues modulo the q_i are summed in the load of one inverse transform, their
-            // residues modulo P are transformed apart, and one element-wise kernel divides.  Same values as dividing
-            // each term in the transform domain (the transform is linear, the rotation commutes with the centred lift).
-            RotBatch rb;
-            memset(&rb, 0, sizeof(rb));
-            rb.n = (int)(g - 1);
-            for (u32 j = 1; j < g; ++j) rb.key[j - 1] = giant_key[j];
-            ModDownEpilogue epi;
-            memset(&epi, 0, sizeof(epi));
-            epi.u = (const u64*)ctx->Ubig.p;
-            epi.aext = (const u64*)ctx->Aext.p;
-            epi.aext_stride = (long long)xw;
-            epi.n_sum = g - 1;
-            epi.n_out = n_out;
-            epi.assemble = 1;
-            const u32 n_t = g + 3;
-            memset(&B, 0, sizeof(B));
-            B.src = epi.aext;                                   // (read through epi)
-            B.dst = ct_out;
-            B.dst_so = (long long)ctw;
-            B.dst_sm = N;
-            B.n_m = 2 * r + n_t;
-            B.mod_wrap = r;
-            B.mod0 = 0;
-            B.mod_step = 1;
-            B.tail_m = 2 * r;                                   // the residues modulo P
-            B.tail_dst = (u64*)ctx->Tc.p;
-            B.tail_so = (long long)n_t * N;
-            B.store_centred = 2;
-            CK(ntt_inverse_gathersum(ctx->ring, B, n_out, rb, epi, ctx->stream));
-            CK(finish_division(ctx->ring, ct_out, (long long)ctw, (const u64*)ctx->Tc.p, n_t, n_out, ctx->stream,
-                               ct_low ? &rcs : nullptr, ct_low));
-            stamp(ctx, 3);
-            stamp(ctx, 4);
-            if (!pt_weights) TRY(check_overflow(ctx));
-            return BF_OK;
-        }
-        if (per_output) {
-            // sum over the giant steps of each output in the extended basis (each term read through its rotation),
-            // then one division by P per output and component; the rotated c0 parts join in the same epilogue
-            RotBatch rb;
-            memset(&rb, 0, sizeof(rb));
-            rb.n = (int)(g - 1);
-            for (u32 j = 1; j < g; ++j) rb.key[j - 1] = giant_key[j];
-            ModDownEpilogue epi;
-            memset(&epi, 0, sizeof(epi));
-            epi.u = (const u64*)ctx->Ubig.p;
-            epi.c0_base = A + (size_t)n_out * ctw;              // ciphertexts with j >= 1, index (j - 1) * n_out + p
-            epi.c0_stride = (long long)ctw;
-            epi.pinv = ctx->perms;
-            epi.perm = ctx->perms_fwd;
-            epi.out_base = Rres;
-            epi.out_stride = (long long)ctw;
-            epi.n_sum = g - 1;
-            epi.n_out = n_out;
-            memset(&B, 0, sizeof(B));
-            B.src = (const u64*)ctx->Ubig.p;                    // (read through epi)
-            B.dst = (u64*)ctx->Tc.p;
-            B.dst_so = N;
-            B.n_m = 1;
-            B.mod0 = r;
-            B.mod_step = 0;
-            B.store_centred = 1;
-            CK(ntt_inverse_gathersum(ctx->ring, B, n_out * 2, rb, epi, ctx->stream));
-            memset(&B, 0, sizeof(B));
-            B.src = (const u64*)ctx->Tc.p;
-            B.dst = (u64*)ctx->Tn.p;
-            B.src_so = N;
-            B.src_sm = 0;
-            B.dst_so = (long long)r * N;
-            B.dst_sm = N;
-            B.n_m = r;
-            B.mod0 = 0;
-            B.mod_step = 1;
-            B.lift_mod = ctx->ring.q[r];
-            CK(ntt_forward_moddown(ctx->ring, B, n_out * 2, rb, epi, ctx->stream));
-        }
     }
     stamp(ctx, 3);
 
-    // ---- back to the coefficient domain; the sum over giant steps happens in the transform's load:
-    // Y[p] = A[0][p] + sum_{j >= 1} (rotated A[j][p])
+    // ---- output, in the coefficient domain
     memset(&B, 0, sizeof(B));
-    B.src = A;
+    B.src = A;                          // (assembly: read through `as`)
     B.dst = ct_out;
     B.src_so = B.dst_so = (long long)ctw;
     B.src_sm = B.dst_sm = N;
@@ -1395,14 +1243,23 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
     B.mod_wrap = r;
     B.mod0 = 0;
     B.mod_step = 1;
-    B.sum_src = Rres;
-    B.sum_terms = per_output ? 1 : g - 1;
-    B.sum_stride = (long long)n_out * ctw;
+    if (assemble) {
+        B.n_m += as.n_t();
+        B.tail_m = 2 * r;               // the residues modulo P
+        B.tail_dst = (u64*)ctx->Tc.p;
+        B.tail_so = (long long)as.n_t() * N;
+        B.store_centred = 2;
+        CK(ntt_inverse_assembly(ctx->ring, B, n_out, as, ctx->stream));
+        CK(finish_division(ctx->ring, ct_out, (long long)ctw, (const u64*)ctx->Tc.p, as.n_u(), as.n_t(), n_out, ctx->stream,
+                           ct_low ? &rcs : nullptr, ct_low));
+        stamp(ctx, 4);
+        if (!pt_weights) TRY(check_overflow(ctx));
+        return BF_OK;
+    }
     CK(ntt_inverse(ctx->ring, B, n_out, ctx->stream));
     if (ct_low) CK(launch_rescale(ctx->ring, ct_out, ct_low, n_out, r, rcs.inv, rcs.invs, rcs.qlmod, ctx->stream));
     stamp(ctx, 4);
     if (!pt_weights) TRY(check_overflow(ctx));
-    (void)nb;
     return BF_OK;
 }
 
@@ -1593,7 +1450,8 @@ extern "C" int bf_rotate(bf_ctx* ctx, const uint64_t* ct_in, uint32_t steps, uin
     int key = -1;
     TRY(find_key(ctx, steps, &key));
     TRY(ensure(ctx, ctx->X, 2 * ctw * 8));
-    TRY(ensure_rot_scratch(ctx, 1, 1));
+    TRY(ensure(ctx, ctx->Dig, (size_t)r * (r + 1) * N * 8));
+    TRY(ensure_rot_scratch(ctx, 1));
     u64* X = (u64*)ctx->X.p;
     PolyBatch B;
     memset(&B, 0, sizeof(B));
@@ -1642,7 +1500,8 @@ extern "C" int bf_fold(bf_ctx* ctx, uint64_t* ct, uint32_t n_ct) {
     u32 batch = giant_batch(ctx);
     if (batch > n_ct) batch = n_ct;
     TRY(ensure(ctx, ctx->X, (size_t)batch * 2 * ctw * 8));
-    TRY(ensure_rot_scratch(ctx, batch, batch));
+    TRY(ensure(ctx, ctx->Dig, (size_t)batch * r * (r + 1) * N * 8));
+    TRY(ensure_rot_scratch(ctx, batch));
     u64* X = (u64*)ctx->X.p;                             // [t][0] = NTT(ct_t), [t][1] = its rotation
     const Lane lane = main_lane(ctx);
     for (u32 t0 = 0; t0 < n_ct; t0 += batch) {

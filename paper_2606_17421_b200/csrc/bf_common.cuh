@@ -190,18 +190,10 @@ struct RotBatch {                     // one key-switch launch over n rotations
     unsigned char grp_first[MAX_ROT_BATCH], grp_cnt[MAX_ROT_BATCH];
 };
 
-// Epilogue of the division by P, fused into the forward transform of the lifted P-residue
+// Epilogue of the division by P of a rotated input, fused into the forward transform of the lifted P-residue
 // (polynomial (o, m) = (rotation*2 + component, prime i)):  instead of storing t = NTT(lift),
 //   v = (u[o][i][n] - t) * P^{-1} + (component == 0 ? c0[c0(rot)][i][n] : 0)
 // is scattered to out[out(rot)][component][i][pinv[key(rot)][n]].
-//
-// Per-output form (n_sum > 0; one division by P per output ciphertext and component): polynomial (o, m) =
-// (output p * 2 + component, prime i).  The inner products of the n_sum giant rotations of output p sit in u at
-// rotation index jj * n_out + p (jj < n_sum, key rb.key[jj]), un-rotated; they are summed through each
-// rotation's permutation (rotated[n] = unrotated[perm[n]]), the inverse transform reads the P-residues that
-// way, and the forward transform's last store computes
-//   v[n] = (sum_jj u[jj][i][perm_jj[n]] - t[n]) * P^{-1} + (component == 0 ? sum_jj c0[jj][i][perm_jj[n]] : 0)
-// into out[p][component][i][n] (no scatter), with c0 of rotation index jj * n_out + p at c0_base + index * c0_stride.
 struct ModDownEpilogue {
     const u64* u;                 // [rot][2][r+1][N]
     const u64* c0_base;
@@ -209,31 +201,38 @@ struct ModDownEpilogue {
     const u32* pinv;              // [n_keys][N]
     u64* out_base;
     long long out_stride;
-    const u32* perm;              // [n_keys][N] (per-output form)
-    u32 n_sum, n_out;             // per-output form: giant steps summed per output, number of outputs
-    u32 plain;                    // division by P of inner sums kept in the extended basis (double hoisting):
-                                  //   polynomial (o, i): out_base[o*out_stride + i*N + n] = (u[o][i][n] - t[n]) * P^{-1},
-                                  //   no rotation, nothing added
-    // Output assembly in the extended basis (double hoisting with one division per output; inverse transforms only).
-    // aext[(j*n_out + p)][comp][r+1][N] are the inner sums, u[((j-1)*n_out + p)*2 + comp][r+1][N] the key-switch
-    // results of the giant steps j >= 1; what is rotated (u, and component 0 of the inner sums with j >= 1) was stored
-    // through rotation j's permutation by its producer.  Polynomial (o = p, m):
-    //   modulus i < r, m = comp*r + i:  aext[p][comp][i] + sum_j u[j][p][comp][i] + (comp == 0) sum_j aext[j*n_out+p][0][i]
-    //   modulus P, m = 0, 1:            sum_j u[j][p][comp = m][P]
-    //               m = 2, 3:            aext[p][comp = m - 2][P]
-    //               m = 3 + j:           aext[j*n_out + p][0][P]
-    // (the residues modulo P stay apart because each of those terms is divided by P, i.e. rounded, by itself)
-    const u64* aext;
-    long long aext_stride;
-    u32 assemble;
 };
 
-// Double hoisting with one division per output: component 0 of inner sum (j, p), j >= 1, is only ever used rotated
-// by giant step j, so the multiply-accumulate stores it through that rotation (group pj0 + pj has j = (pj0 + pj) / n_out;
-// on = 0: plain stores).
+// Output assembly (load of an inverse transform).  Output p is a sum of the inner sum of giant step 0, the rotated c0 parts of
+// the other inner sums and the key-switch results of their c1 parts, which live over {q_i, P} and are divided by P, each by
+// itself or once for their sum.  The result is wanted in the coefficient domain, where that division is element-wise
+// (finish_division): so the terms are summed modulo every q_i here and what is rounded by itself is transformed modulo P by
+// itself; no lifted P-residue is transformed forward.  Inner sum (j, p) is a + (j*n_out + p)*a_stride, [2][r or r+1][N];
+// u[((j-1)*n_out + p)*2 + comp][r+1][N] are the key-switch results of giant steps j >= 1.  What is rotated (u, and component
+// 0 of the inner sums with j >= 1) was stored through rotation j's permutation by its producer.  Polynomial (o = p, m):
+//   modulus i < r, m = comp*r + i:  F a[p][comp][i] + sum_j u[j][p][comp][i] + (comp == 0) F sum_j a[j][p][0][i]
+//       (F = 1 where the inner sums live in the extended basis, else P)
+//   modulus P, the separately rounded terms, m - 2r =
+//       0, 1:                        sum_j u[j][p][comp][P]             (one division per output)
+//       2 (j - 1) + comp:            u[j][p][comp][P]                   (each: one division per rotation)
+//     and, n_u such terms further on, where the inner sums live in the extended basis,
+//       comp:                        a[p][comp][P]
+//       1 + j:                       a[j][p][0][P]
+struct OutputAssembly {
+    const u64 *u, *a;
+    long long a_stride;
+    u32 g1, n_out;                // giant steps j >= 1, outputs
+    u32 ext;                      // the inner sums live in the extended basis (double hoisting)
+    u32 each;                     // every key-switch result is divided by itself
+    __host__ __device__ __forceinline__ u32 n_u() const { return g1 == 0 ? 0u : each ? 2u * g1 : 2u; }
+    __host__ __device__ __forceinline__ u32 n_t() const { return n_u() + (ext ? g1 + 2u : 0u); }
+};
+
+// Component 0 of inner sum (j, p), j >= 1, is only ever used rotated by giant step j, so the multiply-accumulate stores it
+// through that rotation (group pj0 + pj has j = (pj0 + pj) / n_out; on = 0: plain stores).
 struct MacScatter {
     u32 on, n_out, pj0;
-    u32 gal_inv[MAX_ROT_BATCH + 1];     // inverse Galois element of giant step j
+    u32 gal_inv;                        // inverse Galois element of giant step 1: step j has its j-th power
 };
 
 // Baby rotations computed inside the multiply-accumulate (double hoisting): input q's term k is its rotation by key[k].

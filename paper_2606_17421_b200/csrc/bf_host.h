@@ -72,13 +72,12 @@ cudaError_t ntt_inverse(const RingHost& ring, const PolyBatch& B, u32 n_outer, c
 // Forward transform of the centred lifts of P-residues with the ModDown epilogue fused into its last store.
 cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
                                 const ModDownEpilogue& epi, cudaStream_t stream);
-// Inverse transform of the P-residues summed over the giant rotations of each output (per-output form of epi).
-cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
-                                  const ModDownEpilogue& epi, cudaStream_t stream);
-// ct[p][comp][i] = (ct[p][comp][i] - sum of the centred P-residues T[p][.]) * P^{-1}: the division that ends the output
-// assembly in the extended basis (ModDownEpilogue::assemble names the n_t polynomials of T per output)
+// Inverse transforms of the output assembly (see OutputAssembly; B: n_m = 2r + as.n_t() slots of every output, tail_m = 2r,
+// store_centred = 2), and the division that ends it: ct[p][comp][i] = (ct[p][comp][i] - sum of the centred P-residues T[p][.])
+// * P^{-1}, T the n_t polynomials per output, the first n_u of them of key-switch results.
 // rc, low non-null: the rescale from r primes follows in the same kernel; the result goes to low ([n_out][2][r-1][N])
-cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_t, u32 n_out,
+cudaError_t ntt_inverse_assembly(const RingHost& ring, const PolyBatch& B, u32 n_outer, const OutputAssembly& as, cudaStream_t stream);
+cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_u, u32 n_t, u32 n_out,
                             cudaStream_t stream, const RescaleConsts* rc = nullptr, u64* low = nullptr);
 cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, void* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream);

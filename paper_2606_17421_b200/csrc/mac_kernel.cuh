@@ -33,6 +33,15 @@ __device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
     return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
 }
 
+// g^j modulo 2^32
+__device__ __forceinline__ u32 power32(u32 g, u32 j) {
+    u32 v = j & 1u ? g : 1u;
+    while (j >>= 1) {
+        g *= g;
+        if (j & 1u) v *= g;
+    }
+    return v;
+}
 
 // Accumulator of one output word of the multiply-accumulate and the form its operands have: weights as stored (two
 // 32-bit halves), the X word as it sits in shared memory.
@@ -218,7 +227,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         if (++ch == n_chunks) {
             u64* ap = a + ((size_t)pj * 2 * np + i) * N;
             u32 at0 = n0 + c;                                           // where component 0 goes (see MacScatter)
-            if (sc.on && sc.pj0 + pj >= sc.n_out) at0 = automorphism_index(at0, sc.gal_inv[(sc.pj0 + pj) / sc.n_out], logN);
+            if (sc.on && sc.pj0 + pj >= sc.n_out) at0 = automorphism_index(at0, power32(sc.gal_inv, (sc.pj0 + pj) / sc.n_out), logN);
             ap[at0] = a0.reduce(R, i);
             ap[(size_t)np * N + n0 + c] = a1.reduce(R, i);
             a0 = {};

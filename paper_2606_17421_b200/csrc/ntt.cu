@@ -720,10 +720,16 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // Forward: second pass (final reduction to [0, q), then the store functors).  Inverse: first pass
 // (reads the batch source: plain residues, tiled/limb-split plaintexts, or a sum of arrays).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
-// EPI: 0 = none; 1 = division by P per rotation (scatter through the rotation's permutation); 2 = per output
-// (sum over the output's giant rotations, gathered through their permutations); 3 = plain; 4 = output assembly (see
-// ModDownEpilogue); 5 = ingest (see PolyBatch): the digits into the operand array, component c of the inputs times P into
-// lift_ptr.
+// EPI: 0 = none; 1 = division by P per rotation (see ModDownEpilogue); 4 = output assembly (see OutputAssembly); 5 = ingest
+// (see PolyBatch): the digits into the operand array, component c of the inputs times P into lift_ptr.
+struct NoEpilogue {};
+struct RotationDivision {
+    ModDownEpilogue e;
+    RotBatch rb;
+};
+template <int EPI> struct EpiArg { typedef NoEpilogue T; };
+template <> struct EpiArg<1> { typedef RotationDivision T; };
+template <> struct EpiArg<4> { typedef OutputAssembly T; };
 constexpr int CONTIG_THREADS = 128, CONTIG_WARPS = CONTIG_THREADS / 32;
 // Forward launches of up to that many chunks: see ntt_contig_short.  Plain forward launches over 6 primes of 40 bits, one of 50 and
 // one of 60 (N = 2^15), with 4 and with 8 points a thread: 7168 chunks 15.1 and 15.0 us, 10240 19.0 and 18.4, 13312 22.8 and 21.3,
@@ -795,7 +801,7 @@ __device__ __forceinline__ void contig_forward_far(const T* gsrc, u32 slice, int
 // (THREADS: see contig_forward_far; the inverse pass always has 64)
 template <bool FWD, int EPI, int PATH, bool TILED, int THREADS>
 __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B, u64* sm_raw, u32 o, u32 m, u32 mod,
-                                            u32 chunk, int lane, const RotBatch& rb, const ModDownEpilogue& epi) {
+                                            u32 chunk, int lane, const typename EpiArg<EPI>::T& epi) {
     typedef typename Elem<PATH>::T T;
     constexpr int LEN = 1 << LOG_C;
     T* sm = (T*)sm_raw;
@@ -839,58 +845,18 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
             // the epilogue's operands do not depend on the transform: ask for them before the last butterflies
             u64 uu[4] = {0, 0, 0, 0}, cc[4] = {0, 0, 0, 0};
             u32 pp[4] = {0, 0, 0, 0};
-            if (EPI == 2) {
-                const u32 pp_out = o >> 1, comp = o & 1, ip = mod, nb = R.r + 1;
-                const size_t n = (size_t)chunk * LEN + 4 * s;
-                // three rotations at a time: their permutation entries are requested together, then all the words they
-                // point at, so that a group costs two round trips instead of two per rotation
-                for (u32 j0 = 0; j0 < epi.n_sum; j0 += 3) {
-                    uint4 pv[3];
-                    u64 uv[3][4], cv[3][4];
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h < epi.n_sum) pv[h] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + h] * R.N + n);
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h) {
-                        if (j0 + h >= epi.n_sum) continue;
-                        const size_t rot = (size_t)(j0 + h) * epi.n_out + pp_out;
-                        const u64* up = epi.u + ((rot * 2 + comp) * nb + ip) * R.N;
-                        uv[h][0] = __ldg(up + pv[h].x); uv[h][1] = __ldg(up + pv[h].y);
-                        uv[h][2] = __ldg(up + pv[h].z); uv[h][3] = __ldg(up + pv[h].w);
-                        if (comp == 0) {
-                            const u64* cp = epi.c0_base + rot * epi.c0_stride + (size_t)ip * R.N;
-                            cv[h][0] = __ldg(cp + pv[h].x); cv[h][1] = __ldg(cp + pv[h].y);
-                            cv[h][2] = __ldg(cp + pv[h].z); cv[h][3] = __ldg(cp + pv[h].w);
-                        }
-                    }
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h) {
-                        if (j0 + h >= epi.n_sum) continue;
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            uu[w] = add_mod(uu[w], uv[h][w], q);
-                            if (comp == 0) cc[w] = add_mod(cc[w], cv[h][w], q);
-                        }
-                    }
-                }
-            }
-            if (EPI == 3) {         // plain division: only the inner sum's residue is needed
-                const u64* up = epi.u + ((size_t)o * (R.r + 1) + mod) * R.N + (size_t)chunk * LEN + 4 * s;
-                const ulonglong2 u0 = *(const ulonglong2*)up, u1 = *(const ulonglong2*)(up + 2);
-                uu[0] = u0.x; uu[1] = u0.y; uu[2] = u1.x; uu[3] = u1.y;
-            }
-            if (EPI == 1) {
+            if constexpr (EPI == 1) {
                 const u32 rot = o >> 1, comp = o & 1, ip = mod, nb = R.r + 1;
                 const size_t n = (size_t)chunk * LEN + 4 * s;
-                const u64* up = epi.u + ((size_t)o * nb + ip) * R.N + n;
+                const u64* up = epi.e.u + ((size_t)o * nb + ip) * R.N + n;
                 const ulonglong2 u0 = *(const ulonglong2*)up, u1 = *(const ulonglong2*)(up + 2);
                 uu[0] = u0.x; uu[1] = u0.y; uu[2] = u1.x; uu[3] = u1.y;
                 if (comp == 0) {
-                    const u64* cp = epi.c0_base + (size_t)rb.c0[rot] * epi.c0_stride + (size_t)ip * R.N + n;
+                    const u64* cp = epi.e.c0_base + (size_t)epi.rb.c0[rot] * epi.e.c0_stride + (size_t)ip * R.N + n;
                     const ulonglong2 c0 = *(const ulonglong2*)cp, c1 = *(const ulonglong2*)(cp + 2);
                     cc[0] = c0.x; cc[1] = c0.y; cc[2] = c1.x; cc[3] = c1.y;
                 }
-                const uint4 pv = *(const uint4*)(epi.pinv + (size_t)rb.key[rot] * R.N + n);
+                const uint4 pv = *(const uint4*)(epi.e.pinv + (size_t)epi.rb.key[rot] * R.N + n);
                 pp[0] = pv.x; pp[1] = pv.y; pp[2] = pv.z; pp[3] = pv.w;
             }
             set_butterflies<2, true, PATH, false>(e, tw, 64u * mult + s, c);
@@ -911,27 +877,9 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 }
                 continue;
             }
-            if (EPI == 2) {
-                const u32 pp_out = o >> 1, comp = o & 1, ip = mod, r = R.r;
-                u64* op = epi.out_base + (size_t)pp_out * epi.out_stride + ((size_t)comp * r + ip) * R.N + (size_t)chunk * LEN + 4 * s;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    v4[i] = add_mod(mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[ip], R.pinvs[ip], q), cc[i], q);
-                ((ulonglong2*)op)[0] = make_ulonglong2(v4[0], v4[1]);
-                ((ulonglong2*)op)[1] = make_ulonglong2(v4[2], v4[3]);
-                continue;
-            }
-            if (EPI == 3) {
-                u64* op = epi.out_base + (size_t)o * epi.out_stride + (size_t)mod * R.N + (size_t)chunk * LEN + 4 * s;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v4[i] = mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[mod], R.pinvs[mod], q);
-                ((ulonglong2*)op)[0] = make_ulonglong2(v4[0], v4[1]);
-                ((ulonglong2*)op)[1] = make_ulonglong2(v4[2], v4[3]);
-                continue;
-            }
-            if (EPI == 1) {
+            if constexpr (EPI == 1) {
                 const u32 rot = o >> 1, comp = o & 1, ip = mod, r = R.r;
-                u64* op = epi.out_base + (size_t)rb.out[rot] * epi.out_stride + ((size_t)comp * r + ip) * R.N;
+                u64* op = epi.e.out_base + (size_t)epi.rb.out[rot] * epi.e.out_stride + ((size_t)comp * r + ip) * R.N;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     u64 v = mul_shoup(sub_mod(uu[i], v4[i], q), R.pinv[ip], R.pinvs[ip], q);
@@ -985,86 +933,55 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
         for (int it = 0; it < 64 / THREADS; ++it) {
             const int s = lane + 32 * it;
             u64 v4[4];
-            if constexpr (EPI == 2) {   // the residues of this output's giant rotations, each read through its rotation, summed
-                const u32 pp_out = o >> 1, comp = o & 1, nb = R.r + 1;
+            if constexpr (EPI == 4) {   // see OutputAssembly
+                const u32 g1 = epi.g1, rows = epi.ext ? R.r + 1 : R.r, nu = epi.n_u();
                 const size_t n = (size_t)chunk * LEN + 4 * s;
-                v4[0] = v4[1] = v4[2] = v4[3] = 0;
-                // three rotations at a time: their permutation entries are requested together, then all the words they
-                // point at, so that a group costs two round trips instead of two per rotation (these launches are a few
-                // polynomials only: latency is all they cost)
-                for (u32 j0 = 0; j0 < epi.n_sum; j0 += 3) {
-                    uint4 pv[3];
-                    u64 uv[3][4];
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h < epi.n_sum) pv[h] = *(const uint4*)(epi.perm + (size_t)rb.key[j0 + h] * R.N + n);
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h) {
-                        if (j0 + h >= epi.n_sum) continue;
-                        const u64* up = epi.u + ((((size_t)(j0 + h) * epi.n_out + pp_out) * 2 + comp) * nb + mod) * R.N;
-                        uv[h][0] = __ldg(up + pv[h].x); uv[h][1] = __ldg(up + pv[h].y);
-                        uv[h][2] = __ldg(up + pv[h].z); uv[h][3] = __ldg(up + pv[h].w);
-                    }
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h) {
-                        if (j0 + h >= epi.n_sum) continue;
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) v4[w] = add_mod(v4[w], uv[h][w], q);
-                    }
-                }
-            } else if constexpr (EPI == 4) {   // output assembly in the extended basis (see ModDownEpilogue::assemble)
-                const u32 nb = R.r + 1, g1 = epi.n_sum, mt = m - B.tail_m;
-                const size_t n = (size_t)chunk * LEN + 4 * s;
-                u32 comp = 0, ju = 0, jc_lo = 1, jc_hi = 0;    // u-terms of giant steps 1..ju, rotated c0 parts of jc_lo..jc_hi
+                u32 comp = 0, ju_lo = 1, ju_hi = 0, jc_lo = 1, jc_hi = 0;     // u of giant steps ju_lo..ju_hi, rotated c0 parts of jc_lo..jc_hi
                 bool ident = false;
-                if (mod < R.r) { comp = m / R.r; ident = true; ju = g1; if (comp == 0) jc_hi = g1; }
-                else if (mt < 2) { comp = mt; ju = g1; }
-                else if (mt < 4) { comp = mt - 2; ident = true; }
-                else { jc_lo = jc_hi = mt - 3; }
-                v4[0] = v4[1] = v4[2] = v4[3] = 0;
-                if (ident) {
-                    const u64* ap = epi.aext + (size_t)o * epi.aext_stride + ((size_t)comp * nb + mod) * R.N + n;
-                    const ulonglong2 a = *(const ulonglong2*)ap, b = *(const ulonglong2*)(ap + 2);
-                    v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
+                if (mod < R.r) {
+                    comp = m / R.r; ident = true; ju_hi = g1;
+                    if (comp == 0) jc_hi = g1;
+                } else if (m - B.tail_m < nu) {
+                    const u32 mt = m - B.tail_m;
+                    comp = mt & 1;
+                    if (epi.each) ju_lo = ju_hi = 1 + mt / 2;
+                    else ju_hi = g1;
+                } else {
+                    const u32 mt = m - B.tail_m - nu;
+                    if (mt < 2) { comp = mt; ident = true; }
+                    else jc_lo = jc_hi = mt - 1;
                 }
+                v4[0] = v4[1] = v4[2] = v4[3] = 0;
                 // (the producers stored every rotated term through its rotation already: plain loads; the words of
                 // three giant steps are requested together)
-                const u64* ub = epi.u + (((size_t)o * 2 + comp) * nb + mod) * R.N + n;          // giant step 1
-                const size_t u_step = (size_t)epi.n_out * 2 * nb * R.N;
-                for (u32 j0 = 1; j0 <= ju; j0 += 3) {
-                    ulonglong2 a2[3], b2[3];
+                auto add_terms = [&](const u64* base, size_t step, u32 count) {
+                    for (u32 j0 = 0; j0 < count; j0 += 3) {
+                        ulonglong2 a2[3], b2[3];
 #pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h <= ju) {
-                            const u64* up = ub + (size_t)(j0 + h - 1) * u_step;
-                            a2[h] = *(const ulonglong2*)up;
-                            b2[h] = *(const ulonglong2*)(up + 2);
-                        }
+                        for (u32 h = 0; h < 3; ++h)
+                            if (j0 + h < count) {
+                                const u64* p = base + (size_t)(j0 + h) * step;
+                                a2[h] = *(const ulonglong2*)p;
+                                b2[h] = *(const ulonglong2*)(p + 2);
+                            }
 #pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h <= ju) {
-                            v4[0] = add_mod(v4[0], a2[h].x, q); v4[1] = add_mod(v4[1], a2[h].y, q);
-                            v4[2] = add_mod(v4[2], b2[h].x, q); v4[3] = add_mod(v4[3], b2[h].y, q);
-                        }
+                        for (u32 h = 0; h < 3; ++h)
+                            if (j0 + h < count) {
+                                v4[0] = add_mod(v4[0], a2[h].x, q); v4[1] = add_mod(v4[1], a2[h].y, q);
+                                v4[2] = add_mod(v4[2], b2[h].x, q); v4[3] = add_mod(v4[3], b2[h].y, q);
+                            }
+                    }
+                };
+                const u64* ap = epi.a + (size_t)o * epi.a_stride + n;
+                if (ident) add_terms(ap + ((size_t)comp * rows + mod) * R.N, 0, 1);
+                const size_t c_step = (size_t)epi.n_out * epi.a_stride;
+                add_terms(ap + (size_t)mod * R.N + jc_lo * c_step, c_step, jc_hi + 1 - jc_lo);
+                if (!epi.ext && mod < R.r) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v4[i] = times_p(R, mod, v4[i]);
                 }
-                const u64* cb = epi.aext + (size_t)o * epi.aext_stride + (size_t)mod * R.N + n;  // inner sum (0, p), c0
-                const size_t c_step = (size_t)epi.n_out * epi.aext_stride;
-                for (u32 j0 = jc_lo; j0 <= jc_hi; j0 += 3) {
-                    ulonglong2 a2[3], b2[3];
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h <= jc_hi) {
-                            const u64* cp = cb + (size_t)(j0 + h) * c_step;
-                            a2[h] = *(const ulonglong2*)cp;
-                            b2[h] = *(const ulonglong2*)(cp + 2);
-                        }
-#pragma unroll
-                    for (u32 h = 0; h < 3; ++h)
-                        if (j0 + h <= jc_hi) {
-                            v4[0] = add_mod(v4[0], a2[h].x, q); v4[1] = add_mod(v4[1], a2[h].y, q);
-                            v4[2] = add_mod(v4[2], b2[h].x, q); v4[3] = add_mod(v4[3], b2[h].y, q);
-                        }
-                }
+                const size_t u_step = (size_t)epi.n_out * 2 * (R.r + 1) * R.N;
+                add_terms(epi.u + (((size_t)o * 2 + comp) * (R.r + 1) + mod) * R.N + n + (ju_lo - 1) * u_step, u_step, ju_hi + 1 - ju_lo);
             } else if constexpr (TILED) {  // read back from the tile-major plaintext cache
                 const unsigned char* stage = tile_stage + (size_t)it * tile_step;
                 const u32 at = tile_at, fmt = tile_fmt;
@@ -1139,12 +1056,9 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
 }
 
 // grid: x = group of 2^log_wo outer indices, y = slot m, z = group of chunks.
-// (the per-output forms run on a few polynomials per launch and hold the operands of three rotations at once: they
-// trade resident blocks for registers)
 template <int EPI, bool TILED>
-__global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 ? 5 : 8) ntt_contig(const RingDev R, const PolyBatch B,
-                                                                       u32 n_outer, u32 log_wo, const RotBatch rb,
-                                                                       const ModDownEpilogue epi) {
+__global__ void __launch_bounds__(CONTIG_THREADS, 8) ntt_contig(const RingDev R, const PolyBatch B, u32 n_outer, u32 log_wo,
+                                                              const typename EpiArg<EPI>::T epi) {
     __shared__ __align__(128) u64 sm_all[CONTIG_WARPS << LOG_C];
     grid_dependency_enter();
     const u32 m = slot_of_block(blockIdx.y, B.n_m);
@@ -1157,9 +1071,9 @@ __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 ? 5 : 8) ntt_contig(c
     if (own_prime(R, B, o, mod)) return;
     u64* sm = sm_all + (warp << LOG_C);
     const int path = path_of(R, mod);
-    if (path == PATH_DP) contig_body<true, EPI, PATH_DP, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else if (path == PATH_WIDE) contig_body<true, EPI, PATH_WIDE, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else contig_body<true, EPI, PATH_INT, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    if (path == PATH_DP) contig_body<true, EPI, PATH_DP, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, epi);
+    else if (path == PATH_WIDE) contig_body<true, EPI, PATH_WIDE, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, epi);
+    else contig_body<true, EPI, PATH_INT, TILED, 32>(R, B, sm, o, m, mod, chunk, lane, epi);
 }
 
 // The same with a block of 64 threads per chunk, 4 points a thread: the inverse pass, and forward launches too small to run
@@ -1167,9 +1081,11 @@ __global__ void __launch_bounds__(CONTIG_THREADS, EPI == 2 ? 5 : 8) ntt_contig(c
 // chunks and all inverse ones: the calls of a 0.6B layer 1362 -> 1327 us, a 64 x 64 product on a ring of 2^12 70 -> 61 us.
 // Inverse launches of a LLaMA-3-8B layer, up to 36000 chunks: 549 -> 477 us.  Forward launches of 200000 chunks: 783 us with
 // 8 points, 938 us with 4, for an exchange through shared memory more.)  grid: x = outer index, y = slot m, z = chunk.
+// (the output assembly runs on a few polynomials per launch and holds the operands of three giant steps at once: it trades
+// resident blocks for registers)
 template <bool FWD, int EPI, bool TILED>
-__global__ void __launch_bounds__(64, EPI == 2 || EPI == 4 ? 10 : 16) ntt_contig_short(const RingDev R, const PolyBatch B, const RotBatch rb,
-                                                                                    const ModDownEpilogue epi) {
+__global__ void __launch_bounds__(64, EPI == 4 ? 10 : 16) ntt_contig_short(const RingDev R, const PolyBatch B,
+                                                                        const typename EpiArg<EPI>::T epi) {
     __shared__ __align__(128) u64 sm[1 << LOG_C];
     grid_dependency_enter();
     const u32 m = slot_of_block(blockIdx.y, B.n_m), o = blockIdx.x, chunk = blockIdx.z;
@@ -1177,9 +1093,9 @@ __global__ void __launch_bounds__(64, EPI == 2 || EPI == 4 ? 10 : 16) ntt_contig
     if (EPI == 5 && m > R.r) mod = o % R.r;         // (component 0, in the prime it is a residue of)
     if (FWD && own_prime(R, B, o, mod)) return;
     const int path = path_of(R, mod), lane = threadIdx.x;
-    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
-    else contig_body<FWD, EPI, PATH_INT, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, rb, epi);
+    if (path == PATH_DP) contig_body<FWD, EPI, PATH_DP, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, epi);
+    else if (path == PATH_WIDE) contig_body<FWD, EPI, PATH_WIDE, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, epi);
+    else contig_body<FWD, EPI, PATH_INT, TILED, 64>(R, B, sm, o, m, mod, chunk, lane, epi);
 }
 
 // Key-switch products (Sec. 4.2 "key-switching primitives"): the contiguous pass of the digits' transforms and their inner
@@ -1395,43 +1311,37 @@ static cudaError_t launch_strided(const RingHost& ring, const PolyBatch& B, u32 
     return cudaGetLastError();
 }
 
-template <bool FWD>
+template <bool FWD, int EPI = 0>
 static cudaError_t launch_contig(const RingHost& ring, const PolyBatch& B_in, u32 n_polys, cudaStream_t stream,
-                                 const RotBatch* rb = nullptr, const ModDownEpilogue* epi = nullptr) {
+                                 const typename EpiArg<EPI>::T& epi = {}) {
     if (n_polys == 0) return cudaSuccess;
     ProfScope prof(ring.prof, FWD ? CAT_NTT_FWD_CONTIG : CAT_NTT_INV_CONTIG, stream);
     PolyBatch B = B_in;
     const u32 n_outer = n_polys / B.n_m;
     set_magics(B, n_outer);
     const u32 chunks = ring.dev.N >> LOG_C;
-    static const RotBatch no_rb = {};
-    static const ModDownEpilogue no_epi = {};
-    const RotBatch& rots = rb ? *rb : no_rb;
-    const ModDownEpilogue& ep = epi ? *epi : no_epi;
     // the four warps of a block take the same chunk of four polynomials where the batch has enough of them (one fetch of the
     // chunk's twiddles serves them), else of two, else neighbouring chunks
     const u32 log_wo = n_outer % 4 == 0 || n_outer >= 16 ? 2u : n_outer % 2 == 0 || n_outer >= 7 ? 1u : 0u;
     const u32 per = CONTIG_WARPS >> log_wo;
     const dim3 grid((n_outer + (1u << log_wo) - 1) >> log_wo, B.n_m, (chunks + per - 1) / per), grid_short(n_outer, B.n_m, chunks);
-    auto go = [&](auto epi_c, auto tiled_c) {
-        constexpr int EPI = decltype(epi_c)::value;
+    auto go = [&](auto tiled_c) {
         constexpr bool TILED = decltype(tiled_c)::value;
         if constexpr (FWD) {
             if ((size_t)n_polys * chunks > CONTIG_SHORT_CHUNKS) {
-                launch_dependent(ring, ntt_contig<EPI, TILED>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, rots, ep);
+                launch_dependent(ring, ntt_contig<EPI, TILED>, grid, dim3(CONTIG_THREADS), 0, stream, ring.dev, B, n_outer, log_wo, epi);
                 return;
             }
         }
-        launch_dependent(ring, ntt_contig_short<FWD, EPI, TILED>, grid_short, dim3(64), 0, stream, ring.dev, B, rots, ep);
+        launch_dependent(ring, ntt_contig_short<FWD, EPI, TILED>, grid_short, dim3(64), 0, stream, ring.dev, B, epi);
     };
-    const std::integral_constant<bool, false> plain_store;
-    if (FWD && epi && epi->plain) go(std::integral_constant<int, FWD ? 3 : 0>(), plain_store);
-    else if (FWD && B.ingest) go(std::integral_constant<int, FWD ? 5 : 0>(), plain_store);
-    else if (!FWD && epi && epi->assemble) go(std::integral_constant<int, FWD ? 0 : 4>(), plain_store);
-    else if (epi && epi->n_sum) go(std::integral_constant<int, 2>(), plain_store);
-    else if (FWD && epi) go(std::integral_constant<int, FWD ? 1 : 0>(), plain_store);
-    else if (B.tile_ptr) go(std::integral_constant<int, 0>(), std::integral_constant<bool, true>());
-    else go(std::integral_constant<int, 0>(), plain_store);
+    if constexpr (EPI == 0) {
+        if (B.tile_ptr) {
+            go(std::integral_constant<bool, true>());
+            return cudaGetLastError();
+        }
+    }
+    go(std::integral_constant<bool, false>());
     return cudaGetLastError();
 }
 
@@ -1455,7 +1365,7 @@ cudaError_t ntt_forward_ingest(const RingHost& ring, const PolyBatch& B0, u32 n_
     cudaError_t e = launch_strided<true, LOAD_INGEST>(ring, B, n_in * 2 * r * B.n_m, stream);
     if (e != cudaSuccess) return e;
     B.n_m = r + 2;
-    return launch_contig<true>(ring, B, n_in * r * B.n_m, stream);
+    return launch_contig<true, 5>(ring, B, n_in * r * B.n_m, stream);
 }
 
 cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
@@ -1463,7 +1373,7 @@ cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_
     const u32 n_polys = n_outer * B.n_m;
     cudaError_t e = launch_strided<true, LOAD_CENTRED>(ring, B, n_polys, stream);
     if (e != cudaSuccess) return e;
-    return launch_contig<true>(ring, B, n_polys, stream, &rb, &epi);
+    return launch_contig<true, 1>(ring, B, n_polys, stream, RotationDivision{epi, rb});
 }
 
 // Forward transform whose final store is permuted: polynomial (o, m) ends up at
@@ -1549,22 +1459,25 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
     return launch_contig_inner<2>(ring, B_in, rb, keys, u, xext, pinv, stream);
 }
 
-cudaError_t ntt_inverse_gathersum(const RingHost& ring, const PolyBatch& B, u32 n_outer, const RotBatch& rb,
-                                  const ModDownEpilogue& epi, cudaStream_t stream) {
+cudaError_t ntt_inverse_assembly(const RingHost& ring, const PolyBatch& B, u32 n_outer, const OutputAssembly& as, cudaStream_t stream) {
     const u32 n_polys = n_outer * B.n_m;
-    cudaError_t e = launch_contig<false>(ring, B, n_polys, stream, &rb, &epi);
+    cudaError_t e = launch_contig<false, 4>(ring, B, n_polys, stream, as);
     if (e != cudaSuccess) return e;
     return launch_strided<false, LOAD_PLAIN>(ring, B, n_polys, stream);
 }
 
-// Last step of the output assembly in the extended basis: the inverse transforms above left, per output p and
+// Last step of the output assembly: the inverse transforms above left, per output p and
 // component, the sum of all terms modulo every q_i (in ct) and each separately rounded term's residue modulo P as a
-// centred lift plus 2^59 (in T, n_t polynomials per output, indexed as ModDownEpilogue::assemble lists them):
+// centred lift plus 2^59 (in T, n_t polynomials per output, indexed as OutputAssembly lists them):
 //   ct[p][comp][i][n] = (ct[p][comp][i][n] - sum_terms t_term[n]) * P^{-1}  (mod q_i)
 // low non-null: the rescale (Sec. 2.1) follows in the same thread, which holds all residues of its coefficient: the
 // result goes to low[p][comp][r-1][N] as c'_i = (c_i - centred(c_{r-1})) * q_{r-1}^{-1} and ct only held the sums.
+// the k-th of component comp's terms, as the polynomials of T are numbered, and how many there are
+__device__ __forceinline__ u32 assembly_term(u32 k, u32 comp, u32 n_u) { return 2 * k < n_u ? comp + 2 * k : 2 * k == n_u ? n_u + comp : n_u + 1 + k - n_u / 2; }
+__device__ __forceinline__ u32 assembly_terms(u32 comp, u32 n_u, u32 n_t) { return n_u / 2 + (n_t == n_u ? 0u : comp ? 1u : n_t - n_u - 1); }
+
 __global__ void __launch_bounds__(128, 8) finish_division_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
-                                                              const u64* __restrict__ T, u32 n_t, const RescaleConsts rc,
+                                                              const u64* __restrict__ T, u32 n_u, u32 n_t, const RescaleConsts rc,
                                                               u64* __restrict__ low) {
     grid_dependency_enter();
     const u32 n = blockIdx.x * 128 + threadIdx.x;
@@ -1575,14 +1488,13 @@ __global__ void __launch_bounds__(128, 8) finish_division_kernel(const RingDev R
 #pragma unroll
     for (int i = 0; i < MAX_MODULI; ++i)
         if ((u32)i < R.r) v[i] = cp[(size_t)i * R.N];
-    // this component's terms: polynomials comp, comp + 2 and, for component 0, 4 .. n_t - 1.  Their centred values are
-    // added as integers, eight at a time (each is below 2^59 in magnitude), and the sum is reduced once per prime
-    const u32 nt = comp == 0 ? n_t - 2 : 2u;
+    // the centred values of this component's terms are added as integers, eight at a time (each is below 2^59 in magnitude),
+    // and the sum is reduced once per prime
+    const u32 nt = assembly_terms(comp, n_u, n_t);
     for (u32 k0 = 0; k0 < nt; k0 += 8) {
         i64 S = 0;
         for (u32 k = k0; k < nt && k < k0 + 8; ++k) {
-            const u32 m = k < 2 ? comp + 2 * k : k + 2;
-            S += (i64)(tp[(size_t)m * R.N] - (1ull << 59));
+            S += (i64)(tp[(size_t)assembly_term(k, comp, n_u) * R.N] - (1ull << 59));
         }
         const bool neg = S < 0;
         const u64 a = neg ? (u64)(-S) : (u64)S;
@@ -1635,7 +1547,7 @@ __device__ __forceinline__ double fp_times_const(double x, bool wide, double w, 
 }
 
 __global__ void __launch_bounds__(128, 8) finish_division_fp_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
-                                                                 const u64* __restrict__ T, u32 n_t, const RescaleConsts rc,
+                                                                 const u64* __restrict__ T, u32 n_u, u32 n_t, const RescaleConsts rc,
                                                                  u64* __restrict__ low) {
     grid_dependency_enter();
     const u32 n = blockIdx.x * 128 + threadIdx.x;
@@ -1646,12 +1558,11 @@ __global__ void __launch_bounds__(128, 8) finish_division_fp_kernel(const RingDe
 #pragma unroll
     for (int i = 0; i < MAX_MODULI; ++i)
         if ((u32)i < R.r) v[i] = u2d(cp[(size_t)i * R.N]);
-    const u32 nt = comp == 0 ? n_t - 2 : 2u;
+    const u32 nt = assembly_terms(comp, n_u, n_t);
     for (u32 k0 = 0; k0 < nt; k0 += 8) {
         i64 S = 0;
         for (u32 k = k0; k < nt && k < k0 + 8; ++k) {
-            const u32 m = k < 2 ? comp + 2 * k : k + 2;
-            S += (i64)(tp[(size_t)m * R.N] - (1ull << 59));
+            S += (i64)(tp[(size_t)assembly_term(k, comp, n_u) * R.N] - (1ull << 59));
         }
         const i64 s_hi = S >> 30;                               // |s_hi| < 2^33
         const double lo = u2d((u64)(S & ((1ll << 30) - 1)));
@@ -1694,7 +1605,7 @@ __global__ void __launch_bounds__(128, 8) finish_division_fp_kernel(const RingDe
         }
 }
 
-cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_t, u32 n_out,
+cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_u, u32 n_t, u32 n_out,
                             cudaStream_t stream, const RescaleConsts* rc, u64* low) {
     ProfScope prof(ring.prof, CAT_DIVIDE, stream);
     RescaleConsts none;
@@ -1704,11 +1615,11 @@ cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, 
     if (rc && ring.q[ring.dev.r - 1] >= (1ull << 46)) fp = false;
     if (fp) {
         launch_dependent(ring, finish_division_fp_kernel, dim3(ring.dev.N / 128, n_out * 2), dim3(128), 0, stream, ring.dev,
-                         ct, ct_stride, T, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
+                         ct, ct_stride, T, n_u, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
         return cudaGetLastError();
     }
     launch_dependent(ring, finish_division_kernel, dim3(ring.dev.N / 128, n_out * 2), dim3(128), 0, stream, ring.dev, ct,
-                     ct_stride, T, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
+                     ct_stride, T, n_u, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
     return cudaGetLastError();
 }
 

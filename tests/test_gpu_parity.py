@@ -636,6 +636,19 @@ def test_wide_inputs_take_no_more_scratch_than_the_batched_rotations(n_primes, n
         g.close()
 
 
+@pytest.mark.parametrize("modes", [{}, dict(hoist="double"), dict(moddown="per_output")], ids=["plain", "double_hoist", "per_output"])
+@pytest.mark.parametrize("plan_t,shape", [
+    ((128, 1, 2, 64), (130, 128)),          # 63 giant steps, two outputs: launches of several batches, 2 * 63 separate terms
+    ((128, 1, 1, 128), (128, 100)),         # more giant steps than a launch has rotations (refused with one division per output)
+    ((64, 8, 8, 1), (64, 64)),              # none: nothing to assemble, or the inner sums alone
+])
+def test_output_assembly_for_few_and_many_giant_steps(plan_t, shape, modes):
+    if plan_t[3] > 65 and "moddown" in modes:
+        return
+    par = ckks.Params(1 << 10, ckks.find_primes(1 << 40, 2 << 10, 3), ckks.find_primes(1 << 60, 2 << 10, 1)[0], 2.0 ** 40)
+    run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 19, 1e-2, "giants", tight=1e-2)
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
