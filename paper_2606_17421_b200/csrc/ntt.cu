@@ -128,7 +128,7 @@ __device__ __forceinline__ double load_src_fp(const void* src, size_t idx, const
 // How a modulus is transformed.
 //   PATH_DP    primes below 2^41: signed integer-valued doubles, reduced lazily
 //   PATH_WIDE  primes from 2^41 up to 2^50: integer-valued doubles in [0, 4q) (forward) or [0, 2q) (inverse)
-//   PATH_INT   larger primes: 64-bit integers, Harvey's lazy butterflies with Shoup products, the same ranges
+//   PATH_INT   larger primes: 64-bit integers below 16q (forward) or 4q (inverse), Shoup products with a short quotient
 enum Path : int { PATH_INT = 0, PATH_WIDE = 1, PATH_DP = 2 };
 __device__ __forceinline__ int path_of(const RingDev& R, u32 mod) { return !R.fp_ok[mod] ? PATH_INT : (R.q[mod] >> 41) ? PATH_WIDE : PATH_DP; }
 template <int PATH> struct Elem { typedef double T; };
@@ -139,7 +139,21 @@ __device__ __forceinline__ void from_u64(double& dst, u64 v) { dst = u2d(v); }
 struct ModConsts {
     u64 q;
     double qd, qinv;
+    u32 mu;             // floor(2^64 / q), PATH_INT (q above 2^50: below 2^14)
+    __device__ __forceinline__ ModConsts(const RingDev& R, u32 mod) : q(R.q[mod]), qd(R.qd[mod]), qinv(R.qinv_d[mod]), mu((u32)R.mu[mod]) {}
 };
+
+// x * w - h q for any 64-bit x and a constant w < q < 2^60 with companion ws = floor(w 2^64 / q): h is the high word of x * ws short
+// of what its low parts would carry in, i.e. by less than 3, so the result is congruent to x * w and in [0, 4q).  (Three wide
+// multiplications instead of four and their carries.)
+__device__ __forceinline__ u64 mul_shoup_short(u64 x, u64 w, u64 ws, u64 q) {
+    const u32 x0 = (u32)x, x1 = (u32)(x >> 32), s0 = (u32)ws, s1 = (u32)(ws >> 32);
+    const u64 h = (u64)x1 * s1 + __umulhi(x1, s0) + __umulhi(x0, s1);
+    return x * w - h * q;
+}
+// any 64-bit x (so x < 16q) minus a multiple of q, q above 2^50: in [0, 3q).  The quotient floor(x_hi mu / 2^32) is short of x / q
+// by less than 1 + 2^-18 + x / 2^64.
+__device__ __forceinline__ u64 reduce_16q(u64 x, const ModConsts& c) { return x - (u64)__umulhi((u32)(x >> 32), c.mu) * c.q; }
 
 // 32 bytes at once (the widest global access of sm_100)
 __device__ __forceinline__ void ldg4(const double* p, double& a, double& b, double& c, double& d) {
@@ -182,6 +196,12 @@ __device__ __forceinline__ void load_twiddles(const double* tab, u32 idx, double
 // keeps Harvey's invariant [0, 4q) with one conditional subtraction: (X, Y) -> (X~ + T, X~ - T + 2q), X~ = X reduced
 // below 2q, T = Y*w + q in (0.25q, 1.75q); the inverse is (a, b) -> (a + b reduced below 2q, (a - b + 2q)*w + q in
 // (0.25q, 1.75q)): values in [0, 2q).
+// PATH_INT: products come back below 4q (see mul_shoup_short).  Forward, (X, Y) -> (X + T, X - T + 4q): any 64-bit Y will do, X
+// grows by 4q per stage, and where a group starts the X of its first stage are brought below 3q: K <= 3 stages end below 15q.
+// Inverse, (a, b) -> (a + b, (a - b + 4q) w): every second stage, and the last of a group, brings its sums below 3q; the stage
+// before leaves them below 8q, so that its successor's differences take an offset of 8q.
+// (768 -> 2304 on 2^13, two of whose five moduli are 60-bit primes: 234.2 us with products below 2q, which a conditional
+// subtraction per butterfly keeps, 230.9 us like this; 64 x 64 on 2^12: 59.8 and 59.4 us.)
 template <int ST, int K, bool FWD, int PATH, bool SM, int OFF, typename T>
 __device__ __forceinline__ void stage_butterflies(T (&e)[8], const void* __restrict__ tab, u32 base, const ModConsts& c) {
     constexpr int d = (1 << K) >> (ST + 1);
@@ -209,7 +229,6 @@ __device__ __forceinline__ void stage_butterflies(T (&e)[8], const void* __restr
         }
     } else {
         const double q2d = __dadd_rn(c.qd, c.qd);
-        const u64 q = c.q, q2 = 2 * c.q;
 #pragma unroll
         for (int sub = 0; sub < (1 << ST); ++sub) {
             const ulonglong2 wb = SM ? ((const ulonglong2*)tab)[idx + sub] : __ldg((const ulonglong2*)tab + idx + sub);
@@ -232,17 +251,15 @@ __device__ __forceinline__ void stage_butterflies(T (&e)[8], const void* __restr
                         e[i + d] = __dadd_rn(fp_mul_centred(__dadd_rn(__dsub_rn(a, b), q2d), w, wq, c.qd), c.qd);
                     }
                 } else if (FWD) {
-                    u64 x = e[i];
-                    if (x >= q2) x -= q2;
-                    const u64 t = mul_shoup_lazy(e[i + d], wb.x, wb.y, q);
+                    const u64 x = ST == 0 ? reduce_16q(e[i], c) : e[i];
+                    const u64 t = mul_shoup_short(e[i + d], wb.x, wb.y, c.q);
                     e[i] = x + t;
-                    e[i + d] = x - t + q2;
+                    e[i + d] = x - t + 4 * c.q;
                 } else {
+                    constexpr int POS = K - 1 - ST;             // (stages of the group before this one)
                     const u64 a = e[i], b = e[i + d];
-                    u64 s2 = a + b;
-                    if (s2 >= q2) s2 -= q2;
-                    e[i] = s2;
-                    e[i + d] = mul_shoup_lazy(a - b + q2, wb.x, wb.y, q);
+                    e[i] = POS % 2 == 1 || ST == 0 ? reduce_16q(a + b, c) : a + b;
+                    e[i + d] = mul_shoup_short(a - b + (POS % 2 == 1 ? 8 : 4) * c.q, wb.x, wb.y, c.q);
                 }
             }
         }
@@ -401,10 +418,7 @@ __device__ __forceinline__ void strided_body(const RingDev& R, const PolyBatch& 
     typedef typename Elem<PATH>::T T;
     constexpr int LEN = G::LEN, LANES = G::LANES, NT = G::NT, NG = n_groups(LOG_R);
     T* sm = (T*)sm_raw;
-    ModConsts c;
-    c.q = R.q[mod];
-    c.qd = R.qd[mod];
-    c.qinv = R.qinv_d[mod];
+    const ModConsts c(R, mod);
     u64* dst = nullptr;
     if constexpr (INGEST) {
         u32 o_hi, o_lo;
@@ -746,6 +760,7 @@ __device__ __forceinline__ u64 canonical(T x, const ModConsts& c, bool bits) {
         const double v = fp_canonical(x, c.qd, c.qinv);
         return bits ? (u64)__double_as_longlong(v) : d2u(v);
     } else {
+        x = reduce_16q(x, c);
         if (x >= 2 * c.q) x -= 2 * c.q;
         return x >= c.q ? x - c.q : x;
     }
@@ -805,10 +820,7 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
     typedef typename Elem<PATH>::T T;
     constexpr int LEN = 1 << LOG_C;
     T* sm = (T*)sm_raw;
-    ModConsts c;
-    c.q = R.q[mod];
-    c.qd = R.qd[mod];
-    c.qinv = R.qinv_d[mod];
+    const ModConsts c(R, mod);
     const u64 q = c.q;
     const void* tw = twiddle_table(R, FWD, PATH, mod);
     u64* dst = EPI == 5 && m > R.r ? B.tail_dst + (size_t)o * R.N : batch_dst<EPI == 4>(B, o, m);
@@ -1174,10 +1186,7 @@ ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const vo
     const u32 warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
     const int path = path_of(R, m);
-    ModConsts c;
-    c.q = R.q[m];
-    c.qd = R.qd[m];
-    c.qinv = R.qinv_d[m];
+    const ModConsts c(R, m);
     const bool dp = R.dp[m] != 0;
     if (threadIdx.x < cb * 2 && chunk0 + threadIdx.x / 2 < (N >> LOG_C)) {      // the first rotation's keys, on their way to L2
         const unsigned char* kp = key_tile(R, keys, (u32)rb.key[first], m, chunk0 * 2 + threadIdx.x);
