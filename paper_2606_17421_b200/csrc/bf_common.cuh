@@ -113,8 +113,8 @@ __device__ __forceinline__ double fp_centre(double v, double q, double qinv) {
     const double qh = __dsub_rn(__fma_rn(v, qinv, magic), magic);
     return __fma_rn(-qh, q, v);
 }
-// v mod q in [0, q) for a signed integer-valued |v| < 2^46, q < 2^41: (v + 1/2) / q is at least 2^-42 away from any integer,
-// which the errors of the product (2^-52 of at most 2^5 where v is within 32 q) do not bridge, so its floor is exact
+// v mod q in [0, q) for a signed integer-valued |v| < 2^50, q < 2^41: (v + 1/2) / q is at least 1 / (2q) away from any integer,
+// which the error of 1/q (2^-53 of at most 2^50 / q) does not bridge, so its floor is exact
 __device__ __forceinline__ double fp_canonical(double v, double q, double qinv) {
     const double magic = 6755399441055744.0;
     const double qh = __dsub_rn(__fma_rd(__dadd_rn(v, 0.5), qinv, magic), magic);
@@ -431,19 +431,19 @@ constexpr u32 LIMB_NARROW = 25, LIMB_WIDE = 30;
 // fma(a, b, h - h') is the part rounded away, an integer of magnitude at most 2^39; l collects those.  Exact while
 // |sum| < 2^91 and |l| < 2^53: 2048 terms.
 struct DpAcc {
-    double h = 7427640236712282150480740352.0;       // 1.5 * 2^92
+    double h = 7427640235712281649394745344.0;       // 1.5 * 2^92
     double l = 0.0;
     __device__ __forceinline__ void mac(double a, double b) {
         const double h2 = __fma_rn(a, b, h);
         l = __dadd_rn(l, __fma_rn(a, b, __dsub_rn(h, h2)));
         h = h2;
     }
-    // the sum modulo q in [0, q), as an integer-valued double: (h / 2^40) (2^40 mod q) + l, h / 2^40 below 2^51
-    __device__ __forceinline__ double reduce(double q, double qinv, double c40, double c40q) const {
-        const double hi = __dmul_rn(__dsub_rn(h, 7427640236712282150480740352.0), 9.094947017729282379150390625e-13);   // 2^-40
-        const double v = __dadd_rn(fp_mul_centred_signed(fp_centre(hi, q, qinv), c40, c40q, q), l);
-        const double r = fp_centre(v, q, qinv);
-        return r < 0.0 ? __dadd_rn(r, q) : r;
+    // the sum modulo q as an integer-valued double, (h / 2^40) (2^40 mod q) + l: within 0.54q plus 2^39 a term.  The product takes
+    // |h / 2^40| < 2^47, i.e. sums below 2^87: 128 products of residues below 2^40.  `many`: more than that, up to 2^91.
+    __device__ __forceinline__ double lazy(double q, double qinv, double c40, double c40q, bool many) const {
+        double hi = __fma_rn(h, 9.094947017729282379150390625e-13, -6755399441055744.0);       // (h - 1.5 * 2^92) 2^-40, exact
+        if (many) hi = fp_centre(hi, q, qinv);
+        return __dadd_rn(fp_mul_centred_signed(hi, c40, c40q, q), l);
     }
 };
 
@@ -543,7 +543,9 @@ template <>
 struct DigitDot<OP_DP> {
     DpAcc a;
     __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1) { a.mac(__hiloint2double((int)d.y, (int)d.x), __hiloint2double((int)k1, (int)k0)); }
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const { return d2u(a.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m])); }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const {
+        return d2u(fp_canonical(a.lazy(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m], false), R.qd[m], R.qinv_d[m]));
+    }
 };
 
 // One output pair of the key-switch inner product: digit j (d[j * ds]) times key words (2j, 2j + 1) (k[s * ks]) summed
@@ -569,10 +571,6 @@ struct KeyDot<OP_DP> {
         const double dd = __hiloint2double((int)d.y, (int)d.x);
         a0.mac(dd, __hiloint2double((int)k1, (int)k0));
         a1.mac(dd, __hiloint2double((int)l1, (int)l0));
-    }
-    __device__ __forceinline__ void reduce(const RingDev& R, u32 m, u64& v0, u64& v1) const {
-        v0 = d2u(a0.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));
-        v1 = d2u(a1.reduce(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m]));
     }
 };
 

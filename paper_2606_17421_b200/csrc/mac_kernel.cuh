@@ -19,6 +19,10 @@
 // time.  Loads go straight to registers: a stream that every thread consumes in the pattern it loads needs no staging, no
 // barriers and no producer; what hides the latency is the number of independent loads per thread (2r key words at a time;
 // two batches of 8 weights, three where they are packed) times resident warps.
+// Since issue slots come next, index arithmetic is done per warp where it can be, X is held as pairs of its two components (one
+// 16-byte read per weight), and what stays in the block is only reduced as far as its next use needs: the four products of a 0.6B
+// layer take 55 us less than with canonical residues, divisions for an item's place and an automorphism evaluated per
+// coefficient (the layer 1373 -> 1314 us, one of an 8B model 9430 -> 9087 us).
 #pragma once
 #include "bf_host.h"
 
@@ -26,12 +30,20 @@ namespace bf {
 
 constexpr int MAC_THREADS = 256;
 
-// position of the evaluation that an automorphism X -> X^gal moves to position n (and, with the inverse exponent, where
-// position n goes)
-__device__ __forceinline__ u32 automorphism_index(u32 n, u32 gal, u32 logN) {
-    const u32 e = 2u * (__brev(n) >> (32u - logN)) + 1u;
-    return __brev(((e * gal) & ((2u << logN) - 1u)) >> 1) >> (32u - logN);
-}
+// Position n holds the evaluation at exponent e = 2 brev(n) + 1; an automorphism X -> X^gal moves to it the one at e * gal, and
+// with the inverse exponent that is where it goes.  The positions n0 + c of an aligned tile have exponents e0 + brev(c) 2^k,
+// k = log2(2N / tile): their images lie in the tile whose first position is `tile`, at brev(brev(c) * gal + top) inside it.  All
+// but that last step is the same for the whole tile.
+template <int LOG_TN>
+struct TileMove {
+    u32 tile, top, gal;
+    __device__ __forceinline__ TileMove(u32 n0, u32 gal_, u32 logN) : gal(gal_) {
+        const u32 e = ((2u * (__brev(n0) >> (32u - logN)) + 1u) * gal) & ((2u << logN) - 1u);
+        tile = (__brev(e >> 1) >> (32u - logN)) & ~((1u << LOG_TN) - 1u);
+        top = e >> (logN + 1 - LOG_TN);
+    }
+    __device__ __forceinline__ u32 inside(u32 c_rev) const { return __brev(c_rev * gal + top) >> (32 - LOG_TN); }     // c_rev = brev(c)
+};
 
 // g^j modulo 2^32
 __device__ __forceinline__ u32 power32(u32 g, u32 j) {
@@ -44,15 +56,17 @@ __device__ __forceinline__ u32 power32(u32 g, u32 j) {
 }
 
 // Accumulator of one output word of the multiply-accumulate and the form its operands have: weights as stored (two
-// 32-bit halves), the X word as it sits in shared memory.
+// 32-bit halves), the X word as it sits in shared memory (x_word: of a residue; x_stored: of a word of the un-rotated inputs, which
+// are residues except modulo primes of class OP_DP, where they are doubles).
 template <int CLS>
 struct MacAcc {                                          // OP_NARROW
     static constexpr u32 L = LIMB_NARROW;
     LimbAcc<false> a;
     __device__ __forceinline__ void mac(u32 w0, u32 w1, u64 x) { a.mac(w0, w1, w0 + w1, (u32)x, (u32)(x >> 32)); }
     __device__ __forceinline__ void end_chunk(const RingDev&, u32, u32) {}
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const { return a.reduce(R.q[i], (u32)R.qneg[i]); }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i, bool) const { return a.reduce(R.q[i], (u32)R.qneg[i]); }
     static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
+    static __device__ __forceinline__ u64 x_stored(u64 v) { return x_word(v); }
 };
 template <>
 struct MacAcc<OP_WIDE> {
@@ -73,10 +87,11 @@ struct MacAcc<OP_WIDE> {
         a = {};
         if ((chunk & 15u) == 15u) v = ((unsigned __int128)barrett64((u64)(v >> 64), R.q[i], R.mu[i]) << 64) | (u64)v;
     }
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const {
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i, bool) const {
         return redc_2x32(barrett64((u64)(v >> 64), R.q[i], R.mu[i]), (u64)v, R.q[i], (u32)R.qneg[i]);
     }
     static __device__ __forceinline__ u64 x_word(u64 v) { return limb_split(v, L); }
+    static __device__ __forceinline__ u64 x_stored(u64 v) { return x_word(v); }
 };
 template <>
 struct MacAcc<OP_DP> {
@@ -85,40 +100,54 @@ struct MacAcc<OP_DP> {
         a.mac(__hiloint2double((int)w1, (int)w0), __longlong_as_double((long long)x));
     }
     __device__ __forceinline__ void end_chunk(const RingDev&, u32, u32) {}
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i) const {
-        return d2u(a.reduce(R.qd[i], R.qinv_d[i], R.c40_d[i], R.c40_q[i]));
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 i, bool many) const {
+        return d2u(fp_canonical(a.lazy(R.qd[i], R.qinv_d[i], R.c40_d[i], R.c40_q[i], many), R.qd[i], R.qinv_d[i]));
     }
     static __device__ __forceinline__ u64 x_word(u64 v) { return (u64)__double_as_longlong(u2d(v)); }
+    static __device__ __forceinline__ u64 x_stored(u64 v) { return v; }
 };
 
+// The X tile: [term][TN] pairs (component 0, component 1).
 template <int CLS, int LOG_TN, bool BABY, int RC>
 __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict__ pt, const TileLayout& lay,
                                          const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 pj_begin, u32 pj_end,
-                                         u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, u64* xs) {
+                                         u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, ulonglong2* xs) {
     constexpr u32 TN = 1u << LOG_TN, PL = MAC_THREADS >> LOG_TN;
     typedef MacAcc<CLS> Acc;
     const u32 N = R.N, logN = R.logN;
     const u32 np = lay.n_primes;
-    const u32 tid = threadIdx.x, c = tid & (TN - 1), l = tid >> LOG_TN;
+    const u32 tid = threadIdx.x, c = tid & (TN - 1), c_rev = __brev(c) >> (32 - LOG_TN);
+    u32 l = tid >> LOG_TN;
+    if constexpr (LOG_TN >= 5) l = __shfl_sync(0xffffffffu, l, 0);      // (so that what depends on it is computed once per warp)
     const u32 n0 = tile << LOG_TN;
-    const u64 q = R.q[i];
     const u64 pol = stream_policy();
     if constexpr (BABY) {
         const u32 r = R.r;
         const u32 b = bs.b, n_in = bs.n_in;
-        // term (q, 0): P times the un-rotated input
-        for (u32 e = l; e < n_in * 2; e += PL)      // (zero modulo P, and not stored there)
-            xs[(size_t)((e >> 1) * b * 2 + (e & 1)) * TN + c] = Acc::x_word(i < r ? __ldg(x + ((size_t)e * np + i) * N + n0 + c) : 0ull);
+        // term (q, 0): P times the un-rotated input (zero modulo P, and not stored there)
+        const u64* xg = x + (size_t)i * N + c;
+        const size_t comp_stride = (size_t)np * N;
+        for (u32 e = l; e < n_in; e += PL) {
+            const u64* xp = xg + e * 2 * comp_stride + n0;
+            xs[e * b * TN + c] = i < r ? make_ulonglong2(Acc::x_stored(__ldg(xp)), Acc::x_stored(__ldg(xp + comp_stride)))
+                                       : make_ulonglong2(Acc::x_word(0), Acc::x_word(0));
+        }
         // rotations: an item is a key and a part of the inputs that share it
-        const u32 n_items = (b - 1) * bs.parts;
-        for (u32 it = l; it < n_items; it += PL) {
-            const u32 k = 1 + it / bs.parts, part = it % bs.parts;
-            const u32 q_end = min(n_in, (part + 1) * bs.per_part);
-            const u32 src = (automorphism_index(n0, bs.gal[k], logN) & ~(TN - 1)) + c;
-            const u32 cd = automorphism_index(src, bs.gal_inv[k], logN) & (TN - 1);
-            const KeyTile<CLS> kt(key_tile(R, bs.keys, bs.key[k], i, src / KS_TILE), src % KS_TILE, r);
-            const u64* dp = bs.dig + ks_tile_base(N, r + 1, r, part * bs.per_part, 0u, i) + (size_t)(src / KS_TILE) * r * KS_TILE + src % KS_TILE;
-            const size_t dig_stride = ks_tile_base(N, r + 1, r, 1u, 0u, 0u);
+        const u32 parts = bs.parts, per_part = bs.per_part;
+        const size_t dig_stride = ks_tile_base(N, r + 1, r, 1u, 0u, 0u);
+        const u64* dig0 = bs.dig + ks_tile_base(N, r + 1, r, 0u, 0u, i);
+        u32 k = 1, part = l;
+        for (;; part += PL) {
+            while (part >= parts) { part -= parts; ++k; }
+            if (k >= b) break;
+            const u32 src = TileMove<LOG_TN>(n0, bs.gal[k], logN).tile;
+            const u32 cd = TileMove<LOG_TN>(src, bs.gal_inv[k], logN).inside(c_rev);
+            const u32 in_tile = (src + c) % KS_TILE;
+            const KeyTile<CLS> kt(key_tile(R, bs.keys, bs.key[k], i, src / KS_TILE), in_tile, r);
+            const u32 q_end = min(n_in, (part + 1) * per_part);
+            const u64* dp = dig0 + part * per_part * dig_stride + (src / KS_TILE) * (r * KS_TILE) + in_tile;
+            const u64* cp = xg + part * per_part * 2 * comp_stride + src;
+            ulonglong2* xp = xs + (part * per_part * b + k) * TN + cd;
             u32 k0[RC > 0 ? 2 * RC : 1], k1[RC > 0 ? 2 * RC : 1];
             if constexpr (RC > 0) {
                 u32 high[(2 * RC + 3) / 4];
@@ -129,9 +158,9 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 #pragma unroll
                 for (int s = 0; s < 2 * RC; ++s) KeyTile<CLS>::cut(s, high[s / 4], k0[s], k1[s]);
             }
-            for (u32 qi = part * bs.per_part; qi < q_end; ++qi, dp += dig_stride) {
+            for (u32 qi = part * per_part; qi < q_end; ++qi, dp += dig_stride, cp += 2 * comp_stride, xp += b * TN) {
                 KeyDot<CLS> dot;
-                const u64 pc0 = i < r ? __ldg(x + ((size_t)qi * 2 * np + i) * N + src) : 0ull;
+                const u64 pc0 = i < r ? __ldg(cp) : 0ull;
                 if constexpr (RC > 0) {
                     uint2 dw[RC];
 #pragma unroll
@@ -150,29 +179,37 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
                         dot.mac(__ldg((const uint2*)(dp + j * KS_TILE)), ka.x, ka.y, kb.x, kb.y);
                     }
                 }
-                u64 v0, v1;
-                dot.reduce(R, i, v0, v1);
-                u64* xp = xs + (size_t)(qi * b + k) * 2 * TN + cd;
-                xp[0] = Acc::x_word(add_mod(v0, pc0, q));
-                xp[TN] = Acc::x_word(v1);
+                if constexpr (CLS == OP_DP) {           // (centred: what the weights multiply may have either sign)
+                    const double qd = R.qd[i], qinv = R.qinv_d[i], c40 = R.c40_d[i], c40q = R.c40_q[i];
+                    const double v0 = __dadd_rn(dot.a0.lazy(qd, qinv, c40, c40q, false), __longlong_as_double((long long)pc0));
+                    const double v1 = dot.a1.lazy(qd, qinv, c40, c40q, false);
+                    *xp = make_ulonglong2((u64)__double_as_longlong(fp_centre(v0, qd, qinv)), (u64)__double_as_longlong(fp_centre(v1, qd, qinv)));
+                } else {
+                    u64 v0, v1;
+                    dot.reduce(R, i, v0, v1);
+                    *xp = make_ulonglong2(Acc::x_word(add_mod(v0, pc0, R.q[i])), Acc::x_word(v1));
+                }
             }
         }
     } else {
         // X tile: all of a thread's words are requested in batches, one round trip each
         const u64* xg = x + (size_t)i * N + n0 + c;
-        const u32 n_seg = n_terms * 2;
+        const size_t comp_stride = (size_t)np * N;
         u32 e = l;
-        for (; e + 7 * PL < n_seg; e += 8 * PL) {
+        for (; e + 3 * PL < n_terms; e += 4 * PL) {
             u64 v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __ldg(xg + (size_t)(e + j * PL) * np * N);
+            for (int j = 0; j < 8; ++j) v[j] = __ldg(xg + ((size_t)(e + j / 2 * PL) * 2 + j % 2) * comp_stride);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) xs[(size_t)(e + j * PL) * TN + c] = Acc::x_word(v[j]);
+            for (int j = 0; j < 4; ++j) xs[(e + j * PL) * TN + c] = make_ulonglong2(Acc::x_word(v[2 * j]), Acc::x_word(v[2 * j + 1]));
         }
-        for (; e < n_seg; e += PL) xs[(size_t)e * TN + c] = Acc::x_word(__ldg(xg + (size_t)e * np * N));
+        for (; e < n_terms; e += PL) {
+            const u64* xp = xg + (size_t)e * 2 * comp_stride;
+            xs[e * TN + c] = make_ulonglong2(Acc::x_word(__ldg(xp)), Acc::x_word(__ldg(xp + comp_stride)));
+        }
     }
     // terms up to a whole chunk are zero, and so are the padding words of a group's last stage once they are in registers
-    for (u32 e = 2 * n_terms + l; e < 2 * TILE_TS * lay.C; e += PL) xs[(size_t)e * TN + c] = 0;
+    for (u32 e = n_terms + l; e < TILE_TS * lay.C; e += PL) xs[e * TN + c] = make_ulonglong2(0, 0);
     __syncthreads();
 
     // ---------------- the weight stream: a lane's words of successive stages lie one stage apart
@@ -204,8 +241,15 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
     };
     Acc a0, a1;
     u32 pj = pj_begin + l, ch = 0;
-    const u64* xt = xs + c;
+    const ulonglong2* xt = xs + c;
     const u32 tail = n_terms % TILE_TS;
+    // the giant step of group pj and the Galois element of its rotation (see MacScatter)
+    u32 step_rem = 0, step_gal = 1, step = 0;
+    if (sc.on) {
+        step = (sc.pj0 + pj) / sc.n_out;
+        step_rem = sc.pj0 + pj - step * sc.n_out;
+        step_gal = power32(sc.gal_inv, step);
+    }
     auto use = [&](u32 (&wa)[TS], u32 (&wb)[TH]) {
         if constexpr (!PACKED) {        // (packed padding is a finite number times a zero of X, whatever it is)
             if (tail && ch + 1 == n_chunks) {
@@ -218,21 +262,30 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         for (int ts = 0; ts < TS; ++ts) {
             u32 w0 = wa[ts], w1 = wb[PACKED ? ts / 4 : ts];
             if constexpr (PACKED) unpack40(ts, w1, w0, w1);
-            a0.mac(w0, w1, xt[(ts * 2) * TN]);
-            a1.mac(w0, w1, xt[(ts * 2 + 1) * TN]);
+            const ulonglong2 xw = xt[ts * TN];
+            a0.mac(w0, w1, xw.x);
+            a1.mac(w0, w1, xw.y);
         }
         a0.end_chunk(R, i, ch);
         a1.end_chunk(R, i, ch);
-        xt += TS * 2 * TN;
+        xt += TS * TN;
         if (++ch == n_chunks) {
             u64* ap = a + ((size_t)pj * 2 * np + i) * N;
             u32 at0 = n0 + c;                                           // where component 0 goes (see MacScatter)
-            if (sc.on && sc.pj0 + pj >= sc.n_out) at0 = automorphism_index(at0, power32(sc.gal_inv, (sc.pj0 + pj) / sc.n_out), logN);
-            ap[at0] = a0.reduce(R, i);
-            ap[(size_t)np * N + n0 + c] = a1.reduce(R, i);
+            if (step) {
+                const TileMove<LOG_TN> to(n0, step_gal, logN);
+                at0 = to.tile + to.inside(c_rev);
+            }
+            ap[at0] = a0.reduce(R, i, n_terms > 128);
+            ap[(size_t)np * N + n0 + c] = a1.reduce(R, i, n_terms > 128);
             a0 = {};
             a1 = {};
             pj += PL;
+            if (sc.on)
+                for (step_rem += PL; step_rem >= sc.n_out; step_rem -= sc.n_out) {
+                    step_gal *= sc.gal_inv;
+                    ++step;
+                }
             ch = 0;
             xt = xs + c;
         }
@@ -255,7 +308,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
 // grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
 // operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
-// Four blocks an SM (64 registers; the key part spills 80 bytes at r = 7, 236 at r = 9) because resident warps are what hides the latency: two,
+// Four blocks an SM (64 registers; the key part spills 108 bytes at r = 9 in tiles of 128, none at r = 7) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
 template <bool NARROW, int LOG_TN, bool BABY, int RC>
@@ -263,7 +316,7 @@ __global__ void __launch_bounds__(MAC_THREADS, 4)
 mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const __grid_constant__ TileLayout lay,
            const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 n_pj, u32 pj_per_block,
            const __grid_constant__ MacScatter sc, const __grid_constant__ BabySteps bs) {
-    extern __shared__ __align__(128) u64 mac_xs[];
+    extern __shared__ __align__(128) ulonglong2 mac_xs[];
     grid_dependency_enter();
     const u32 tiles_log = R.logN - LOG_TN;
     const u32 i = lay.n_primes - 1 - blockIdx.x % lay.n_primes;

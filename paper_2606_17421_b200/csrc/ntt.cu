@@ -882,9 +882,11 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 split_index(o, B.dtile_div, B.dtile_magic, q_in, j);
                 if (m <= R.r) stg4(B.dtile_ptr + ks_tile_base(R.N, nbp, R.r, q_in, j, m) + (size_t)(n / KS_TILE) * R.r * KS_TILE + n % KS_TILE, v4[0], v4[1], v4[2], v4[3]);
                 if (mod == j) {             // its own prime: the un-rotated input, times P
-                    u64 p4[4];
+                    u64 p4[4];                  // (the multiply-accumulate, which reads them, takes doubles where it takes digits as such)
+                    const double pd = u2d(R.pmod[mod]), pq = __dmul_rn(pd, c.qinv);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) p4[i] = times_p(R, mod, dp ? d2u(__longlong_as_double((long long)v4[i])) : v4[i]);
+                    for (int i = 0; i < 4; ++i)
+                        p4[i] = dp ? (u64)__double_as_longlong(fp_mul_centred_signed(__longlong_as_double((long long)v4[i]), pd, pq, c.qd)) : times_p(R, mod, v4[i]);
                     stg4(B.lift_ptr + (size_t)q_in * B.lift_so + ((size_t)(m <= R.r ? nbp : 0u) + mod) * R.N + n, p4[0], p4[1], p4[2], p4[3]);
                 }
                 continue;
