@@ -311,10 +311,6 @@ struct PolyBatch {
     u32 mod_wrap;                 // > 0: modulus index = mod0 + (m % mod_wrap) * mod_step (e.g. m = component*r + prime)
     u32 o_div;                    // > 0: source = src + (o / o_div)*src_so2 + (o % o_div)*src_so + m*src_sm
     long long src_so2;
-    // inverse only: the input is a sum  src + sum_{t < sum_terms} (sum_src + t*sum_stride)  of residues in [0, q)
-    const u64* sum_src;
-    long long sum_stride;
-    u32 sum_terms;
     u64 lift_mod;                 // LOAD_CENTRED: the modulus M the source residues live in
     u32 src32;                    // LOAD_I64_MONT: the source words are 32-bit integers
     u32 src_digits;               // LOAD_REDUCE: the source of outer index o is a residue modulo prime o % r

@@ -79,6 +79,9 @@ cudaError_t ntt_forward_moddown(const RingHost& ring, const PolyBatch& B, u32 n_
 cudaError_t ntt_inverse_assembly(const RingHost& ring, const PolyBatch& B, u32 n_outer, const OutputAssembly& as, cudaStream_t stream);
 cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, const u64* T, u32 n_u, u32 n_t, u32 n_out,
                             cudaStream_t stream, const RescaleConsts* rc = nullptr, u64* low = nullptr);
+// out = (u0, u1) / P + (phi(c0), 0), plus ct where `add`, for n_ct ciphertexts [2][r][N] in the coefficient domain: u, [2][r+1][N] each,
+// is the rotated key-switch result with its residue modulo P as a centred lift plus 2^59.  out must not overlap ct.
+cudaError_t finish_rotation(const RingHost& ring, const u64* u, const u64* ct, u64* out, u32 n_ct, u32 gal_inv, bool add, cudaStream_t stream);
 cudaError_t ntt_forward_split(const RingHost& ring, const PolyBatch& B, u32 n_outer, int load, void* final_dst,
                               const u32* scatter, u32 scatter_div, cudaStream_t stream);
 

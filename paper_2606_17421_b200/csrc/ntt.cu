@@ -732,7 +732,7 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // with 691 warp instructions (68 % of the issue slots), 324 of them fp64 (64 % of that pipe) and about 165 wavefronts of the
 // L1 pipe (65 %); small launches are bound by the latency of one chunk.
 // Forward: second pass (final reduction to [0, q), then the store functors).  Inverse: first pass
-// (reads the batch source: plain residues, tiled/limb-split plaintexts, or a sum of arrays).
+// (reads the batch source: plain residues or tiled/limb-split plaintexts).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
 // EPI: 0 = none; 1 = division by P per rotation (see ModDownEpilogue); 4 = output assembly (see OutputAssembly); 5 = ingest
 // (see PolyBatch): the digits into the operand array, component c of the inputs times P into lift_ptr.
@@ -1018,30 +1018,6 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 const ulonglong2* gp = (const ulonglong2*)(gsrc + 4 * s);
                 const ulonglong2 a = gp[0], b = gp[1];
                 v4[0] = a.x; v4[1] = a.y; v4[2] = b.x; v4[3] = b.y;
-            }
-            if (B.sum_terms) {      // the input is a sum of several arrays of the same shape
-                const u64* sp = B.sum_src + (size_t)o * B.src_so + (size_t)m * B.src_sm + (size_t)chunk * LEN + 4 * s;
-                // three arrays at a time, all their loads in flight together (g - 1 = 3 is the common case)
-                u32 h = 0;
-                for (; h + 3 <= B.sum_terms; h += 3) {
-                    ulonglong2 a2[3], b2[3];
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        a2[j] = *(const ulonglong2*)(sp + (size_t)(h + j) * B.sum_stride);
-                        b2[j] = *(const ulonglong2*)(sp + (size_t)(h + j) * B.sum_stride + 2);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        v4[0] = add_mod(v4[0], a2[j].x, q); v4[1] = add_mod(v4[1], a2[j].y, q);
-                        v4[2] = add_mod(v4[2], b2[j].x, q); v4[3] = add_mod(v4[3], b2[j].y, q);
-                    }
-                }
-                for (; h < B.sum_terms; ++h) {
-                    const ulonglong2 a2 = *(const ulonglong2*)(sp + (size_t)h * B.sum_stride);
-                    const ulonglong2 b2 = *(const ulonglong2*)(sp + (size_t)h * B.sum_stride + 2);
-                    v4[0] = add_mod(v4[0], a2.x, q); v4[1] = add_mod(v4[1], a2.y, q);
-                    v4[2] = add_mod(v4[2], b2.x, q); v4[3] = add_mod(v4[3], b2.y, q);
-                }
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) from_u64(e[i], v4[i]);
@@ -1631,6 +1607,56 @@ cudaError_t finish_division(const RingHost& ring, u64* ct, long long ct_stride, 
     }
     launch_dependent(ring, finish_division_kernel, dim3(ring.dev.N / 128, n_out * 2), dim3(128), 0, stream, ring.dev, ct,
                      ct_stride, T, n_u, n_t, rc ? *rc : none, rc ? low : (u64*)nullptr);
+    return cudaGetLastError();
+}
+
+// The last step of a rotation whose key-switch result u is at hand in the coefficient domain, rotated, over {q_i, P} (its residue
+// modulo P as a centred lift plus 2^59): out = (u0, u1) / P + (phi(c0), 0), plus (c0, c1) where `add`.  phi moves coefficient k to
+// k * gal mod 2N, with a sign beyond N.  A thread has all residues of its coefficient, so that the lift is cut once.
+template <bool FP>
+__global__ void __launch_bounds__(128, 8) finish_rotation_kernel(const RingDev R, const u64* __restrict__ u, const u64* __restrict__ ct,
+                                                                 u64* __restrict__ out, u32 gal_inv, u32 add) {
+    grid_dependency_enter();
+    const u32 n = blockIdx.x * 128 + threadIdx.x, comp = blockIdx.y & 1;
+    const size_t N = R.N, poly = (size_t)blockIdx.y * R.r * N;
+    const u64* up = u + (size_t)blockIdx.y * (R.r + 1) * N + n;
+    const u64* cp = ct + poly;
+    const u32 k = (n * gal_inv) & (2 * R.N - 1), from = k & (R.N - 1);
+    const bool minus = k >= R.N;
+    const i64 S = (i64)(up[R.r * N] - (1ull << 59));
+    const i64 s_hi = S >> 30;
+    const bool neg = S < 0;
+    const u64 mag = neg ? (u64)(-S) : (u64)S;
+    const double lo = u2d((u64)(S & ((1ll << 30) - 1))), ah = u2d((u64)(s_hi < 0 ? -s_hi : s_hi));
+#pragma unroll
+    for (int i = 0; i < MAX_MODULI; ++i)
+        if ((u32)i < R.r) {
+            const u64 q = R.q[i];
+            u64 v;
+            if (FP) {
+                const double sm = fp_mul_centred(ah, R.c30_d[i], R.c30_q[i], R.qd[i]);
+                const double x = __dsub_rn(__dsub_rn(u2d(up[i * N]), neg ? -sm : sm), lo);
+                v = d2u(fp_times_const(fp_centre(x, R.qd[i], R.qinv_d[i]), (q >> 41) != 0, R.pinv_d[i], R.pinv_q[i], R.qd[i], R.qinv_d[i]));
+            } else {
+                u64 t = barrett64(mag, q, R.mu[i]);
+                if (neg && t) t = q - t;
+                v = mul_shoup(sub_mod(up[i * N], t, q), R.pinv[i], R.pinvs[i], q);
+            }
+            if (comp == 0) {
+                const u64 c = cp[i * N + from];
+                v = minus ? sub_mod(v, c, q) : add_mod(v, c, q);
+            }
+            if (add) v = add_mod(v, cp[i * N + n], q);
+            out[poly + i * N + n] = v;
+        }
+}
+
+cudaError_t finish_rotation(const RingHost& ring, const u64* u, const u64* ct, u64* out, u32 n_ct, u32 gal_inv, bool add, cudaStream_t stream) {
+    ProfScope prof(ring.prof, CAT_DIVIDE, stream);
+    bool fp = true;
+    for (u32 i = 0; i < ring.dev.r; ++i) fp = fp && ring.dev.fp_ok[i];
+    launch_dependent(ring, fp ? finish_rotation_kernel<true> : finish_rotation_kernel<false>, dim3(ring.dev.N / 128, n_ct * 2), dim3(128), 0,
+                     stream, ring.dev, u, ct, out, gal_inv, add ? 1u : 0u);
     return cudaGetLastError();
 }
 

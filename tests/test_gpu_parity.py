@@ -1038,6 +1038,30 @@ def test_fold_in_ciphertext_matches_oracle(pkey, plan_t, shape):
         g.close()
 
 
+@pytest.mark.parametrize("pkey", ["n12", "paper_n13"])        # ciphertext primes below 2^50, and one of 60 bits
+@pytest.mark.parametrize("tau", [2, 8])                       # one round (which ends in the other buffer), an odd number of them
+def test_fold_rounds_and_rotation_in_place(pkey, tau):
+    par = oracle_params(pkey)
+    plan = ckks.Plan(8 * tau, tau, 4, 2)
+    s = ckks.keygen(par, 47)
+    keys = ckks.make_rotation_keys(par, s, plan, 47, extra_steps=ckks.fold_rotations(plan))
+    cts = np.stack([np.ascontiguousarray(wl.gen_uniform_residues(47, f"fold{t}", par.primes, (2, par.N)).transpose(1, 0, 2))
+                    for t in range(3)])
+    g = GpuSide(par, plan)
+    try:
+        steps = g.load_keys(keys, extra_steps=ckks.fold_rotations(plan))
+        d = g.to_dev(cts)
+        g.bf.bf_fold(g.ctx, d, len(cts))
+        got = g.to_host_u64(d)
+        for t in range(len(cts)):
+            assert np.array_equal(got[t], ckks.fold_in_ciphertext(par, plan, cts[t], keys)), t
+        d = g.to_dev(cts[0])
+        g.bf.bf_rotate(g.ctx, d, steps[-1], d)
+        assert np.array_equal(g.to_host_u64(d), ckks.rotate(par, cts[0], steps[-1], keys))
+    finally:
+        g.close()
+
+
 def test_fold_of_more_ciphertexts_than_one_key_switch_batch():
     # 70 ciphertexts: the rounds run in two batches (64 + 6); sampled ones are compared with the oracle
     par = oracle_params("n12")
