@@ -1156,7 +1156,7 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
         baby.keys = ctx->keys;
         baby.dig = Dig;
         for (u32 k = 1; k < b; ++k) {
-            baby.key[k] = (u32)baby_key[k];
+            baby.key_at[k] = (u64)baby_key[k] * ctx->ring.dev.key_bytes;
             baby.gal[k] = ctx->gal[baby_key[k]];
             baby.gal_inv[k] = ctx->gal_inv[baby_key[k]];
         }

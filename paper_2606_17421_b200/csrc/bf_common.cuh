@@ -235,13 +235,13 @@ struct MacScatter {
     u32 gal_inv;                        // inverse Galois element of giant step 1: step j has its j-th power
 };
 
-// Baby rotations computed inside the multiply-accumulate (double hoisting): input q's term k is its rotation by key[k].
+// Baby rotations computed inside the multiply-accumulate (double hoisting): input q's term k is its rotation by the key at key_at[k].
 struct BabySteps {
     u32 n_in, b;
     u32 parts, per_part;                // how the inputs are dealt out to a block's lanes (set by the launcher)
     const void* keys;                   // resident keys
     const u64* dig;                     // digit set q of input q (tile-major, see KS_TILE)
-    u32 key[MAX_ROT_BATCH + 1];
+    u64 key_at[MAX_ROT_BATCH + 1];      // byte offset of the key
     u32 gal[MAX_ROT_BATCH + 1], gal_inv[MAX_ROT_BATCH + 1];
 };
 

@@ -122,7 +122,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
     const u32 n0 = tile << LOG_TN;
     const u64 pol = stream_policy();
     if constexpr (BABY) {
-        const u32 r = R.r;
+        const u32 r = RC > 0 ? (u32)RC : R.r;
         const u32 b = bs.b, n_in = bs.n_in;
         // term (q, 0): P times the un-rotated input (zero modulo P, and not stored there)
         const u64* xg = x + (size_t)i * N + c;
@@ -132,22 +132,26 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             xs[e * b * TN + c] = i < r ? make_ulonglong2(Acc::x_stored(__ldg(xp)), Acc::x_stored(__ldg(xp + comp_stride)))
                                        : make_ulonglong2(Acc::x_word(0), Acc::x_word(0));
         }
-        // rotations: an item is a key and a part of the inputs that share it
+        // rotations: an item is a key and a part of the inputs that share it.  The tile has the exponents e0 + brev(c) 2^k; a
+        // rotation reads the tile of e0 * gal, whose own first exponent is that less its top bits T, so that the word at c there
+        // goes to brev((brev(c) - T) / gal) here (see TileMove)
         const u32 parts = bs.parts, per_part = bs.per_part;
         const size_t dig_stride = ks_tile_base(N, r + 1, r, 1u, 0u, 0u);
-        const u64* dig0 = bs.dig + ks_tile_base(N, r + 1, r, 0u, 0u, i);
+        const u64* dig0 = bs.dig + ks_tile_base(N, r + 1, r, 0u, 0u, i) + c;
+        const unsigned char* key0 = (const unsigned char*)bs.keys + R.key_base[i];
+        const u32 e0 = 2u * (__brev(n0) >> (32u - logN)) + 1u, tile_bytes = key_tile_bytes(CLS == OP_DP, r);
         u32 k = 1, part = l;
         for (;; part += PL) {
             while (part >= parts) { part -= parts; ++k; }
             if (k >= b) break;
-            const u32 src = TileMove<LOG_TN>(n0, bs.gal[k], logN).tile;
-            const u32 cd = TileMove<LOG_TN>(src, bs.gal_inv[k], logN).inside(c_rev);
-            const u32 in_tile = (src + c) % KS_TILE;
-            const KeyTile<CLS> kt(key_tile(R, bs.keys, bs.key[k], i, src / KS_TILE), in_tile, r);
-            const u32 q_end = min(n_in, (part + 1) * per_part);
-            const u64* dp = dig0 + part * per_part * dig_stride + (src / KS_TILE) * (r * KS_TILE) + in_tile;
-            const u64* cp = xg + part * per_part * 2 * comp_stride + src;
-            ulonglong2* xp = xs + (part * per_part * b + k) * TN + cd;
+            const u32 e = (e0 * bs.gal[k]) & ((2u << logN) - 1u), T = e >> (logN + 1 - LOG_TN);
+            const u32 src = (__brev(e >> 1) >> (32u - logN)) & ~(TN - 1), ks = src / KS_TILE, in_tile = src % KS_TILE;
+            const u32 cd = __brev((c_rev - T) * bs.gal_inv[k]) >> (32 - LOG_TN);
+            const KeyTile<CLS> kt(key0 + bs.key_at[k] + ks * tile_bytes, in_tile + c, r);
+            const u32 q0 = part * per_part, q_end = min(n_in, q0 + per_part);
+            const u64* dp = dig0 + q0 * dig_stride + ks * (r * KS_TILE) + in_tile;
+            const u64* cp = xg + q0 * 2 * comp_stride + src;
+            ulonglong2* xp = xs + (q0 * b + k) * TN + cd;
             u32 k0[RC > 0 ? 2 * RC : 1], k1[RC > 0 ? 2 * RC : 1];
             if constexpr (RC > 0) {
                 u32 high[(2 * RC + 3) / 4];
@@ -158,7 +162,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 #pragma unroll
                 for (int s = 0; s < 2 * RC; ++s) KeyTile<CLS>::cut(s, high[s / 4], k0[s], k1[s]);
             }
-            for (u32 qi = part * per_part; qi < q_end; ++qi, dp += dig_stride, cp += 2 * comp_stride, xp += b * TN) {
+            for (u32 qi = q0; qi < q_end; ++qi, dp += dig_stride, cp += 2 * comp_stride, xp += b * TN) {
                 KeyDot<CLS> dot;
                 const u64 pc0 = i < r ? __ldg(cp) : 0ull;
                 if constexpr (RC > 0) {
@@ -240,7 +244,10 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         stage += stage_bytes;
     };
     Acc a0, a1;
-    u32 pj = pj_begin + l, ch = 0;
+    u32 ch = 0;
+    const size_t comp1 = (size_t)np * N;                // from component 0 to component 1
+    const u32 pj = pj_begin + l;
+    u64* ap = a + ((size_t)pj * 2 * np + i) * N;
     const ulonglong2* xt = xs + c;
     const u32 tail = n_terms % TILE_TS;
     // the giant step of group pj and the Galois element of its rotation (see MacScatter)
@@ -270,17 +277,16 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         a1.end_chunk(R, i, ch);
         xt += TS * TN;
         if (++ch == n_chunks) {
-            u64* ap = a + ((size_t)pj * 2 * np + i) * N;
             u32 at0 = n0 + c;                                           // where component 0 goes (see MacScatter)
             if (step) {
                 const TileMove<LOG_TN> to(n0, step_gal, logN);
                 at0 = to.tile + to.inside(c_rev);
             }
             ap[at0] = a0.reduce(R, i, n_terms > 128);
-            ap[(size_t)np * N + n0 + c] = a1.reduce(R, i, n_terms > 128);
+            ap[comp1 + n0 + c] = a1.reduce(R, i, n_terms > 128);
+            ap += 2 * PL * comp1;
             a0 = {};
             a1 = {};
-            pj += PL;
             if (sc.on)
                 for (step_rem += PL; step_rem >= sc.n_out; step_rem -= sc.n_out) {
                     step_gal *= sc.gal_inv;
