@@ -400,6 +400,14 @@ __device__ __forceinline__ u64 redc_2x32(u64 H, u64 L, u64 q, u32 qneg32) {
     return t >= q ? t - q : t;
 }
 
+// A pointer kept whole in a thread's registers, so that loads around it take immediate offsets.  (Left to itself the compiler adds
+// each offset to the part of the address that a warp shares: two instructions a load.)
+template <typename T>
+__device__ __forceinline__ const T* thread_pointer(const T* p) {
+    asm("" : "+l"(p));
+    return p;
+}
+
 // words that are read exactly once: not kept in L1, first to leave L2
 __device__ __forceinline__ u64 stream_policy() {
     u64 pol;
@@ -507,7 +515,7 @@ template <int CLS>
 struct KeyTile {
     const unsigned char* at;
     u32 r;
-    __device__ __forceinline__ KeyTile(const unsigned char* tile, u32 c, u32 r_) : at(tile + (CLS == OP_DP ? 4 : 8) * c), r(r_) {}
+    __device__ __forceinline__ KeyTile(const unsigned char* tile, u32 c, u32 r_) : at(thread_pointer(tile + (CLS == OP_DP ? 4 : 8) * c)), r(r_) {}
     __device__ __forceinline__ u32 high(u32 group, u64 pol) const { return CLS == OP_DP ? ld_stream32(at + (2 * r + group) * KS_TILE * 4, pol) : 0u; }
     __device__ __forceinline__ void word(u32 s, u64 pol, u32& k0, u32& k1) const {
         if (CLS == OP_DP) k0 = ld_stream32(at + s * KS_TILE * 4, pol);
@@ -523,7 +531,10 @@ struct KeyTile {
 };
 
 // One output word of the key-switch inner product: digits times key words (cut), summed, in [0, q).  The keys carry a
-// factor 2^64 except where the class is OP_DP.
+// factor 2^64 except where the class is OP_DP; there the digits may be lazy, as a forward transform leaves them: within 13q, so
+// that a sum of LAZY_DIGITS products stays below 2^87 (`many`: more of them; see DpAcc::lazy).  (Four fp64 operations and a
+// conversion less for every point of a digit's transform: three rotations of 7 digits at N = 2^15 36.1 -> 34.0 us.)
+constexpr u32 LAZY_DIGITS = 9;
 template <int CLS>
 struct DigitDot {
     static constexpr u32 L = CLS == OP_WIDE ? LIMB_WIDE : LIMB_NARROW;
@@ -533,14 +544,14 @@ struct DigitDot {
         cut_limbs(d.x, d.y, L, d0, d1);
         a.mac(d0, d1, d0 + d1, k0, k1);
     }
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const { return a.reduce(R.q[m], (u32)R.qneg[m]); }
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m, bool) const { return a.reduce(R.q[m], (u32)R.qneg[m]); }
 };
 template <>
 struct DigitDot<OP_DP> {
     DpAcc a;
     __device__ __forceinline__ void mac(uint2 d, u32 k0, u32 k1) { a.mac(__hiloint2double((int)d.y, (int)d.x), __hiloint2double((int)k1, (int)k0)); }
-    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m) const {
-        return d2u(fp_canonical(a.lazy(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m], false), R.qd[m], R.qinv_d[m]));
+    __device__ __forceinline__ u64 reduce(const RingDev& R, u32 m, bool many) const {
+        return d2u(fp_canonical(a.lazy(R.qd[m], R.qinv_d[m], R.c40_d[m], R.c40_q[m], many), R.qd[m], R.qinv_d[m]));
     }
 };
 

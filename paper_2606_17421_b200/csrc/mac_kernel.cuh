@@ -185,8 +185,8 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
                 }
                 if constexpr (CLS == OP_DP) {           // (centred: what the weights multiply may have either sign)
                     const double qd = R.qd[i], qinv = R.qinv_d[i], c40 = R.c40_d[i], c40q = R.c40_q[i];
-                    const double v0 = __dadd_rn(dot.a0.lazy(qd, qinv, c40, c40q, false), __longlong_as_double((long long)pc0));
-                    const double v1 = dot.a1.lazy(qd, qinv, c40, c40q, false);
+                    const double v0 = __dadd_rn(dot.a0.lazy(qd, qinv, c40, c40q, r > LAZY_DIGITS), __longlong_as_double((long long)pc0));
+                    const double v1 = dot.a1.lazy(qd, qinv, c40, c40q, r > LAZY_DIGITS);
                     *xp = make_ulonglong2((u64)__double_as_longlong(fp_centre(v0, qd, qinv)), (u64)__double_as_longlong(fp_centre(v1, qd, qinv)));
                 } else {
                     u64 v0, v1;

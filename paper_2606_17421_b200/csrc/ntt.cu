@@ -735,7 +735,7 @@ __device__ __forceinline__ void swz_load_set(u32 a_thread, T (&e)[8]) {
 // (reads the batch source: plain residues or tiled/limb-split plaintexts).
 // TILED: the transform-domain side of the batch lives in the tile-major plaintext cache (B.tile_ptr).
 // EPI: 0 = none; 1 = division by P per rotation (see ModDownEpilogue); 4 = output assembly (see OutputAssembly); 5 = ingest
-// (see PolyBatch): the digits into the operand array, component c of the inputs times P into lift_ptr.
+// (see PolyBatch): the digits into the operand array (lazy doubles modulo primes of class OP_DP), component c of the inputs times P into lift_ptr.
 struct NoEpilogue {};
 struct RotationDivision {
     ModDownEpilogue e;
@@ -751,14 +751,15 @@ constexpr int CONTIG_THREADS = 128, CONTIG_WARPS = CONTIG_THREADS / 32;
 // Whole calls do not tell lines from 7000 to 40000 apart (within 1 % but for 768 -> 2304 without flags: 477, 485, 485 us).
 constexpr size_t CONTIG_SHORT_CHUNKS = 12000;
 
-// a point of the forward transform, brought to [0, q): a word, or the bits of a double where `bits`
+__device__ __forceinline__ u64 word_of(u64 v) { return v; }
+__device__ __forceinline__ u64 word_of(double v) { return (u64)__double_as_longlong(v); }
+// a point of the forward transform, brought to [0, q)
 template <int PATH, typename T>
-__device__ __forceinline__ u64 canonical(T x, const ModConsts& c, bool bits) {
+__device__ __forceinline__ u64 canonical(T x, const ModConsts& c) {
     if constexpr (PATH == PATH_WIDE) {
         return d2u(fp_reduce(x, c.qd, c.qinv));
     } else if constexpr (PATH == PATH_DP) {
-        const double v = fp_canonical(x, c.qd, c.qinv);
-        return bits ? (u64)__double_as_longlong(v) : d2u(v);
+        return d2u(fp_canonical(x, c.qd, c.qinv));
     } else {
         x = reduce_16q(x, c);
         if (x >= 2 * c.q) x -= 2 * c.q;
@@ -872,10 +873,16 @@ __device__ __forceinline__ void contig_body(const RingDev& R, const PolyBatch& B
                 pp[0] = pv.x; pp[1] = pv.y; pp[2] = pv.z; pp[3] = pv.w;
             }
             set_butterflies<2, true, PATH, false>(e, tw, 64u * mult + s, c);
-            // (doubles stay doubles where they are stored as such)
+            // (what is stored as doubles stays lazy: see LAZY_DIGITS)
             u64 v4[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c, EPI == 5 && dp);
+            for (int i = 0; i < 4; ++i) v4[i] = EPI == 5 && PATH == PATH_DP ? word_of(e[i]) : canonical<PATH>(e[i], c);
+            if constexpr (EPI == 5 && PATH == PATH_DP) {
+                if (!dp) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v4[i] = canonical<PATH>(e[i], c);
+                }
+            }
             if constexpr (EPI == 5) {
                 const u32 n = chunk * LEN + 4 * s, nbp = R.r + 1;
                 u32 q_in, j;
@@ -1141,7 +1148,7 @@ __device__ __forceinline__ void inner_products(const RingDev& R, const RotBatch&
                 KeyTile<CLS>::cut(2 * j + comp, high[j / 2], k0[j], k1[j]);
                 dot.mac(*(const uint2*)&sd[(j << LOG_C) + at], k0[j], k1[j]);
             }
-            return dot.reduce(R, m);
+            return dot.reduce(R, m, RC > LAZY_DIGITS);
         };
         const u64 v0 = component(0), v1 = component(1);
         // xext (double hoisting): the rotated input in the extended basis is (P*c0 + u0, u1) moved through the rotation's
@@ -1185,8 +1192,9 @@ ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const vo
         const u32 mult = (N >> LOG_C) + chunk;
         const void* tw = twiddle_table(R, true, path, m);
         const u32 a_near = slice + 8u * (u32)swz(4 * lane);
-        auto finish = [&](auto path_c) {
+        auto finish = [&](auto path_c, auto lazy_c) {
             constexpr int PATH = decltype(path_c)::value;
+            constexpr bool LAZY = decltype(lazy_c)::value;          // (digits of class OP_DP stay lazy: see LAZY_DIGITS)
             typedef typename Elem<PATH>::T T;
             contig_forward_far<PATH>((const T*)gsrc, slice, lane, tw, mult, c);
 #pragma unroll
@@ -1196,13 +1204,14 @@ ntt_contig_inner(const RingDev R, const PolyBatch B, const RotBatch rb, const vo
                 set_butterflies<2, true, PATH, false>(e, tw, 64u * mult + lane + 32 * it, c);
                 u64 v[8];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = canonical<PATH>(e[i], c, dp);
+                for (int i = 0; i < 4; ++i) v[i] = LAZY ? word_of(e[i]) : canonical<PATH>(e[i], c);
                 swz_store_set<4, 0>(a_near + (u32)(it * 8 * swz(128)), v);
             }
         };
-        if (path == PATH_DP) finish(std::integral_constant<int, PATH_DP>());
-        else if (path == PATH_WIDE) finish(std::integral_constant<int, PATH_WIDE>());
-        else finish(std::integral_constant<int, PATH_INT>());
+        if (dp) finish(std::integral_constant<int, PATH_DP>(), std::true_type());
+        else if (path == PATH_DP) finish(std::integral_constant<int, PATH_DP>(), std::false_type());
+        else if (path == PATH_WIDE) finish(std::integral_constant<int, PATH_WIDE>(), std::false_type());
+        else finish(std::integral_constant<int, PATH_INT>(), std::false_type());
     }
     __syncthreads();
     const u64 pol = stream_policy();
@@ -1239,6 +1248,7 @@ static void launch_shared_src_t(const RingHost& ring, const PolyBatch& B_in, u32
     typedef StridedGeo<LOG_R, LOG_LANES> G;
     PolyBatch B = B_in;
     set_magics(B, n_outer);
+    constexpr bool INGEST = LOAD == LOAD_INGEST;
     // targets per block: fewer blocks share the source better but quantise into waves; cost model =
     // waves x (targets per block + half a unit for staging the source)
     const u32 slots = 148u * G::BLOCKS;
@@ -1248,7 +1258,14 @@ static void launch_shared_src_t(const RingHost& ring, const PolyBatch& B_in, u32
         const u32 slices = (B.n_m + per - 1) / per;
         if ((B.n_m + slices - 1) / slices != per) continue;         // keep the slices balanced
         const u32 blocks = G::TILES * n_outer * slices;
-        const double cost = (double)((blocks + slots - 1) / slots) * (per + 0.5);
+        double cost = (double)((blocks + slots - 1) / slots) * (per + 0.5);
+        // (an ingest batch has half as many blocks of that length and one of a single target for every other source: the work, or
+        // one block where that is longer, and half a block for the end.  us for 1, 2, 4, 8 targets a block, N = 2^15, r = 7: one
+        // input 13.1, 12.7, 14.7, 18.0, three 31.6, 29.9, 31.4, 34.9; N = 2^16, r = 9, four inputs, 1, 2, 5, 10: 134, 119, 114, 117)
+        if (INGEST) {
+            const double work = (blocks * (per + 0.5) + G::TILES * n_outer * 1.5) / 2 / slots;
+            cost = (work > per + 0.5 ? work : per + 0.5) + (per + 0.5) / 2;
+        }
         if (cost <= best_cost) { best_cost = cost; best = per; }
     }
     const dim3 grid(G::TILES, n_outer, (B.n_m + best - 1) / best);
