@@ -389,7 +389,13 @@ static cudaError_t launch_mac_tile(const MacLaunch& m) {
 template <bool NARROW>
 static cudaError_t launch_mac_ring(const MacLaunch& m) {
     if (!m.baby) return launch_mac_tile<NARROW, false, 0>(m);
-    // (digit counts of the shipped parameter sets: the key words of a rotation in registers)
+    // (digit counts of the shipped parameter sets: the key words of a rotation in registers.  300 -> 1000 on a ring of 2^12, three
+    // digits: 11.7 us with a loop over them, 10.9 us like this)
+    if constexpr (NARROW) {
+        if (m.ring->dev.r == 3) return launch_mac_tile<NARROW, true, 3>(m);
+    } else {
+        if (m.ring->dev.r == 4) return launch_mac_tile<NARROW, true, 4>(m);
+    }
     switch (m.ring->dev.r) {
         case 7: return launch_mac_tile<NARROW, true, 7>(m);
         case 9: return launch_mac_tile<NARROW, true, 9>(m);

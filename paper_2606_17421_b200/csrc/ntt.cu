@@ -1118,7 +1118,7 @@ __global__ void __launch_bounds__(64, EPI == 4 ? 10 : 16) ntt_contig_short(const
 // and more: as many warps as digits leave fewer blocks to an SM (15 digits, loop: 1801 us).
 template <int RC>
 struct InnerGeo {
-    static constexpr int WARPS = RC == 9 ? 9 : 8, CHUNKS = RC > 8 ? 1 : WARPS / RC;    // (few digits leave room for several chunks)
+    static constexpr int WARPS = RC == 9 ? 9 : 8;                           // (few digits leave room for several chunks)
     static constexpr int BLOCKS = RC == 9 ? 3 : 4;
 };
 template <int CLS, int RC>
@@ -1402,9 +1402,9 @@ cudaError_t ntt_forward_first(const RingHost& ring, const PolyBatch& B, u32 n_ou
 
 template <int RC>
 static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const void* keys, u64* u, u64* xext,
-                                         const u32* pinv, cudaStream_t stream) {
+                                         const u32* pinv, u32 cb, cudaStream_t stream) {
     typedef InnerGeo<RC> G;
-    const u32 chunks = ring.dev.N >> LOG_C, cb = (u32)G::CHUNKS < chunks ? (u32)G::CHUNKS : chunks;
+    const u32 chunks = ring.dev.N >> LOG_C;
     return launch_dependent(ring, ntt_contig_inner<RC>, dim3(rb.n_groups, (chunks + cb - 1) / cb, RC + 1), dim3(32 * G::WARPS),
                             (size_t)8 * (cb * RC << LOG_C), stream, ring.dev, B, rb, keys, u, xext, pinv, cb);
 }
@@ -1412,9 +1412,9 @@ static cudaError_t launch_contig_inner_t(const RingHost& ring, const PolyBatch& 
 // (a context has 2 to MAX_MODULI - 1 digits: see bf_ctx_create)
 template <int RC>
 static cudaError_t launch_contig_inner(const RingHost& ring, const PolyBatch& B, const RotBatch& rb, const void* keys, u64* u, u64* xext,
-                                       const u32* pinv, cudaStream_t stream) {
-    if (ring.dev.r == RC) return launch_contig_inner_t<RC>(ring, B, rb, keys, u, xext, pinv, stream);
-    if constexpr (RC + 1 < MAX_MODULI) return launch_contig_inner<RC + 1>(ring, B, rb, keys, u, xext, pinv, stream);
+                                       const u32* pinv, u32 cb, cudaStream_t stream) {
+    if (ring.dev.r == RC) return launch_contig_inner_t<RC>(ring, B, rb, keys, u, xext, pinv, cb, stream);
+    if constexpr (RC + 1 < MAX_MODULI) return launch_contig_inner<RC + 1>(ring, B, rb, keys, u, xext, pinv, cb, stream);
     else return cudaErrorInvalidValue;
 }
 
@@ -1431,11 +1431,16 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
     // are on the integer path, whose transforms cost several times as much (N = 2^15, 1024 -> 2048 without double hoisting:
     // 55-bit primes 422 us in three, 409 us in one; 40-bit primes, 3072 -> 768, 632 and 641 us)
     RotBatch rb = rb_in;
-    const u32 cb = r > 8 ? 1u : 8u / r;
+    // (as many chunks a block as digits leave warps for, fewer where a block per rotation and chunks would not fill the GPU once:
+    // six rotations of three digits on a ring of 2^12 6.6 us with two chunks a block, 5.7 us with one)
+    const u32 chunks = ring.dev.N >> LOG_C;
+    u32 cb = r > 8 ? 1u : 8u / r;
+    if (cb > chunks) cb = chunks;
+    while (cb > 1 && (u32)rb.n * ((chunks + cb - 1) / cb) * (r + 1) < 592u) cb = (cb + 1) / 2;
     u32 runs = 0, n_int = 0;
     for (int t = 0; t < rb.n; ++t) runs += t == 0 || rb.dig[t] != rb.dig[t - 1];
     for (u32 m = 0; m <= r; ++m) n_int += ring.dev.fp_ok[m] ? 0u : 1u;
-    const u32 blocks = runs * (((ring.dev.N >> LOG_C) + cb - 1) / cb) * (r + 1), fill = 2 * n_int > r + 1 ? 592u : 1776u;
+    const u32 blocks = runs * ((chunks + cb - 1) / cb) * (r + 1), fill = 2 * n_int > r + 1 ? 592u : 1776u;
     const u32 parts = blocks < fill ? fill / blocks : 1u;
     rb.n_groups = 0;
     for (int t = 0; t < rb.n;) {
@@ -1460,7 +1465,7 @@ cudaError_t ntt_forward_inner(const RingHost& ring, const PolyBatch& B_in, u32 n
         ring.prof->key_bytes_per_rotation += (u64)rb.n * key_bytes;
     }
     ProfScope prof(ring.prof, CAT_KEY_INNER, stream);
-    return launch_contig_inner<2>(ring, B_in, rb, keys, u, xext, pinv, stream);
+    return launch_contig_inner<2>(ring, B_in, rb, keys, u, xext, pinv, cb, stream);
 }
 
 cudaError_t ntt_inverse_assembly(const RingHost& ring, const PolyBatch& B, u32 n_outer, const OutputAssembly& as, cudaStream_t stream) {
@@ -1480,6 +1485,18 @@ cudaError_t ntt_inverse_assembly(const RingHost& ring, const PolyBatch& B, u32 n
 __device__ __forceinline__ u32 assembly_term(u32 k, u32 comp, u32 n_u) { return 2 * k < n_u ? comp + 2 * k : 2 * k == n_u ? n_u + comp : n_u + 1 + k - n_u / 2; }
 __device__ __forceinline__ u32 assembly_terms(u32 comp, u32 n_u, u32 n_t) { return n_u / 2 + (n_t == n_u ? 0u : comp ? 1u : n_t - n_u - 1); }
 
+// the centred values of terms k0 .. k0 + 7 (each below 2^59 in magnitude), requested together: two outputs of five terms at N = 2^15
+// 8.6 us one after the other, 6.8 us like this
+__device__ __forceinline__ i64 assembly_sum(const u64* __restrict__ tp, size_t N, u32 k0, u32 nt, u32 comp, u32 n_u) {
+    u64 t[8];
+#pragma unroll
+    for (u32 h = 0; h < 8; ++h) t[h] = k0 + h < nt ? __ldg(tp + assembly_term(k0 + h, comp, n_u) * N) : 1ull << 59;
+    i64 S = 0;
+#pragma unroll
+    for (u32 h = 0; h < 8; ++h) S += (i64)(t[h] - (1ull << 59));
+    return S;
+}
+
 __global__ void __launch_bounds__(128, 8) finish_division_kernel(const RingDev R, u64* __restrict__ ct, long long ct_stride,
                                                               const u64* __restrict__ T, u32 n_u, u32 n_t, const RescaleConsts rc,
                                                               u64* __restrict__ low) {
@@ -1496,10 +1513,7 @@ __global__ void __launch_bounds__(128, 8) finish_division_kernel(const RingDev R
     // and the sum is reduced once per prime
     const u32 nt = assembly_terms(comp, n_u, n_t);
     for (u32 k0 = 0; k0 < nt; k0 += 8) {
-        i64 S = 0;
-        for (u32 k = k0; k < nt && k < k0 + 8; ++k) {
-            S += (i64)(tp[(size_t)assembly_term(k, comp, n_u) * R.N] - (1ull << 59));
-        }
+        const i64 S = assembly_sum(tp, R.N, k0, nt, comp, n_u);
         const bool neg = S < 0;
         const u64 a = neg ? (u64)(-S) : (u64)S;
 #pragma unroll
@@ -1564,10 +1578,7 @@ __global__ void __launch_bounds__(128, 8) finish_division_fp_kernel(const RingDe
         if ((u32)i < R.r) v[i] = u2d(cp[(size_t)i * R.N]);
     const u32 nt = assembly_terms(comp, n_u, n_t);
     for (u32 k0 = 0; k0 < nt; k0 += 8) {
-        i64 S = 0;
-        for (u32 k = k0; k < nt && k < k0 + 8; ++k) {
-            S += (i64)(tp[(size_t)assembly_term(k, comp, n_u) * R.N] - (1ull << 59));
-        }
+        const i64 S = assembly_sum(tp, R.N, k0, nt, comp, n_u);
         const i64 s_hi = S >> 30;                               // |s_hi| < 2^33
         const double lo = u2d((u64)(S & ((1ll << 30) - 1)));
         const bool sneg = s_hi < 0;
