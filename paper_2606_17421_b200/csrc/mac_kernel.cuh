@@ -314,7 +314,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
 // grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
 // operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
-// Four blocks an SM (64 registers; the key part spills 108 bytes at r = 9 in tiles of 128, none at r = 7) because resident warps are what hides the latency: two,
+// Four blocks an SM (64 registers, which the key part of 7 and of 9 digits fits) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
 template <bool NARROW, int LOG_TN, bool BABY, int RC>
