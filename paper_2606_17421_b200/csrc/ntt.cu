@@ -1248,24 +1248,22 @@ static void launch_shared_src_t(const RingHost& ring, const PolyBatch& B_in, u32
     typedef StridedGeo<LOG_R, LOG_LANES> G;
     PolyBatch B = B_in;
     set_magics(B, n_outer);
-    constexpr bool INGEST = LOAD == LOAD_INGEST;
-    // targets per block: fewer blocks share the source better but quantise into waves; cost model =
-    // waves x (targets per block + half a unit for staging the source)
-    const u32 slots = 148u * G::BLOCKS;
+    // targets per block: fewer blocks share the source better, but a launch lasts as long as its longest block and ends raggedly.
+    // Cost = the work over the resident blocks, or one block where that is longer, and half a block for the end (not for digits that need
+    // no division: their launches mostly run beside one another, and long blocks suit that: 768 -> 2304 without flags 445 us, 454 us with
+    // it); a block costs its targets and the staging of its source, a whole target's worth where that divides by P (an ingest batch has
+    // half as many blocks and one of a single target for every other source).  us for 1, 2, 4, 8 targets a block, N = 2^15, r = 7: one
+    // input 13.1, 12.7, 14.7, 18.0, three 31.6, 29.9, 31.4, 34.9, digits of six rotations 64.4, 52.4, 48.3, 47.9; N = 2^16, r = 9, for 1, 2,
+    // 5, 10: four inputs 134, 119, 114, 117, six rotations 332, 256, 220, 217.
+    const double slots = 148.0 * G::BLOCKS, stage = B.div_t ? 1.0 : 0.5, tail = LOAD == LOAD_REDUCE && !B.div_t ? 0.0 : 0.5;
     u32 best = 1;
     double best_cost = 1e30;
     for (u32 per = 1; per <= B.n_m; ++per) {
         const u32 slices = (B.n_m + per - 1) / per;
         if ((B.n_m + slices - 1) / slices != per) continue;         // keep the slices balanced
-        const u32 blocks = G::TILES * n_outer * slices;
-        double cost = (double)((blocks + slots - 1) / slots) * (per + 0.5);
-        // (an ingest batch has half as many blocks of that length and one of a single target for every other source: the work, or
-        // one block where that is longer, and half a block for the end.  us for 1, 2, 4, 8 targets a block, N = 2^15, r = 7: one
-        // input 13.1, 12.7, 14.7, 18.0, three 31.6, 29.9, 31.4, 34.9; N = 2^16, r = 9, four inputs, 1, 2, 5, 10: 134, 119, 114, 117)
-        if (INGEST) {
-            const double work = (blocks * (per + 0.5) + G::TILES * n_outer * 1.5) / 2 / slots;
-            cost = (work > per + 0.5 ? work : per + 0.5) + (per + 0.5) / 2;
-        }
+        double work = (double)G::TILES * n_outer * slices * (per + stage) / slots;
+        if (LOAD == LOAD_INGEST) work = work / 2 + (double)G::TILES * n_outer * 1.5 / 2 / slots;
+        const double cost = (work > per + stage ? work : per + stage) + tail * (per + stage);
         if (cost <= best_cost) { best_cost = cost; best = per; }
     }
     const dim3 grid(G::TILES, n_outer, (B.n_m + best - 1) / best);
