@@ -649,6 +649,34 @@ def test_output_assembly_for_few_and_many_giant_steps(plan_t, shape, modes):
     run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 19, 1e-2, "giants", tight=1e-2)
 
 
+@pytest.mark.parametrize("bits,modes", [(40, {}), (55, dict(moddown="per_output")), (40, dict(hoist="double"))],
+                         ids=["fp64", "integer_per_output", "fp64_double_hoist"])
+def test_more_outputs_than_the_second_dimension_of_a_grid_holds(bits, modes):
+    # 32770 output ciphertexts of two components: the division that ends them has 65540 polynomials
+    par = ckks.Params(1 << 10, ckks.find_primes(1 << bits, 2 << 10, 2), ckks.find_primes(1 << 60, 2 << 10, 1)[0], 2.0 ** 30)
+    plan = ckks.Plan(2, 1, 1, 2, **modes)
+    d_out, d_in, n_out = 65539, 2, 32770
+    s = ckks.keygen(par, 23)
+    keys = ckks.make_rotation_keys(par, s, plan, 23)
+    W = wl.gen_weights(23, "tall", d_out, d_in)
+    cts = ckks.encrypt_vector(par, plan, s, wl.gen_activation(23, "tall", d_in), 23)
+    sample = [0, 1, 32766, 32767, 32768, n_out - 1]
+    expect = ckks.linear(par, plan, cts, W, keys, blocks=sample)
+    g = GpuSide(par, plan)
+    try:
+        g.load_keys(keys)
+        w = g.bf.bf_encode_weights(g.ctx, g.to_dev(W), d_out, d_in)
+        out = g.linear(cts, W, d_out, d_in, weights=w)
+        assert out.shape[0] == n_out
+        low = g.empty_u64(n_out, 2, par.r - 1, par.N)
+        g.bf.bf_linear_rescaled(g.ctx, g.to_dev(np.stack(cts)), 1, w, None, d_out, d_in, low, n_out)
+        for p in sample:
+            assert np.array_equal(g.to_host_u64(out[p]), expect[p]), p
+            assert np.array_equal(g.to_host_u64(low[p]), ckks.rescale(par, expect[p])), ("rescaled", p)
+    finally:
+        g.close()
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
