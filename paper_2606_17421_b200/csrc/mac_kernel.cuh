@@ -26,6 +26,8 @@
 #pragma once
 #include "bf_host.h"
 
+#include <type_traits>
+
 namespace bf {
 
 constexpr int MAC_THREADS = 256;
@@ -107,18 +109,41 @@ struct MacAcc<OP_DP> {
     static __device__ __forceinline__ u64 x_stored(u64 v) { return v; }
 };
 
-// The X tile: [term][TN] pairs (component 0, component 1).
+// A row of the tile fills a warp: its threads share their lane, and what depends on the lane is worked out once for all of them.
+__host__ __device__ constexpr bool warp_has_one_lane(int log_tn) { return log_tn >= 5; }
+
+// The X tile: [term][TN] pairs (component 0, component 1), one 16-byte read per weight; rows of 16, [term][component][TN] words, because
+// the halves of a warp read such a row alike and 8-byte reads serve both at once.  (Tiles of 16, a product of 4096 -> 1024 in 128 terms on
+// 2^15, us: without rotations inside 371 with pairs and what a lane needs carried along as below, 330 like this; with them 686 and 633.)
+template <int LOG_TN>
+struct XRow {
+    static constexpr bool PAIRS = warp_has_one_lane(LOG_TN);
+    static constexpr u32 TN = 1u << LOG_TN, WORDS = PAIRS ? TN : 2 * TN;
+    typedef typename std::conditional<PAIRS, ulonglong2, u64>::type Word;
+    static __device__ __forceinline__ void put(Word* at, ulonglong2 v) {
+        if constexpr (PAIRS) *at = v;
+        else { at[0] = v.x; at[TN] = v.y; }
+    }
+    static __device__ __forceinline__ ulonglong2 get(const Word* at) {
+        if constexpr (PAIRS) return *at;
+        else return make_ulonglong2(at[0], at[TN]);
+    }
+};
+
 template <int CLS, int LOG_TN, bool BABY, int RC>
 __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict__ pt, const TileLayout& lay,
                                          const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 pj_begin, u32 pj_end,
-                                         u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, ulonglong2* xs) {
+                                         u32 tile, u32 i, const MacScatter& sc, const BabySteps& bs, typename XRow<LOG_TN>::Word* xs) {
     constexpr u32 TN = 1u << LOG_TN, PL = MAC_THREADS >> LOG_TN;
     typedef MacAcc<CLS> Acc;
+    typedef XRow<LOG_TN> Row;
+    constexpr u32 RW = Row::WORDS;
     const u32 N = R.N, logN = R.logN;
     const u32 np = lay.n_primes;
     const u32 tid = threadIdx.x, c = tid & (TN - 1), c_rev = __brev(c) >> (32 - LOG_TN);
     u32 l = tid >> LOG_TN;
-    if constexpr (LOG_TN >= 5) l = __shfl_sync(0xffffffffu, l, 0);      // (so that what depends on it is computed once per warp)
+    constexpr bool ONE_LANE = warp_has_one_lane(LOG_TN);
+    if constexpr (ONE_LANE) l = __shfl_sync(0xffffffffu, l, 0);
     const u32 n0 = tile << LOG_TN;
     const u64 pol = stream_policy();
     if constexpr (BABY) {
@@ -129,8 +154,8 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         const size_t comp_stride = (size_t)np * N;
         for (u32 e = l; e < n_in; e += PL) {
             const u64* xp = xg + e * 2 * comp_stride + n0;
-            xs[e * b * TN + c] = i < r ? make_ulonglong2(Acc::x_stored(__ldg(xp)), Acc::x_stored(__ldg(xp + comp_stride)))
-                                       : make_ulonglong2(Acc::x_word(0), Acc::x_word(0));
+            Row::put(xs + e * b * RW + c, i < r ? make_ulonglong2(Acc::x_stored(__ldg(xp)), Acc::x_stored(__ldg(xp + comp_stride)))
+                                                : make_ulonglong2(Acc::x_word(0), Acc::x_word(0)));
         }
         // rotations: an item is a key and a part of the inputs that share it.  The tile has the exponents e0 + brev(c) 2^k; a
         // rotation reads the tile of e0 * gal, whose own first exponent is that less its top bits T, so that the word at c there
@@ -141,8 +166,12 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         const unsigned char* key0 = (const unsigned char*)bs.keys + R.key_base[i];
         const u32 e0 = 2u * (__brev(n0) >> (32u - logN)) + 1u, tile_bytes = key_tile_bytes(CLS == OP_DP, r);
         u32 k = 1, part = l;
-        for (;; part += PL) {
-            while (part >= parts) { part -= parts; ++k; }
+        const u32 step_k = PL / parts, step_part = PL % parts;      // (used by tiles of 16)
+        if constexpr (!ONE_LANE) { k += l / parts; part = l % parts; }
+        for (;;) {
+            if constexpr (ONE_LANE) {
+                while (part >= parts) { part -= parts; ++k; }
+            }
             if (k >= b) break;
             const u32 e = (e0 * bs.gal[k]) & ((2u << logN) - 1u), T = e >> (logN + 1 - LOG_TN);
             const u32 src = (__brev(e >> 1) >> (32u - logN)) & ~(TN - 1), ks = src / KS_TILE, in_tile = src % KS_TILE;
@@ -151,7 +180,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             const u32 q0 = part * per_part, q_end = min(n_in, q0 + per_part);
             const u64* dp = dig0 + q0 * dig_stride + ks * (r * KS_TILE) + in_tile;
             const u64* cp = xg + q0 * 2 * comp_stride + src;
-            ulonglong2* xp = xs + (q0 * b + k) * TN + cd;
+            typename Row::Word* xp = xs + (q0 * b + k) * RW + cd;
             u32 k0[RC > 0 ? 2 * RC : 1], k1[RC > 0 ? 2 * RC : 1];
             if constexpr (RC > 0) {
                 u32 high[(2 * RC + 3) / 4];
@@ -162,7 +191,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 #pragma unroll
                 for (int s = 0; s < 2 * RC; ++s) KeyTile<CLS>::cut(s, high[s / 4], k0[s], k1[s]);
             }
-            for (u32 qi = q0; qi < q_end; ++qi, dp += dig_stride, cp += 2 * comp_stride, xp += b * TN) {
+            for (u32 qi = q0; qi < q_end; ++qi, dp += dig_stride, cp += 2 * comp_stride, xp += b * RW) {
                 KeyDot<CLS> dot;
                 const u64 pc0 = i < r ? __ldg(cp) : 0ull;
                 if constexpr (RC > 0) {
@@ -187,12 +216,18 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
                     const double qd = R.qd[i], qinv = R.qinv_d[i], c40 = R.c40_d[i], c40q = R.c40_q[i];
                     const double v0 = __dadd_rn(dot.a0.lazy(qd, qinv, c40, c40q, r > LAZY_DIGITS), __longlong_as_double((long long)pc0));
                     const double v1 = dot.a1.lazy(qd, qinv, c40, c40q, r > LAZY_DIGITS);
-                    *xp = make_ulonglong2((u64)__double_as_longlong(fp_centre(v0, qd, qinv)), (u64)__double_as_longlong(fp_centre(v1, qd, qinv)));
+                    Row::put(xp, make_ulonglong2((u64)__double_as_longlong(fp_centre(v0, qd, qinv)), (u64)__double_as_longlong(fp_centre(v1, qd, qinv))));
                 } else {
                     u64 v0, v1;
                     dot.reduce(R, i, v0, v1);
-                    *xp = make_ulonglong2(Acc::x_word(add_mod(v0, pc0, R.q[i])), Acc::x_word(v1));
+                    Row::put(xp, make_ulonglong2(Acc::x_word(add_mod(v0, pc0, R.q[i])), Acc::x_word(v1)));
                 }
+            }
+            if constexpr (ONE_LANE) part += PL;
+            else {
+                k += step_k;
+                part += step_part;
+                if (part >= parts) { part -= parts; ++k; }
             }
         }
     } else {
@@ -205,15 +240,15 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 #pragma unroll
             for (int j = 0; j < 8; ++j) v[j] = __ldg(xg + ((size_t)(e + j / 2 * PL) * 2 + j % 2) * comp_stride);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) xs[(e + j * PL) * TN + c] = make_ulonglong2(Acc::x_word(v[2 * j]), Acc::x_word(v[2 * j + 1]));
+            for (int j = 0; j < 4; ++j) Row::put(xs + (e + j * PL) * RW + c, make_ulonglong2(Acc::x_word(v[2 * j]), Acc::x_word(v[2 * j + 1])));
         }
         for (; e < n_terms; e += PL) {
             const u64* xp = xg + (size_t)e * 2 * comp_stride;
-            xs[e * TN + c] = make_ulonglong2(Acc::x_word(__ldg(xp)), Acc::x_word(__ldg(xp + comp_stride)));
+            Row::put(xs + e * RW + c, make_ulonglong2(Acc::x_word(__ldg(xp)), Acc::x_word(__ldg(xp + comp_stride))));
         }
     }
     // terms up to a whole chunk are zero, and so are the padding words of a group's last stage once they are in registers
-    for (u32 e = n_terms + l; e < TILE_TS * lay.C; e += PL) xs[e * TN + c] = make_ulonglong2(0, 0);
+    for (u32 e = n_terms + l; e < TILE_TS * lay.C; e += PL) Row::put(xs + e * RW + c, make_ulonglong2(0, 0));
     __syncthreads();
 
     // ---------------- the weight stream: a lane's words of successive stages lie one stage apart
@@ -246,17 +281,20 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
     Acc a0, a1;
     u32 ch = 0;
     const size_t comp1 = (size_t)np * N;                // from component 0 to component 1
-    const u32 pj = pj_begin + l;
+    u32 pj = pj_begin + l;
     u64* ap = a + ((size_t)pj * 2 * np + i) * N;
-    const ulonglong2* xt = xs + c;
+    const typename Row::Word* xt = xs + c;
     const u32 tail = n_terms % TILE_TS;
-    // the giant step of group pj and the Galois element of its rotation (see MacScatter)
+    // the giant step of group pj and the Galois element of its rotation (see MacScatter): carried along from group to group where
+    // a warp's threads share them, else (they would take registers of every thread) made when the group ends
     u32 step_rem = 0, step_gal = 1, step = 0;
-    if (sc.on) {
+    auto set_step = [&] {
+        if (!sc.on) return;
         step = (sc.pj0 + pj) / sc.n_out;
         step_rem = sc.pj0 + pj - step * sc.n_out;
         step_gal = power32(sc.gal_inv, step);
-    }
+    };
+    if constexpr (ONE_LANE) set_step();
     auto use = [&](u32 (&wa)[TS], u32 (&wb)[TH]) {
         if constexpr (!PACKED) {        // (packed padding is a finite number times a zero of X, whatever it is)
             if (tail && ch + 1 == n_chunks) {
@@ -269,14 +307,19 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
         for (int ts = 0; ts < TS; ++ts) {
             u32 w0 = wa[ts], w1 = wb[PACKED ? ts / 4 : ts];
             if constexpr (PACKED) unpack40(ts, w1, w0, w1);
-            const ulonglong2 xw = xt[ts * TN];
+            const ulonglong2 xw = Row::get(xt + ts * RW);
             a0.mac(w0, w1, xw.x);
             a1.mac(w0, w1, xw.y);
         }
         a0.end_chunk(R, i, ch);
         a1.end_chunk(R, i, ch);
-        xt += TS * TN;
+        xt += TS * RW;
         if (++ch == n_chunks) {
+            if constexpr (!ONE_LANE) {
+                set_step();
+                ap = a + ((size_t)pj * 2 * np + i) * N;
+                pj += PL;
+            }
             u32 at0 = n0 + c;                                           // where component 0 goes (see MacScatter)
             if (step) {
                 const TileMove<LOG_TN> to(n0, step_gal, logN);
@@ -284,10 +327,10 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
             }
             ap[at0] = a0.reduce(R, i, n_terms > 128);
             ap[comp1 + n0 + c] = a1.reduce(R, i, n_terms > 128);
-            ap += 2 * PL * comp1;
+            if constexpr (ONE_LANE) ap += 2 * PL * comp1;
             a0 = {};
             a1 = {};
-            if (sc.on)
+            if (ONE_LANE && sc.on)
                 for (step_rem += PL; step_rem >= sc.n_out; step_rem -= sc.n_out) {
                     step_gal *= sc.gal_inv;
                     ++step;
@@ -314,7 +357,8 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
 // grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
 // operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
-// Four blocks an SM (64 registers, which the key part of 7 and of 9 digits fits) because resident warps are what hides the latency: two,
+// Four blocks an SM (64 registers, which the key part of 7 and of 9 digits fits in tiles of 32 and more; in tiles of 16 it spills 4
+// bytes at 7 digits and 196 at 9) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.
 template <bool NARROW, int LOG_TN, bool BABY, int RC>
@@ -322,7 +366,8 @@ __global__ void __launch_bounds__(MAC_THREADS, 4)
 mac_kernel(const __grid_constant__ RingDev R, const u64* __restrict__ pt, const __grid_constant__ TileLayout lay,
            const u64* __restrict__ x, u64* __restrict__ a, u32 n_terms, u32 n_pj, u32 pj_per_block,
            const __grid_constant__ MacScatter sc, const __grid_constant__ BabySteps bs) {
-    extern __shared__ __align__(128) ulonglong2 mac_xs[];
+    extern __shared__ __align__(128) u64 mac_xs_words[];
+    typename XRow<LOG_TN>::Word* mac_xs = (typename XRow<LOG_TN>::Word*)mac_xs_words;
     grid_dependency_enter();
     const u32 tiles_log = R.logN - LOG_TN;
     const u32 i = lay.n_primes - 1 - blockIdx.x % lay.n_primes;

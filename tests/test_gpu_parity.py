@@ -677,6 +677,18 @@ def test_more_outputs_than_the_second_dimension_of_a_grid_holds(bits, modes):
         g.close()
 
 
+@pytest.mark.parametrize("bits", [(50, 40, 40), (60, 40, 30), (50,) + (40,) * 6], ids=["narrow", "wide", "seven_digits"])
+@pytest.mark.parametrize("modes", [{}, BEST, dict(hoist="double")], ids=["plain", "best", "double_hoist"])
+def test_tiles_of_16_coefficients(bits, modes):
+    # 100 terms a group (the last stage half empty) in tiles of 16: a warp has two lanes.  96 groups, or 48 with two row blocks in one:
+    # several per lane, of four giant steps; three keys and 25 inputs in 9 parts
+    two_n = 2 << 10
+    P, base = ckks.find_primes(1 << 60, two_n, 2)
+    primes = [base if b == 60 else ckks.find_primes(1 << b, two_n, 8)[i] for i, b in enumerate(bits)]
+    run_case(ckks.Params(1 << 10, primes, P, 2.0 ** 40), ckks.Plan(16, 1, 4, 4, **modes), 24 * 16 - 5, 25 * 16 - 3, 29, 1e-2,
+             "tiles16", tight=1e-2)
+
+
 def test_linear_gpt2_qkv_config_bit_exact():
     w = wl.WORKLOADS["gpt2_qkv"]
     par = oracle_params(w.params)
