@@ -431,21 +431,23 @@ static cudaError_t launch_mac_tile(const MacLaunch& m) {
     }
 }
 
+// The 2 r key words of a rotation in registers, asked for together and once for all inputs it is applied to: an instance for every digit
+// count up to 11.  Beyond that too many are spilled (in tiles of 32 and more at most 4 bytes up to 9 digits, 172 at 10, 296 at 11, 352 at
+// 12) and a loop over the digits is used, which asks for the words again for every input.  us with the loop and with an instance, one input
+// and 1024 -> 2048 on 2^15: 2 digits 95 and 87, 3 125 and 113, 5 168 and 157, 6 205 and 180, 8 256 and 244, 10 363 and 338, 11 433 and
+// 396, 12 441 and 452.
+constexpr int MAC_MOST_DIGITS = 11;
+template <bool NARROW, int RC>
+static cudaError_t launch_mac_digits(const MacLaunch& m) {
+    if (m.ring->dev.r == RC) return launch_mac_tile<NARROW, true, RC>(m);
+    if constexpr (RC < MAC_MOST_DIGITS) return launch_mac_digits<NARROW, RC + 1>(m);
+    else return launch_mac_tile<NARROW, true, 0>(m);
+}
+
 template <bool NARROW>
 static cudaError_t launch_mac_ring(const MacLaunch& m) {
     if (!m.baby) return launch_mac_tile<NARROW, false, 0>(m);
-    // (digit counts of the shipped parameter sets: the key words of a rotation in registers.  300 -> 1000 on a ring of 2^12, three
-    // digits: 11.7 us with a loop over them, 10.9 us like this)
-    if constexpr (NARROW) {
-        if (m.ring->dev.r == 3) return launch_mac_tile<NARROW, true, 3>(m);
-    } else {
-        if (m.ring->dev.r == 4) return launch_mac_tile<NARROW, true, 4>(m);
-    }
-    switch (m.ring->dev.r) {
-        case 7: return launch_mac_tile<NARROW, true, 7>(m);
-        case 9: return launch_mac_tile<NARROW, true, 9>(m);
-        default: return launch_mac_tile<NARROW, true, 0>(m);
-    }
+    return launch_mac_digits<NARROW, 2>(m);
 }
 
 cudaError_t launch_mac_narrow(const MacLaunch& m);      // every ciphertext prime below 2^50

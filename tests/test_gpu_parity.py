@@ -590,6 +590,17 @@ def test_operand_classes_and_tile_edges(logN, bits, plan_t, shape, modes):
     run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 31, 1e-2, "classes", tight=1e-2)
 
 
+@pytest.mark.parametrize("base", [50, 60], ids=["narrow", "wide"])
+@pytest.mark.parametrize("n_primes", [2, 3, 4, 5, 6, 8, 10, 11, 12, 15])
+def test_baby_steps_inside_the_product_for_every_digit_count(n_primes, base):
+    # an instance for each count up to 11, a loop beyond, where all ciphertext primes are below 2^50 and where one is not (7 and 9
+    # digits: see above)
+    two_n = 2 << 10
+    P, wide = ckks.find_primes(1 << 60, two_n, 2)
+    primes = [wide if base == 60 else ckks.find_primes(1 << 50, two_n, 1)[0]] + ckks.find_primes(1 << 40, two_n, n_primes - 1)
+    run_case(ckks.Params(1 << 10, primes, P, 2.0 ** 40), ckks.Plan(16, 1, 4, 4, **BEST), 40, 40, 41, 1e-2, "digits", tight=1e-2)
+
+
 @pytest.mark.parametrize("moddown", ["per_rotation", "per_output"])
 @pytest.mark.parametrize("plan_t", [(32, 2, 4, 4), (32, 4, 1, 8)], ids=["baby_steps", "none"])
 @pytest.mark.parametrize("bits,special_bits", [
