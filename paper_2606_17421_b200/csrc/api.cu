@@ -1209,8 +1209,9 @@ static int linear_enqueue(bf_ctx* ctx, const uint64_t* ct_in, uint32_t n_in, con
                 B.mod_step = 1;
                 B.store_centred = 2;
                 CK(ntt_inverse(ctx->ring, B, cnt, lane[c].s));
-                const PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)mid_primes * N, lane[c].Dig, c1, (long long)xw,
-                                                 dh ? lane[c].Cc + (size_t)r * N : nullptr);
+                PolyBatch D0 = modup_batch(ctx, lane[c].Cc, (long long)mid_primes * N, lane[c].Dig, c1, (long long)xw,
+                                           dh ? lane[c].Cc + (size_t)r * N : nullptr);
+                D0.beside = used > 1;
                 RotBatch rb;
                 memset(&rb, 0, sizeof(rb));
                 rb.n = (int)cnt;

@@ -350,6 +350,9 @@ struct PolyBatch {
     long long div_so;             //   i = o % o_div of set s = o / o_div is the residue modulo q_i of a polynomial in the
                                   //   extended basis, coefficient domain, and t = div_t + s*div_so holds its residue
                                   //   modulo P as a centred lift plus 2^59: the digit is (source - t) * P^{-1} mod q_i
+    u32 beside;                   // forward from a shared source: digits of giant steps that run as several chains, whose launches
+                                  //   overlap (for the launcher.  The lifts of baby rotations in two chains, in fewer
+                                  //   blocks, do better without it: 1024 -> 512 without flags 293 us, 298 with it)
 };
 
 // The digit sets that the multiply-accumulate reads are kept tile-major, so that what a block needs of one (set, modulus,

@@ -1249,13 +1249,15 @@ static void launch_shared_src_t(const RingHost& ring, const PolyBatch& B_in, u32
     PolyBatch B = B_in;
     set_magics(B, n_outer);
     // targets per block: fewer blocks share the source better, but a launch lasts as long as its longest block and ends raggedly.
-    // Cost = the work over the resident blocks, or one block where that is longer, and half a block for the end (not for digits that need
-    // no division: their launches mostly run beside one another, and long blocks suit that: 768 -> 2304 without flags 445 us, 454 us with
-    // it); a block costs its targets and the staging of its source, a whole target's worth where that divides by P (an ingest batch has
-    // half as many blocks and one of a single target for every other source).  us for 1, 2, 4, 8 targets a block, N = 2^15, r = 7: one
-    // input 13.1, 12.7, 14.7, 18.0, three 31.6, 29.9, 31.4, 34.9, digits of six rotations 64.4, 52.4, 48.3, 47.9; N = 2^16, r = 9, for 1, 2,
-    // 5, 10: four inputs 134, 119, 114, 117, six rotations 332, 256, 220, 217.
-    const double slots = 148.0 * G::BLOCKS, stage = B.div_t ? 1.0 : 0.5, tail = LOAD == LOAD_REDUCE && !B.div_t ? 0.0 : 0.5;
+    // Cost = the work over the resident blocks, or one block where that is longer, and half a block for the end, unless another chain's
+    // launches fill it (PolyBatch::beside); a block costs its targets and the staging of its source, a whole target's worth where that
+    // divides by P (an ingest batch has half as many blocks and one of a single target for every other source).  us for 1, 2, 4, 8
+    // targets a block, N = 2^15, r = 7, what is taken marked: digits of one ciphertext 15.2*, 15.7, 16.9, 20.5, of three 31.0, 29.0*, 30.7,
+    // 31.1, of six 53.7, 49.6, 49.2*, 50.0, of 40 322, 284, 269, 261*; ingest of one input 13.1*, 12.7, 14.7, 18.0, of three 31.6, 29.9*,
+    // 31.4, 34.9; for 1, 2, 5, 10, N = 2^16, r = 9: digits of one ciphertext 36.2, 33.1*, 33.1, 34.7, of six 174, 154, 146*, 146, ingest of
+    // four inputs 134, 119, 114*, 117.  Whole calls whose giant steps run as two chains, the end counted and not: 768 -> 2304 without flags
+    // 454 and 445 us, with double hoisting alone 392 and 389; 1024 -> 6144 with all flags 389 and 384.
+    const double slots = 148.0 * G::BLOCKS, stage = B.div_t ? 1.0 : 0.5, tail = B.beside ? 0.0 : 0.5;
     u32 best = 1;
     double best_cost = 1e30;
     for (u32 per = 1; per <= B.n_m; ++per) {
