@@ -147,8 +147,8 @@ def test_rotate_matches_oracle(pkey):
 
 @pytest.mark.parametrize("logN,n_primes", [(10, 2), (10, 5), (11, 8), (10, 10), (10, 15)])
 def test_rotate_for_every_arrangement_of_digits_in_a_block(logN, n_primes):
-    # the fused transform and inner product: several chunks per block where digits are few (all that the smallest ring has),
-    # one chunk and idle warps, a warp per digit, digits in two rounds of 8 warps
+    # the fused transform and inner product of one rotation, a launch that does not fill the GPU: one chunk a block, idle warps, a warp
+    # per digit, digits in two rounds of 8 warps (several chunks a block: see the folds of many ciphertexts)
     par = ckks.Params(1 << logN, ckks.find_primes(1 << 40, 2 << logN, n_primes), ckks.find_primes(1 << 60, 2 << logN, 1)[0], 2.0 ** 30)
     plan = ckks.Plan(8, 1, 4, 2)
     s = ckks.keygen(par, 5)
@@ -564,10 +564,22 @@ def test_random_small_ring_cases(case):
 
 
 @pytest.mark.parametrize("n_out", [124, 126])
-def test_one_division_per_output_on_both_sides_of_the_short_launches(n_out):
-    # forward passes of up to 12000 chunks have 4 points a thread, longer ones 8: n_out * 2 components * 3 primes * 16 chunks
+def test_one_division_per_output_with_many_outputs(n_out):
     par = oracle_params("n12")
     run_case(par, ckks.Plan(16, 1, 8, 2, moddown="per_output"), n_out * 16, 16, 37, 1e-2, "short", tight=1e-2)
+
+
+@pytest.mark.parametrize("pkey,plan_t,n_in,modes", [
+    ("n12", (16, 1, 1, 16), 125, {}),                       # the inputs' transforms: n_in x 2 components x 3 primes x 16 chunks
+    ("n12", (16, 1, 1, 16), 126, {}),
+    ("paper_n13", (32, 2, 16, 1), 3, {}),                   # baby rotations divided by P: 15 n_in x 2 x 4 primes x 32 chunks
+    ("paper_n13", (32, 2, 16, 1), 4, {}),
+    ("n12", (16, 1, 2, 8), 50, dict(hoist="double")),       # inputs and digits at once: n_in x 3 digits x 5 x 16 chunks
+    ("n12", (16, 1, 2, 8), 51, dict(hoist="double")),
+])
+def test_forward_passes_on_both_sides_of_the_short_launches(pkey, plan_t, n_in, modes):
+    # forward passes of up to 12000 chunks have 4 points a thread, longer ones 8
+    run_case(oracle_params(pkey), ckks.Plan(*plan_t, **modes), plan_t[0], plan_t[0] * n_in, 37, 1e-2, "short", tight=1e-2)
 
 
 @pytest.mark.parametrize("modes", [{}, dict(moddown="per_output", hoist="double")], ids=["plain", "extended"])
@@ -647,15 +659,17 @@ def test_wide_inputs_take_no_more_scratch_than_the_batched_rotations(n_primes, n
         g.close()
 
 
-@pytest.mark.parametrize("modes", [{}, dict(hoist="double"), dict(moddown="per_output")], ids=["plain", "double_hoist", "per_output"])
-@pytest.mark.parametrize("plan_t,shape", [
-    ((128, 1, 2, 64), (130, 128)),          # 63 giant steps, two outputs: launches of several batches, 2 * 63 separate terms
-    ((128, 1, 1, 128), (128, 100)),         # more giant steps than a launch has rotations (refused with one division per output)
-    ((64, 8, 8, 1), (64, 64)),              # none: nothing to assemble, or the inner sums alone
+@pytest.mark.parametrize("plan_t,shape,modes", [
+    ((128, 1, 2, 64), (130, 128), {}),              # 63 giant steps, two outputs: launches of several batches, 2 * 63 separate terms
+    ((128, 1, 2, 64), (130, 128), dict(hoist="double")),
+    ((128, 1, 2, 64), (130, 128), dict(moddown="per_output")),
+    ((128, 1, 1, 128), (128, 100), {}),             # more giant steps than a launch has rotations (with one division per output
+    ((128, 1, 1, 128), (128, 100), dict(hoist="double")),       # the library refuses them: see the test of its refusals)
+    ((64, 8, 8, 1), (64, 64), {}),                  # none: nothing to assemble, or the inner sums alone
+    ((64, 8, 8, 1), (64, 64), dict(hoist="double")),
+    ((64, 8, 8, 1), (64, 64), dict(moddown="per_output")),
 ])
 def test_output_assembly_for_few_and_many_giant_steps(plan_t, shape, modes):
-    if plan_t[3] > 65 and "moddown" in modes:
-        return
     par = ckks.Params(1 << 10, ckks.find_primes(1 << 40, 2 << 10, 3), ckks.find_primes(1 << 60, 2 << 10, 1)[0], 2.0 ** 40)
     run_case(par, ckks.Plan(*plan_t, **modes), shape[0], shape[1], 19, 1e-2, "giants", tight=1e-2)
 
@@ -1131,6 +1145,30 @@ def test_fold_of_more_ciphertexts_than_one_key_switch_batch():
         g.bf.bf_fold(g.ctx, d, n_ct)
         got = g.to_host_u64(d)
         for t in (0, 1, 63, 64, 69):
+            assert np.array_equal(got[t], ckks.fold_in_ciphertext(par, plan, cts[t], keys)), t
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("n_primes,n_ct", [
+    (2, 55),        # 16 chunks of a ring of 2^12, two digits: four chunks a block
+    (2, 27),        # ... two, so that the launch fills the GPU
+    (4, 16),        # four digits, two chunks: all eight warps
+])
+def test_fold_with_several_chunks_in_a_block(n_primes, n_ct):
+    par = ckks.Params(1 << 12, ckks.find_primes(1 << 40, 2 << 12, n_primes), ckks.find_primes(1 << 60, 2 << 12, 1)[0], 2.0 ** 30)
+    plan = ckks.Plan(4, 2, 2, 1)
+    s = ckks.keygen(par, 53)
+    keys = ckks.make_rotation_keys(par, s, plan, 53, extra_steps=ckks.fold_rotations(plan))
+    cts = np.stack([np.ascontiguousarray(wl.gen_uniform_residues(53, f"fold{t}", par.primes, (2, par.N)).transpose(1, 0, 2))
+                    for t in range(n_ct)])
+    g = GpuSide(par, plan)
+    try:
+        g.load_keys(keys, extra_steps=ckks.fold_rotations(plan))
+        d = g.to_dev(cts)
+        g.bf.bf_fold(g.ctx, d, n_ct)
+        got = g.to_host_u64(d)
+        for t in (0, 1, n_ct // 2, n_ct - 1):
             assert np.array_equal(got[t], ckks.fold_in_ciphertext(par, plan, cts[t], keys)), t
     finally:
         g.close()
