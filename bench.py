@@ -169,48 +169,39 @@ def split_specs(text: str):
 def transform_counts(runner) -> dict:
     """Transforms one step launches, by direction and by arithmetic path.  Moduli below 2^41 run in
     fp64 with 8 fp64 operations per butterfly (signed lazy values), moduli from 2^41 up to 2^50 in fp64
-    with a conditional subtraction and offsets (12 operations), the 60-bit special prime in integers
-    (at least 10 32-bit multiply-adds per butterfly)."""
+    with a conditional subtraction and offsets (12 operations), 60-bit primes in integers (at least 9
+    32-bit multiply-adds per butterfly, and one reduction more in every second or third stage)."""
     import math
     r, N = runner.r, runner.N
     per = (N // 2) * int(math.log2(N))           # butterflies of a transform
     moduli = list(runner.primes) + [runner.P]
-    cost = [8 if q < (1 << 41) else 12 if q < (1 << 50) else 10 for q in moduli]
+    cost = [8 if q < (1 << 41) else 12 if q < (1 << 50) else 9 for q in moduli]
     fp = [q < (1 << 50) for q in moduli]
     fwd = [0] * (r + 1)
     inv = [0] * (r + 1)
     fused = [0] * (r + 1)       # ModUp digits whose second pass (8 of the log2 N stages) is part of the key-switch product
+    double, per_output = runner.plan.hoist == "double", runner.plan.moddown == "per_output"
     for e in runner.layers:
         n_in, n_out, b, g = e["n_in"], e["n_out"], e["b"], e["g"]
-        n_giant = (g - 1) * n_out
-        sets = (n_in if b > 1 else 0) + n_giant            # ModUp digit sets
-        products = sets if runner.plan.hoist != "double" else n_giant      # digit sets multiplied in a launch of their own
-        in_place = r if runner.plan.hoist == "double" and runner.plan.moddown == "per_output" else r - 1
+        n_giant, baby_sets = (g - 1) * n_out, n_in if b > 1 else 0
+        # ModUp digits modulo each ciphertext prime: a baby step's in its own prime is the transform of the input, a giant
+        # step's that of the inner sum, unless the sum is still to be divided by P (double hoisting)
+        baby, giant = baby_sets * (r - 1), n_giant * (r if double else r - 1)
+        # divisions by P in the transform domain: baby rotations without double hoisting, each of two components
+        lifts = 0 if double else 2 * n_in * (b - 1)
+        # separately rounded terms of the output assembly: key-switch results of the giant steps, both components, in one sum or
+        # each by itself; with double hoisting also the inner sums' (components 0 of all, component 1 of the first)
+        terms = ((0 if g == 1 else 2 if per_output else 2 * (g - 1)) + (g + 1 if double else 0)) * n_out
         for i in range(r):
-            fused[i] += products * in_place
-        fused[r] += products * r
-        # divisions by P: one per rotation and component, or (per_output) one per baby rotation and per output
-        n_baby_lift = 2 * n_out * g if runner.plan.hoist == "double" else 2 * n_in * (b - 1)
-        n_lift = n_baby_lift + 2 * (n_out if runner.plan.moddown == "per_output" and n_giant else n_giant)
-        if runner.plan.hoist == "double" and runner.plan.moddown == "per_output" and n_giant:
-            # inner sums stay in the extended basis: no lifted P-residue is transformed; the giant steps' ModUp divides in
-            # its first load (and transforms each digit in its own prime too); the outputs are assembled by one inverse
-            # transform per residue, g + 3 of them modulo P per output
-            baby_sets = n_in if b > 1 else 0
-            for i in range(r):
-                fwd[i] += 2 * n_in + baby_sets * (r - 1) + n_giant * r
-                inv[i] += n_giant + 2 * n_out
-            fwd[r] += sets * r
-            inv[r] += n_giant + n_out * (g + 3)
-        else:
-            for i in range(r):
-                fwd[i] += 2 * n_in + sets * (r - 1) + n_lift   # inputs; digits of the other primes; lifted P-residues
-                inv[i] += n_giant + 2 * n_out                  # c1 of the giant-step inputs; outputs
-            fwd[r] += sets * r
-            inv[r] += n_lift                                   # P-residues of the inner products
+            fwd[i] += 2 * n_in + baby + giant + lifts
+            inv[i] += n_giant + 2 * n_out
+            fused[i] += giant + (0 if double else baby)        # (double hoisting: the multiply-accumulate makes the baby products)
+        fwd[r] += (baby_sets + n_giant) * r
+        inv[r] += lifts + terms + (n_giant if double else 0)
+        fused[r] += (n_giant + (0 if double else baby_sets)) * r
         if runner.transforms_weights_per_call(e):          # on the fly or kept as coefficients: every diagonal is transformed on each call
             n_diag = n_in * n_out * b * g
-            for i in range(r + (1 if runner.plan.hoist == "double" else 0)):
+            for i in range(r + (1 if double else 0)):
                 fwd[i] += n_diag
     fwd = [c - f * 8.0 / math.log2(N) for c, f in zip(fwd, fused)]
     def summary(cnt):
