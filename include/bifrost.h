@@ -191,8 +191,8 @@ int bf_set_graph_replay(bf_ctx* ctx, int on);
 int bf_set_dependent_launch(bf_ctx* ctx, int on);
 
 /* The key switches of a call are independent per rotation.  bf_linear deals the baby rotations of a
- * batch, and then the giant rotations, out to n_lanes chains (inner product, then division by the
- * special prime) that run on streams of the library's own between a fork from and a join into the
+ * batch, and then the giant rotations, out to n_lanes chains (baby: inner product, then division by the
+ * special prime; giant: digits, then inner product) that run on streams of the library's own between a fork from and a join into the
  * context's stream, so that one chain's HBM-bound inner product overlaps another chain's
  * arithmetic-bound transforms.  n_lanes is an upper bound: a stage is split only where that was
  * measured to pay (at most 24 baby rotations in the batch; 6 to 20 giant rotations; counts weighted
@@ -228,7 +228,7 @@ int bf_linear_host(bf_ctx* ctx, const uint64_t* host_ct_in, uint32_t n_in, const
                    const float* W_raw, uint32_t d_out, uint32_t d_in, uint64_t* host_ct_out, uint32_t n_out);
 
 /* One key-switched left rotation of a full-level ciphertext by `steps` slots (the primitive the
- * baby and giant steps are made of).  ct_in, ct_out: device, boundary layout.  Asynchronous. */
+ * baby and giant steps are made of).  ct_in, ct_out: device, boundary layout; they may overlap.  Asynchronous. */
 int bf_rotate(bf_ctx* ctx, const uint64_t* ct_in, uint32_t steps, uint64_t* ct_out);
 
 /* Products in Z_q[X]/(X^N + 1): out[t] = a[t] * b[t] for n_polys polynomials, polynomial t modulo

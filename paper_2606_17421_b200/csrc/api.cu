@@ -88,6 +88,7 @@ struct bf_weights {
     u32 coef_bits = 0;
 };
 
+constexpr u32 MAX_GIANT_PER_OUTPUT = 64;        // giant rotations of BF_PLAN_MODDOWN_PER_OUTPUT, as bifrost.h states it
 constexpr size_t ENCODE_PASS_BYTES = (size_t)1536 << 20, ENCODE_PASS_BYTES_MIN = (size_t)512 << 20;
 
 struct bf_ctx {
@@ -241,7 +242,8 @@ extern "C" int bf_ctx_create(bf_ctx** out, uint32_t N, const uint64_t* primes, u
         return BF_ERR_SHAPE;
     if (plan->bsgs_b - 1 > (u32)MAX_ROT_BATCH) return BF_ERR_SHAPE;
     if (plan->flags & ~(u32)(BF_PLAN_COMPLEX_PACK | BF_PLAN_MODDOWN_PER_OUTPUT | BF_PLAN_DOUBLE_HOIST)) return BF_ERR_INVALID_ARG;
-    if ((plan->flags & BF_PLAN_MODDOWN_PER_OUTPUT) && plan->bsgs_g - 1 > (u32)MAX_ROT_BATCH) return BF_ERR_SHAPE;
+    // (a bound of the interface: the output assembly itself sums any number of giant steps)
+    if ((plan->flags & BF_PLAN_MODDOWN_PER_OUTPUT) && plan->bsgs_g - 1 > MAX_GIANT_PER_OUTPUT) return BF_ERR_SHAPE;
 
     bf_ctx* ctx = new (std::nothrow) bf_ctx();
     if (!ctx) return BF_ERR_OOM;
@@ -601,7 +603,7 @@ extern "C" uint64_t bf_weights_bytes(const bf_ctx* ctx, uint32_t d_out, uint32_t
 static bool split_ok(const bf_ctx* ctx, u32 b, u32 g) {
     if (!b || !g || (b & (b - 1)) || (g & (g - 1))) return false;
     if ((u64)b * g != ctx->plan.tile_D / ctx->plan.tau || b - 1 > (u32)MAX_ROT_BATCH) return false;
-    return !((ctx->plan.flags & BF_PLAN_MODDOWN_PER_OUTPUT) && g - 1 > (u32)MAX_ROT_BATCH);
+    return !((ctx->plan.flags & BF_PLAN_MODDOWN_PER_OUTPUT) && g - 1 > MAX_GIANT_PER_OUTPUT);
 }
 
 // Encode diagonals [d0, d0 + count) of W (order [j][p][q][k], i.e. group pj = d / n_terms, term d % n_terms)

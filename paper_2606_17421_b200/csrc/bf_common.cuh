@@ -1,6 +1,6 @@
 // Shared device-side types and modular arithmetic for the CKKS linear-layer kernels (sm_100a).
 //
-// Residues are 64-bit words modulo primes q < 2^60, so lazily reduced values up to 4q fit a word
+// Residues are 64-bit words modulo primes q < 2^60, so lazily reduced values up to 16q fit a word
 // and a sum of up to 2^8 products of two residues fits 128 bits.
 #pragma once
 #include <cstdint>

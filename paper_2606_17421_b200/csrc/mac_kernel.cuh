@@ -13,16 +13,17 @@
 // in place, coalesced, and permutes inside the tile on the way to shared memory.  X itself (2 (r+1) N words per term) is
 // never written to memory.
 //
-// What bounds it: no resource alone.  The 768 -> 2304 call of a GPT-2 layer (510 MB of keys and weights, read once, 5 bytes a
-// word modulo the primes below 2^40) takes 126 us: 4.3 TB/s of DRAM traffic, 61 % of the issue slots, 45 % of the warps
-// resident, waits for loads ahead of every other stall; weights in 5 bytes instead of 8 took 13 % of its bytes and none of its
-// time.  Loads go straight to registers: a stream that every thread consumes in the pattern it loads needs no staging, no
-// barriers and no producer; what hides the latency is the number of independent loads per thread (2r key words at a time;
-// two batches of 8 weights, three where they are packed) times resident warps.
+// What bounds it: the stream where one input meets the keys, issue where several do.  In one layer of a 0.6B decoder (N = 2^15, r = 7,
+// 5 bytes a word modulo the primes below 2^40) 1024 -> 4096 reads 534 MB of keys and weights in 110 us, 4.9 TB/s, and 1024 -> 6144 with 31
+// keys 974 MB in 187 us, 5.2 TB/s, where a plain sequential read reaches 5.5; two and three inputs 4.2 and 3.8 TB/s, with 58 to 62 % of the
+// issue slots taken, 45 % of the warps resident and waits for loads ahead of every other stall.  Loads go straight to registers: a
+// stream that every thread consumes in the pattern it loads needs no staging, no barriers and no producer; what hides the latency
+// is the number of independent loads per thread (2r key words at a time; two batches of 8 weights, three where they are packed)
+// times resident warps.
 // Since issue slots come next, index arithmetic is done per warp where it can be, X is held as pairs of its two components (one
 // 16-byte read per weight), and what stays in the block is only reduced as far as its next use needs: the four products of a 0.6B
 // layer take 55 us less than with canonical residues, divisions for an item's place and an automorphism evaluated per
-// coefficient (the layer 1373 -> 1314 us, one of an 8B model 9430 -> 9087 us).
+// coefficient (the layer 1373 -> 1314 us, one of an 8B model 9430 -> 9087 us).  Tiles of 16 differ in two of these: see XRow.
 #pragma once
 #include "bf_host.h"
 
@@ -357,7 +358,7 @@ __device__ __forceinline__ void mac_body(const RingDev& R, const u64* __restrict
 
 // grid: x = slice of the output groups * tiles * primes, primes fastest: the blocks that share an SM then work in different
 // operand classes, i.e. on different pipes (4 % of the kernel against tiles fastest on a 1024 -> 6144 product).
-// Four blocks an SM (64 registers, which the key part of 7 and of 9 digits fits in tiles of 32 and more; in tiles of 16 it spills 4
+// Four blocks an SM (64 registers, which the key part of up to 9 digits fits in tiles of 32 and more; in tiles of 16 it spills 4
 // bytes at 7 digits and 196 at 9) because resident warps are what hides the latency: two,
 // three and four blocks took 791, 671 and 653 us over the four products of a 0.6B decoder layer (N = 2^15, r = 7; 3.34 GB of
 // keys and weights), where the separate inner product and multiply-accumulate this kernel replaces took 867 us.

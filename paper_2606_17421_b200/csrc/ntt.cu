@@ -151,7 +151,7 @@ __device__ __forceinline__ u64 mul_shoup_short(u64 x, u64 w, u64 ws, u64 q) {
     const u64 h = (u64)x1 * s1 + __umulhi(x1, s0) + __umulhi(x0, s1);
     return x * w - h * q;
 }
-// any 64-bit x (so x < 16q) minus a multiple of q, q above 2^50: in [0, 3q).  The quotient floor(x_hi mu / 2^32) is short of x / q
+// any 64-bit x, in particular any below 16q, minus a multiple of q, q above 2^50: in [0, 3q).  The quotient floor(x_hi mu / 2^32) is short of x / q
 // by less than 1 + 2^-18 + x / 2^64.
 __device__ __forceinline__ u64 reduce_16q(u64 x, const ModConsts& c) { return x - (u64)__umulhi((u32)(x >> 32), c.mu) * c.q; }
 

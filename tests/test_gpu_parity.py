@@ -445,7 +445,7 @@ def test_weights_kept_as_coefficients_give_the_same_ciphertexts(bits, modes):
         g.close()
 
 
-def test_per_output_division_refuses_more_giant_steps_than_it_can_sum():
+def test_per_output_division_refuses_more_giant_steps_than_its_interface_allows():
     from paper_2606_17421_b200 import bifrost as bf
     ps = wl.PARAM_SETS["n12"]
     basis = list(ps["primes"]) + [ps["special"]]
